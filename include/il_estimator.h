@@ -144,7 +144,7 @@ typedef struct {
     double  sim_ms;          /* device time of the simulation kernels (CUDA events)      */
     double  select_ms;       /* device time of the percentile kernels (CUDA events)      */
     double  total_ms;        /* device time of all stream work of the call               */
-    int64_t fallback_candidates; /* candidates the lane kernel gave up on (stream ring overflow) and the
+    int64_t fallback_candidates; /* candidates the lane kernel gave up on (spill ring overflow) and the
                                 warp-per-candidate kernel evaluated instead; results are the same     */
     int64_t stage_runs;      /* (stage, candidate) simulations carried out: candidates * S unless
                                 candidates with a common configuration prefix shared them            */
@@ -257,7 +257,7 @@ IL_API int il_estimate_device(il_estimator *est, const il_stage_config *d_config
  *   il_feasible         configs HOST [n][S], out_feasible HOST [n] bytes; candidates validated on the host
  *   il_feasible_device  DEVICE pointers; an invalid candidate makes the call return BAD_CONFIG
  * Work on the handle's stream; returns after completion.  Errors as il_estimate / il_estimate_device.
- * If the lane kernel gives candidates up on stream ring overflow (see il_set_variant), they are
+ * If the lane kernel gives candidates up on spill ring overflow (see il_set_variant), they are
  * evaluated by the warp-per-candidate kernel in the same call, which then allocates temporaries.
  */
 IL_API int il_feasible(il_estimator *est, const il_stage_config *configs, int64_t n, int64_t slo_us,
@@ -378,15 +378,14 @@ IL_API int il_set_workspace(il_estimator *est, void *d_workspace, size_t bytes);
  * IL_VARIANT_LANES: one lane per (candidate, stage); the stages of a candidate
  *   run side by side as a pipeline inside one warp, floor(32 / S) candidates per
  *   warp; a group of lanes takes its next candidate as soon as it has finished
- *   one.  While the inter-stage streams of all resident candidates fit 48 GiB
- *   every stage keeps its whole arrival stream in the workspace.  Beyond that
- *   (long traces through deep pipelines) a stage's stream lives in a ring of
- *   8,192 records, so the scratch per resident candidate does not grow with the
- *   trace, and a parent stage waits when it would overrun its child's ring.  A
- *   candidate in which one batch stays in flight while more than a ring of later
- *   records passes through the other replicas of its stage cannot be finished
- *   that way: it is evaluated by the IL_VARIANT_PACKED kernel in the same call
- *   (il_stats.fallback_candidates counts them).
+ *   one.  The stream between two stages is a ring of a few records in shared
+ *   memory; a parent stage waits when its child's ring is full.  Examined records
+ *   wait in shared memory for their batch to leave, and beyond that in a spill
+ *   ring of up to 8,192 words per lane in the workspace (whole streams with
+ *   fan-out).  A candidate in which one batch stays in flight while more than a
+ *   spill ring of later records passes through the other replicas of its stage
+ *   cannot be finished that way: it is evaluated by the IL_VARIANT_PACKED kernel
+ *   in the same call (il_stats.fallback_candidates counts them).
  * IL_VARIANT_PACKED: one candidate per warp, stages one after the other, replica
  *   slots across the lanes, warp-level primitives for the queue count and the
  *   slot to reuse.
@@ -408,9 +407,8 @@ IL_API int il_set_variant(il_estimator *est, int variant);
 
 /*
  * Hooks for the library's own tests; not for production use.
- *   IL_KNOB_LANE_RING_LOG2  value 6..24: the lane kernel keeps its streams in rings of at most 2^value
- *                           records whatever the sizes (by default the library chooses between whole
- *                           streams and rings of 2^13).  Small rings force the overflow path.
+ *   IL_KNOB_LANE_RING_LOG2  value 6..24: the lane kernel's spill rings hold at most 2^value words
+ *                           (2^13 by default).  Small rings force the overflow path.
  *   IL_KNOB_ITER_LIMIT      value >= 0: iteration bound of the simulation kernels' loops; 0 restores
  *                           the bound each loop derives from its input.  A small bound makes a call
  *                           return IL_ERR_ITER_LIMIT; the handle stays usable.
@@ -419,7 +417,7 @@ IL_API int il_set_variant(il_estimator *est, int variant);
  *                           preconditions hold; 2: never; 3: always, and the distinct stage runs are
  *                           simulated one by one even where a covering set of whole candidates on
  *                           the lane kernel would do.
- *   IL_KNOB_LANE_CTAS       value 0..16: resident CTAs (of two warps) per SM of the lane kernel; 0 restores
+ *   IL_KNOB_LANE_CTAS       value 0..16: resident CTAs (of four warps) per SM of the lane kernel; 0 restores
  *                           the library's choice (4).  For measurements.
  *   IL_KNOB_BITS_IN_RECORDS value 0 or 1: whether the lane kernel's stream records carry the queries' branch
  *                           bits (1, the default where the time range leaves room) or every stage looks

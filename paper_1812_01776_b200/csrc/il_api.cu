@@ -26,6 +26,7 @@ static constexpr int kCounters = 8;
 struct il_estimator {
     int device = 0;
     int num_sms = 0;
+    size_t smem_per_sm = 0, smem_per_cta = 0;   // shared memory of an SM, and the most a CTA can have of it
     int ctas_per_sm = 0;
     cudaStream_t stream = nullptr;
 
@@ -49,16 +50,14 @@ struct il_estimator {
     bool lane_ok = false;              // the lane kernel applies (packed records, stream offsets fit 31 bits)
     int variant = IL_VARIANT_AUTO;
     int ctas_per_sm_wide = 0, ctas_per_sm_packed = 0, ctas_per_sm_staged = 0, ctas_per_sm_lane = 0;
-    int64_t lane_elems = 0;            // lane kernel: stream records per candidate (all rings of a candidate)
-    int lane_ring_log2 = 0;            // lane kernel: a stream ring holds 2^this records
-    int lane_ring_cap_log2 = 0;        // test knob: force rings of at most 2^this records (0: the library's choice)
+    int lane_ring_log2 = 0;            // lane kernel: a lane's spill ring holds 2^this words
+    int lane_ring_cap_log2 = 0;        // test knob: force rings of at most 2^this words (0: the library's choice)
     bool lane_wrap = false;            // the rings are shorter than the longest stream
     unsigned long long iter_limit = 0; // test knob: iteration bound of the device loops (0 = their own)
     int share_mode = 0;                // shared-prefix evaluation: 0 when it pays, 1 always (tests), 2 never, 3 always and node by node
     int32_t parent[IL_MAX_STAGES] = {};
     int cpw = 1;                       // lane kernel: candidates per warp
-    size_t smem_lane[2] = {0, 0};       // lane kernel with 16 / 32 batch ring positions per lane
-    int ctas_lane[2] = {0, 0};
+    int ctas_lane[2] = {0, 0};         // lane kernel with 16 / 32 batch ring positions per lane: CTAs that fit an SM
     int lane_slots = 32;               // batch ring positions used by the current call
     int64_t setup_launches = 0;        // kernels a call launched before its simulation: the replica reduction, the node probe
     int lane_ctas_knob = 0;            // test knob: resident CTAs per SM of the lane kernel (0: the library's choice)
@@ -94,6 +93,7 @@ constexpr int kOneWaveCtasPerSm = 6;
 struct Plan {
     int64_t slots = 0;       // warp slots with stream buffers
     int64_t chunk = 0;       // candidates per (simulate, select) pair
+    int64_t cps = 1;         // candidates per warp slot
     int64_t fb_slots = 0;    // lane kernel with wrapping rings: warp slots of the kernel that takes over
                              // the candidates given up on ring overflow
     size_t off_time = 0, off_qid = 0, off_slab = 0, off_order = 0, off_ovf = 0, off_fb = 0, total = 0;
@@ -101,13 +101,12 @@ struct Plan {
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// Resident CTAs (of two warps) per SM for the lane kernel.  Every stream record reaches its lane through
-// L1, and L1 is what the 256 KB of an SM have left after the shared-memory carve-out, which the launch
-// sets to what the resident CTAs use (des_lane_kernel.cu).  More CTAs mean more lanes sharing less L1:
-// on B200, 3 / 4 / 5 / 6 / 8 CTAs gave 42.8 / 39.3 / 43.0 / 46.8 / 70.4 ms on workload 2 with 16,384
-// candidates and 298 / 245 / 336 / 336 / 335 ms on workload 3 with 16,384.  (Left to the driver, the
-// carve-out was the largest one whatever the grid, and the same cases took 70 and 336 ms.)
+// Resident CTAs (of four warps) per SM for the lane kernel: what shared memory holds, at most four.
 constexpr int kLaneCtasPerSm = 4;
+
+// Words of examined records a lane keeps in shared memory before it spills: this many where the grid needs every
+// resident CTA, more where it leaves shared memory unused.
+constexpr int kLaneWords = 64, kLaneWordsMost = 256;
 
 bool use_packed(const il_estimator *e)
 {
@@ -137,11 +136,18 @@ int ctas_for(const il_estimator *e)
 // kernel cpw candidates.
 bool is_lane(const il_estimator *e) { return sim_kernel(e) == kSimLane; }
 int warps_per_cta(const il_estimator *e) { return is_lane(e) ? des_lane_warps_per_cta() : kWarpsPerCta; }
-int64_t cands_per_slot(const il_estimator *e) { return is_lane(e) ? e->cpw : 1; }
+// A batch that leaves schedulers idle is spread over them first: a warp that has its scheduler to itself takes
+// the same time for one candidate as for cpw, and less where its lanes diverge.
+int64_t cands_per_slot(const il_estimator *e, int64_t n_cand)
+{
+    if (!is_lane(e)) return 1;
+    const int64_t schedulers = (int64_t)e->num_sms * 4;
+    return std::max<int64_t>(1, std::min<int64_t>(e->cpw, (n_cand + schedulers - 1) / schedulers));
+}
 
 size_t slot_time_bytes(const il_estimator *e)
 {
-    return is_lane(e) ? (size_t)e->cpw * e->lane_elems * 8 : (size_t)e->slot_elems * 8;
+    return is_lane(e) ? (size_t)32 * 4 << e->lane_ring_log2 : (size_t)e->slot_elems * 8;
 }
 size_t slot_qid_bytes(const il_estimator *e) { return is_lane(e) ? 0 : (size_t)e->slot_elems * 4; }
 size_t slot_bytes(const il_estimator *e) { return slot_time_bytes(e) + slot_qid_bytes(e); }
@@ -149,22 +155,23 @@ size_t cand_bytes(const il_estimator *e) { return (size_t)e->n_pad * 8 + 5; }   
 bool lane_fallback(const il_estimator *e) { return is_lane(e) && e->lane_wrap; }
 size_t fb_slot_bytes(const il_estimator *e) { return (size_t)e->slot_elems * 8; }
 
-int lane_ctas(const il_estimator *e)
+int lane_ctas(const il_estimator *e, int lane_slots)
 {
-    const int fit = e->ctas_lane[e->lane_slots == 16 ? 0 : 1];
+    const int fit = e->ctas_lane[lane_slots == 16 ? 0 : 1];
     return std::max(1, std::min(fit, e->lane_ctas_knob > 0 ? e->lane_ctas_knob : kLaneCtasPerSm));
 }
 
-int64_t full_slots(const il_estimator *e)
+// Warp slots that can be resident at once; the lane kernel has more of them with 16 batch ring positions per lane.
+int64_t full_slots(const il_estimator *e, int lane_slots)
 {
-    return (int64_t)e->num_sms * (is_lane(e) ? lane_ctas(e) : e->ctas_per_sm) * warps_per_cta(e);
+    return (int64_t)e->num_sms * (is_lane(e) ? lane_ctas(e, lane_slots) : e->ctas_per_sm) * warps_per_cta(e);
 }
 
-int64_t wanted_slots(const il_estimator *e, int64_t n_cand)
+int64_t wanted_slots(const il_estimator *e, int64_t n_cand, int lane_slots)
 {
-    const int64_t w = warps_per_cta(e), cps = cands_per_slot(e);
+    const int64_t w = warps_per_cta(e), cps = cands_per_slot(e, n_cand);
     const int64_t need = ((n_cand + cps - 1) / cps + w - 1) / w * w;
-    return std::max<int64_t>(w, std::min(full_slots(e), need));
+    return std::max<int64_t>(w, std::min(full_slots(e, lane_slots), need));
 }
 
 size_t layout(const il_estimator *e, Plan &pl)
@@ -193,9 +200,9 @@ size_t recommended_bytes(const il_estimator *e, int64_t n_cand)
 {
     Plan pl;
     n_cand = std::max<int64_t>(n_cand, 1);
-    pl.slots = wanted_slots(e, n_cand);
-    pl.chunk = std::max<int64_t>(std::min<int64_t>(n_cand, 8 * full_slots(e) * cands_per_slot(e)),
-                                 2 * pl.slots * cands_per_slot(e));
+    pl.slots = wanted_slots(e, n_cand, 16);
+    const int64_t cps = cands_per_slot(e, n_cand);
+    pl.chunk = std::max<int64_t>(std::min<int64_t>(n_cand, 8 * full_slots(e, 16) * cps), 2 * pl.slots * cps);
     pl.fb_slots = lane_fallback(e) ? (int64_t)e->num_sms * kWarpsPerCta : 0;
     return layout(e, pl) + 2048;
 }
@@ -218,14 +225,16 @@ bool make_plan(const il_estimator *e, size_t bytes, int64_t n_cand, Plan &pl)
     if (pl.fb_slots > 0) usable -= (size_t)pl.fb_slots * fb_slot_bytes(e) + 256;
     const size_t sb = slot_bytes(e), cb = cand_bytes(e);
     const int64_t w = warps_per_cta(e);
-    int64_t slots = std::min<int64_t>(wanted_slots(e, n_cand), (int64_t)(usable / (sb + 2 * cands_per_slot(e) * cb)));
+    const int64_t cps = cands_per_slot(e, n_cand);
+    int64_t slots = std::min<int64_t>(wanted_slots(e, n_cand, e->lane_slots), (int64_t)(usable / (sb + 2 * cps * cb)));
     slots = slots / w * w;
     if (slots < w) return false;
     pl.slots = slots;
+    pl.cps = cps;
     pl.chunk = std::min<int64_t>(n_cand, (int64_t)((usable - (size_t)slots * sb) / cb));
     // several chunks: whole waves of the resident warps per chunk, so that only the last chunk has a
     // partly filled wave
-    const int64_t wave = slots * cands_per_slot(e);
+    const int64_t wave = slots * cps;
     if (pl.chunk < n_cand && pl.chunk > wave) pl.chunk = pl.chunk / wave * wave;
     // alignment padding may push the layout over: shrink the chunk until it fits
     while (pl.chunk > 0 && layout(e, pl) > bytes) pl.chunk -= std::max<int64_t>(1, pl.chunk / 64);
@@ -308,44 +317,23 @@ int64_t plan_stream_buffers(const il_profiles *pr, const int64_t *visits, int32_
     return top;
 }
 
-// Layout of a candidate's inter-stage streams in the lane kernel.  While the streams of all resident
-// candidates fit kLaneExactBytes, every stage keeps its whole arrival stream (nothing wraps, and the
-// kernel instantiation without the ring protocol runs, which is the faster one per iteration).  Beyond
-// that -- long traces through deep pipelines -- a stage's stream lives in a ring of 2^13 records and the
-// scratch per resident candidate no longer grows with the trace.  lane_ring_cap_log2 > 0 (test knob)
-// forces rings of at most that length.
-constexpr int64_t kLaneExactBytes = INT64_C(48) << 30;
+// Spill rings of the lane kernel: where more examined records wait for their batch to leave than a lane keeps in
+// shared memory, they go to a ring of 2^13 words per lane (shorter where no stream is longer).  With fan-out the
+// rings hold whole streams, since no other kernel can take a candidate over half-way.  lane_ring_cap_log2 > 0
+// (test knob) forces rings of at most that length.
 constexpr int kLaneRingLog2 = 13;
 
 void configure_lane_rings(il_estimator *e)
 {
-    DesParams &bp = e->base;
-    int64_t longest = 8, exact = 0;
-    for (int s = 1; s < e->S; s++) {
-        longest = std::max(longest, e->visits[s]);
-        exact += (e->visits[s] + 3) / 4 * 4;
-    }
-    const int64_t resident = (int64_t)e->num_sms * kLaneCtasPerSm * des_lane_warps_per_cta() * e->cpw;
-    const bool rings = !e->fork && (e->lane_ring_cap_log2 > 0 || exact * 8 * resident > kLaneExactBytes ||
-                                    exact >= (INT64_C(1) << 31));
-    bp.lane_off[0] = 0;
-    if (!rings) {
-        int64_t off = 0;
-        for (int s = 1; s < e->S; s++) { bp.lane_off[s] = (int32_t)off; off += (e->visits[s] + 3) / 4 * 4; }
-        e->lane_elems = std::max<int64_t>(exact, 4);
-        e->lane_ring_log2 = 31;
-        e->lane_wrap = false;
-    } else {
-        int need = 3;
-        while ((INT64_C(1) << need) < longest) need++;
-        e->lane_ring_log2 = std::min(need, e->lane_ring_cap_log2 > 0 ? e->lane_ring_cap_log2 : kLaneRingLog2);
-        e->lane_wrap = (INT64_C(1) << e->lane_ring_log2) < longest;
-        for (int s = 1; s < e->S; s++) bp.lane_off[s] = (int32_t)((int64_t)(s - 1) << e->lane_ring_log2);
-        e->lane_elems = std::max<int64_t>((int64_t)(e->S - 1) << e->lane_ring_log2, 4);
-    }
-    bp.lane_elems = e->lane_elems;
-    bp.lane_ring_log2 = e->lane_ring_log2;
-    bp.lane_wrap = e->lane_wrap ? 1 : 0;
+    int64_t longest = 1;
+    for (int s = 0; s < e->S; s++) longest = std::max(longest, e->visits[s]);
+    int need = 6;                      // ring positions are told apart over the reach of a spill, 2 x 8 records more
+    while ((INT64_C(1) << need) < longest) need++;
+    const int cap = e->lane_ring_cap_log2 > 0 ? e->lane_ring_cap_log2 : kLaneRingLog2;
+    e->lane_ring_log2 = e->fork ? need : std::min(need, cap);
+    e->lane_wrap = e->lane_ring_log2 < need;
+    e->base.lane_ring_log2 = e->lane_ring_log2;
+    e->base.lane_wrap = e->lane_wrap ? 1 : 0;
 }
 
 void free_device(il_estimator *e)
@@ -450,14 +438,13 @@ static DesParams chunk_params(const il_estimator *e, const Plan &pl, char *ws, c
     p.ovf = reinterpret_cast<uint8_t *>(ws + pl.off_ovf);
     p.iter_limit = e->iter_limit;
     p.lane_slots = e->lane_slots;
-    p.lane_ctas_per_sm = lane_ctas(e);
+    p.cpw = (int32_t)pl.cps;
     return p;
 }
 
-// Batch ring positions per lane for this batch: 16 when no candidate has more than 14 replicas at any
-// stage (the ring must hold the slots in use and the batches waiting to be handed on; with 16 replicas on
-// 16 positions a stage stalls until each batch has been handed on, and workload 4 ran 1.6x slower), else 32.  One
-// small reduction over the configurations and a 4-byte read-back.
+// Batch ring positions per lane for this batch: 16 when no candidate has more than 16 replicas at any
+// stage (the ring must hold the batches in use), else 32.  One small reduction over the configurations
+// and a 4-byte read-back.
 static int choose_lane_slots(il_estimator *e, const il_stage_config *d_configs, int64_t n_cand)
 {
     e->lane_slots = 32;
@@ -469,8 +456,18 @@ static int choose_lane_slots(il_estimator *e, const il_stage_config *d_configs, 
     IL_CUDA(launch_max_replicas(d_configs, n_cand * e->S, e->d_maxrep, e->stream));
     IL_CUDA(cudaMemcpyAsync(&h, e->d_maxrep, sizeof(int), cudaMemcpyDeviceToHost, e->stream));
     IL_CUDA(cudaStreamSynchronize(e->stream));
-    e->lane_slots = h <= 14 ? 16 : 32;
+    e->lane_slots = h <= 16 ? 16 : 32;
     return IL_OK;
+}
+
+static cudaError_t launch_lane(const il_estimator *e, DesParams p, int64_t ctas, cudaStream_t st)
+{
+    const size_t per_sm = (size_t)((ctas + e->num_sms - 1) / e->num_sms);
+    int words = kLaneWordsMost;
+    while (words > kLaneWords && ((des_lane_smem(e->S * e->H, e->Bmax, e->lane_slots, words) + 1024) * per_sm > e->smem_per_sm ||
+                                  des_lane_smem(e->S * e->H, e->Bmax, e->lane_slots, words) > e->smem_per_cta)) words >>= 1;
+    p.lane_words = words;
+    return launch_des_lane(p, (int)ctas, des_lane_smem(e->S * e->H, e->Bmax, e->lane_slots, words), st);
 }
 
 // Enqueues the simulation of one chunk whose work counter is zero: the kernel the handle uses
@@ -485,7 +482,8 @@ static int enqueue_simulation(il_estimator *e, const DesParams &p, const Plan &p
     // fan-out: the lane kernel keeps per query the largest leaving record, starting from zero
     if (kernel == kSimLane && e->fork)
         IL_CUDA(cudaMemsetAsync(p.slab, 0, (size_t)p.n_cand * p.slab_stride * 8, st));
-    IL_CUDA(launch_simulation(p, kernel, (int)ctas, kernel == kSimLane ? e->smem_lane[e->lane_slots == 16 ? 0 : 1] : e->smem, st));
+    if (kernel == kSimLane) IL_CUDA(launch_lane(e, p, ctas, st));
+    else IL_CUDA(launch_simulation(p, kernel, (int)ctas, e->smem, st));
     (*launches)++;
     if (fb) {
         IL_CUDA(launch_overflow_list(p.ovf, p.n_cand, const_cast<int32_t *>(p.order), e->d_counters, st));
@@ -529,9 +527,9 @@ static int finish_shared(il_estimator *e, int64_t n_cand, int64_t launches, int6
 // that contains it); those are simulated like any batch, and a node's leaving records are the region
 // of its stage in the slab row of its candidate.  Candidates of the set repeat the work of the
 // prefixes they share, but they run on the kernel that is an order of magnitude faster per stage run
-// than the node-by-node one, and all at once instead of level by level.  Needs whole streams (no
-// rings, so that every row has the region layout) and room for all rows in one chunk; *done stays
-// false when that is not so, and the caller simulates the nodes one by one.
+// than the node-by-node one, and all at once instead of level by level.  (A candidate evaluated by the
+// fallback has its row laid out the same way.)  Needs room for all rows in one chunk; *done stays false
+// when that is not so, and the caller simulates the nodes one by one.
 // On entry `off` bytes of the workspace are in use; events[0] has been recorded.
 struct SharedCommon {
     const il_stage_config *d_configs;
@@ -546,7 +544,7 @@ static int shared_by_cover(il_estimator *e, const SharedCommon &c, char *ws, siz
                            int64_t *launches, int64_t *stage_runs, bool *done)
 {
     *done = false;
-    if (e->share_mode == 3 || !is_lane(e) || e->lane_wrap) return IL_OK;
+    if (e->share_mode == 3 || !is_lane(e)) return IL_OK;
     const int S = e->S;
     const int64_t n_cand = c.n_cand;
     auto take = [&](size_t bytes) { const size_t at = off; off = align_up(off + bytes, 256); return at; };
@@ -596,7 +594,7 @@ static int shared_by_cover(il_estimator *e, const SharedCommon &c, char *ws, siz
     char *sim_ws = ws + off;
     DesParams p = chunk_params(e, pl, sim_ws, cfg, m);
     const int64_t wpc = warps_per_cta(e);
-    const int64_t groups = (m + cands_per_slot(e) - 1) / cands_per_slot(e);
+    const int64_t groups = (m + pl.cps - 1) / pl.cps;
     const int64_t ctas = std::min<int64_t>(pl.slots / wpc, (groups + wpc - 1) / wpc);
     int rc = enqueue_simulation(e, p, pl, sim_ws, ctas, st, launches);
     if (rc) return rc;
@@ -858,6 +856,8 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
     if (!e) return IL_ERR_NOMEM;
     e->device = dev;
     e->num_sms = prop.multiProcessorCount;
+    e->smem_per_sm = prop.sharedMemPerMultiprocessor;
+    e->smem_per_cta = prop.sharedMemPerBlockOptin;
     e->S = S; e->H = H; e->Bmax = B; e->n = n;
     e->n_pad = (n + 31) / 32 * 32;
     e->span_us = (float)std::max<int64_t>(1, tr->arrival_us[n - 1] - tr->arrival_us[0]);
@@ -954,9 +954,7 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
         }
     }
     for (int s = 0; s < S; s++) bp.n_s[s] = (int32_t)e->visits[s];
-    // lane kernel: every stage but the root reads its arrival stream from a ring
     e->cpw = 32 / S;
-    bp.cpw = e->cpw;
     configure_lane_rings(e);
     bp.S = S; bp.H = H; bp.Bmax = B; bp.n = (int32_t)n;
     e->smem = (size_t)S * H * B * sizeof(int32_t);
@@ -970,12 +968,12 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
     IL_CUDA_E(cudaMalloc(&e->d_arrival, (size_t)n * 8));
     IL_CUDA_E(cudaMalloc(&e->d_bits, (size_t)n));
     e->can_pack = can_pack;
-    e->lane_ok = can_pack && !e->join && e->lane_elems < (INT64_C(1) << 31);   // (with fan-out the streams are kept whole)
+    e->lane_ok = can_pack && !e->join;
     bp.qbits = qbits;
     if (can_pack) {
         // padded with "never" records to whole tiles, so that bulk copies always move full tiles
         const int64_t tile = trace_tile_records();
-        const int64_t n_padded = (n + tile - 1) / tile * tile;
+        const int64_t n_padded = (n + 2 + tile - 1) / tile * tile;      // (two at least: the lane kernel reads ahead)
         std::vector<uint64_t> packed((size_t)n_padded, ~0ull);
         for (int64_t i = 0; i < n; i++)
             packed[(size_t)i] = ((uint64_t)tr->arrival_us[i] << qbits) | (uint64_t)i;
@@ -986,7 +984,7 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
         int nb = 0;
         for (int s = 0; s < pr->n_stages; s++)
             if (pr->cond_bit[s] >= 0) nb = std::max(nb, (int)pr->cond_bit[s] + 1);
-        if (nb > 0 && tr->branch_bits && !e->join &&
+        if (nb > 0 && tr->branch_bits && !e->join && qbits + nb <= 31 &&
             tr->arrival_us[n - 1] + worst < (INT64_C(1) << (63 - qbits - nb))) {
             for (int64_t i = 0; i < n; i++)
                 packed[(size_t)i] = ((uint64_t)tr->arrival_us[i] << (qbits + nb)) |
@@ -1015,8 +1013,7 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
     e->ctas_per_sm_packed = des_packed_max_ctas_per_sm(false, e->smem);
     e->ctas_per_sm_staged = des_packed_max_ctas_per_sm(true, e->smem);
     for (int k = 0; k < 2; k++) {
-        e->smem_lane[k] = des_lane_smem(S * H * B, B, k == 0 ? 16 : 32);
-        e->ctas_lane[k] = des_lane_max_ctas_per_sm(e->smem_lane[k]);
+        e->ctas_lane[k] = des_lane_max_ctas_per_sm(des_lane_smem(S * H, B, k == 0 ? 16 : 32, kLaneWords));
     }
     e->ctas_per_sm_lane = std::min(e->ctas_lane[1], kLaneCtasPerSm);
     if (e->ctas_per_sm_wide < 1 || e->ctas_per_sm_packed < 1 || e->ctas_per_sm_staged < 1 ||
@@ -1175,7 +1172,7 @@ int il_estimate_device(il_estimator *e, const il_stage_config *d_configs, int64_
         if (ch > 0) IL_CUDA(cudaMemsetAsync(e->d_counters, 0, sizeof(unsigned long long), st));
         const bool lane = is_lane(e);
         const int64_t wpc = warps_per_cta(e);
-        const int64_t groups = (cnt + cands_per_slot(e) - 1) / cands_per_slot(e);
+        const int64_t groups = (cnt + pl.cps - 1) / pl.cps;
         int64_t ctas = std::min<int64_t>(pl.slots / wpc, (groups + wpc - 1) / wpc);
         if (!lane) {   // the lane kernel's warps take candidates in index order
             OrderParams op;
@@ -1186,7 +1183,7 @@ int il_estimate_device(il_estimator *e, const il_stage_config *d_configs, int64_
             op.order = const_cast<int32_t *>(p.order);
             IL_CUDA(launch_order(op, st));
             launches++;
-            if (2 * cnt <= 3 * full_slots(e))
+            if (2 * cnt <= 3 * full_slots(e, 32))
                 ctas = std::min<int64_t>(ctas, (int64_t)e->num_sms * std::min(e->ctas_per_sm, kOneWaveCtasPerSm));
         }
         IL_CUDA(cudaEventRecord(e->events[2 + 3 * ch], st));
@@ -1358,7 +1355,7 @@ int il_feasible_device(il_estimator *e, const il_stage_config *d_configs, int64_
     const size_t sb = slot_time_bytes(e);
     const size_t tail_bytes = align_up((size_t)n_cand, 256) + align_up((size_t)n_cand * 4, 256) + 1024;
     if (ws_bytes < tail_bytes + (size_t)wpc * sb) return IL_ERR_NOMEM;
-    int64_t slots = std::min<int64_t>(wanted_slots(e, n_cand), (int64_t)((ws_bytes - tail_bytes) / sb)) / wpc * wpc;
+    int64_t slots = std::min<int64_t>(wanted_slots(e, n_cand, e->lane_slots), (int64_t)((ws_bytes - tail_bytes) / sb)) / wpc * wpc;
     if (slots < wpc) return IL_ERR_NOMEM;
     const size_t off_ovf = align_up((size_t)slots * sb, 256);
     const size_t off_order = off_ovf + align_up((size_t)n_cand, 256);
@@ -1374,17 +1371,17 @@ int il_feasible_device(il_estimator *e, const il_stage_config *d_configs, int64_
     p.ovf = reinterpret_cast<uint8_t *>(ws + off_ovf);
     p.iter_limit = e->iter_limit;
     p.lane_slots = e->lane_slots;
-    p.lane_ctas_per_sm = lane_ctas(e);
+    p.cpw = (int32_t)cands_per_slot(e, n_cand);
     p.out_feasible = d_out_feasible;
     // latency > objective is tested on time fields shifted by qbits: keep the objective in that range
     // (latencies are at least 1 and every reachable time is below 2^(63 - qbits))
     p.slo_us = std::min<int64_t>(std::max<int64_t>(slo_us, 0), INT64_C(1) << (62 - p.qbits - p.rec_bits));
     p.miss_allow = (uint32_t)(e->n - (99 * e->n + 99) / 100);
     if (e->lane_wrap) IL_CUDA(cudaMemsetAsync(p.ovf, 0, (size_t)n_cand, st));
-    const int64_t groups = (n_cand + e->cpw - 1) / e->cpw;
+    const int64_t groups = (n_cand + p.cpw - 1) / p.cpw;
     const int64_t ctas = std::min<int64_t>(slots / wpc, (groups + wpc - 1) / wpc);
     IL_CUDA(cudaEventRecord(e->events[0], st));
-    IL_CUDA(launch_des_lane(p, (int)ctas, e->smem_lane[e->lane_slots == 16 ? 0 : 1], st));
+    IL_CUDA(launch_lane(e, p, ctas, st));
     IL_CUDA(cudaEventRecord(e->events[1], st));
     int64_t launches = 1;
     if (e->lane_wrap) {

@@ -73,15 +73,13 @@ struct DesParams {
     unsigned long long *counters; // [0] next candidate, [1] batches dispatched, [2] algorithmic ops
     int *status;                  // first error seen by any warp (0 = none)
     // lane-parallel kernel only (des_lane_kernel.cu)
-    uint64_t *lane_ws;            // [warp slots][cpw][lane_elems] inter-stage streams of packed records
-    int64_t lane_elems;           // stream records per candidate: every stage's arrival stream but the root's
-    int32_t lane_off[IL_MAX_STAGES]; // record offset of stage s's arrival stream inside a candidate's block
-    int32_t cpw;                  // candidates per warp, floor(32 / S)
+    uint64_t *lane_ws;            // [warp slots][32][2^lane_ring_log2] words: the lanes' spill rings
+    int32_t cpw;                  // candidates per warp, at most floor(32 / S)
     int32_t lane_slots;           // positions of a lane's batch ring in shared memory: 16 or 32, at least the
                                   // largest replica count among the launch's candidates
-    int32_t lane_ctas_per_sm;     // CTAs the host keeps resident per SM (sizes the shared-memory carve-out); 0: unknown
-    int32_t lane_ring_log2;       // a stream ring holds 2^this records
-    int32_t lane_wrap;            // the rings are shorter than the longest stream: positions wrap
+    int32_t lane_ring_log2;       // a lane's spill ring in lane_ws holds 2^this words
+    int32_t lane_words;           // words of examined records a lane keeps in shared memory (a power of two)
+    int32_t lane_wrap;            // the rings are shorter than the longest stream
     uint8_t *ovf;                 // [n_cand] set to 1 for a candidate given up on ring overflow (lane_wrap only)
     // lane kernel, feasibility only: set out_feasible to select that instantiation
     uint8_t *out_feasible;        // [n_cand] 1: P99 <= slo_us, 0: not, 2: given up on ring overflow (see ovf)
@@ -131,7 +129,8 @@ int trace_tile_records();     // the packed trace is padded to a multiple of thi
 // lane-parallel kernel: one lane per (candidate, stage); smem from des_lane_smem
 cudaError_t launch_des_lane(const DesParams &p, int grid, size_t smem, cudaStream_t stream);
 int des_lane_warps_per_cta();
-size_t des_lane_smem(int n_tab, int Bmax, int ring_slots);   // ring_slots: 16 or 32 batch ring positions per lane
+// ring_slots: 16 or 32 batch ring positions per lane; ring_words: words of examined records (a power of two)
+size_t des_lane_smem(int table_rows, int Bmax, int ring_slots, int ring_words);
 int des_lane_max_ctas_per_sm(size_t smem);
 enum SimKernel { kSimWide = 0, kSimPacked = 1, kSimPackedStaged = 2, kSimLane = 3 };
 inline cudaError_t launch_simulation(const DesParams &p, int kernel, int grid, size_t smem,

@@ -1,0 +1,63 @@
+"""The lane kernel where its rings can go wrong: records in flight around what a lane keeps in shared memory and in
+its spill ring, replica counts around the two sizes of the batch ring, trace lengths around a turn and around a tile
+of the packed trace, and more candidates than the device holds at once."""
+import numpy as np
+import pytest
+
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+
+def same(w, oracle, ring=0):
+    import torch
+    import paper_1812_01776_b200 as il
+    exp = oracle.estimate_workload(w)
+    with il.Estimator.from_workload(w) as est:
+        if ring:
+            est.set_test_knob(1, ring)
+        est.set_test_knob(3, 2)
+        a, b = est.estimate_device(torch.from_numpy(w.configs).cuda(), w.slo_us)
+        st = est.stats()
+        assert np.array_equal(a.cpu().numpy(), exp[0]) and np.array_equal(b.cpu().numpy(), exp[1])
+        assert np.array_equal(est.feasible(w.configs, w.slo_us), exp[0] <= w.slo_us)
+    return st
+
+
+@pytest.mark.parametrize("ring", [0, 7, 9])
+@pytest.mark.parametrize("burst", [30, 47, 65, 130, 260, 1100])
+def test_records_in_flight(oracle, burst, ring):
+    """Bursts of arrivals at one instant, on as many replicas as take them all: that many records wait at once."""
+    w = workloads.random_small(burst, S=3, H=2, Bmax=64, n=4000, C=48, max_replicas=32, lat_lo=500, lat_hi=900000)
+    w.arrival_us = (np.arange(4000) // burst * 400_000).astype(np.int64)
+    w.configs[::2, :, 2] = 32
+    st = same(w, oracle, ring)
+    assert ring or st["fallback_candidates"] == 0
+
+
+@pytest.mark.parametrize("replicas", [1, 2, 14, 15, 16, 17, 31, 32])
+def test_replicas_around_the_ring_sizes(oracle, replicas):
+    w = workloads.random_small(replicas, S=4, H=2, Bmax=4, n=1500, C=40, max_replicas=replicas, qps=900.0, cv=4.0,
+                               lat_lo=1, lat_hi=60000, equal_stamp_every=2)
+    w.configs[::3, :, 2] = replicas
+    same(w, oracle)
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 15, 16, 17, 32, 33, 510, 511, 512, 513, 1024])
+def test_trace_lengths(oracle, n):
+    w = workloads.random_small(n, S=5, H=2, Bmax=8, n=n, C=33, max_replicas=3, tree=n % 2 == 1)
+    same(w, oracle)
+
+
+@pytest.mark.parametrize("S", [1, 3])
+def test_more_candidates_than_resident_groups(oracle, S):
+    w = workloads.random_small(S, S=S, H=2, Bmax=4, n=60, C=90_001, max_replicas=3)
+    w.configs = np.ascontiguousarray(w.configs[np.arange(90_001) % 5_000])
+    exp = oracle.estimate_workload(workloads.Workload(w.name, w.parent, w.cond_bit, w.cond_val, w.latency_us, w.arrival_us,
+                                                      w.branch_bits, w.configs[:5_000].copy(), w.slo_us))
+    import torch
+    import paper_1812_01776_b200 as il
+    with il.Estimator.from_workload(w) as est:
+        est.set_test_knob(3, 2)
+        a, _ = est.estimate_device(torch.from_numpy(w.configs).cuda(), w.slo_us)
+    assert np.array_equal(a.cpu().numpy(), exp[0][np.arange(w.n_candidates) % 5_000])
