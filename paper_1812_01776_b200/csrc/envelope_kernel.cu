@@ -1,17 +1,27 @@
 // Traffic envelope of the bound trace (Section 5): for each window length, the
 // largest number of arrivals inside any window of that length.  A maximising
-// window can be moved right until it starts at an arrival, so thread j counts
-// the arrivals in [a_j, a_j + window) for every window length -- a binary search
-// for the first arrival at or after a_j + window, started where the search for
-// the previous (shorter) window ended when the lengths ascend -- and the
-// per-window maxima are combined with a warp reduction and one atomic per warp.
-// The trace is read-only and L2-resident; the work is n * W searches.
+// window can be moved right until it starts at an arrival, so the answer is the
+// maximum over j of end(j) - j, end(j) being the first arrival at or after
+// a_j + window.
+//
+// What bounds it: the binary searches for end(j) in the L2-resident trace (their
+// latency, and a sector of L2 per step), so most of them are not made.  end()
+// never decreases, so for neighbouring starts j .. k - 1 the counts are at most
+// end(k) - j.  A CTA searches every 256th start of its stretch, all windows side
+// by side; these counts also are lower bounds of the answer, which the CTAs share
+// as they go.  Only where 256 starts could still beat the best count known so
+// far, a warp looks closer: start m can only be better than B if arrival m + B still
+// lies in its window, one coalesced load and a compare, and only a start that passes
+// is searched.  10^6 arrivals, 12 windows: the whole call 361 -> 48 us (before:
+// 12 x 10^6 searches in two launches).
 #include "il_internal.h"
 
 namespace il {
 
 namespace {
 constexpr int kEnvThreads = 256;
+constexpr int kEnvGroups = 4;                    // groups of 256 starts per CTA
+constexpr int kEnvGroup = 256;
 constexpr int kMaxWindows = 64;
 }
 
@@ -23,42 +33,66 @@ struct EnvParams {
     int *out;                  // [n_windows], zero on entry
 };
 
+// First index in [lo, hi] whose arrival is `window` or more after a (hi if there is none before it).
+__device__ __forceinline__ int first_at(const int64_t *arrival, int lo, int hi, int64_t a, int64_t window)
+{
+    while (lo < hi) {
+        const int mid = lo + (hi - lo) / 2;
+        if (__ldg(arrival + mid) - a < window) lo = mid + 1; else hi = mid;
+    }
+    return lo;
+}
+
 __global__ void __launch_bounds__(kEnvThreads) envelope_kernel(const __grid_constant__ EnvParams p)
 {
-    for (int j0 = blockIdx.x * kEnvThreads; j0 < p.n; j0 += gridDim.x * kEnvThreads) {
-        const int j = j0 + threadIdx.x;
-        const bool act = j < p.n;
-        const int64_t a = act ? p.arrival[j] : 0;
-        int lo_hint = j;
-        int64_t prev_win = 0;
-        for (int w = 0; w < p.n_windows; w++) {
-            int count = 0;
-            if (act) {
-                // first index hi with arrival[hi] - a >= window; the arrivals before it are inside
-                int lo = p.window[w] >= prev_win ? lo_hint : j, hi = p.n;
-                while (lo < hi) {
-                    const int mid = lo + (hi - lo) / 2;
-                    if (p.arrival[mid] - a < p.window[w]) lo = mid + 1; else hi = mid;
-                }
-                count = lo - j;
-                lo_hint = lo;
-                prev_win = p.window[w];
-            }
-            count = __reduce_max_sync(0xffffffffu, count);
-            if ((threadIdx.x & 31) == 0 && count > 0) atomicMax(&p.out[w], count);
+    __shared__ int end[kMaxWindows][kEnvGroups + 1];
+    __shared__ int best[kMaxWindows];
+    const int j0 = blockIdx.x * (kEnvGroups * kEnvGroup);
+    const int W = p.n_windows;
+    for (int w = threadIdx.x; w < W; w += kEnvThreads) best[w] = 0;
+    __syncthreads();
+    for (int k = threadIdx.x; k < W * (kEnvGroups + 1); k += kEnvThreads) {
+        const int w = k / (kEnvGroups + 1), g = k - w * (kEnvGroups + 1);
+        const int64_t j = (int64_t)j0 + g * kEnvGroup;
+        int e = p.n;
+        if (j < p.n) {
+            e = first_at(p.arrival, (int)j, p.n, __ldg(p.arrival + j), p.window[w]);
+            atomicMax(&best[w], e - (int)j);
         }
+        end[w][g] = e;
+    }
+    __syncthreads();
+    for (int w = threadIdx.x; w < W; w += kEnvThreads) best[w] = max(best[w], atomicMax(&p.out[w], best[w]));
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    for (int k = threadIdx.x >> 5; k < W * kEnvGroups; k += kEnvThreads / 32) {
+        const int w = k / kEnvGroups, g = k - w * kEnvGroups;
+        const int64_t j = (int64_t)j0 + g * kEnvGroup;
+        if (j >= p.n || end[w][g + 1] - (int)j <= best[w]) continue;       // none of these 256 can be better
+        const int known = best[w];
+        int count = 0;
+#pragma unroll
+        for (int i = 0; i < kEnvGroup; i += 32) {
+            const int64_t m = j + i + lane;
+            if (m + known >= p.n) continue;
+            const int64_t a = __ldg(p.arrival + m);
+            if (__ldg(p.arrival + m + known) - a < p.window[w])
+                count = max(count, first_at(p.arrival, (int)m + known + 1, end[w][g + 1], a, p.window[w]) - (int)m);
+        }
+        count = __reduce_max_sync(0xffffffffu, count);
+        if (lane == 0 && count > best[w]) best[w] = max(count, atomicMax(&p.out[w], count));
+        __syncwarp();
     }
 }
 
 cudaError_t launch_envelope(const int64_t *d_arrival, int n, const int64_t *h_windows, int n_windows,
-                            int *d_out, int num_sms, cudaStream_t stream)
+                            int *d_out, cudaStream_t stream)
 {
     EnvParams p;
     p.arrival = d_arrival; p.n = n; p.n_windows = n_windows; p.out = d_out;
     for (int w = 0; w < n_windows; w++) p.window[w] = h_windows[w];
-    const int blocks = (n + kEnvThreads - 1) / kEnvThreads;
-    const int grid = blocks < num_sms * 8 ? blocks : num_sms * 8;
-    envelope_kernel<<<grid, kEnvThreads, 0, stream>>>(p);
+    const int64_t per_cta = kEnvGroups * kEnvGroup;
+    envelope_kernel<<<(int)((n + per_cta - 1) / per_cta), kEnvThreads, 0, stream>>>(p);
     return cudaGetLastError();
 }
 

@@ -69,6 +69,7 @@ struct il_estimator {
     int *d_status = nullptr;
     unsigned long long *h_counters = nullptr;   // pinned: [kCounters] counters, then the status word
     int *h_status = nullptr;
+    int *d_envelope = nullptr, *h_envelope = nullptr;   // counts of the traffic envelope, one per window length
 
     void *user_ws = nullptr; size_t user_ws_bytes = 0;
     void *own_ws = nullptr;  size_t own_ws_bytes = 0;
@@ -339,7 +340,7 @@ void configure_lane_rings(il_estimator *e)
 void free_device(il_estimator *e)
 {
     cudaFree(e->d_arrival); cudaFree(e->d_ptrace); cudaFree(e->d_ptrace_b); cudaFree(e->d_bits); cudaFree(e->d_lat);
-    cudaFree(e->d_counters); cudaFree(e->d_status); cudaFree(e->d_maxrep);
+    cudaFree(e->d_counters); cudaFree(e->d_status); cudaFree(e->d_maxrep); cudaFree(e->d_envelope);
     cudaFree(e->own_ws); cudaFree(e->d_cfg); cudaFree(e->d_out);
     if (e->h_counters) cudaFreeHost(e->h_counters);
     for (cudaEvent_t ev : e->events) cudaEventDestroy(ev);
@@ -998,8 +999,10 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
     IL_CUDA_E(cudaMalloc(&e->d_counters, kCounters * sizeof(unsigned long long)));
     IL_CUDA_E(cudaMalloc(&e->d_status, sizeof(int)));
     IL_CUDA_E(cudaMalloc(&e->d_maxrep, sizeof(int)));
-    IL_CUDA_E(cudaMallocHost(&e->h_counters, (kCounters + 2) * sizeof(unsigned long long)));
+    IL_CUDA_E(cudaMalloc(&e->d_envelope, envelope_max_windows() * sizeof(int)));
+    IL_CUDA_E(cudaMallocHost(&e->h_counters, (kCounters + 2) * sizeof(unsigned long long) + envelope_max_windows() * sizeof(int)));
     e->h_status = reinterpret_cast<int *>(e->h_counters + kCounters);
+    e->h_envelope = reinterpret_cast<int *>(e->h_counters + kCounters + 2);
     IL_CUDA_E(cudaMemcpy(e->d_arrival, tr->arrival_us, (size_t)n * 8, cudaMemcpyHostToDevice));
     if (tr->branch_bits) IL_CUDA_E(cudaMemcpy(e->d_bits, tr->branch_bits, (size_t)n, cudaMemcpyHostToDevice));
     else IL_CUDA_E(cudaMemset(e->d_bits, 0, (size_t)n));
@@ -1264,19 +1267,12 @@ int il_traffic_envelope(il_estimator *e, const int64_t *window_us, int32_t n_win
     if (!window_us || !out_max_count) return IL_ERR_INVALID_ARG;
     for (int w = 0; w < n_windows; w++) if (window_us[w] < 1) return IL_ERR_INVALID_ARG;
     IL_CUDA(cudaSetDevice(e->device));
-    // the counts fit the 4-word counter block that every estimate call clears before use
-    static_assert(sizeof(unsigned long long) * kCounters >= sizeof(int) * 8, "counter block too small");
-    int host_out[64];
     cudaStream_t st = e->stream;
-    for (int w0 = 0; w0 < n_windows; w0 += 8) {
-        const int cnt = std::min(8, n_windows - w0);
-        IL_CUDA(cudaMemsetAsync(e->d_counters, 0, kCounters * sizeof(unsigned long long), st));
-        IL_CUDA(launch_envelope(e->d_arrival, (int)e->n, window_us + w0, cnt,
-                                reinterpret_cast<int *>(e->d_counters), e->num_sms, st));
-        IL_CUDA(cudaMemcpyAsync(host_out + w0, e->d_counters, cnt * sizeof(int), cudaMemcpyDeviceToHost, st));
-    }
+    IL_CUDA(cudaMemsetAsync(e->d_envelope, 0, n_windows * sizeof(int), st));
+    IL_CUDA(launch_envelope(e->d_arrival, (int)e->n, window_us, n_windows, e->d_envelope, st));
+    IL_CUDA(cudaMemcpyAsync(e->h_envelope, e->d_envelope, n_windows * sizeof(int), cudaMemcpyDeviceToHost, st));
     IL_CUDA(cudaStreamSynchronize(st));
-    for (int w = 0; w < n_windows; w++) out_max_count[w] = host_out[w];
+    for (int w = 0; w < n_windows; w++) out_max_count[w] = e->h_envelope[w];
     return IL_OK;
 }
 

@@ -76,3 +76,18 @@ def test_gpu_envelope_matches_oracle(oracle, cid, n):
         from paper_1812_01776_b200 import estimator as E
         with pytest.raises(E.ILError):
             est.traffic_envelope(np.array([0], np.int64))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [1, 2, 31, 255, 256, 257, 1023, 1024, 1025, 5000])
+def test_gpu_envelope_around_group_sizes(oracle, n):
+    """Trace lengths around the groups of starts that the kernel rules out together, 64 windows from one
+    microsecond to far beyond the trace, runs of equal stamps."""
+    import paper_1812_01776_b200 as il
+    w = workloads.random_small(n, S=1, H=1, Bmax=1, n=n, C=1, cv=4.0, equal_stamp_every=3 if n % 2 else 0)
+    wins = np.unique(np.geomspace(1, 10 ** 11, 64).astype(np.int64))
+    with il.Estimator.from_workload(w) as est:
+        got = est.traffic_envelope(wins)
+    a = w.arrival_us
+    exp = [(np.searchsorted(a, a + int(win), side="left") - np.arange(n)).max() for win in wins]
+    assert np.array_equal(got, exp)
