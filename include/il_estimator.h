@@ -187,10 +187,13 @@ typedef struct {
 
 /*
  * il_estimator_create for a pipeline with joins; `joins` may be NULL (then the
- * two calls are the same).  A handle with a join runs on the kernel with
- * separate streams (kernel name "des_kernel") whatever variant is set: that
- * kernel builds the join's arrival stream from the two incoming streams before
- * it simulates the stage.  Every entry point works on such a handle and gives
+ * two calls are the same).  A handle with a join runs on one of the two kernels
+ * that merge incoming streams, both reported as "des_kernel", whatever variant
+ * is set: with IL_VARIANT_AUTO and IL_VARIANT_LANES the lane-parallel form, in
+ * which a join has a lane of its own that merges the streams as they come, else
+ * (or where times do not fit a record) the kernel with separate streams, which
+ * builds the join's arrival stream before it simulates the stage.  Every entry
+ * point works on such a handle and gives
  * the same results as on any other; il_feasible* evaluate it without early exit.
  * Errors: as il_estimator_create; BAD_TOPOLOGY also for a second edge outside
  * the form above or a third outgoing edge; TOO_LARGE if the streams of one

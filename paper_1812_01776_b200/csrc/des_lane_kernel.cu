@@ -163,6 +163,11 @@ constexpr uint32_t kXBytes = kX * 256u;
 __host__ __device__ inline size_t table_bytes(int rows, int Bmax) { return ((size_t)rows * (Bmax | 1) + 1) * 4; }
 __host__ __device__ inline size_t ring_bytes(int kr, int nq) { return (size_t)kLaneWarps * (key_bytes(kr) + nq * 128u + kXBytes); }
 constexpr size_t kTailBytes = 256 + kLaneWarps * 128;
+constexpr int kSeen = 64;                     // joins: words of the queries' bits that are kept in shared memory
+// joins: per warp and per (group, join) the counts and the windows of the two incoming streams, then the cached words
+// of the queries' bits with their numbers, then which branch bits follow both edges (256 bits)
+__host__ __device__ inline uint32_t join_lane_bytes(int window) { return 2u * (window + 1) * 8u + kSeen * 8u + 32u; }
+__host__ __device__ inline size_t join_bytes(int cpw, int joins, int window) { return (size_t)kLaneWarps * cpw * joins * join_lane_bytes(window); }
 
 }  // namespace
 
@@ -172,11 +177,17 @@ constexpr size_t kTailBytes = 256 + kLaneWarps * 128;
 //       have missed the objective than the P99 rule allows.
 // FORK: fan-out -- a query goes down every edge whose condition holds, a copy that finds none leaves, and
 //       the slab keeps per query the record of the copy that left last (only with BRANCHY, without FEAS).
-template <bool BRANCHY, bool FEAS, bool FORK = false>
-__global__ void __launch_bounds__(kLaneWarps * 32)
-des_lane_kernel(const __grid_constant__ DesParams p)
+// JOIN: some stage has two incoming edges (with FORK: a query goes down both before it gets there).  A join has a
+//       lane of its own, behind the stages' lanes: it merges the two incoming streams in time order, at equal
+//       times the first parent's records first, swallows the record of an input that is not its query's last one
+//       (one bit per query and join in global memory: the other input has been seen) and feeds the stage's ring.
+//       The incoming streams have no back-pressure -- either parent may have to run ahead of the other by all
+//       that the slower branch keeps in flight -- so they go to global memory whole, and the latest
+//       64 to 512 records of each to shared memory, from where the join nearly always reads them.  511 candidates
+//       of a diamond, 50,000 queries: 130 ms on the warp-per-candidate kernel, 65 ms here.
+template <bool BRANCHY, bool FEAS, bool FORK, bool JOIN>
+__device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned char *smem_raw)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
     // A stream record is (time << q) | low part; the low part is the query index, below the query's
     // branch bits when the records carry them (rb > 0: no stage then looks the bits up).  Keys of batches
     // use the same q, with the index of the batch's first arrival in the low part.
@@ -191,6 +202,7 @@ des_lane_kernel(const __grid_constant__ DesParams p)
     const int lane = threadIdx.x & 31;
     const int kr = p.lane_slots == 16 ? 16 : 32;      // batch ring positions of a lane
     const int S = p.S, cpw = p.cpw, rowlen = p.Bmax | 1;
+    const int L = JOIN ? S + p.n_join : S;            // lanes of a candidate
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem_raw);
     if (sbase != kSmemBase) { atomicCAS(p.status, 0, IL_ERR_CUDA); return; }
     const uint32_t tab0 = sbase + 4u;
@@ -200,7 +212,8 @@ des_lane_kernel(const __grid_constant__ DesParams p)
     const uint32_t xb0 = rings + kLaneWarps * key_bytes(kr);
     const uint32_t xbw = xb0 + (uint32_t)wid * kXBytes, xb = xbw + (uint32_t)lane * 8u;
     const uint32_t nowhere = xb0 + kLaneWarps * kXBytes;
-    const uint32_t qb = nowhere + (uint32_t)kTailBytes + (uint32_t)wid * nq * 128u + (uint32_t)lane * 4u;
+    const uint32_t qb0 = nowhere + (uint32_t)kTailBytes;
+    const uint32_t qb = qb0 + (uint32_t)wid * nq * 128u + (uint32_t)lane * 4u;
     unsigned *missw = reinterpret_cast<unsigned *>(smem_raw + (nowhere - sbase) + 256u + (uint32_t)wid * 128u);   // per group
     const uint32_t rm = (uint32_t)(kr - 1) << 8;      // ring counters epos, lpos, tpos count in bytes of a row
 
@@ -211,8 +224,10 @@ des_lane_kernel(const __grid_constant__ DesParams p)
     for (int k = 0; k < kX; k++) sts64(xb + (uint32_t)k * 256u, kInf);       // lanes without a stage see no record either
     __syncthreads();
 
-    const int j = lane / S, s = lane - j * S;
+    const int j = lane / L, row = lane - j * L;
     const bool lane_used = j < cpw;
+    const bool is_join = JOIN && lane_used && row >= S;      // a lane that merges the incoming streams of a join
+    const int s = JOIN && row >= S ? p.join_stage[row - S] : row;
 
     // static facts of this lane's stage
     int exit_off = 0;
@@ -228,19 +243,50 @@ des_lane_kernel(const __grid_constant__ DesParams p)
     const int cbit_a = p.cbit_a[s], cbit_b = p.cbit_b[s];
     const unsigned cval_a = p.cval_a[s], cval_b = p.cval_b[s];
     const int bit = FORK ? ((cbit_a >= 0 || cbit_b >= 0) ? 0 : -1) : p.bit[s];
-    const uint32_t n_in = lane_used ? (uint32_t)p.n_s[s] : 0u;
-    const unsigned group_mask = lane_used ? (((1u << S) - 1u) << (j * S)) : 0u;
-    const int root_lane = lane_used ? j * S : 0;
-    const bool is_root = s == 0;
+    const uint32_t n_in = lane_used && !is_join ? (uint32_t)p.n_s[s] : 0u;
+    const unsigned group_mask = lane_used ? (((1u << L) - 1u) << (j * L)) : 0u;
+    const int root_lane = lane_used ? j * L : 0;
+    const bool is_root = row == 0;
     // the child's stream on either side; towards the outside (or nowhere) the row of empty records
-    const bool has_a = lane_used && da >= 0, has_b = BRANCHY && lane_used && db >= 0;
-    const uint32_t xa = has_a ? xbw + (uint32_t)(j * S + da) * 8u : nowhere + (uint32_t)lane * 8u;
-    const uint32_t xc = has_b ? xbw + (uint32_t)(j * S + db) * 8u : nowhere + (uint32_t)lane * 8u;
+    const bool join_a = JOIN && da >= 0 && p.join_b[da >= 0 ? da : 0] >= 0, join_b = JOIN && db >= 0 && p.join_b[db >= 0 ? db : 0] >= 0;
+    const bool has_a = lane_used && !is_join && da >= 0 && !join_a, has_b = BRANCHY && lane_used && !is_join && db >= 0 && !join_b;
+    const uint32_t xa = has_a ? xbw + (uint32_t)(j * L + da) * 8u : nowhere + (uint32_t)lane * 8u;
+    const uint32_t xc = has_b ? xbw + (uint32_t)(j * L + db) * 8u : nowhere + (uint32_t)lane * 8u;
     const uint32_t xam = has_a ? (kX - 1) * 256u : 0u, xcm = has_b ? (kX - 1) * 256u : 0u;
     const uint32_t leaving = (uint32_t)p.n - (uint32_t)exit_off;      // slab entries from this stage's region on
     (void)leaving;
 
     const int64_t wslot = (int64_t)blockIdx.x * kLaneWarps + wid;
+    // joins: where a stage's records for a join go (global stream, window and count in shared memory), and where the
+    // join's lane finds them
+    const uint32_t jbase = qb0 + kLaneWarps * nq * 128u + (uint32_t)(wid * cpw * p.n_join) * join_lane_bytes(p.join_window);
+    uint64_t *jg_a = nullptr, *jg_b = nullptr;
+    uint32_t jw_a = nowhere, jw_b = nowhere, seen_cache = nowhere;      // (lanes that are no join's read there, and store nothing)
+    uint32_t *seen = nullptr;
+    (void)jbase;
+    if (JOIN && lane_used) {
+        uint64_t *streams = p.join_ws + (wslot * cpw + j) * p.join_elems;
+        auto window = [&](int t, int side) {
+            return jbase + (uint32_t)(j * p.n_join + p.join_no[t]) * join_lane_bytes(p.join_window) + (uint32_t)side * ((p.join_window + 1u) * 8u);
+        };
+        auto stream = [&](int t, int side) { return streams + (side ? p.join_lane_b[t] : p.join_lane_a[t]); };
+        if (is_join) {
+            jg_a = stream(s, 0); jw_a = window(s, 0);
+            jg_b = stream(s, 1); jw_b = window(s, 1);
+            seen_cache = jw_b + (p.join_window + 1u) * 8u;
+            seen = p.join_seen + ((wslot * cpw + j) * p.n_join + (row - S)) * p.join_seen_words;
+            for (int k = 0; k < 4; k++) sts64(seen_cache + kSeen * 8u + (uint32_t)k * 8u, p.join_both[s][k]);
+        } else {
+            if (join_a) { const int side = p.join_b[da] == s; jg_a = stream(da, side); jw_a = window(da, side); }
+            if (join_b) { const int side = p.join_b[db] == s; jg_b = stream(db, side); jw_b = window(db, side); }
+        }
+    }
+    const uint32_t join_na = is_join ? (uint32_t)p.join_na[s] << 8 : 0u, join_nb = is_join ? (uint32_t)p.join_nb[s] << 8 : 0u;
+    const uint32_t seen_mask = is_join ? kSeen - 1u : 0u, seen_both = is_join ? seen_cache + kSeen * 8u : nowhere;
+    const uint32_t win_mask = (p.join_window - 1u) * 8u, win_reach = (p.join_window - 1u) * 256u;     // (of a window's records, in bytes)
+    const bool join_always = JOIN && !p.any_bits;     // no conditional edges: every query goes down both edges into a join
+    const uint32_t xj = is_join && lane_used ? xbw + (uint32_t)(j * L + s) * 8u : nowhere + (uint32_t)lane * 8u;
+    const uint32_t xjm = is_join && lane_used ? (kX - 1) * 256u : 0u;
     const uint32_t gmask = (uint32_t)((1ull << p.lane_ring_log2) - 1ull);
     uint32_t *spill_ring = reinterpret_cast<uint32_t *>(p.lane_ws) + ((wslot * 32 + lane) << p.lane_ring_log2);
     const unsigned long long n_cand = (unsigned long long)p.n_cand;
@@ -281,8 +327,12 @@ des_lane_kernel(const __grid_constant__ DesParams p)
     uint32_t low = 0, next_idx = 0;
     uint64_t next_key = 0;
     unsigned nb = 0;
+    uint32_t ja = 0, jb = 0;     // joins: records of either incoming stream consumed
+    uint32_t seen_new = 0;       // joins: words of the queries' bits from here on have not been touched
     uint32_t turns = 1, turns_hi = 0;        // iteration bound, in turns
     bool any_spill = false;
+    uint32_t have_a = 0, have_b = 0;         // joins: records of either incoming stream delivered so far
+    (void)have_a; (void)have_b;
     uint64_t late_fin = 0, late_arr = 0;     // feasibility only: finish and arrival record of a query that has just left
     uint32_t miss_local = 0;
 
@@ -304,11 +354,14 @@ des_lane_kernel(const __grid_constant__ DesParams p)
             next_key = lk;
         }
         if (is_root && i + 64u < (uint32_t)p.n) asm volatile("prefetch.global.L1 [%0];" ::"l"(trace + i + 64u));
-        bool attn = !exhausted && (i == n_cur || cap == 0u || --turns == 0u);
+        turns--;
+        bool attn = !exhausted && ((is_join ? ja == join_na && jb == join_nb : i == n_cur || cap == 0u) || turns == 0u);
+        if (JOIN) attn |= !exhausted && !has;
         attn |= i - low > reach || spill;
         if (FEAS) attn |= has && missw[j] > p.miss_allow;
         if (__any_sync(full, attn)) {
         bool done = i == n_cur && bm == ~0u && epos == tpos && !e_act && !(FEAS && late_fin != 0ull);
+        if (is_join && has && !cand_bad) done = ja == join_na && jb == join_nb;
         bool stop = FEAS && has && missw[j] > p.miss_allow;       // this lane ends its group's candidate here
         bool give_up = false;
         if (i - low > reach || spill) {
@@ -335,7 +388,7 @@ des_lane_kernel(const __grid_constant__ DesParams p)
                 stop = true;
             }
         }
-        if (FEAS) stop = (__ballot_sync(full, stop) & group_mask) != 0u;      // decided: the whole group
+        stop = (__ballot_sync(full, stop) & group_mask) != 0u;                // the whole group
         if (p.lane_wrap) {
             const bool group_gives_up = (__ballot_sync(full, give_up) & group_mask) != 0u;
             if (group_gives_up && !over) { over = true; if (has) p.ovf[c] = 1; }
@@ -343,11 +396,12 @@ des_lane_kernel(const __grid_constant__ DesParams p)
         }
         if (stop) {
             n_cur = i; bm = ~0u; epos = tpos; e_act = false; late_fin = 0; cap = 0;
+            ja = join_na; jb = join_nb;
             done = true;
         }
         // The first record of a stream opens a batch on an unused replica, and the last batch is closed by the
         // end of the stream; both once per candidate, so here and not in every iteration.
-        if (!done && cap == 0u) {
+        if (!done && cap == 0u && !is_join) {
             const uint64_t rec = is_root ? rr : lds64_shared(xb);
             if ((int64_t)rec >= 0) {
                 tk = rec | qmask;
@@ -358,7 +412,7 @@ des_lane_kernel(const __grid_constant__ DesParams p)
                 if (is_root) rn = trace[2];
                 cap = rm + 256u;
             }
-        } else if (!done && i == n_cur && bm != ~0u && tpos - epos < cap) {
+        } else if (!done && !is_join && i == n_cur && bm != ~0u && tpos - epos < cap) {
             const uint64_t key = ((tk + (uint64_t)lds32(tab + bm * 4u) * tick) & ~(uint64_t)qmask) | (i - 1u - bm);
             uint32_t pos = tpos;
             for (; pos != lpos; pos -= 256u) {
@@ -401,7 +455,7 @@ des_lane_kernel(const __grid_constant__ DesParams p)
             g = __shfl_sync(full, g, root_lane);
             il_stage_config cfg = {0, 1, 1, 0};
             const bool got = turn && g < n_cand;
-            if (got) cfg = p.configs[g * S + s];
+            if (got && !is_join) cfg = p.configs[g * S + s];
             const bool bad = got && (cfg.hw >= p.H || cfg.max_batch < 1 || cfg.max_batch > p.Bmax ||
                                      cfg.replicas < 1 || cfg.replicas > IL_MAX_REPLICAS);
             const bool grp_bad = (__ballot_sync(full, bad) & group_mask) != 0u;
@@ -414,9 +468,15 @@ des_lane_kernel(const __grid_constant__ DesParams p)
                 uint64_t *slab = FEAS ? nullptr : reinterpret_cast<uint64_t *>(p.slab + (got ? c : 0) * p.slab_stride);
                 if (got && cand_bad) {
                     if (is_root) atomicCAS(p.status, 0, IL_ERR_BAD_CONFIG);
-                    if (!FEAS) for (int k = s; k < p.n; k += S) slab[k] = 0;
+                    if (!FEAS) for (int k = row; k < p.n; k += L) slab[k] = 0;
                 }
                 live = got && !cand_bad && n_in > 0;
+                ja = is_join && got && !cand_bad ? 0u : join_na; jb = is_join && got && !cand_bad ? 0u : join_nb;
+                seen_new = 0u;
+                if (is_join) {
+                    sts32(jw_a, 0u); sts32(jw_b, 0u);
+                    for (int k = 0; k < kSeen; k++) sts64(seen_cache + (uint32_t)k * 8u, kInf);
+                }
                 Rm1 = (cfg.replicas - 1u) << 8;
                 cap = 0;
                 mbm1 = cfg.max_batch - 1u;
@@ -445,6 +505,61 @@ des_lane_kernel(const __grid_constant__ DesParams p)
         any_spill = __any_sync(full, spill);
         }
 
+        // joins: a record for a join.  Records of its two streams are counted in bytes of a row, as tails are.
+        auto deliver = [&](bool c, uint64_t *stream, uint32_t win, uint32_t tail, uint64_t rec) {
+            stg64_if(c && IL_IN_RANGE(stream + (tail >> 8) - p.join_ws, p.join_size, p.status), stream + (tail >> 8), rec);
+            sts64_if(c, win + 8u + ((tail >> 5) & win_mask), rec);
+            sts32_if(c, win, tail + 256u);
+        };
+        // joins: takes the next record of the two incoming streams, if what comes next on both sides is known.
+        // Straight-line code but for a parent that is far ahead and for the first query of a word of bits.
+        // (A parent may add one record to what have_a / have_b say before the next barrier.)
+        auto merge_step = [&]() {
+            uint64_t va = lds64(jw_a + 8u + ((ja >> 5) & win_mask)), vb = lds64(jw_b + 8u + ((jb >> 5) & win_mask));
+            const uint32_t slot = xj | (tail_a & xjm);
+            const bool room = is_join && (int)lds32_shared(slot + 4u) < 0;
+            const bool end_a = ja == join_na, end_b = jb == join_nb;
+            const bool far_a = !end_a && have_a - ja > win_reach, far_b = !end_b && have_b - jb > win_reach;
+            if (far_a || far_b) {
+                // (the lines from here on are complete, so they may come through L1)
+                if (far_a && IL_IN_RANGE(jg_a + (ja >> 8) - p.join_ws, p.join_size, p.status)) va = jg_a[ja >> 8];
+                if (far_a && (ja & 0xf00u) == 0u) asm volatile("prefetch.global.L1 [%0];" ::"l"(jg_a + (ja >> 8) + 32u));
+                if (far_b && IL_IN_RANGE(jg_b + (jb >> 8) - p.join_ws, p.join_size, p.status)) vb = jg_b[jb >> 8];
+                if (far_b && (jb & 0xf00u) == 0u) asm volatile("prefetch.global.L1 [%0];" ::"l"(jg_b + (jb >> 8) + 32u));
+            }
+            const bool known = room && (end_a || have_a != ja) && (end_b || have_b != jb) && !(end_a && end_b);
+            va = end_a ? kInf : va;
+            vb = end_b ? kInf : vb;
+            const bool from_a = (va | qmask) <= (vb | qmask);
+            const uint64_t rec = from_a ? va : vb;
+            const uint32_t low = (uint32_t)rec & qmask, qid = low & imask, w = qid >> 5;
+            bool both = known && join_always;
+            if (!join_always) {
+                uint32_t bits = rb > 0 ? low >> qi : 0u;
+                if (rb == 0 && known && IL_IN_RANGE(qid, p.n, p.status)) bits = p.bits[qid];
+                both = known && ((lds32(seen_both + (bits >> 5) * 4u) >> (bits & 31u)) & 1u);
+            }
+            const uint32_t at = seen_cache + (w & seen_mask) * 8u;
+            uint64_t e = lds64(at);                      // number of the word << 32 | word
+            if (both && (uint32_t)(e >> 32) != w) {
+                // the cache of the queries' bits: queries come in nearly in order, so a word is new when first needed
+                const uint32_t old = (uint32_t)(e >> 32);
+                if (old != ~0u && IL_IN_RANGE(old, p.join_seen_words, p.status)) seen[old] = (uint32_t)e;
+                e = (uint64_t)w << 32;
+                if (w < seen_new && IL_IN_RANGE(w, p.join_seen_words, p.status)) e |= seen[w];
+#pragma unroll 1
+                for (; seen_new < w; seen_new++)         // passed over: it may come later
+                    if (IL_IN_RANGE(seen_new, p.join_seen_words, p.status)) seen[seen_new] = 0u;
+                seen_new = max(seen_new, w + 1u);
+            }
+            const uint32_t mine = 1u << (qid & 31u);
+            sts64_if(both, at, e ^ mine);
+            const bool last_input = known && (!both || ((uint32_t)e & mine) != 0u);
+            sts64_shared_if(last_input, slot, rec);
+            tail_a += last_input ? 256u : 0u;
+            ja += (known && from_a) ? 256u : 0u;
+            jb += (known && !from_a) ? 256u : 0u;
+        };
         auto step = [&](auto spilling) {
             constexpr bool SPILL = decltype(spilling)::value;
             // ---- everything the iteration needs from shared memory
@@ -527,8 +642,12 @@ des_lane_kernel(const __grid_constant__ DesParams p)
                     const bool go_a = da >= 0 && (cbit_a < 0 || ((bits >> cbit_a) & 1u) == cval_a);
                     const bool go_b = db >= 0 && (cbit_b < 0 || ((bits >> cbit_b) & 1u) == cval_b);
                     hand = e_act && (!go_a || free_a) && (!go_b || free_b);
-                    sts64_shared_if(hand && go_a, sa, e_base | qv);
-                    sts64_shared_if(hand && go_b, sc, e_base | qv);
+                    sts64_shared_if(hand && go_a && !join_a, sa, e_base | qv);
+                    sts64_shared_if(hand && go_b && !join_b, sc, e_base | qv);
+                    if (JOIN) {
+                        deliver(hand && go_a && join_a, jg_a, jw_a, tail_a, e_base | qv);
+                        deliver(hand && go_b && join_b, jg_b, jw_b, tail_b, e_base | qv);
+                    }
                     tail_a += (hand && go_a) ? 256u : 0u;
                     tail_b += (hand && go_b) ? 256u : 0u;
                     // this copy leaves: the query's slab entry keeps the latest of its copies
@@ -571,6 +690,13 @@ des_lane_kernel(const __grid_constant__ DesParams p)
             e_base = fetch ? fkey & ~(uint64_t)qmask : e_base;
             epos += fetch ? 256u : 0u;
             e_act = goes_on || fetch;
+            if (JOIN) {
+                __syncwarp();        // what was delivered is there for the joins' lanes
+                have_a = is_join ? lds32(jw_a) : 0u;
+                have_b = is_join ? lds32(jw_b) : 0u;
+                merge_step();        // two records: every query can come from both sides
+                merge_step();
+            }
         };
         if (any_spill) {
 #pragma unroll 1
@@ -595,6 +721,23 @@ des_lane_kernel(const __grid_constant__ DesParams p)
     }
 }
 
+template <bool BRANCHY, bool FEAS, bool FORK = false>
+__global__ void __launch_bounds__(kLaneWarps * 32) des_lane_kernel(const __grid_constant__ DesParams p)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    lane_simulation<BRANCHY, FEAS, FORK, false>(p, smem_raw);
+}
+
+// Pipelines with joins: des_kernel in the lane-parallel form (des_kernel.cu holds the form for times that do not fit
+// a record).
+namespace lanes {
+__global__ void __launch_bounds__(kLaneWarps * 32) des_kernel(const __grid_constant__ DesParams p)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    lane_simulation<true, false, true, true>(p, smem_raw);
+}
+}  // namespace lanes
+
 namespace {
 bool any_branch(const DesParams &p)
 {
@@ -617,6 +760,13 @@ cudaError_t launch_one(const DesParams &p, int grid, size_t smem, cudaStream_t s
 // never combines the two, nor fan-out with spill rings shorter than the longest stream).
 cudaError_t launch_des_lane(const DesParams &p, int grid, size_t smem, cudaStream_t stream)
 {
+    if (p.n_join > 0) {
+        if (p.lane_wrap || p.out_feasible) return cudaErrorInvalidValue;
+        cudaError_t e = cudaFuncSetAttribute(lanes::des_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        lanes::des_kernel<<<grid, kLaneWarps * 32, smem, stream>>>(p);
+        return cudaGetLastError();
+    }
     if (p.fork) {
         if (p.lane_wrap || p.out_feasible) return cudaErrorInvalidValue;
         return launch_one<true, false, true>(p, grid, smem, stream);
@@ -628,10 +778,10 @@ cudaError_t launch_des_lane(const DesParams &p, int grid, size_t smem, cudaStrea
 
 int des_lane_warps_per_cta() { return kLaneWarps; }
 
-size_t des_lane_smem(int table_rows, int Bmax, int ring_slots, int ring_words)
+size_t des_lane_smem(int table_rows, int Bmax, int ring_slots, int ring_words, int cpw, int joins, int window)
 {
     return (kSmemBase + table_bytes(table_rows, Bmax) + key_bytes(ring_slots) - 1) / key_bytes(ring_slots) * key_bytes(ring_slots) -
-           kSmemBase + ring_bytes(ring_slots, ring_words) + kTailBytes;
+           kSmemBase + ring_bytes(ring_slots, ring_words) + kTailBytes + join_bytes(cpw, joins, window);
 }
 
 int des_lane_max_ctas_per_sm(size_t smem)

@@ -108,6 +108,8 @@ constexpr int kLaneCtasPerSm = 4;
 // Words of examined records a lane keeps in shared memory before it spills: this many where the grid needs every
 // resident CTA, more where it leaves shared memory unused.
 constexpr int kLaneWords = 64, kLaneWordsMost = 256;
+// Records of a join's incoming streams kept there, likewise.
+constexpr int kJoinWindow = 64, kJoinWindowMost = 512;
 
 bool use_packed(const il_estimator *e)
 {
@@ -116,7 +118,7 @@ bool use_packed(const il_estimator *e)
 
 int sim_kernel(const il_estimator *e)
 {
-    if (!use_packed(e) || e->join) return kSimWide;     // joins: only the kernel with separate streams merges them
+    if (!use_packed(e)) return kSimWide;
     // fan-out is implemented by the lane kernel and by the kernel with separate streams
     if (e->fork) return (e->variant == IL_VARIANT_AUTO || e->variant == IL_VARIANT_LANES) && e->lane_ok ? kSimLane : kSimWide;
     if (e->variant == IL_VARIANT_LANES && e->lane_ok) return kSimLane;
@@ -150,7 +152,12 @@ size_t slot_time_bytes(const il_estimator *e)
 {
     return is_lane(e) ? (size_t)32 * 4 << e->lane_ring_log2 : (size_t)e->slot_elems * 8;
 }
-size_t slot_qid_bytes(const il_estimator *e) { return is_lane(e) ? 0 : (size_t)e->slot_elems * 4; }
+// joins on the lane kernel: per slot the bits of the queries of which one input has come in, and the incoming streams
+size_t slot_seen_bytes(const il_estimator *e) { return (size_t)e->cpw * e->base.n_join * e->base.join_seen_words * 4; }
+size_t slot_qid_bytes(const il_estimator *e)
+{
+    return is_lane(e) ? slot_seen_bytes(e) + (size_t)e->cpw * e->base.join_elems * 8 : (size_t)e->slot_elems * 4;
+}
 size_t slot_bytes(const il_estimator *e) { return slot_time_bytes(e) + slot_qid_bytes(e); }
 size_t cand_bytes(const il_estimator *e) { return (size_t)e->n_pad * 8 + 5; }   // slab row, order entry, overflow mark
 bool lane_fallback(const il_estimator *e) { return is_lane(e) && e->lane_wrap; }
@@ -440,6 +447,12 @@ static DesParams chunk_params(const il_estimator *e, const Plan &pl, char *ws, c
     p.iter_limit = e->iter_limit;
     p.lane_slots = e->lane_slots;
     p.cpw = (int32_t)pl.cps;
+    if (e->join) {
+        const size_t seen = ((size_t)pl.slots * slot_seen_bytes(e) + 7) / 8 * 8;
+        p.join_seen = reinterpret_cast<uint32_t *>(ws + pl.off_qid);
+        p.join_ws = reinterpret_cast<uint64_t *>(ws + pl.off_qid + seen);
+        p.join_size = pl.slots * e->cpw * e->base.join_elems;
+    }
     return p;
 }
 
@@ -464,11 +477,13 @@ static int choose_lane_slots(il_estimator *e, const il_stage_config *d_configs, 
 static cudaError_t launch_lane(const il_estimator *e, DesParams p, int64_t ctas, cudaStream_t st)
 {
     const size_t per_sm = (size_t)((ctas + e->num_sms - 1) / e->num_sms);
-    int words = kLaneWordsMost;
-    while (words > kLaneWords && ((des_lane_smem(e->S * e->H, e->Bmax, e->lane_slots, words) + 1024) * per_sm > e->smem_per_sm ||
-                                  des_lane_smem(e->S * e->H, e->Bmax, e->lane_slots, words) > e->smem_per_cta)) words >>= 1;
-    p.lane_words = words;
-    return launch_des_lane(p, (int)ctas, des_lane_smem(e->S * e->H, e->Bmax, e->lane_slots, words), st);
+    p.lane_words = kLaneWordsMost;
+    p.join_window = kJoinWindowMost;
+    auto smem = [&] { return des_lane_smem(e->S * e->H, e->Bmax, e->lane_slots, p.lane_words, p.cpw, p.n_join, p.join_window); };
+    auto fits = [&] { return smem() <= e->smem_per_cta && (smem() + 1024) * per_sm <= e->smem_per_sm; };
+    while (!fits() && p.n_join > 0 && p.join_window > kJoinWindow) p.join_window >>= 1;
+    while (!fits() && p.lane_words > kLaneWords) p.lane_words >>= 1;
+    return launch_des_lane(p, (int)ctas, smem(), st);
 }
 
 // Enqueues the simulation of one chunk whose work counter is zero: the kernel the handle uses
@@ -955,7 +970,32 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
         }
     }
     for (int s = 0; s < S; s++) bp.n_s[s] = (int32_t)e->visits[s];
-    e->cpw = 32 / S;
+    bp.n_join = 0;
+    bp.any_bits = any_cond ? 1 : 0;
+    bp.join_elems = 0;
+    if (e->join) {
+        // lane kernel: which queries follow both edges into a join is a function of their branch bits
+        bp.join_seen_words = (int32_t)((n + 31) / 32);
+        for (int c = 1; c < S; c++) {
+            if (bp.join_b[c] < 0) continue;
+            bp.join_no[c] = (int8_t)bp.n_join;
+            bp.join_stage[bp.n_join++] = (int8_t)c;
+            bp.join_lane_a[c] = bp.join_elems; bp.join_elems += edge_a[c];
+            bp.join_lane_b[c] = bp.join_elems; bp.join_elems += edge_b[c];
+        }
+        for (unsigned bits = 0; bits < 256; bits++) {
+            bool reach[IL_MAX_STAGES] = {};
+            reach[0] = true;
+            for (int c = 1; c < S; c++) {
+                const bool a = reach[pr->parent[c]] && (pr->cond_bit[c] < 0 || ((bits >> pr->cond_bit[c]) & 1u) == pr->cond_val[c]);
+                const bool b = bp.join_b[c] >= 0 && reach[jn->parent2[c]] &&
+                               (jn->cond_bit2[c] < 0 || ((bits >> jn->cond_bit2[c]) & 1u) == jn->cond_val2[c]);
+                reach[c] = a || b;
+                if (a && b) bp.join_both[c][bits >> 6] |= 1ull << (bits & 63u);
+            }
+        }
+    }
+    e->cpw = std::max(1, 32 / (S + bp.n_join));
     configure_lane_rings(e);
     bp.S = S; bp.H = H; bp.Bmax = B; bp.n = (int32_t)n;
     e->smem = (size_t)S * H * B * sizeof(int32_t);
@@ -969,7 +1009,7 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
     IL_CUDA_E(cudaMalloc(&e->d_arrival, (size_t)n * 8));
     IL_CUDA_E(cudaMalloc(&e->d_bits, (size_t)n));
     e->can_pack = can_pack;
-    e->lane_ok = can_pack && !e->join;
+    e->lane_ok = can_pack && (!e->join || n < (INT64_C(1) << 24));     // (a join counts its records in 24 bits)
     bp.qbits = qbits;
     if (can_pack) {
         // padded with "never" records to whole tiles, so that bulk copies always move full tiles
@@ -984,8 +1024,11 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
         // kernel then routes a query by the record it hands on instead of looking its bits up.
         int nb = 0;
         for (int s = 0; s < pr->n_stages; s++)
+        {
             if (pr->cond_bit[s] >= 0) nb = std::max(nb, (int)pr->cond_bit[s] + 1);
-        if (nb > 0 && tr->branch_bits && !e->join && qbits + nb <= 31 &&
+            if (jn && jn->parent2[s] >= 0 && jn->cond_bit2[s] >= 0) nb = std::max(nb, (int)jn->cond_bit2[s] + 1);
+        }
+        if (nb > 0 && tr->branch_bits && qbits + nb <= 31 &&
             tr->arrival_us[n - 1] + worst < (INT64_C(1) << (63 - qbits - nb))) {
             for (int64_t i = 0; i < n; i++)
                 packed[(size_t)i] = ((uint64_t)tr->arrival_us[i] << (qbits + nb)) |
@@ -1016,7 +1059,7 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
     e->ctas_per_sm_packed = des_packed_max_ctas_per_sm(false, e->smem);
     e->ctas_per_sm_staged = des_packed_max_ctas_per_sm(true, e->smem);
     for (int k = 0; k < 2; k++) {
-        e->ctas_lane[k] = des_lane_max_ctas_per_sm(des_lane_smem(S * H, B, k == 0 ? 16 : 32, kLaneWords));
+        e->ctas_lane[k] = des_lane_max_ctas_per_sm(des_lane_smem(S * H, B, k == 0 ? 16 : 32, kLaneWords, e->cpw, e->base.n_join, kJoinWindow));
     }
     e->ctas_per_sm_lane = std::min(e->ctas_lane[1], kLaneCtasPerSm);
     if (e->ctas_per_sm_wide < 1 || e->ctas_per_sm_packed < 1 || e->ctas_per_sm_staged < 1 ||
@@ -1091,7 +1134,7 @@ const char *il_kernel_name(const il_estimator *e)
 {
     if (!e) return "";
     switch (sim_kernel(e)) {
-    case kSimLane: return "des_lane_kernel";
+    case kSimLane: return e->join ? "des_kernel" : "des_lane_kernel";      // (lanes::des_kernel)
     case kSimPacked: return "des_packed_kernel";
     case kSimPackedStaged: return "des_packed_kernel<staged>";
     default: return "des_kernel";

@@ -80,6 +80,17 @@ struct DesParams {
     int32_t lane_ring_log2;       // a lane's spill ring in lane_ws holds 2^this words
     int32_t lane_words;           // words of examined records a lane keeps in shared memory (a power of two)
     int32_t lane_wrap;            // the rings are shorter than the longest stream
+    // lane kernel, joins: join_stage[0 .. n_join) are the stages with two incoming edges, join_no[s] their number
+    int32_t n_join;
+    int8_t  join_stage[IL_MAX_STAGES], join_no[IL_MAX_STAGES];
+    uint64_t join_both[IL_MAX_STAGES][4];    // bit b: a query with branch bits b follows both incoming edges of the stage
+    uint64_t *join_ws;            // [warp slots][cpw][join_elems] incoming streams of the joins, stage s's at
+    int64_t join_lane_a[IL_MAX_STAGES], join_lane_b[IL_MAX_STAGES];
+    int64_t join_elems, join_size;           // records per candidate; and in all of join_ws
+    uint32_t *join_seen;          // [warp slots][cpw][n_join][join_seen_words]: one input of this query has come in
+    int32_t join_seen_words;
+    int32_t join_window;          // records of an incoming stream kept in shared memory (a power of two)
+    int32_t any_bits;             // some edge is conditional
     uint8_t *ovf;                 // [n_cand] set to 1 for a candidate given up on ring overflow (lane_wrap only)
     // lane kernel, feasibility only: set out_feasible to select that instantiation
     uint8_t *out_feasible;        // [n_cand] 1: P99 <= slo_us, 0: not, 2: given up on ring overflow (see ovf)
@@ -129,8 +140,9 @@ int trace_tile_records();     // the packed trace is padded to a multiple of thi
 // lane-parallel kernel: one lane per (candidate, stage); smem from des_lane_smem
 cudaError_t launch_des_lane(const DesParams &p, int grid, size_t smem, cudaStream_t stream);
 int des_lane_warps_per_cta();
-// ring_slots: 16 or 32 batch ring positions per lane; ring_words: words of examined records (a power of two)
-size_t des_lane_smem(int table_rows, int Bmax, int ring_slots, int ring_words);
+// ring_slots: 16 or 32 batch ring positions per lane; ring_words: words of examined records (a power of two);
+// cpw candidates per warp with so many joins each, whose streams keep `window` records
+size_t des_lane_smem(int table_rows, int Bmax, int ring_slots, int ring_words, int cpw, int joins, int window);
 int des_lane_max_ctas_per_sm(size_t smem);
 enum SimKernel { kSimWide = 0, kSimPacked = 1, kSimPackedStaged = 2, kSimLane = 3 };
 inline cudaError_t launch_simulation(const DesParams &p, int kernel, int grid, size_t smem,

@@ -61,3 +61,21 @@ def test_more_candidates_than_resident_groups(oracle, S):
         est.set_test_knob(3, 2)
         a, _ = est.estimate_device(torch.from_numpy(w.configs).cuda(), w.slo_us)
     assert np.array_equal(a.cpu().numpy(), exp[0][np.arange(w.n_candidates) % 5_000])
+
+
+@pytest.mark.parametrize("slow", [1, 2])
+@pytest.mark.parametrize("shape", ["diamond", "guarded", "two_joins", "skip"])
+def test_joins_with_one_slow_input(oracle, shape, slow):
+    """One of two branches falls behind the other by hundreds to thousands of queries: more than a join keeps in
+    shared memory of its incoming streams, and of its queries' bits."""
+    import torch
+    import paper_1812_01776_b200 as il
+    w = workloads.join_small(slow, n=6000, C=40, max_replicas=4, Bmax=8, shape=shape)
+    if shape == "skip" and slow == 2:
+        slow = 1                                  # (the other input there comes straight from stage 0)
+    w.configs[:20, slow] = (0, 1, 1, 0)
+    w.latency_us[slow, 0, 0] = 9000               # 110 a second of 300
+    exp = oracle.estimate_workload(w)
+    with il.Estimator.from_workload(w) as est:
+        a, b = est.estimate_device(torch.from_numpy(w.configs).cuda(), w.slo_us)
+        assert np.array_equal(a.cpu().numpy(), exp[0]) and np.array_equal(b.cpu().numpy(), exp[1])
