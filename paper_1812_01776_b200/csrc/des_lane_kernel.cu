@@ -54,6 +54,8 @@
 //     whose distance outgrows that ring as well gives its candidate up (marked in
 //     the overflow array; the host's fallback evaluates it with the
 //     warp-per-candidate kernel).
+//   * A root's records are copied to shared memory two turns of kTurn iterations
+//     before their use (cp.async, all lanes of the group).
 //   * The profile tables are shared by the CTA, rows padded to an odd length so
 //     that rows of different lanes start in different banks.
 //   * What happens once per candidate or rarely (its first and last batch, spills,
@@ -61,25 +63,15 @@
 //     iteration only, behind one vote.
 //
 // Measured on B200 against the version whose streams lay in global memory (three
-// gathers of 8 bytes per lane and iteration through L1, 208 instructions): 144
-// instructions per iteration and 155 instead of 290 ns for a warp on its own;
-// 4,096 candidates x 4 stages x 50,000 queries 15.4 -> 8.6 ms, 4,096 x 10 x 10^6
-// 720 -> 476 ms.  With two or three warps per scheduler the ALU pipe (compares,
-// selects and logic, half the issue rate) is what bounds it.
-//
-// Scheduling.  The groups of a warp are independent: when the lanes of a group
-// have finished their candidate (looked at every eighth iteration), the group
-// takes the next one from a global work counter.  In the feasibility-only
-// instantiation (Section 4.3, "Feasible") the leaves compare each leaving query
-// with the objective instead of writing it to the slab, and a group drops its
-// candidate as soon as more queries have missed the objective than the P99 rule
-// allows.
-//
-// Records and keys are packed 64-bit words: (time << q) | low part for records,
-// (finish << q) | index of the batch's first record for batches, whose unsigned
-// order is (finish, dispatch order).  q is at most 31, so the low part lies in
-// the low 32-bit word.  The host selects this kernel only when every reachable
-// time fits.
+// gathers of 8 bytes per lane and iteration through L1, 208 instructions): about
+// 120 instructions per iteration and 120 instead of 290 ns for a warp on its own;
+// 4,096 candidates x 4 stages x 50,000 queries 15.4 -> 6.7 ms, 4,096 x 10 x 10^6
+// 720 -> 367 ms.  With two or three warps per scheduler the ALU pipe (compares,
+// selects and logic, half the issue rate) is what bounds it.  What took the loop
+// from 155 to 120 ns: the trace copied ahead of its use by all lanes of a group
+// (8 instructions less, no stall on the load), the word to hand on loaded an
+// iteration early, comparisons as doubles, one counter per lane for the records
+// it passes on.
 #include "il_internal.h"
 
 #include <type_traits>
@@ -90,8 +82,10 @@ namespace {
 
 constexpr int kLaneWarps = 4;                 // warps per CTA: one per scheduler even in a grid of few CTAs
 constexpr uint64_t kInf = ~0ull;
+constexpr uint64_t kLatest = 0x7fefffffffffffffull;      // no record or key is larger
 constexpr int kX = 4;                         // records of a stream between two stages
 constexpr uint32_t kLast = 0x80000000u;       // flag of a batch's last record in that ring
+constexpr int kAhead = 32;                    // records of the trace a root has before it: two turns, a power of two
 constexpr int kTurn = 16;                     // iterations between two looks at finished groups, spills, bounds (8: 5 % slower)
 
 __device__ __forceinline__ uint64_t lds64(uint32_t a)
@@ -106,6 +100,12 @@ __device__ __forceinline__ uint32_t lds32(uint32_t a)
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
     return v;
 }
+// Order of two records or keys.  Words below 0x7ff0... order the same as the doubles of their bits, and a double
+// is compared by one instruction on a pipe that is idle otherwise, where a 64-bit integer takes two on the ALU pipe
+// (5 % of a launch with three warps per scheduler).  A word with the sign or all exponent bits set compares as false.
+__device__ __forceinline__ bool before(uint64_t a, uint64_t b) { return __longlong_as_double((long long)a) < __longlong_as_double((long long)b); }
+__device__ __forceinline__ bool not_after(uint64_t a, uint64_t b) { return __longlong_as_double((long long)a) <= __longlong_as_double((long long)b); }
+
 // Words that two lanes share (stream records): each is complete in itself, so no ordering between words is needed.
 __device__ __forceinline__ uint64_t lds64_shared(uint32_t a)
 {
@@ -130,7 +130,7 @@ __device__ __forceinline__ void sts32_shared_if(bool c, uint32_t a, uint32_t v)
 __device__ __forceinline__ void sts64(uint32_t a, uint64_t v) { asm volatile("st.shared.u64 [%0], %1;" ::"r"(a), "l"(v) : "memory"); }
 __device__ __forceinline__ void sts32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
 
-// The same under a predicate, and a predicated load that leaves its destination alone otherwise: a lane's steps
+// The same under a predicate: a lane's steps
 // are straight-line code (a branch costs the warp more than the few instructions it would skip).
 __device__ __forceinline__ void sts64_if(bool c, uint32_t a, uint64_t v)
 {
@@ -148,20 +148,26 @@ __device__ __forceinline__ void stg64_if(bool c, uint64_t *a, uint64_t v)
 {
     asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p st.global.u64 [%1], %2; }" ::"r"((uint32_t)c), "l"(a), "l"(v) : "memory");
 }
-__device__ __forceinline__ void ldg64_if(bool c, const uint64_t *a, uint64_t &v)
+// 8 bytes from global to shared memory, asynchronously
+__device__ __forceinline__ void copy8(uint32_t dst, const uint64_t *src)
 {
-    asm volatile("{ .reg .pred p; setp.ne.u32 p, %1, 0; @p ld.global.nc.u64 %0, [%2]; }" : "+l"(v) : "r"((uint32_t)c), "l"(a));
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
 }
+__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Shared memory of a CTA: the tables ([S * H] rows of Bmax | 1 words, one word in front of them), then per warp
 // the batch keys [kr][lane] (aligned to their size: a ring address is (counter & mask) | base), per warp the
 // streams [kX][lane], a row of empty records (the "child" of a leaf), per warp the miss counts of the groups
-// (feasibility only), and per warp the words of examined records [nq][lane].
+// (feasibility only), per warp the words of examined records [nq][lane], and per warp the next records of the trace
+// [kAhead][group].
 constexpr uint32_t kSmemBase = 1024;          // where a CTA's dynamic shared memory starts (checked by the kernel)
 __host__ __device__ inline uint32_t key_bytes(int kr) { return (uint32_t)kr * 256u; }
 constexpr uint32_t kXBytes = kX * 256u;
 __host__ __device__ inline size_t table_bytes(int rows, int Bmax) { return ((size_t)rows * (Bmax | 1) + 1) * 4; }
-__host__ __device__ inline size_t ring_bytes(int kr, int nq) { return (size_t)kLaneWarps * (key_bytes(kr) + nq * 128u + kXBytes); }
+__host__ __device__ inline size_t ring_bytes(int kr, int nq, int cpw)
+{
+    return (size_t)kLaneWarps * (key_bytes(kr) + nq * 128u + kXBytes + (size_t)kAhead * cpw * 8);
+}
 constexpr size_t kTailBytes = 256 + kLaneWarps * 128;
 constexpr int kSeen = 64;                     // joins: words of the queries' bits that are kept in shared memory
 // joins: per warp and per (group, join) the counts and the windows of the two incoming streams, then the cached words
@@ -214,6 +220,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
     const uint32_t nowhere = xb0 + kLaneWarps * kXBytes;
     const uint32_t qb0 = nowhere + (uint32_t)kTailBytes;
     const uint32_t qb = qb0 + (uint32_t)wid * nq * 128u + (uint32_t)lane * 4u;
+    const uint32_t tb0 = qb0 + kLaneWarps * nq * 128u;        // per warp the next records of the trace, [kAhead][group]
     unsigned *missw = reinterpret_cast<unsigned *>(smem_raw + (nowhere - sbase) + 256u + (uint32_t)wid * 128u);   // per group
     const uint32_t rm = (uint32_t)(kr - 1) << 8;      // ring counters epos, lpos, tpos count in bytes of a row
 
@@ -239,27 +246,36 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
         exit_off += p.n_s[u] - kids;
     }
     const int da = FORK ? p.child_a[s] : p.dest_a[s], db = FORK ? p.child_b[s] : p.dest_b[s];
-    // fan-out: the guard of either edge; the branch bits are needed if one of them is conditional
-    const int cbit_a = p.cbit_a[s], cbit_b = p.cbit_b[s];
-    const unsigned cval_a = p.cval_a[s], cval_b = p.cval_b[s];
-    const int bit = FORK ? ((cbit_a >= 0 || cbit_b >= 0) ? 0 : -1) : p.bit[s];
+    // (with fan-out the branch bits are needed if one of the edges is conditional)
+    const int bit = FORK ? ((p.cbit_a[s] >= 0 || p.cbit_b[s] >= 0) ? 0 : -1) : p.bit[s];
+    // Routing by the bits of a record's low part: without fan-out to side b if (bits & mask_b), with fan-out down
+    // either edge if (bits & mask) == want.
+    auto bit_at = [&](int b) { return b >= 0 ? 1u << (rb > 0 ? qi + b : b) : 0u; };      // (rb = 0: bits looked up)
+    const uint32_t mask_a = FORK && da >= 0 ? bit_at(p.cbit_a[s]) : 0u;
+    const uint32_t mask_b = FORK ? (db >= 0 ? bit_at(p.cbit_b[s]) : 0u) : bit_at(p.bit[s]);
+    const uint32_t want_a = da < 0 ? ~0u : (p.cval_a[s] ? mask_a : 0u), want_b = db < 0 ? ~0u : (p.cval_b[s] ? mask_b : 0u);
     const uint32_t n_in = lane_used && !is_join ? (uint32_t)p.n_s[s] : 0u;
     const unsigned group_mask = lane_used ? (((1u << L) - 1u) << (j * L)) : 0u;
     const int root_lane = lane_used ? j * L : 0;
     const bool is_root = row == 0;
+    // arrival stream: the lane's ring, for a root the group's stretch of the trace
+    const uint32_t tb = tb0 + (uint32_t)(wid * kAhead * cpw + (lane_used ? j : 0)) * 8u;
+    const bool from_trace = is_root && lane_used;
+    const uint32_t xin = from_trace ? tb : xb, xin_mask = from_trace ? kAhead - 1u : kX - 1u, xin_row = from_trace ? (uint32_t)cpw * 8u : 256u;
     // the child's stream on either side; towards the outside (or nowhere) the row of empty records
     const bool join_a = JOIN && da >= 0 && p.join_b[da >= 0 ? da : 0] >= 0, join_b = JOIN && db >= 0 && p.join_b[db >= 0 ? db : 0] >= 0;
     const bool has_a = lane_used && !is_join && da >= 0 && !join_a, has_b = BRANCHY && lane_used && !is_join && db >= 0 && !join_b;
     const uint32_t xa = has_a ? xbw + (uint32_t)(j * L + da) * 8u : nowhere + (uint32_t)lane * 8u;
     const uint32_t xc = has_b ? xbw + (uint32_t)(j * L + db) * 8u : nowhere + (uint32_t)lane * 8u;
     const uint32_t xam = has_a ? (kX - 1) * 256u : 0u, xcm = has_b ? (kX - 1) * 256u : 0u;
+    const uint32_t tail_step = da >= 0 ? 256u : 8u;
     const uint32_t leaving = (uint32_t)p.n - (uint32_t)exit_off;      // slab entries from this stage's region on
     (void)leaving;
 
     const int64_t wslot = (int64_t)blockIdx.x * kLaneWarps + wid;
     // joins: where a stage's records for a join go (global stream, window and count in shared memory), and where the
     // join's lane finds them
-    const uint32_t jbase = qb0 + kLaneWarps * nq * 128u + (uint32_t)(wid * cpw * p.n_join) * join_lane_bytes(p.join_window);
+    const uint32_t jbase = tb0 + (uint32_t)(kLaneWarps * kAhead * cpw) * 8u + (uint32_t)(wid * cpw * p.n_join) * join_lane_bytes(p.join_window);
     uint64_t *jg_a = nullptr, *jg_b = nullptr;
     uint32_t jw_a = nowhere, jw_b = nowhere, seen_cache = nowhere;      // (lanes that are no join's read there, and store nothing)
     uint32_t *seen = nullptr;
@@ -304,6 +320,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
     bool exhausted = !lane_used; // the group will get no further candidate
     bool live = false, cand_bad = false, over = false;
     uint32_t Rm1 = 0;            // replicas less one, in bytes of a ring row
+    uint32_t kfb = nowhere, kfm = 0;         // where the first batch in use is looked up (one replica: kInf, which compares as later)
     uint32_t cap = 0;            // positions of the batch ring the lane may fill; 0 until its first record has opened a batch
     uint32_t mbm1 = 0;
     uint32_t tab = tab0;         // the lane's row of the tables
@@ -317,10 +334,11 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
     uint32_t tpos_seen = 0;      // tpos when batches were last counted
     uint32_t prev = 0;           // low part of record i - 1, with its flag
     bool e_act = false;          // a batch is being handed on:
-    uint64_t e_base = 0;         //   its finish << q
+    uint64_t e_key = 0;          //   its key
     uint32_t e_idx = 0;          //   the record to hand on next
     uint32_t tail_a = 0, tail_b = 0;         // records handed to the children, in bytes of a row
-    uint64_t rr = kInf, rn = kInf;           // root: records i and i + 1 of the trace
+    uint32_t fed = 0;            // records of the trace requested for the group's root
+    uint32_t qv = 0;             // low part of the record to hand on (where there is one)
     bool spill = false;
     // No record before low_idx is needed any more once every batch up to low_key has been handed on (next_*: the
     // same for a later moment)
@@ -353,7 +371,8 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
             next_idx = i - (bm + 1u);
             next_key = lk;
         }
-        if (is_root && i + 64u < (uint32_t)p.n) asm volatile("prefetch.global.L1 [%0];" ::"l"(trace + i + 64u));
+        copies_done();
+        __syncwarp();
         turns--;
         bool attn = !exhausted && ((is_join ? ja == join_na && jb == join_nb : i == n_cur || cap == 0u) || turns == 0u);
         if (JOIN) attn |= !exhausted && !has;
@@ -402,14 +421,12 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
         // The first record of a stream opens a batch on an unused replica, and the last batch is closed by the
         // end of the stream; both once per candidate, so here and not in every iteration.
         if (!done && cap == 0u && !is_join) {
-            const uint64_t rec = is_root ? rr : lds64_shared(xb);
+            const uint64_t rec = lds64_shared(xin);
             if ((int64_t)rec >= 0) {
                 tk = rec | qmask;
                 bm = 0; i = 1;
                 prev = (uint32_t)rec & qmask;
-                sts32_shared_if(true, xb + 4u, ~0u);
-                rr = rn;
-                if (is_root) rn = trace[2];
+                sts32_shared_if(true, xin + 4u, ~0u);
                 cap = rm + 256u;
             }
         } else if (!done && !is_join && i == n_cur && bm != ~0u && tpos - epos < cap) {
@@ -423,7 +440,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
             sts64(kb | (pos & rm), key);
             tpos += 256u;
             bm = ~0u;
-            tk = kInf;          // nothing more will be dispatched: every batch may leave
+            tk = kLatest;       // nothing more will be dispatched: every batch may leave
             prev |= kLast;
             sts32(qb + (((i - 1u) & (nq - 1u)) << 7), prev);
             if (spill && IL_IN_RANGE((i - 1u) & gmask, gmask + 1ull, p.status)) spill_ring[(i - 1u) & gmask] = prev;
@@ -440,7 +457,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
                 const bool decided = FEAS && missw[j] > p.miss_allow;
                 // every query of a candidate that ran to its end must have left through exactly one
                 // leaf (checked over all candidates of the warp when the kernel ends)
-                if (live && !over && !decided && (BRANCHY || da < 0)) exits_seen += n_left;
+                if (live && !over && !decided) exits_seen += BRANCHY ? n_left : da < 0 ? tail_a >> 3 : 0u;
                 if (is_root && !cand_bad && !over && !decided)
                     exits_due += FORK ? (unsigned long long)p.total_leaving : (unsigned long long)(unsigned)p.n;
                 if (FEAS && is_root) {
@@ -478,6 +495,8 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
                     for (int k = 0; k < kSeen; k++) sts64(seen_cache + (uint32_t)k * 8u, kInf);
                 }
                 Rm1 = (cfg.replicas - 1u) << 8;
+                kfb = Rm1 != 0u ? kb : nowhere + (uint32_t)lane * 8u;
+                kfm = Rm1 != 0u ? rm : 0u;
                 cap = 0;
                 mbm1 = cfg.max_batch - 1u;
                 tab = tab0 + (uint32_t)((live ? s * p.H + cfg.hw : 0) * rowlen) * 4u;
@@ -496,13 +515,21 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
                 nb = 0;
                 turns = (uint32_t)limit; turns_hi = (uint32_t)(limit >> 32);
                 late_fin = 0;
-                rr = kInf; rn = kInf;
-                if (is_root && live) { rr = trace[0]; rn = trace[1]; }      // (two records of padding at the end)
+                fed = 0u;
+                if (is_root) for (int k = 0; k < kAhead; k++) sts64(tb + (uint32_t)(k * cpw) * 8u, kInf);
             }
             __syncwarp();     // the rings are empty before anybody looks
             if (__all_sync(full, exhausted)) break;
         }
         any_spill = __any_sync(full, spill);
+        }
+
+        // The root's next records: requested two turns before their use, by all lanes of the group.
+        {
+            const uint32_t at = __shfl_sync(full, i, root_lane);
+            const uint32_t to = has && !cand_bad ? min(at + (uint32_t)kAhead, (uint32_t)p.n) : 0u;
+            for (uint32_t k = fed + (uint32_t)row; k < to; k += (uint32_t)L) copy8(tb + (k & (kAhead - 1u)) * (uint32_t)cpw * 8u, trace + k);
+            fed = max(fed, to);
         }
 
         // joins: a record for a join.  Records of its two streams are counted in bytes of a row, as tails are.
@@ -563,39 +590,43 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
         auto step = [&](auto spilling) {
             constexpr bool SPILL = decltype(spilling)::value;
             // ---- everything the iteration needs from shared memory
-            const uint32_t xs = xb + ((i & (kX - 1)) << 8);
-            const uint64_t x = lds64_shared(xs);
+            const uint32_t xs = xin + (i & xin_mask) * xin_row;
+            const uint64_t rec = lds64_shared(xs);                    // record to examine
             const uint32_t lat = lds32(tab + bm * 4u);                // time of the open batch
-            const uint64_t kf = lds64(kb | (lpos & rm));              // first batch in use (if there is one)
+            const uint64_t kf = lds64(kfb | (lpos & kfm));            // first batch in use (one replica: kInf)
             const uint64_t k1 = lds64(kb | ((tpos - 256u) & rm)), k2 = lds64(kb | ((tpos - 512u) & rm));    // the last two batches
             const uint64_t fkey = lds64(kb | (epos & rm));            // first batch not handed on (if there is one)
-            uint32_t qv = lds32(qb + ((e_idx & (nq - 1u)) << 7));      // record to hand on
             const uint32_t sa = xa | (tail_a & xam), sc = xc | (tail_b & xcm);
-            const bool free_a = (int)lds32_shared(sa + 4u) < 0;
-            const bool free_b = BRANCHY && (int)lds32_shared(sc + 4u) < 0;
-            const bool far = i - e_idx > nq;                // (only where the lane spills)
-            const uint64_t rec = is_root ? rr : x;
-            const bool f_ok = epos != tpos && fkey <= tk;
+            // where the record in hand goes, and whether there is room: towards the outside always
+            uint32_t bits = 0;
+            if (BRANCHY && rb == 0 && e_act && bit >= 0 && IL_IN_RANGE(qv & imask, p.n, p.status)) bits = p.bits[qv & imask];
+            else if (BRANCHY) bits = qv;
+            const bool to_b = BRANCHY && !FORK && (bits & mask_b) != 0u;
+            const bool go_a = FORK && (bits & mask_a) == want_a, go_b = FORK && (bits & mask_b) == want_b;
+            const uint32_t sd = to_b ? sc : sa;
+            const bool free_d = (int)lds32_shared(sd + 4u) < 0;
+            const bool free_b = FORK && (int)lds32_shared(sc + 4u) < 0;
+            const bool f_ok = epos != tpos && not_after(fkey, tk);
 
             // ---- examine record i, if it is there: it joins the open batch, or the open batch is closed and it
             // opens the next one
             const bool taken = (int64_t)rec >= 0 && tpos - epos < cap;
-            const bool join = taken && bm < mbm1 && rec <= tk;
-            const bool open = taken && !(bm < mbm1 && rec <= tk);
+            const bool joins = bm < mbm1 && not_after(rec, tk);
+            const bool join = taken && joins, open = taken && !joins;
             const uint64_t key = ((tk + (uint64_t)lat * tick) & ~(uint64_t)qmask) | (i - 1u - bm);
             // the next batch goes to a replica never used so far (free from time 0), else to the one that is
             // free first -- maybe the one whose batch is closed just now
             const uint32_t in_use = tpos - lpos;
             const bool pop = in_use == Rm1;
-            const uint64_t first = (in_use == 0u || key < kf) ? key : kf;
-            const uint64_t start = ((pop && first > rec) ? first : rec) | qmask;
+            const uint64_t first = before(kf, key) ? kf : key;
+            const uint64_t start = ((pop && before(rec, first)) ? first : rec) | qmask;
             // its place in the ring: behind the last one, nearly always, or just before it (a batch that finishes
             // before one dispatched earlier); further ahead is rare enough for a loop
             const uint32_t at0 = kb | (tpos & rm), at1 = kb | ((tpos - 256u) & rm);
-            const bool overtakes = key < k1;
-            sts64_if(open, at0, overtakes ? k1 : key);
-            sts64_if(open && overtakes, at1, key);
-            if (open && overtakes && key < k2) {
+            const bool overtakes = before(key, k1);
+            sts64_if(open, overtakes ? at1 : at0, key);
+            sts64_if(open && overtakes, at0, k1);
+            if (open && overtakes && before(key, k2)) {
                 uint32_t pos = tpos - 256u;
                 for (;;) {       // four at a time: the loads overlap, and most of the time one round does it
                     const uint32_t left = pos - lpos;
@@ -621,27 +652,20 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
             sts32_shared_if(taken, xs + 4u, ~0u);
             if (SPILL) {
                 stg32_if(spill && taken && IL_IN_RANGE((i - 1u) & gmask, gmask + 1ull, p.status), spill_ring + ((i - 1u) & gmask), word);
-                if (spill && far && IL_IN_RANGE(e_idx & gmask, gmask + 1ull, p.status)) qv = __ldcg(spill_ring + (e_idx & gmask));
             }
             prev = taken ? (uint32_t)rec & qmask : prev;
             i += taken ? 1u : 0u;
-            rr = taken ? rn : rr;
-            ldg64_if(taken && is_root, trace + (i + 1u), rn);
 
             // ---- hand on
             if (FEAS) miss_local += (late_fin > late_arr + slo_q) ? 1u : 0u;
             const bool last = (int)qv < 0;
+            const uint64_t e_base = e_key & ~(uint64_t)qmask;         // finish << q
             qv &= ~kLast;
             const uint32_t qid = BRANCHY ? qv & imask : qv;
             bool hand;
             if (BRANCHY) {
-                uint32_t bits = 0;
-                if (rb > 0) bits = qv >> qi;
-                else if (e_act && bit >= 0 && IL_IN_RANGE(qid, p.n, p.status)) bits = p.bits[qid];
                 if (FORK) {
-                    const bool go_a = da >= 0 && (cbit_a < 0 || ((bits >> cbit_a) & 1u) == cval_a);
-                    const bool go_b = db >= 0 && (cbit_b < 0 || ((bits >> cbit_b) & 1u) == cval_b);
-                    hand = e_act && (!go_a || free_a) && (!go_b || free_b);
+                    hand = e_act && (!go_a || free_d) && (!go_b || free_b);
                     sts64_shared_if(hand && go_a && !join_a, sa, e_base | qv);
                     sts64_shared_if(hand && go_b && !join_b, sc, e_base | qv);
                     if (JOIN) {
@@ -657,10 +681,9 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
                         n_left++;
                     }
                 } else {
-                    const bool to_b = bit >= 0 && ((bits >> bit) & 1u);
                     const bool leaves = to_b ? db < 0 : da < 0;
-                    hand = e_act && (to_b ? free_b : free_a);
-                    sts64_shared_if(hand && !leaves, to_b ? sc : sa, e_base | qv);
+                    hand = e_act && free_d;
+                    sts64_shared_if(hand && !leaves, sd, e_base | qv);
                     // (slab records are plain (finish, query) records whatever the streams carry)
                     if (!FEAS) stg64_if(hand && leaves && IL_IN_RANGE(n_left, leaving, p.status), out + n_left, (e_base >> rb) | qid);
                     if (FEAS) {
@@ -672,11 +695,12 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
                     n_left += (hand && leaves) ? 1u : 0u;
                 }
             } else {
-                hand = e_act && free_a;
+                hand = e_act && free_d;
                 sts64_shared_if(hand && da >= 0, sa, e_base | qv);
-                if (!FEAS) stg64_if(hand && da < 0 && IL_IN_RANGE(n_left, leaving, p.status), out + n_left, e_base | qv);
-                tail_a += hand ? 256u : 0u;
-                n_left += hand ? 1u : 0u;             // (only looked at on a leaf)
+                // (one counter: bytes of ring rows towards the child, of the slab on a leaf)
+                if (!FEAS) stg64_if(hand && da < 0 && IL_IN_RANGE(tail_a >> 3, leaving, p.status),
+                                    reinterpret_cast<uint64_t *>(reinterpret_cast<char *>(out) + tail_a), e_base | qv);
+                tail_a += hand ? tail_step : 0u;
                 if (FEAS) {
                     late_fin = (hand && da < 0) ? e_base : 0ull;
                     late_arr = __ldg(trace + (hand && da < 0 && IL_IN_RANGE(qid, p.n, p.status) ? qid : 0u));
@@ -687,9 +711,11 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
             const bool fetch = f_ok && !goes_on;
             e_idx += hand ? 1u : 0u;
             e_idx = fetch ? (uint32_t)fkey & qmask : e_idx;
-            e_base = fetch ? fkey & ~(uint64_t)qmask : e_base;
+            e_key = fetch ? fkey : e_key;
             epos += fetch ? 256u : 0u;
             e_act = goes_on || fetch;
+            qv = lds32(qb + ((e_idx & (nq - 1u)) << 7));
+            if (SPILL && spill && i - e_idx > nq && IL_IN_RANGE(e_idx & gmask, gmask + 1ull, p.status)) qv = __ldcg(spill_ring + (e_idx & gmask));
             if (JOIN) {
                 __syncwarp();        // what was delivered is there for the joins' lanes
                 have_a = is_join ? lds32(jw_a) : 0u;
@@ -702,7 +728,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
 #pragma unroll 1
             for (int k = 0; k < kTurn; k++) step(std::true_type{});
         } else {
-#pragma unroll 1
+#pragma unroll 2
             for (int k = 0; k < kTurn; k++) step(std::false_type{});
         }
     }
@@ -781,7 +807,7 @@ int des_lane_warps_per_cta() { return kLaneWarps; }
 size_t des_lane_smem(int table_rows, int Bmax, int ring_slots, int ring_words, int cpw, int joins, int window)
 {
     return (kSmemBase + table_bytes(table_rows, Bmax) + key_bytes(ring_slots) - 1) / key_bytes(ring_slots) * key_bytes(ring_slots) -
-           kSmemBase + ring_bytes(ring_slots, ring_words) + kTailBytes + join_bytes(cpw, joins, window);
+           kSmemBase + ring_bytes(ring_slots, ring_words, cpw) + kTailBytes + join_bytes(cpw, joins, window);
 }
 
 int des_lane_max_ctas_per_sm(size_t smem)

@@ -1009,12 +1009,14 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
     IL_CUDA_E(cudaMalloc(&e->d_arrival, (size_t)n * 8));
     IL_CUDA_E(cudaMalloc(&e->d_bits, (size_t)n));
     e->can_pack = can_pack;
-    e->lane_ok = can_pack && (!e->join || n < (INT64_C(1) << 24));     // (a join counts its records in 24 bits)
+    const int64_t latest = tr->arrival_us[n - 1] + worst;
+    // lane kernel: its words stay below 0x7fe0 << 48; a lane counts its records in bytes of rings and slab rows
+    e->lane_ok = can_pack && latest < (INT64_C(0x7fe0000000000000) >> qbits) && n < (INT64_C(1) << (e->join ? 24 : 29));
     bp.qbits = qbits;
     if (can_pack) {
         // padded with "never" records to whole tiles, so that bulk copies always move full tiles
         const int64_t tile = trace_tile_records();
-        const int64_t n_padded = (n + 2 + tile - 1) / tile * tile;      // (two at least: the lane kernel reads ahead)
+        const int64_t n_padded = (n + tile - 1) / tile * tile;
         std::vector<uint64_t> packed((size_t)n_padded, ~0ull);
         for (int64_t i = 0; i < n; i++)
             packed[(size_t)i] = ((uint64_t)tr->arrival_us[i] << qbits) | (uint64_t)i;
@@ -1029,7 +1031,7 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
             if (jn && jn->parent2[s] >= 0 && jn->cond_bit2[s] >= 0) nb = std::max(nb, (int)jn->cond_bit2[s] + 1);
         }
         if (nb > 0 && tr->branch_bits && qbits + nb <= 31 &&
-            tr->arrival_us[n - 1] + worst < (INT64_C(1) << (63 - qbits - nb))) {
+            latest < (INT64_C(0x7fe0000000000000) >> (qbits + nb))) {
             for (int64_t i = 0; i < n; i++)
                 packed[(size_t)i] = ((uint64_t)tr->arrival_us[i] << (qbits + nb)) |
                                     ((uint64_t)(tr->branch_bits[i] & ((1u << nb) - 1u)) << qbits) | (uint64_t)i;
