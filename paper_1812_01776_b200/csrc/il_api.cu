@@ -22,6 +22,8 @@ static thread_local int g_last_cuda_error = 0;
     } while (0)
 
 static constexpr int kCounters = 8;
+// device and pinned block: the counters, the status word, the largest replica count of a batch
+static constexpr size_t kCounterBytes = kCounters * sizeof(unsigned long long) + 2 * sizeof(int);
 
 struct il_estimator {
     int device = 0;
@@ -61,7 +63,7 @@ struct il_estimator {
     int lane_slots = 32;               // batch ring positions used by the current call
     int64_t setup_launches = 0;        // kernels a call launched before its simulation: the replica reduction, the node probe
     int lane_ctas_knob = 0;            // test knob: resident CTAs per SM of the lane kernel (0: the library's choice)
-    int *d_maxrep = nullptr;           // device word: largest replica count of a batch
+    int *d_maxrep = nullptr;           // device word behind the status: largest replica count of a batch
     uint8_t *d_bits = nullptr;
     int32_t *d_lat = nullptr;
     unsigned long long *d_counters = nullptr;   // [kCounters]: next candidate, batches, algorithmic ops,
@@ -74,6 +76,9 @@ struct il_estimator {
     void *user_ws = nullptr; size_t user_ws_bytes = 0;
     void *own_ws = nullptr;  size_t own_ws_bytes = 0;
 
+    // results that go to pinned memory behind the kernels of a call, so that a host entry point waits once
+    void *copy_dst = nullptr; const void *copy_src = nullptr; size_t copy_bytes = 0;
+    char *h_out = nullptr; int64_t h_out_cap = 0;              // pinned: 16 bytes per candidate
     il_stage_config *d_cfg = nullptr; int64_t d_cfg_cap = 0;   // staging for il_estimate
     int64_t *d_out = nullptr; int64_t d_out_cap = 0;           // [2][cap]
 
@@ -347,9 +352,10 @@ void configure_lane_rings(il_estimator *e)
 void free_device(il_estimator *e)
 {
     cudaFree(e->d_arrival); cudaFree(e->d_ptrace); cudaFree(e->d_ptrace_b); cudaFree(e->d_bits); cudaFree(e->d_lat);
-    cudaFree(e->d_counters); cudaFree(e->d_status); cudaFree(e->d_maxrep); cudaFree(e->d_envelope);
+    cudaFree(e->d_counters); cudaFree(e->d_envelope);
     cudaFree(e->own_ws); cudaFree(e->d_cfg); cudaFree(e->d_out);
     if (e->h_counters) cudaFreeHost(e->h_counters);
+    if (e->h_out) cudaFreeHost(e->h_out);
     for (cudaEvent_t ev : e->events) cudaEventDestroy(ev);
 }
 
@@ -429,6 +435,34 @@ static int ensure_staging(il_estimator *e, int64_t n_cand)
     return IL_OK;
 }
 
+// Pinned memory for the results of a host entry point, so that they come back with the counters and the call waits
+// once; nullptr for batches so large that a second wait does not matter (or when there is no such memory).
+static char *host_results(il_estimator *e, int64_t n_cand)
+{
+    constexpr int64_t kMost = 32768;
+    if (n_cand > kMost) return nullptr;
+    if (e->h_out_cap < n_cand) {
+        if (e->h_out) cudaFreeHost(e->h_out);
+        e->h_out = nullptr; e->h_out_cap = 0;
+        const int64_t cap = std::min(kMost, std::max<int64_t>(1024, 2 * n_cand));
+        if (cudaMallocHost(&e->h_out, (size_t)cap * 16) != cudaSuccess) { cudaGetLastError(); e->h_out = nullptr; return nullptr; }
+        e->h_out_cap = cap;
+    }
+    return e->h_out;
+}
+
+// The largest replica count among host configurations, 0 if one of them is out of range.
+static int check_configs(const il_estimator *e, const il_stage_config *configs, int64_t total)
+{
+    int most = 0;
+    for (int64_t i = 0; i < total; i++) {
+        const il_stage_config &c = configs[i];
+        if (c.hw >= e->H || c.max_batch < 1 || c.max_batch > e->Bmax || c.replicas < 1 || c.replicas > IL_MAX_REPLICAS) return 0;
+        most = std::max(most, (int)c.replicas);
+    }
+    return most;
+}
+
 // Kernel parameters of one chunk: the bound inputs plus this chunk's scratch.
 static DesParams chunk_params(const il_estimator *e, const Plan &pl, char *ws, const il_stage_config *d_configs,
                               int64_t cnt)
@@ -456,21 +490,40 @@ static DesParams chunk_params(const il_estimator *e, const Plan &pl, char *ws, c
     return p;
 }
 
-// Batch ring positions per lane for this batch: 16 when no candidate has more than 16 replicas at any
-// stage (the ring must hold the batches in use), else 32.  One small reduction over the configurations
-// and a 4-byte read-back.
-static int choose_lane_slots(il_estimator *e, const il_stage_config *d_configs, int64_t n_cand)
+// Start of a call: clears the counter block and chooses the batch ring positions per lane: 16 when no candidate has
+// more than 16 replicas at any stage (the ring must hold the batches in use), else 32.  The larger ring only costs
+// shared memory, so a grid of at most one CTA per SM takes it without looking; a host entry point knows the largest
+// replica count (max_replicas > 0); otherwise one small reduction over the configurations and a read-back find it.
+static int start_call(il_estimator *e, const il_stage_config *d_configs, int64_t n_cand, int max_replicas)
 {
     e->lane_slots = 32;
     e->setup_launches = 0;
-    if (!is_lane(e)) return IL_OK;
+    if (!is_lane(e)) {
+        IL_CUDA(cudaMemsetAsync(e->d_counters, 0, kCounterBytes, e->stream));
+        return IL_OK;
+    }
     e->setup_launches = 1;
-    int h = 0;
-    IL_CUDA(cudaMemsetAsync(e->d_maxrep, 0, sizeof(int), e->stream));
+    const int64_t cps = cands_per_slot(e, n_cand), per_cta = cps * des_lane_warps_per_cta();
+    if (max_replicas > 0 || (n_cand + per_cta - 1) / per_cta <= e->num_sms) {
+        IL_CUDA(launch_clear(e->d_counters, (int)(kCounterBytes / sizeof(unsigned long long)), e->stream));
+        if (max_replicas > 0 && max_replicas <= 16) e->lane_slots = 16;
+        return IL_OK;
+    }
+    int *h = reinterpret_cast<int *>(e->h_counters + kCounters) + 1;
+    IL_CUDA(cudaMemsetAsync(e->d_counters, 0, kCounterBytes, e->stream));
     IL_CUDA(launch_max_replicas(d_configs, n_cand * e->S, e->d_maxrep, e->stream));
-    IL_CUDA(cudaMemcpyAsync(&h, e->d_maxrep, sizeof(int), cudaMemcpyDeviceToHost, e->stream));
+    IL_CUDA(cudaMemcpyAsync(h, e->d_maxrep, sizeof(int), cudaMemcpyDeviceToHost, e->stream));
     IL_CUDA(cudaStreamSynchronize(e->stream));
-    e->lane_slots = h <= 16 ? 16 : 32;
+    e->lane_slots = *h <= 16 ? 16 : 32;
+    return IL_OK;
+}
+
+// End of a call: the counter block and the results asked for come to pinned memory; waits for the stream.
+static int end_call(il_estimator *e)
+{
+    IL_CUDA(cudaMemcpyAsync(e->h_counters, e->d_counters, kCounterBytes, cudaMemcpyDeviceToHost, e->stream));
+    if (e->copy_dst) IL_CUDA(cudaMemcpyAsync(e->copy_dst, e->copy_src, e->copy_bytes, cudaMemcpyDeviceToHost, e->stream));
+    IL_CUDA(cudaStreamSynchronize(e->stream));
     return IL_OK;
 }
 
@@ -517,10 +570,8 @@ static int finish_shared(il_estimator *e, int64_t n_cand, int64_t launches, int6
 {
     cudaStream_t st = e->stream;
     IL_CUDA(cudaEventRecord(e->events[2], st));
-    IL_CUDA(cudaMemcpyAsync(e->h_counters, e->d_counters, kCounters * sizeof(unsigned long long),
-                            cudaMemcpyDeviceToHost, st));
-    IL_CUDA(cudaMemcpyAsync(e->h_status, e->d_status, sizeof(int), cudaMemcpyDeviceToHost, st));
-    IL_CUDA(cudaStreamSynchronize(st));
+    const int erc = end_call(e);
+    if (erc) return erc;
     float ms = 0.f;
     IL_CUDA(cudaEventElapsedTime(&ms, e->events[0], e->events[1]));
     e->stats.sim_ms = ms;
@@ -683,8 +734,6 @@ static int estimate_shared(il_estimator *e, const il_stage_config *d_configs, in
     int rc = ensure_events(e, 5);
     if (rc) return rc;
     cudaStream_t st = e->stream;
-    IL_CUDA(cudaMemsetAsync(e->d_counters, 0, kCounters * sizeof(unsigned long long), st));
-    IL_CUDA(cudaMemsetAsync(e->d_status, 0, sizeof(int), st));
     IL_CUDA(cudaMemsetAsync(d_count, 0, (size_t)IL_MAX_STAGES * 4, st));
     IL_CUDA(cudaMemsetAsync(d_work, 0, (size_t)IL_MAX_STAGES * 8, st));
     IL_CUDA(cudaEventRecord(e->events[0], st));
@@ -794,6 +843,11 @@ static int estimate_shared(il_estimator *e, const il_stage_config *d_configs, in
     launches++;
     return finish_shared(e, n_cand, launches, stage_runs);
 }
+
+static int estimate_device(il_estimator *e, const il_stage_config *d_configs, int64_t n_cand, int64_t slo_us,
+                           int64_t *d_out_p99, int64_t *d_out_miss, int max_replicas);
+static int feasible_device(il_estimator *e, const il_stage_config *d_configs, int64_t n_cand, int64_t slo_us,
+                           uint8_t *d_out_feasible, int max_replicas, void *h_out, bool *h_done);
 
 extern "C" {
 
@@ -1041,9 +1095,9 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
         }
     }
     IL_CUDA_E(cudaMalloc(&e->d_lat, e->smem));
-    IL_CUDA_E(cudaMalloc(&e->d_counters, kCounters * sizeof(unsigned long long)));
-    IL_CUDA_E(cudaMalloc(&e->d_status, sizeof(int)));
-    IL_CUDA_E(cudaMalloc(&e->d_maxrep, sizeof(int)));
+    IL_CUDA_E(cudaMalloc(&e->d_counters, kCounterBytes));
+    e->d_status = reinterpret_cast<int *>(e->d_counters + kCounters);
+    e->d_maxrep = e->d_status + 1;
     IL_CUDA_E(cudaMalloc(&e->d_envelope, envelope_max_windows() * sizeof(int)));
     IL_CUDA_E(cudaMallocHost(&e->h_counters, (kCounters + 2) * sizeof(unsigned long long) + envelope_max_windows() * sizeof(int)));
     e->h_status = reinterpret_cast<int *>(e->h_counters + kCounters);
@@ -1185,13 +1239,21 @@ int il_stage_visits(const il_estimator *e, int64_t *out_visits)
 int il_estimate_device(il_estimator *e, const il_stage_config *d_configs, int64_t n_cand,
                        int64_t slo_us, int64_t *d_out_p99, int64_t *d_out_miss)
 {
+    return estimate_device(e, d_configs, n_cand, slo_us, d_out_p99, d_out_miss, 0);
+}
+
+}  // extern "C"
+
+static int estimate_device(il_estimator *e, const il_stage_config *d_configs, int64_t n_cand, int64_t slo_us,
+                           int64_t *d_out_p99, int64_t *d_out_miss, int max_replicas)
+{
     if (!e || n_cand < 0) return IL_ERR_INVALID_ARG;
     e->stats = il_stats{};
     if (n_cand == 0) return IL_OK;
     if (!d_configs || !d_out_p99 || !d_out_miss) return IL_ERR_INVALID_ARG;
     IL_CUDA(cudaSetDevice(e->device));
 
-    int lrc = choose_lane_slots(e, d_configs, n_cand);
+    int lrc = start_call(e, d_configs, n_cand, max_replicas);
     if (lrc) return lrc;
     char *ws = nullptr;
     size_t ws_bytes = 0;
@@ -1208,8 +1270,6 @@ int il_estimate_device(il_estimator *e, const il_stage_config *d_configs, int64_
     if (rc) return rc;
 
     cudaStream_t st = e->stream;
-    IL_CUDA(cudaMemsetAsync(e->d_counters, 0, kCounters * sizeof(unsigned long long), st));
-    IL_CUDA(cudaMemsetAsync(e->d_status, 0, sizeof(int), st));
     IL_CUDA(cudaEventRecord(e->events[0], st));
 
     int64_t launches = e->setup_launches;
@@ -1249,10 +1309,8 @@ int il_estimate_device(il_estimator *e, const il_stage_config *d_configs, int64_
         launches++;
     }
     IL_CUDA(cudaEventRecord(e->events[1], st));
-    IL_CUDA(cudaMemcpyAsync(e->h_counters, e->d_counters, kCounters * sizeof(unsigned long long),
-                            cudaMemcpyDeviceToHost, st));
-    IL_CUDA(cudaMemcpyAsync(e->h_status, e->d_status, sizeof(int), cudaMemcpyDeviceToHost, st));
-    IL_CUDA(cudaStreamSynchronize(st));
+    rc = end_call(e);
+    if (rc) return rc;
 
     float ms = 0.f;
     IL_CUDA(cudaEventElapsedTime(&ms, e->events[0], e->events[1]));
@@ -1276,6 +1334,8 @@ int il_estimate_device(il_estimator *e, const il_stage_config *d_configs, int64_
     return *e->h_status;
 }
 
+extern "C" {
+
 int il_estimate_latencies(il_estimator *e, const il_stage_config *d_config, int64_t *d_out_latency)
 {
     if (!e || !d_config || !d_out_latency) return IL_ERR_INVALID_ARG;
@@ -1288,8 +1348,7 @@ int il_estimate_latencies(il_estimator *e, const il_stage_config *d_config, int6
     Plan pl;
     if (!make_plan(e, ws_bytes, 1, pl)) return IL_ERR_NOMEM;
     cudaStream_t st = e->stream;
-    IL_CUDA(cudaMemsetAsync(e->d_counters, 0, kCounters * sizeof(unsigned long long), st));
-    IL_CUDA(cudaMemsetAsync(e->d_status, 0, sizeof(int), st));
+    IL_CUDA(cudaMemsetAsync(e->d_counters, 0, kCounterBytes, st));
     DesParams p = chunk_params(e, pl, ws, d_config, 1);
     IL_CUDA(cudaMemsetAsync(ws + pl.off_order, 0, sizeof(int32_t), st));   // the one candidate is number 0
     const int kernel = sim_kernel(e);
@@ -1328,28 +1387,40 @@ int il_estimate(il_estimator *e, const il_stage_config *configs, int64_t n_cand,
     if (n_cand == 0) { e->stats = il_stats{}; return IL_OK; }
     if (!configs || !out_p99 || !out_miss) return IL_ERR_INVALID_ARG;
     const int64_t total = n_cand * e->S;
-    for (int64_t i = 0; i < total; i++) {
-        const il_stage_config &c = configs[i];
-        if (c.hw >= e->H || c.max_batch < 1 || c.max_batch > e->Bmax || c.replicas < 1 ||
-            c.replicas > IL_MAX_REPLICAS)
-            return IL_ERR_BAD_CONFIG;
-    }
+    const int max_replicas = check_configs(e, configs, total);
+    if (max_replicas < 1) return IL_ERR_BAD_CONFIG;
     IL_CUDA(cudaSetDevice(e->device));
     int rc0 = ensure_staging(e, n_cand);
     if (rc0) return rc0;
     IL_CUDA(cudaMemcpyAsync(e->d_cfg, configs, (size_t)total * sizeof(il_stage_config),
                             cudaMemcpyHostToDevice, e->stream));
-    int rc = il_estimate_device(e, e->d_cfg, n_cand, slo_us, e->d_out, e->d_out + e->d_out_cap);
+    char *h = host_results(e, n_cand);
+    e->copy_dst = h; e->copy_src = e->d_out; e->copy_bytes = (size_t)n_cand * 16;
+    const int rc = estimate_device(e, e->d_cfg, n_cand, slo_us, e->d_out, e->d_out + n_cand, max_replicas);
+    e->copy_dst = nullptr;
     if (rc) return rc;
+    if (h) {
+        memcpy(out_p99, h, (size_t)n_cand * 8);
+        memcpy(out_miss, h + (size_t)n_cand * 8, (size_t)n_cand * 8);
+        return IL_OK;
+    }
     IL_CUDA(cudaMemcpyAsync(out_p99, e->d_out, (size_t)n_cand * 8, cudaMemcpyDeviceToHost, e->stream));
-    IL_CUDA(cudaMemcpyAsync(out_miss, e->d_out + e->d_out_cap, (size_t)n_cand * 8,
-                            cudaMemcpyDeviceToHost, e->stream));
+    IL_CUDA(cudaMemcpyAsync(out_miss, e->d_out + n_cand, (size_t)n_cand * 8, cudaMemcpyDeviceToHost, e->stream));
     IL_CUDA(cudaStreamSynchronize(e->stream));
     return IL_OK;
 }
 
 int il_feasible_device(il_estimator *e, const il_stage_config *d_configs, int64_t n_cand, int64_t slo_us,
                        uint8_t *d_out_feasible)
+{
+    return feasible_device(e, d_configs, n_cand, slo_us, d_out_feasible, 0, nullptr, nullptr);
+}
+
+}  // extern "C"
+
+// h_out (pinned, may be nullptr): where the flags go besides; *h_done tells whether they went.
+static int feasible_device(il_estimator *e, const il_stage_config *d_configs, int64_t n_cand, int64_t slo_us,
+                           uint8_t *d_out_feasible, int max_replicas, void *h_out, bool *h_done)
 {
     if (!e || n_cand < 0) return IL_ERR_INVALID_ARG;
     e->stats = il_stats{};
@@ -1363,7 +1434,7 @@ int il_feasible_device(il_estimator *e, const il_stage_config *d_configs, int64_
         // is, so copies cannot be counted as they leave): P99 as usual, then the comparison
         int rc = ensure_staging(e, n_cand);
         if (rc) return rc;
-        rc = il_estimate_device(e, d_configs, n_cand, slo_us, e->d_out, e->d_out + e->d_out_cap);
+        rc = estimate_device(e, d_configs, n_cand, slo_us, e->d_out, e->d_out + e->d_out_cap, max_replicas);
         if (rc) return rc;
         IL_CUDA(launch_feasible_from_p99(e->d_out, nullptr, n_cand, slo_us, d_out_feasible, st));
         IL_CUDA(cudaStreamSynchronize(st));
@@ -1372,7 +1443,7 @@ int il_feasible_device(il_estimator *e, const il_stage_config *d_configs, int64_
     }
 
     // lane kernel: no slab and no percentile pass, so the whole batch is one chunk
-    int rc = choose_lane_slots(e, d_configs, n_cand);
+    int rc = start_call(e, d_configs, n_cand, max_replicas);
     if (rc) return rc;
     char *ws = nullptr;
     size_t ws_bytes = 0;
@@ -1403,8 +1474,6 @@ int il_feasible_device(il_estimator *e, const il_stage_config *d_configs, int64_
     rc = ensure_events(e, 4);
     if (rc) return rc;
 
-    IL_CUDA(cudaMemsetAsync(e->d_counters, 0, kCounters * sizeof(unsigned long long), st));
-    IL_CUDA(cudaMemsetAsync(e->d_status, 0, sizeof(int), st));
     DesParams p = e->base;
     p.configs = d_configs;
     p.n_cand = n_cand;
@@ -1429,10 +1498,11 @@ int il_feasible_device(il_estimator *e, const il_stage_config *d_configs, int64_
         IL_CUDA(launch_overflow_list(p.ovf, n_cand, reinterpret_cast<int32_t *>(ws + off_order), e->d_counters, st));
         launches++;
     }
-    IL_CUDA(cudaMemcpyAsync(e->h_counters, e->d_counters, kCounters * sizeof(unsigned long long),
-                            cudaMemcpyDeviceToHost, st));
-    IL_CUDA(cudaMemcpyAsync(e->h_status, e->d_status, sizeof(int), cudaMemcpyDeviceToHost, st));
-    IL_CUDA(cudaStreamSynchronize(st));
+    e->copy_dst = h_out; e->copy_src = d_out_feasible; e->copy_bytes = (size_t)n_cand;
+    rc = end_call(e);
+    e->copy_dst = nullptr;
+    if (rc) return rc;
+    if (h_done) *h_done = h_out && e->h_counters[3] == 0;
     float ms = 0.f;
     IL_CUDA(cudaEventElapsedTime(&ms, e->events[0], e->events[1]));
     il_stats stats = {};
@@ -1486,6 +1556,8 @@ int il_feasible_device(il_estimator *e, const il_stage_config *d_configs, int64_
     return rc;
 }
 
+extern "C" {
+
 int il_feasible(il_estimator *e, const il_stage_config *configs, int64_t n_cand, int64_t slo_us,
                 uint8_t *out_feasible)
 {
@@ -1493,12 +1565,8 @@ int il_feasible(il_estimator *e, const il_stage_config *configs, int64_t n_cand,
     if (n_cand == 0) { e->stats = il_stats{}; return IL_OK; }
     if (!configs || !out_feasible) return IL_ERR_INVALID_ARG;
     const int64_t total = n_cand * e->S;
-    for (int64_t i = 0; i < total; i++) {
-        const il_stage_config &c = configs[i];
-        if (c.hw >= e->H || c.max_batch < 1 || c.max_batch > e->Bmax || c.replicas < 1 ||
-            c.replicas > IL_MAX_REPLICAS)
-            return IL_ERR_BAD_CONFIG;
-    }
+    const int max_replicas = check_configs(e, configs, total);
+    if (max_replicas < 1) return IL_ERR_BAD_CONFIG;
     IL_CUDA(cudaSetDevice(e->device));
     int rc = ensure_staging(e, n_cand);
     if (rc) return rc;
@@ -1507,8 +1575,11 @@ int il_feasible(il_estimator *e, const il_stage_config *configs, int64_t n_cand,
     // the flags go behind the two output arrays of the staging (which the warp-per-candidate
     // kernels fill with P99 and misses first)
     uint8_t *d_flags = reinterpret_cast<uint8_t *>(e->d_out + 2 * e->d_out_cap);
-    rc = il_feasible_device(e, e->d_cfg, n_cand, slo_us, d_flags);
+    char *h = host_results(e, n_cand);
+    bool done = false;
+    rc = feasible_device(e, e->d_cfg, n_cand, slo_us, d_flags, max_replicas, h, &done);
     if (rc) return rc;
+    if (done) { memcpy(out_feasible, h, (size_t)n_cand); return IL_OK; }
     IL_CUDA(cudaMemcpyAsync(out_feasible, d_flags, (size_t)n_cand, cudaMemcpyDeviceToHost, e->stream));
     IL_CUDA(cudaStreamSynchronize(e->stream));
     return IL_OK;

@@ -232,6 +232,7 @@ struct OrderParams {
     int32_t *order;                  // [n_cand] out
 };
 cudaError_t launch_order(const OrderParams &p, cudaStream_t stream);
+cudaError_t launch_clear(unsigned long long *words, int count, cudaStream_t stream);
 cudaError_t launch_max_replicas(const il_stage_config *configs, int64_t count, int *out, cudaStream_t stream);
 cudaError_t launch_gather_configs(const il_stage_config *configs, const int32_t *list, int64_t count, int S,
                                   il_stage_config *out, cudaStream_t stream);

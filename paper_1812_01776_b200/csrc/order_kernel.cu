@@ -95,6 +95,12 @@ __global__ void __launch_bounds__(256) max_replicas_kernel(const il_stage_config
     if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(out, m);
 }
 
+// a handle's counter block at the start of a call
+__global__ void clear_kernel(unsigned long long *words, int count)
+{
+    for (int i = threadIdx.x; i < count; i += blockDim.x) words[i] = 0ull;
+}
+
 // configs of the listed candidates, packed one after the other
 __global__ void gather_configs_kernel(const il_stage_config *configs, const int32_t *list, int64_t count, int S,
                                       il_stage_config *out)
@@ -112,6 +118,12 @@ __global__ void feasible_from_p99_kernel(const int64_t *p99, const int32_t *list
 }
 
 }  // namespace
+
+cudaError_t launch_clear(unsigned long long *words, int count, cudaStream_t stream)
+{
+    clear_kernel<<<1, 32, 0, stream>>>(words, count);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_max_replicas(const il_stage_config *configs, int64_t count, int *out, cudaStream_t stream)
 {
