@@ -321,7 +321,9 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
     bool live = false, cand_bad = false, over = false;
     uint32_t Rm1 = 0;            // replicas less one, in bytes of a ring row
     uint32_t kfb = nowhere, kfm = 0;         // where the first batch in use is looked up (one replica: kInf, which compares as later)
-    uint32_t cap = 0;            // positions of the batch ring the lane may fill; 0 until its first record has opened a batch
+    uint32_t efull = 0;          // tpos with the batch ring full: epos + its size; epos until a first record has opened a batch
+    uint32_t lfull = 0;          // tpos with every replica in use or about to be: lpos + replicas less one
+    bool started = false;        // a first record has opened a batch
     uint32_t mbm1 = 0;
     uint32_t tab = tab0;         // the lane's row of the tables
     uint64_t *out = nullptr;     // leaving records: the stage's region of the slab row (fan-out: the row)
@@ -337,6 +339,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
     uint64_t e_key = 0;          //   its key
     uint32_t e_idx = 0;          //   the record to hand on next
     uint32_t tail_a = 0, tail_b = 0;         // records handed to the children, in bytes of a row
+    uint32_t at1 = kb | rm, at2 = kb | (rm - 256u);          // where the last two batches of the ring are
     uint32_t fed = 0;            // records of the trace requested for the group's root
     uint32_t qv = 0;             // low part of the record to hand on (where there is one)
     bool spill = false;
@@ -374,7 +377,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
         copies_done();
         __syncwarp();
         turns--;
-        bool attn = !exhausted && ((is_join ? ja == join_na && jb == join_nb : i == n_cur || cap == 0u) || turns == 0u);
+        bool attn = !exhausted && ((is_join ? ja == join_na && jb == join_nb : i == n_cur || !started) || turns == 0u);
         if (JOIN) attn |= !exhausted && !has;
         attn |= i - low > reach || spill;
         if (FEAS) attn |= has && missw[j] > p.miss_allow;
@@ -414,22 +417,23 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
             stop |= group_gives_up;
         }
         if (stop) {
-            n_cur = i; bm = ~0u; epos = tpos; e_act = false; late_fin = 0; cap = 0;
+            n_cur = i; bm = ~0u; epos = tpos; efull = tpos; e_act = false; late_fin = 0; started = false;
             ja = join_na; jb = join_nb;
             done = true;
         }
         // The first record of a stream opens a batch on an unused replica, and the last batch is closed by the
         // end of the stream; both once per candidate, so here and not in every iteration.
-        if (!done && cap == 0u && !is_join) {
+        if (!done && !started && !is_join) {
             const uint64_t rec = lds64_shared(xin);
             if ((int64_t)rec >= 0) {
                 tk = rec | qmask;
                 bm = 0; i = 1;
                 prev = (uint32_t)rec & qmask;
                 sts32_shared_if(true, xin + 4u, ~0u);
-                cap = rm + 256u;
+                started = true;
+                efull = epos + rm + 256u;
             }
-        } else if (!done && !is_join && i == n_cur && bm != ~0u && tpos - epos < cap) {
+        } else if (!done && !is_join && i == n_cur && bm != ~0u && tpos != efull) {
             const uint64_t key = ((tk + (uint64_t)lds32(tab + bm * 4u) * tick) & ~(uint64_t)qmask) | (i - 1u - bm);
             uint32_t pos = tpos;
             for (; pos != lpos; pos -= 256u) {
@@ -497,7 +501,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
                 Rm1 = (cfg.replicas - 1u) << 8;
                 kfb = Rm1 != 0u ? kb : nowhere + (uint32_t)lane * 8u;
                 kfm = Rm1 != 0u ? rm : 0u;
-                cap = 0;
+                started = false; efull = 0; lfull = Rm1;
                 mbm1 = cfg.max_batch - 1u;
                 tab = tab0 + (uint32_t)((live ? s * p.H + cfg.hw : 0) * rowlen) * 4u;
                 out = FORK ? slab : slab + exit_off;
@@ -507,7 +511,8 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
                 if (FEAS && is_root) missw[j] = 0u;
                 i = 0; bm = ~0u; tk = 0;
                 epos = 0; lpos = 0; tpos = 0; tpos_seen = 0;
-                sts64(kb | rm, 0ull); sts64(kb | (rm - 256u), 0ull);       // (no batch before the first one)
+                at1 = kb | rm; at2 = kb | (rm - 256u);
+                sts64(at1, 0ull); sts64(at2, 0ull);       // (no batch before the first one)
                 prev = 0;
                 e_act = false; e_idx = 0;
                 tail_a = 0; tail_b = 0;
@@ -594,7 +599,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
             const uint64_t rec = lds64_shared(xs);                    // record to examine
             const uint32_t lat = lds32(tab + bm * 4u);                // time of the open batch
             const uint64_t kf = lds64(kfb | (lpos & kfm));            // first batch in use (one replica: kInf)
-            const uint64_t k1 = lds64(kb | ((tpos - 256u) & rm)), k2 = lds64(kb | ((tpos - 512u) & rm));    // the last two batches
+            const uint64_t k1 = lds64(at1), k2 = lds64(at2);    // the last two batches
             const uint64_t fkey = lds64(kb | (epos & rm));            // first batch not handed on (if there is one)
             const uint32_t sa = xa | (tail_a & xam), sc = xc | (tail_b & xcm);
             // where the record in hand goes, and whether there is room: towards the outside always
@@ -610,19 +615,17 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
 
             // ---- examine record i, if it is there: it joins the open batch, or the open batch is closed and it
             // opens the next one
-            const bool taken = (int64_t)rec >= 0 && tpos - epos < cap;
+            const bool taken = (int64_t)rec >= 0 && tpos != efull;
             const bool joins = bm < mbm1 && not_after(rec, tk);
             const bool join = taken && joins, open = taken && !joins;
             const uint64_t key = ((tk + (uint64_t)lat * tick) & ~(uint64_t)qmask) | (i - 1u - bm);
             // the next batch goes to a replica never used so far (free from time 0), else to the one that is
             // free first -- maybe the one whose batch is closed just now
-            const uint32_t in_use = tpos - lpos;
-            const bool pop = in_use == Rm1;
+            const bool pop = tpos == lfull;
             const uint64_t first = before(kf, key) ? kf : key;
-            const uint64_t start = ((pop && before(rec, first)) ? first : rec) | qmask;
             // its place in the ring: behind the last one, nearly always, or just before it (a batch that finishes
             // before one dispatched earlier); further ahead is rare enough for a loop
-            const uint32_t at0 = kb | (tpos & rm), at1 = kb | ((tpos - 256u) & rm);
+            const uint32_t at0 = kb | (tpos & rm);
             const bool overtakes = before(key, k1);
             sts64_if(open, overtakes ? at1 : at0, key);
             sts64_if(open && overtakes, at0, k1);
@@ -641,11 +644,16 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
                     pos -= 1024u;
                 }
             }
+            // dispatch time: the record's, or later the time the replica is free
+            const uint64_t start = ((pop && before(rec, first)) ? first : rec) | qmask;
             tk = open ? start : tk;
             tpos += open ? 256u : 0u;
+            at2 = open ? at1 : at2;
+            at1 = open ? at0 : at1;
             lpos += (open && pop) ? 256u : 0u;
-            bm = open ? 0u : bm;
+            lfull += (open && pop) ? 256u : 0u;
             bm += join ? 1u : 0u;
+            bm = open ? 0u : bm;
             // the word of record i - 1 is final now: the last one of its batch or not
             const uint32_t word = prev | (open ? kLast : 0u);
             sts32_if(taken, qb + (((i - 1u) & (nq - 1u)) << 7), word);
@@ -713,6 +721,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
             e_idx = fetch ? (uint32_t)fkey & qmask : e_idx;
             e_key = fetch ? fkey : e_key;
             epos += fetch ? 256u : 0u;
+            efull += fetch ? 256u : 0u;
             e_act = goes_on || fetch;
             qv = lds32(qb + ((e_idx & (nq - 1u)) << 7));
             if (SPILL && spill && i - e_idx > nq && IL_IN_RANGE(e_idx & gmask, gmask + 1ull, p.status)) qv = __ldcg(spill_ring + (e_idx & gmask));
