@@ -590,8 +590,7 @@ static int finish_shared(il_estimator *e, int64_t n_cand, int64_t launches, int6
 }
 
 // Shared-prefix evaluation, simulation by the lane kernel.  The nodes that queries leave after are
-// covered by a set of whole candidates of the batch (per node the candidate with the smallest index
-// that contains it); those are simulated like any batch, and a node's leaving records are the region
+// covered by a set of whole candidates of the batch (prefix_kernel.cu); those are simulated like any batch, and a node's leaving records are the region
 // of its stage in the slab row of its candidate.  Candidates of the set repeat the work of the
 // prefixes they share, but they run on the kernel that is an order of magnitude faster per stage run
 // than the node-by-node one, and all at once instead of level by level.  (A candidate evaluated by the
@@ -637,8 +636,11 @@ static int shared_by_cover(il_estimator *e, const SharedCommon &c, char *ws, siz
     il_stage_config *cfg = reinterpret_cast<il_stage_config *>(ws + o_cfg);
     IL_CUDA(cudaMemsetAsync(flags, 0, (size_t)n_cand, st));
     IL_CUDA(cudaMemsetAsync(d_cnt, 0, 4, st));
-    for (int s = 0; s < S; s++)
-        if (c.leaving[s] > 0) {
+    int by_nodes[IL_MAX_STAGES];
+    for (int s = 0; s < S; s++) by_nodes[s] = s;
+    std::stable_sort(by_nodes, by_nodes + S, [&](int a, int b) { return c.h_count[a] > c.h_count[b]; });
+    for (int k = 0; k < S; k++)
+        if (const int s = by_nodes[k]; c.leaving[s] > 0) {
             IL_CUDA(launch_cover_rep(c.node_of + (size_t)s * n_cand, n_cand, reinterpret_cast<int32_t *>(ws + o_rep[s]),
                                      c.h_count[s], flags, st));
             *launches += 2;
@@ -962,12 +964,16 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
             bp.join_b[c] = (int8_t)jn->parent2[c];
         }
     }
-    // Which stages a query visits follows from its branch bits alone (parents have smaller indices):
-    // count the visits per stage, the records on each edge into a join, and the copies that leave.
+    // Which stages a query visits follows from its branch bits alone (parents have smaller indices): per value of the
+    // bits, times the queries that have it, count the visits per stage, the records on each edge into a join, and
+    // the copies that leave.
     bp.total_leaving = 0;
-    int64_t edge_a[IL_MAX_STAGES] = {}, edge_b[IL_MAX_STAGES] = {};
-    for (int64_t q = 0; q < n; q++) {
-        const unsigned bits = tr->branch_bits ? tr->branch_bits[q] : 0u;
+    int64_t edge_a[IL_MAX_STAGES] = {}, edge_b[IL_MAX_STAGES] = {}, with_bits[256] = {};
+    if (tr->branch_bits) for (int64_t q = 0; q < n; q++) with_bits[tr->branch_bits[q]]++;
+    else with_bits[0] = n;
+    for (unsigned bits = 0; bits < 256; bits++) {
+        const int64_t m = with_bits[bits];
+        if (m == 0) continue;
         bool reach[IL_MAX_STAGES] = {};
         reach[0] = true;
         for (int c = 1; c < S; c++) {
@@ -975,11 +981,11 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
             const bool b = jn && jn->parent2[c] >= 0 && reach[jn->parent2[c]] &&
                            (jn->cond_bit2[c] < 0 || ((bits >> jn->cond_bit2[c]) & 1u) == jn->cond_val2[c]);
             reach[c] = a || b;
-            edge_a[c] += a; edge_b[c] += b;
+            edge_a[c] += a ? m : 0; edge_b[c] += b ? m : 0;
         }
         for (int s = 0; s < S; s++) {
             if (!reach[s]) continue;
-            e->visits[s]++;
+            e->visits[s] += m;
             int taken = 0;
             for (int side = 0; side < 2; side++) {
                 const int c = side == 0 ? bp.child_a[s] : bp.child_b[s];
@@ -988,7 +994,7 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
                 const unsigned val = side == 0 ? bp.cval_a[s] : bp.cval_b[s];
                 taken += (bit < 0 || ((bits >> bit) & 1u) == val);
             }
-            if (taken == 0) bp.total_leaving++;
+            if (taken == 0) bp.total_leaving += m;
         }
     }
     e->events_per_candidate = 0;

@@ -212,8 +212,8 @@ struct CombineParams {
     int64_t *out_p99, *out_miss;
 };
 cudaError_t launch_prefix_combine(const CombineParams &p, cudaStream_t stream);
-// Covering candidates (prefix_kernel.cu): per node of a stage the smallest candidate that contains it
-// (marked in flags), the list of marked candidates with their positions, and per node its candidate's position.
+// Covering candidates (prefix_kernel.cu): per node of a stage a candidate that contains it, one that is
+// marked in flags already if there is one (stages in any order; then marked in flags), the list of marked candidates with their positions, and per node its candidate's position.
 cudaError_t launch_cover_rep(const int32_t *node_of, int64_t n_cand, int32_t *rep, int64_t n_nodes, uint8_t *flags,
                              cudaStream_t stream);
 cudaError_t launch_cover_list(const uint8_t *flags, int64_t n_cand, int32_t *list, int32_t *pos, int *count,
