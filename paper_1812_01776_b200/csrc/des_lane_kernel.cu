@@ -54,13 +54,13 @@
 //     whose distance outgrows that ring as well gives its candidate up (marked in
 //     the overflow array; the host's fallback evaluates it with the
 //     warp-per-candidate kernel).
-//   * A root's records are copied to shared memory two turns of kTurn iterations
+//   * A root's records are copied to shared memory at least one turn (below)
 //     before their use (cp.async, all lanes of the group).
 //   * The profile tables are shared by the CTA, rows padded to an odd length so
 //     that rows of different lanes start in different banks.
 //   * What happens once per candidate or rarely (its first and last batch, spills,
-//     the iteration bound, the next candidate) is looked at every kTurn-th
-//     iteration only, behind one vote.
+//     the iteration bound, the next candidate) is looked at once a turn of 16 or
+//     32 iterations only, behind one vote.
 //
 // Measured on B200 against the version whose streams lay in global memory (three
 // gathers of 8 bytes per lane and iteration through L1, 208 instructions): about
@@ -83,10 +83,10 @@ namespace {
 constexpr int kLaneWarps = 4;                 // warps per CTA: one per scheduler even in a grid of few CTAs
 constexpr uint64_t kInf = ~0ull;
 constexpr uint64_t kLatest = 0x7fefffffffffffffull;      // no record or key is larger
-constexpr int kX = 4;                         // records of a stream between two stages
+constexpr int kX = 8;                         // records of a stream between two stages
 constexpr uint32_t kLast = 0x80000000u;       // flag of a batch's last record in that ring
-constexpr int kAhead = 32;                    // records of the trace a root has before it: two turns, a power of two
-constexpr int kTurn = 16;                     // iterations between two looks at finished groups, spills, bounds (8: 5 % slower)
+constexpr int kAhead = 64;                    // records of the trace a root has before it: two long turns, a power of two
+constexpr int kTurn = 16, kLongTurn = 32;     // iterations between two looks at finished groups, spills, bounds
 
 __device__ __forceinline__ uint64_t lds64(uint32_t a)
 {
@@ -143,6 +143,10 @@ __device__ __forceinline__ void sts32_if(bool c, uint32_t a, uint32_t v)
 __device__ __forceinline__ void stg32_if(bool c, uint32_t *a, uint32_t v)
 {
     asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p st.global.u32 [%1], %2; }" ::"r"((uint32_t)c), "l"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void ldg32_if(bool c, const uint32_t *a, uint32_t &v)      // leaves v alone otherwise
+{
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %1, 0; @p ld.global.ca.u32 %0, [%2]; }" : "+r"(v) : "r"((uint32_t)c), "l"(a) : "memory");
 }
 __device__ __forceinline__ void stg64_if(bool c, uint64_t *a, uint64_t v)
 {
@@ -311,6 +315,8 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
         (p.iter_limit ? p.iter_limit : 8ull * (unsigned)p.n * (unsigned)(S + 1) + 4096ull) / kTurn + 1ull;
     // a spill has to start before a record still needed is overwritten, two turns from now at the latest
     const uint32_t reach = min((uint32_t)(nq - kTurn - 2), gmask - 2u * kTurn);
+    // (and no long turn may start where it would come too late)
+    const uint32_t long_reach = gmask > 2u * kLongTurn && nq > kLongTurn + 2u ? min((uint32_t)(nq - kLongTurn - 2), gmask - 2u * kLongTurn) : 0u;
     unsigned long long batches = 0, alg_ops = 0, exits_seen = 0, exits_due = 0;
     unsigned early = 0;          // candidates dropped before the end of the trace (feasibility only)
 
@@ -358,7 +364,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
     uint32_t miss_local = 0;
 
     for (;;) {
-        // ---- every kTurn-th iteration: does a lane need more than its steps?  A stream at its start or its end, a
+        // ---- every kTurn-th or kLongTurn-th iteration: does a lane need more than its steps?  A stream at its start or its end, a
         // candidate that is decided, records in reach of being overwritten, the iteration bound.  (Kept short: its
         // latency is on the chain of every iteration, a kTurn-th of it.)
         if (FEAS && miss_local) { atomicAdd(missw + j, miss_local); miss_local = 0; }
@@ -390,9 +396,11 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
             // the oldest record still needed, exactly
             low = i - (bm + 1u);
             if (e_act) low = min(low, e_idx);
+#pragma unroll 1
             for (uint32_t k = epos; k != tpos; k += 256u) low = min(low, (uint32_t)lds64(kb | (k & rm)) & qmask);
             const uint32_t span = i - low;
             if (!spill && span > (uint32_t)(nq - kTurn - 2)) {
+#pragma unroll 1
                 for (uint32_t k = low; k != i; k++)
                     if (IL_IN_RANGE(k & gmask, gmask + 1ull, p.status))
                         spill_ring[k & gmask] = lds32(qb + ((k & (nq - 1u)) << 7));
@@ -528,11 +536,13 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
         }
         any_spill = __any_sync(full, spill);
         }
+        const int turn_its = __any_sync(full, i - low > long_reach) ? kTurn : kLongTurn;
 
         // The root's next records: requested two turns before their use, by all lanes of the group.
         {
             const uint32_t at = __shfl_sync(full, i, root_lane);
             const uint32_t to = has && !cand_bad ? min(at + (uint32_t)kAhead, (uint32_t)p.n) : 0u;
+#pragma unroll 1
             for (uint32_t k = fed + (uint32_t)row; k < to; k += (uint32_t)L) copy8(tb + (k & (kAhead - 1u)) * (uint32_t)cpw * 8u, trace + k);
             fed = max(fed, to);
         }
@@ -724,7 +734,8 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
             efull += fetch ? 256u : 0u;
             e_act = goes_on || fetch;
             qv = lds32(qb + ((e_idx & (nq - 1u)) << 7));
-            if (SPILL && spill && i - e_idx > nq && IL_IN_RANGE(e_idx & gmask, gmask + 1ull, p.status)) qv = __ldcg(spill_ring + (e_idx & gmask));
+            // (the lane's own stores, so the words may come through L1: 32 of them with one miss)
+            if (SPILL) ldg32_if(spill && i - e_idx > nq && IL_IN_RANGE(e_idx & gmask, gmask + 1ull, p.status), spill_ring + (e_idx & gmask), qv);
             if (JOIN) {
                 __syncwarp();        // what was delivered is there for the joins' lanes
                 have_a = is_join ? lds32(jw_a) : 0u;
@@ -735,10 +746,10 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
         };
         if (any_spill) {
 #pragma unroll 1
-            for (int k = 0; k < kTurn; k++) step(std::true_type{});
+            for (int k = 0; k < turn_its; k++) step(std::true_type{});
         } else {
-#pragma unroll 2
-            for (int k = 0; k < kTurn; k++) step(std::false_type{});
+#pragma unroll 1
+            for (int k = 0; k < turn_its; k += 2) { step(std::false_type{}); step(std::false_type{}); }
         }
     }
 
@@ -757,7 +768,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
 }
 
 template <bool BRANCHY, bool FEAS, bool FORK = false>
-__global__ void __launch_bounds__(kLaneWarps * 32) des_lane_kernel(const __grid_constant__ DesParams p)
+__global__ void __launch_bounds__(kLaneWarps * 32, 3) des_lane_kernel(const __grid_constant__ DesParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     lane_simulation<BRANCHY, FEAS, FORK, false>(p, smem_raw);
