@@ -220,3 +220,29 @@ def test_planner_on_the_image_pipeline(oracle):
             p, _ = oracle.estimate_many(w.parent, w.cond_bit, w.cond_val, w.latency_us, w.arrival_us,
                                         w.branch_bits, new[None], w.slo_us)
             assert p[0] > w.slo_us
+
+
+@pytest.mark.parametrize("S,H,B", [(1, 1, 1), (1, 3, 8), (3, 2, 16), (4, 3, 64), (5, 3, 32)])
+@pytest.mark.parametrize("seed", range(4))
+def test_questions_asked_ahead_change_nothing(seed, S, H, B):
+    """The same plan by the same steps whether iterations are asked for ahead or one by one, whatever the answers
+    (here drawn per configuration), and no configuration's answers taken from another's."""
+    rng = np.random.default_rng(seed)
+    lat = np.sort(rng.integers(1, 50, (S, H, B)), axis=2)
+    share = rng.uniform(0.6, 0.98)
+
+    def answers(cfg):
+        return np.array([np.random.default_rng([seed, *map(int, c[:, :3].ravel())]).random() < share for c in cfg])
+
+    def plan(room, ahead):
+        pl = Planner(np.arange(-1, S - 1), lat, np.full(S, 100), np.linspace(1.0, 0.1, H), 10 ** 9,
+                     lambda c: (np.zeros(len(c), np.int64), None), feasible=answers)
+        pl.CALL_ROOM, pl.MOST_AHEAD = room, ahead
+        return pl.minimize_cost()
+
+    one_by_one, default, wide = plan(0, 0), plan(Planner.CALL_ROOM, Planner.MOST_AHEAD), plan(900, 5)
+    for got in (default, wide):
+        assert got.steps == one_by_one.steps and got.feasible == one_by_one.feasible
+        assert got.estimator_calls <= one_by_one.estimator_calls
+        if got.feasible:
+            assert np.array_equal(np.stack(got.trajectory), np.stack(one_by_one.trajectory))
