@@ -358,8 +358,6 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
     uint32_t seen_new = 0;       // joins: words of the queries' bits from here on have not been touched
     uint32_t turns = 1, turns_hi = 0;        // iteration bound, in turns
     bool any_spill = false;
-    uint32_t have_a = 0, have_b = 0;         // joins: records of either incoming stream delivered so far
-    (void)have_a; (void)have_b;
     uint64_t late_fin = 0, late_arr = 0;     // feasibility only: finish and arrival record of a query that has just left
     uint32_t miss_local = 0;
 
@@ -553,57 +551,45 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
             sts64_if(c, win + 8u + ((tail >> 5) & win_mask), rec);
             sts32_if(c, win, tail + 256u);
         };
-        // joins: takes the next record of the two incoming streams, if what comes next on both sides is known.
-        // Straight-line code but for a parent that is far ahead and for the first query of a word of bits.
-        // (A parent may add one record to what have_a / have_b say before the next barrier.)
-        auto merge_step = [&]() {
-            uint64_t va = lds64(jw_a + 8u + ((ja >> 5) & win_mask)), vb = lds64(jw_b + 8u + ((jb >> 5) & win_mask));
-            const uint32_t slot = xj | (tail_a & xjm);
-            const bool room = is_join && (int)lds32_shared(slot + 4u) < 0;
-            const bool end_a = ja == join_na, end_b = jb == join_nb;
-            const bool far_a = !end_a && have_a - ja > win_reach, far_b = !end_b && have_b - jb > win_reach;
-            if (far_a || far_b) {
-                // (the lines from here on are complete, so they may come through L1)
-                if (far_a && IL_IN_RANGE(jg_a + (ja >> 8) - p.join_ws, p.join_size, p.status)) va = jg_a[ja >> 8];
-                if (far_a && (ja & 0xf00u) == 0u) asm volatile("prefetch.global.L1 [%0];" ::"l"(jg_a + (ja >> 8) + 32u));
-                if (far_b && IL_IN_RANGE(jg_b + (jb >> 8) - p.join_ws, p.join_size, p.status)) vb = jg_b[jb >> 8];
-                if (far_b && (jb & 0xf00u) == 0u) asm volatile("prefetch.global.L1 [%0];" ::"l"(jg_b + (jb >> 8) + 32u));
-            }
-            const bool known = room && (end_a || have_a != ja) && (end_b || have_b != jb) && !(end_a && end_b);
-            va = end_a ? kInf : va;
-            vb = end_b ? kInf : vb;
-            const bool from_a = (va | qmask) <= (vb | qmask);
-            const uint64_t rec = from_a ? va : vb;
-            const uint32_t low = (uint32_t)rec & qmask, qid = low & imask, w = qid >> 5;
-            bool both = known && join_always;
-            if (!join_always) {
-                uint32_t bits = rb > 0 ? low >> qi : 0u;
-                if (rb == 0 && known && IL_IN_RANGE(qid, p.n, p.status)) bits = p.bits[qid];
-                both = known && ((lds32(seen_both + (bits >> 5) * 4u) >> (bits & 31u)) & 1u);
-            }
-            const uint32_t at = seen_cache + (w & seen_mask) * 8u;
-            uint64_t e = lds64(at);                      // number of the word << 32 | word
-            if (both && (uint32_t)(e >> 32) != w) {
-                // the cache of the queries' bits: queries come in nearly in order, so a word is new when first needed
-                const uint32_t old = (uint32_t)(e >> 32);
-                if (old != ~0u && IL_IN_RANGE(old, p.join_seen_words, p.status)) seen[old] = (uint32_t)e;
-                e = (uint64_t)w << 32;
-                if (w < seen_new && IL_IN_RANGE(w, p.join_seen_words, p.status)) e |= seen[w];
+        // joins: one step of a join's lane takes up to two records of its two incoming streams (every query can come from
+        // both sides), as long as what comes next on both sides is known.  The loads stand at the top of the
+        // iteration and the rest among the stages' work, so that the two hide each other's latency: one after the other,
+        // with the second record's loads behind the first one's stores, an iteration took 0.6 us.
+        // Whether the other input of a record's query has been seen already: the queries' bits are kept in a small
+        // write-back cache; queries come in nearly in order, so a word is new when it is first needed.
+        auto new_word = [&](uint64_t &e, uint32_t w) {
+            const uint32_t old = (uint32_t)(e >> 32);
+            if (old != ~0u && IL_IN_RANGE(old, p.join_seen_words, p.status)) seen[old] = (uint32_t)e;
+            e = (uint64_t)w << 32;
+            if (w < seen_new && IL_IN_RANGE(w, p.join_seen_words, p.status)) e |= seen[w];
 #pragma unroll 1
-                for (; seen_new < w; seen_new++)         // passed over: it may come later
-                    if (IL_IN_RANGE(seen_new, p.join_seen_words, p.status)) seen[seen_new] = 0u;
-                seen_new = max(seen_new, w + 1u);
-            }
-            const uint32_t mine = 1u << (qid & 31u);
-            sts64_if(both, at, e ^ mine);
-            const bool last_input = known && (!both || ((uint32_t)e & mine) != 0u);
-            sts64_shared_if(last_input, slot, rec);
-            tail_a += last_input ? 256u : 0u;
-            ja += (known && from_a) ? 256u : 0u;
-            jb += (known && !from_a) ? 256u : 0u;
+            for (; seen_new < w; seen_new++)         // passed over: it may come later
+                if (IL_IN_RANGE(seen_new, p.join_seen_words, p.status)) seen[seen_new] = 0u;
+            seen_new = max(seen_new, w + 1u);
+        };
+        // joins: whether the query of a record goes down both edges into the join
+        auto goes_both = [&](bool known, uint32_t low) {
+            if (join_always) return known;
+            const uint32_t qid = low & imask;
+            uint32_t bits = rb > 0 ? low >> qi : 0u;
+            if (rb == 0 && known && IL_IN_RANGE(qid, p.n, p.status)) bits = p.bits[qid];
+            return known && ((lds32(seen_both + (bits >> 5) * 4u) >> (bits & 31u)) & 1u) != 0u;
         };
         auto step = [&](auto spilling) {
             constexpr bool SPILL = decltype(spilling)::value;
+            // ---- joins: what has come in, the next two records of either side, room for two
+            // (A parent may add one record to what have_a / have_b say before the barrier at the end.)
+            uint32_t have_a = 0, have_b = 0, slot0 = 0, slot1 = 0;
+            uint64_t va0 = 0, va1 = 0, vb0 = 0, vb1 = 0;
+            bool room0 = false, room1 = false;
+            if (JOIN) {
+                have_a = lds32(jw_a); have_b = lds32(jw_b);
+                va0 = lds64(jw_a + 8u + ((ja >> 5) & win_mask)); va1 = lds64(jw_a + 8u + (((ja + 256u) >> 5) & win_mask));
+                vb0 = lds64(jw_b + 8u + ((jb >> 5) & win_mask)); vb1 = lds64(jw_b + 8u + (((jb + 256u) >> 5) & win_mask));
+                slot0 = xj | (tail_a & xjm); slot1 = xj | ((tail_a + 256u) & xjm);
+                room0 = is_join && (int)lds32_shared(slot0 + 4u) < 0;
+                room1 = (int)lds32_shared(slot1 + 4u) < 0;
+            }
             // ---- everything the iteration needs from shared memory
             const uint32_t xs = xin + (i & xin_mask) * xin_row;
             const uint64_t rec = lds64_shared(xs);                    // record to examine
@@ -622,6 +608,38 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
             const bool free_d = (int)lds32_shared(sd + 4u) < 0;
             const bool free_b = FORK && (int)lds32_shared(sc + 4u) < 0;
             const bool f_ok = epos != tpos && not_after(fkey, tk);
+
+            // ---- joins: the one or two records to take
+            uint64_t jrec0 = 0, jrec1 = 0, je0 = 0, je1 = 0;
+            uint32_t jat0 = 0, jat1 = 0;
+            bool known0 = false, known1 = false, from_a0 = false, from_a1 = false;
+            if (JOIN) {
+                const bool end_a = ja == join_na, end_b = jb == join_nb;
+                const bool far_a = is_join && !end_a && have_a - ja > win_reach, far_b = is_join && !end_b && have_b - jb > win_reach;
+                if (far_a || far_b) {
+                    // (the lines from here on are complete, so they may come through L1)
+                    if (far_a && IL_IN_RANGE(jg_a + (ja >> 8) - p.join_ws, p.join_size, p.status)) va0 = jg_a[ja >> 8];
+                    if (far_a && (ja & 0xf00u) == 0u) asm volatile("prefetch.global.L1 [%0];" ::"l"(jg_a + (ja >> 8) + 32u));
+                    if (far_b && IL_IN_RANGE(jg_b + (jb >> 8) - p.join_ws, p.join_size, p.status)) vb0 = jg_b[jb >> 8];
+                    if (far_b && (jb & 0xf00u) == 0u) asm volatile("prefetch.global.L1 [%0];" ::"l"(jg_b + (jb >> 8) + 32u));
+                }
+                known0 = room0 && (end_a || have_a != ja) && (end_b || have_b != jb) && !(end_a && end_b);
+                va0 = end_a ? kInf : va0;
+                vb0 = end_b ? kInf : vb0;
+                from_a0 = (va0 | qmask) <= (vb0 | qmask);
+                jrec0 = from_a0 ? va0 : vb0;
+                // behind it: on its side the record after it, on the other side the same one as before
+                const uint32_t ja1 = ja + (from_a0 ? 256u : 0u), jb1 = jb + (from_a0 ? 0u : 256u);
+                const bool end_a1 = ja1 == join_na, end_b1 = jb1 == join_nb;
+                known1 = known0 && room1 && !far_a && !far_b && (end_a1 || have_a != ja1) && (end_b1 || have_b != jb1) && !(end_a1 && end_b1);
+                const uint64_t va = end_a1 ? kInf : from_a0 ? va1 : va0, vb = end_b1 ? kInf : from_a0 ? vb0 : vb1;
+                from_a1 = (va | qmask) <= (vb | qmask);
+                jrec1 = from_a1 ? va : vb;
+                jat0 = seen_cache + ((((uint32_t)jrec0 & imask) >> 5) & seen_mask) * 8u;
+                jat1 = seen_cache + ((((uint32_t)jrec1 & imask) >> 5) & seen_mask) * 8u;
+                je0 = lds64(jat0);                       // number of the word << 32 | word
+                je1 = lds64(jat1);
+            }
 
             // ---- examine record i, if it is there: it joins the open batch, or the open batch is closed and it
             // opens the next one
@@ -673,6 +691,27 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
             }
             prev = taken ? (uint32_t)rec & qmask : prev;
             i += taken ? 1u : 0u;
+
+            // ---- joins: the records are counted, and the last input of a query goes to the join's stage
+            if (JOIN) {
+                const uint32_t low0 = (uint32_t)jrec0 & qmask, low1 = (uint32_t)jrec1 & qmask;
+                const uint32_t w0 = (low0 & imask) >> 5, w1 = (low1 & imask) >> 5, mine0 = 1u << (low0 & 31u), mine1 = 1u << (low1 & 31u);
+                const bool both0 = goes_both(known0, low0);
+                bool both1 = goes_both(known1, low1);
+                const bool fresh = both0 && (uint32_t)(je0 >> 32) != w0;
+                if (fresh) new_word(je0, w0);
+                if (fresh || (both1 && (uint32_t)(je1 >> 32) != w1)) { known1 = false; both1 = false; }     // (next time)
+                sts64_if(both0, jat0, je0 ^ mine0);
+                if (both0 && jat0 == jat1) je1 ^= mine0;
+                sts64_if(both1, jat1, je1 ^ mine1);
+                const bool last0 = known0 && (!both0 || ((uint32_t)je0 & mine0) != 0u);
+                const bool last1 = known1 && (!both1 || ((uint32_t)je1 & mine1) != 0u);
+                sts64_shared_if(last0, slot0, jrec0);
+                sts64_shared_if(last1, last0 ? slot1 : slot0, jrec1);
+                ja += (known0 && from_a0 ? 256u : 0u) + (known1 && from_a1 ? 256u : 0u);
+                jb += (known0 && !from_a0 ? 256u : 0u) + (known1 && !from_a1 ? 256u : 0u);
+                tail_a += (last0 ? 256u : 0u) + (last1 ? 256u : 0u);
+            }
 
             // ---- hand on
             if (FEAS) miss_local += (late_fin > late_arr + slo_q) ? 1u : 0u;
@@ -736,13 +775,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
             qv = lds32(qb + ((e_idx & (nq - 1u)) << 7));
             // (the lane's own stores, so the words may come through L1: 32 of them with one miss)
             if (SPILL) ldg32_if(spill && i - e_idx > nq && IL_IN_RANGE(e_idx & gmask, gmask + 1ull, p.status), spill_ring + (e_idx & gmask), qv);
-            if (JOIN) {
-                __syncwarp();        // what was delivered is there for the joins' lanes
-                have_a = is_join ? lds32(jw_a) : 0u;
-                have_b = is_join ? lds32(jw_b) : 0u;
-                merge_step();        // two records: every query can come from both sides
-                merge_step();
-            }
+            if (JOIN) __syncwarp();      // what was delivered is there for the joins' lanes
         };
         if (any_spill) {
 #pragma unroll 1
