@@ -23,6 +23,7 @@ static thread_local int g_last_cuda_error = 0;
 
 static constexpr int kCounters = 8;
 // device and pinned block: the counters, the status word, the largest replica count of a batch
+static constexpr int64_t kSmallResults = 4096;
 static constexpr size_t kCounterBytes = kCounters * sizeof(unsigned long long) + 2 * sizeof(int);
 
 struct il_estimator {
@@ -42,6 +43,7 @@ struct il_estimator {
     size_t smem = 0;
     int64_t slot_elems = 0;
 
+    char *d_bound = nullptr;           // the allocation that holds the bound inputs and the counters (pointers below)
     int64_t *d_arrival = nullptr;
     uint64_t *d_ptrace = nullptr;      // packed root stream
     uint64_t *d_ptrace_b = nullptr;    // the same with the branch bits inside each record (lane kernel)
@@ -78,7 +80,8 @@ struct il_estimator {
 
     // results that go to pinned memory behind the kernels of a call, so that a host entry point waits once
     void *copy_dst = nullptr; const void *copy_src = nullptr; size_t copy_bytes = 0;
-    char *h_out = nullptr; int64_t h_out_cap = 0;              // pinned: 16 bytes per candidate
+    char *h_small = nullptr;                                   // pinned: 16 bytes for each of kSmallResults candidates
+    char *h_out = nullptr; int64_t h_out_cap = 0;              // the same for larger batches
     il_stage_config *d_cfg = nullptr; int64_t d_cfg_cap = 0;   // staging for il_estimate
     int64_t *d_out = nullptr; int64_t d_out_cap = 0;           // [2][cap]
 
@@ -351,8 +354,7 @@ void configure_lane_rings(il_estimator *e)
 
 void free_device(il_estimator *e)
 {
-    cudaFree(e->d_arrival); cudaFree(e->d_ptrace); cudaFree(e->d_ptrace_b); cudaFree(e->d_bits); cudaFree(e->d_lat);
-    cudaFree(e->d_counters); cudaFree(e->d_envelope);
+    cudaFree(e->d_bound);
     cudaFree(e->own_ws); cudaFree(e->d_cfg); cudaFree(e->d_out);
     if (e->h_counters) cudaFreeHost(e->h_counters);
     if (e->h_out) cudaFreeHost(e->h_out);
@@ -440,11 +442,12 @@ static int ensure_staging(il_estimator *e, int64_t n_cand)
 static char *host_results(il_estimator *e, int64_t n_cand)
 {
     constexpr int64_t kMost = 32768;
+    if (n_cand <= kSmallResults) return e->h_small;
     if (n_cand > kMost) return nullptr;
     if (e->h_out_cap < n_cand) {
         if (e->h_out) cudaFreeHost(e->h_out);
         e->h_out = nullptr; e->h_out_cap = 0;
-        const int64_t cap = std::min(kMost, std::max<int64_t>(1024, 2 * n_cand));
+        const int64_t cap = std::min(kMost, 2 * n_cand);
         if (cudaMallocHost(&e->h_out, (size_t)cap * 16) != cudaSuccess) { cudaGetLastError(); e->h_out = nullptr; return nullptr; }
         e->h_out_cap = cap;
     }
@@ -919,17 +922,20 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
     const bool can_pack = tr->arrival_us[n - 1] + worst < (INT64_C(1) << (63 - qbits));
 
     int dev = 0;
-    cudaDeviceProp prop;
+    int major = 0, sms = 0, smem_per_sm = 0, smem_per_cta = 0;
     IL_CUDA(cudaGetDevice(&dev));
-    IL_CUDA(cudaGetDeviceProperties(&prop, dev));
-    if (prop.major != 10) { g_last_cuda_error = (int)cudaErrorNoKernelImageForDevice; return IL_ERR_CUDA; }
+    IL_CUDA(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev));
+    IL_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    IL_CUDA(cudaDeviceGetAttribute(&smem_per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
+    IL_CUDA(cudaDeviceGetAttribute(&smem_per_cta, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    if (major != 10) { g_last_cuda_error = (int)cudaErrorNoKernelImageForDevice; return IL_ERR_CUDA; }
 
     il_estimator *e = new (std::nothrow) il_estimator();
     if (!e) return IL_ERR_NOMEM;
     e->device = dev;
-    e->num_sms = prop.multiProcessorCount;
-    e->smem_per_sm = prop.sharedMemPerMultiprocessor;
-    e->smem_per_cta = prop.sharedMemPerBlockOptin;
+    e->num_sms = sms;
+    e->smem_per_sm = (size_t)smem_per_sm;
+    e->smem_per_cta = (size_t)smem_per_cta;
     e->S = S; e->H = H; e->Bmax = B; e->n = n;
     e->n_pad = (n + 31) / 32 * 32;
     e->span_us = (float)std::max<int64_t>(1, tr->arrival_us[n - 1] - tr->arrival_us[0]);
@@ -1066,48 +1072,59 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
         g_last_cuda_error = (int)e_;                                      \
         return fail(e_ == cudaErrorMemoryAllocation ? IL_ERR_NOMEM : IL_ERR_CUDA); } } while (0)
 
-    IL_CUDA_E(cudaMalloc(&e->d_arrival, (size_t)n * 8));
-    IL_CUDA_E(cudaMalloc(&e->d_bits, (size_t)n));
     e->can_pack = can_pack;
     const int64_t latest = tr->arrival_us[n - 1] + worst;
     // lane kernel: its words stay below 0x7fe0 << 48; a lane counts its records in bytes of rings and slab rows
     e->lane_ok = can_pack && latest < (INT64_C(0x7fe0000000000000) >> qbits) && n < (INT64_C(1) << (e->join ? 24 : 29));
     bp.qbits = qbits;
+    // Branch bits inside the records, where the time range leaves room for them: a stage of the lane
+    // kernel then routes a query by the record it hands on instead of looking its bits up.
+    int nb = 0;
+    for (int s = 0; s < S; s++) {
+        if (pr->cond_bit[s] >= 0) nb = std::max(nb, (int)pr->cond_bit[s] + 1);
+        if (jn && jn->parent2[s] >= 0 && jn->cond_bit2[s] >= 0) nb = std::max(nb, (int)jn->cond_bit2[s] + 1);
+    }
+    const bool with_bits_inside = can_pack && nb > 0 && tr->branch_bits && qbits + nb <= 31 &&
+                                  latest < (INT64_C(0x7fe0000000000000) >> (qbits + nb));
+    // the packed trace is padded with "never" records to whole tiles, so that bulk copies always move full tiles
+    const int64_t tile = trace_tile_records();
+    const int64_t n_padded = can_pack ? (n + tile - 1) / tile * tile : 0;
+
+    // All bound inputs and counters are one device allocation, and what comes back to the host one pinned one, with
+    // room for the results of small batches: each allocation costs more than its few copies.
+    size_t size = 0;
+    auto place = [&](size_t bytes) { const size_t at = size; size = align_up(size + bytes, 256); return at; };
+    const size_t o_arrival = place((size_t)n * 8), o_bits = place((size_t)n), o_ptrace = place((size_t)n_padded * 8);
+    const size_t o_ptrace_b = place(with_bits_inside ? (size_t)n_padded * 8 : 0), o_lat = place(e->smem);
+    const size_t o_counters = place(kCounterBytes), o_envelope = place(envelope_max_windows() * sizeof(int));
+    IL_CUDA_E(cudaMalloc(&e->d_bound, size));
+    e->d_arrival = reinterpret_cast<int64_t *>(e->d_bound + o_arrival);
+    e->d_bits = reinterpret_cast<uint8_t *>(e->d_bound + o_bits);
+    e->d_lat = reinterpret_cast<int32_t *>(e->d_bound + o_lat);
+    e->d_counters = reinterpret_cast<unsigned long long *>(e->d_bound + o_counters);
+    e->d_status = reinterpret_cast<int *>(e->d_counters + kCounters);
+    e->d_maxrep = e->d_status + 1;
+    e->d_envelope = reinterpret_cast<int *>(e->d_bound + o_envelope);
+    const size_t h_head = (kCounters + 2) * sizeof(unsigned long long) + envelope_max_windows() * sizeof(int);
+    IL_CUDA_E(cudaMallocHost(&e->h_counters, h_head + (size_t)kSmallResults * 16));
+    e->h_status = reinterpret_cast<int *>(e->h_counters + kCounters);
+    e->h_envelope = reinterpret_cast<int *>(e->h_counters + kCounters + 2);
+    e->h_small = reinterpret_cast<char *>(e->h_counters) + h_head;
     if (can_pack) {
-        // padded with "never" records to whole tiles, so that bulk copies always move full tiles
-        const int64_t tile = trace_tile_records();
-        const int64_t n_padded = (n + tile - 1) / tile * tile;
+        e->d_ptrace = reinterpret_cast<uint64_t *>(e->d_bound + o_ptrace);
         std::vector<uint64_t> packed((size_t)n_padded, ~0ull);
         for (int64_t i = 0; i < n; i++)
             packed[(size_t)i] = ((uint64_t)tr->arrival_us[i] << qbits) | (uint64_t)i;
-        IL_CUDA_E(cudaMalloc(&e->d_ptrace, (size_t)n_padded * 8));
         IL_CUDA_E(cudaMemcpy(e->d_ptrace, packed.data(), (size_t)n_padded * 8, cudaMemcpyHostToDevice));
-        // Branch bits inside the records, where the time range leaves room for them: a stage of the lane
-        // kernel then routes a query by the record it hands on instead of looking its bits up.
-        int nb = 0;
-        for (int s = 0; s < pr->n_stages; s++)
-        {
-            if (pr->cond_bit[s] >= 0) nb = std::max(nb, (int)pr->cond_bit[s] + 1);
-            if (jn && jn->parent2[s] >= 0 && jn->cond_bit2[s] >= 0) nb = std::max(nb, (int)jn->cond_bit2[s] + 1);
-        }
-        if (nb > 0 && tr->branch_bits && qbits + nb <= 31 &&
-            latest < (INT64_C(0x7fe0000000000000) >> (qbits + nb))) {
+        if (with_bits_inside) {
+            e->d_ptrace_b = reinterpret_cast<uint64_t *>(e->d_bound + o_ptrace_b);
             for (int64_t i = 0; i < n; i++)
                 packed[(size_t)i] = ((uint64_t)tr->arrival_us[i] << (qbits + nb)) |
                                     ((uint64_t)(tr->branch_bits[i] & ((1u << nb) - 1u)) << qbits) | (uint64_t)i;
-            IL_CUDA_E(cudaMalloc(&e->d_ptrace_b, (size_t)n_padded * 8));
             IL_CUDA_E(cudaMemcpy(e->d_ptrace_b, packed.data(), (size_t)n_padded * 8, cudaMemcpyHostToDevice));
             e->rec_bits = nb;
         }
     }
-    IL_CUDA_E(cudaMalloc(&e->d_lat, e->smem));
-    IL_CUDA_E(cudaMalloc(&e->d_counters, kCounterBytes));
-    e->d_status = reinterpret_cast<int *>(e->d_counters + kCounters);
-    e->d_maxrep = e->d_status + 1;
-    IL_CUDA_E(cudaMalloc(&e->d_envelope, envelope_max_windows() * sizeof(int)));
-    IL_CUDA_E(cudaMallocHost(&e->h_counters, (kCounters + 2) * sizeof(unsigned long long) + envelope_max_windows() * sizeof(int)));
-    e->h_status = reinterpret_cast<int *>(e->h_counters + kCounters);
-    e->h_envelope = reinterpret_cast<int *>(e->h_counters + kCounters + 2);
     IL_CUDA_E(cudaMemcpy(e->d_arrival, tr->arrival_us, (size_t)n * 8, cudaMemcpyHostToDevice));
     if (tr->branch_bits) IL_CUDA_E(cudaMemcpy(e->d_bits, tr->branch_bits, (size_t)n, cudaMemcpyHostToDevice));
     else IL_CUDA_E(cudaMemset(e->d_bits, 0, (size_t)n));
