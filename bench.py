@@ -46,25 +46,25 @@ WORKLOADS = {
 # proportion to the query-events processed).  Each entry names the SHA-256 of the kernel source it was taken
 # from; when the source in the tree differs, the figures that depend on the capture are reported as null.
 NCU_CAPTURES = {
-    # whole streams (workloads 1, 2, 3, 5): 16,384 candidates x 8,000 queries of workload 2, all warp slots busy
+    # chains of up to one warp per scheduler (workloads 1, 2): 4,096 candidates x 20,000 queries of workload 2
     "des_lane_kernel": {
         "source": "paper_1812_01776_b200/csrc/des_lane_kernel.cu",
-        "source_sha256": "7ced5906c1a2907bed48cee1217576a44e88a55664f1015da071eca0aecef96a",
-        "dram_bytes_per_query_event": 8.84, "warp_inst_per_query_event": 6.89,
-        "summary": "profiles/des_lane_kernel_config2.md"},
-    # stream rings (workload 4): 3,552 candidates x 20,000 queries of workload 4, all warp slots busy
-    "des_lane_kernel:rings": {
+        "source_sha256": "7c5d8eda70d2d6a3b452f671d6087725aa77045bc2ca4c3b338c9e5c125cbf32",
+        "dram_bytes_per_query_event": 1.84, "warp_inst_per_query_event": 4.37,
+        "summary": "profiles/des_lane_kernel.md"},
+    # two to three warps per scheduler (workload 4): 4,096 candidates x 20,000 queries of workload 4
+    "des_lane_kernel:long": {
         "source": "paper_1812_01776_b200/csrc/des_lane_kernel.cu",
-        "source_sha256": "7ced5906c1a2907bed48cee1217576a44e88a55664f1015da071eca0aecef96a",
-        "dram_bytes_per_query_event": 8.99, "warp_inst_per_query_event": 7.68,
-        "summary": "profiles/des_lane_kernel_config4_rings.md"},
-    # pipelines with branch points (workloads 3, 5; a lane idles while its stage has no query): 5,920 candidates x
-    # 20,000 queries of workload 3, all warp slots busy
+        "source_sha256": "7c5d8eda70d2d6a3b452f671d6087725aa77045bc2ca4c3b338c9e5c125cbf32",
+        "dram_bytes_per_query_event": 0.74, "warp_inst_per_query_event": 4.16,
+        "summary": "profiles/des_lane_kernel.md"},
+    # pipelines with branch points (workloads 3, 5; a lane idles while its stage has no query): 7,001 candidates x
+    # 20,000 queries of workload 3
     "des_lane_kernel:tree": {
         "source": "paper_1812_01776_b200/csrc/des_lane_kernel.cu",
-        "source_sha256": "7ced5906c1a2907bed48cee1217576a44e88a55664f1015da071eca0aecef96a",
-        "dram_bytes_per_query_event": 8.84, "warp_inst_per_query_event": 12.74,
-        "summary": "profiles/des_lane_kernel_config3_branch_bits.md"},
+        "source_sha256": "7c5d8eda70d2d6a3b452f671d6087725aa77045bc2ca4c3b338c9e5c125cbf32",
+        "dram_bytes_per_query_event": 2.09, "warp_inst_per_query_event": 7.81,
+        "summary": "profiles/des_lane_kernel.md"},
     "des_packed_kernel": {
         "source": "paper_1812_01776_b200/csrc/des_packed_kernel.cu",
         "source_sha256": "",       # not captured again since the kernel got its node-stage entry and checks
@@ -111,11 +111,11 @@ def reduce_sum(values, dist=None, device=None):
     return t.tolist()
 
 
-def ncu_capture(kernel: str, rings: bool = False, tree: bool = False):
+def ncu_capture(kernel: str, long: bool = False, tree: bool = False):
     """The capture record of `kernel` if it still describes the source in the tree, else None."""
     import hashlib
     name = kernel.split("<")[0]
-    cap = NCU_CAPTURES.get(name + ":rings") if rings else (NCU_CAPTURES.get(name + ":tree") if tree else None)
+    cap = NCU_CAPTURES.get(name + ":long") if long else (NCU_CAPTURES.get(name + ":tree") if tree else None)
     cap = cap or NCU_CAPTURES.get(name)
     if not cap:
         return None
@@ -362,21 +362,18 @@ def measure(il, torch, w, dev, stream, flush, steps, warmup, e2e_steps, variant,
     total_events = events_per_cand * n_cand
     rec_bytes = 12 if kernel == "des_kernel" else 8  # separate time/query streams, else one 64-bit record
     slab_bytes = 8 * n * n_cand                       # written once by the simulation, read once by the select
-    stream_bytes = (events_per_cand - n) * 2 * rec_bytes * n_cand   # written once, read once
-    # the lane kernel keeps its streams in rings when whole streams of all resident candidates pass 48 GiB
-    rings = kernel == "des_lane_kernel" and (events_per_cand - n) * 8 * 148 * 8 * (32 // S) > 48 * 2**30
-    cap = None if shared else ncu_capture(kernel, rings, tree=bool((w.cond_bit >= 0).any()))
+    # the lane kernel keeps the streams between stages in shared memory; the others write and read them once
+    stream_bytes = 0 if kernel == "des_lane_kernel" else (events_per_cand - n) * 2 * rec_bytes * n_cand
+    cap = None if shared else ncu_capture(kernel, long=S == 10, tree=bool((w.cond_bit >= 0).any()))
     alu_peak = issue_rate * 32.0
-    hbm_note = ("latency slab written once + every inter-stage stream record written once "
+    hbm_note = ("latency slab written once" if kernel == "des_lane_kernel" else
+                "latency slab written once + every inter-stage stream record written once "
                 "and read once (the streams are this design's, not the method's)")
     if shared:
-        # only the simulated stage runs move data: per run its arrival stream read and its output written
-        # (about 16 B per simulated query-event); the method's own count does not apply
-        simulated_events = total_events * st["stage_runs"] / float(n_cand * S)
-        stream_bytes = 16.0 * simulated_events
-        slab_bytes = 0
-        hbm_note = ("shared prefixes: about 16 B per SIMULATED query-event (stage_runs_simulated / "
-                    "stage_runs_of_the_method of the method's count)")
+        # one slab row per covering candidate; the method's own count does not apply
+        stream_bytes = 0
+        slab_bytes = 8 * n * st["stage_runs"] / float(S)
+        hbm_note = "shared prefixes: latency rows of the covering candidates written once"
     rec = {
         "candidates": n_cand, "queries": n, "stages": S, "query_events_per_candidate": events_per_cand,
         "kernel": kernel, "workspace_bytes": ws_bytes, "steps": steps, "warmup": warmup,
