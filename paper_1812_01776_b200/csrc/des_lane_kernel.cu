@@ -87,6 +87,7 @@ constexpr int kX = 8;                         // records of a stream between two
 constexpr uint32_t kLast = 0x80000000u;       // flag of a batch's last record in that ring
 constexpr int kAhead = 64;                    // records of the trace a root has before it: two long turns, a power of two
 constexpr int kTurn = 16, kLongTurn = 32;     // iterations between two looks at finished groups, spills, bounds
+constexpr int kQuickTurn = 8;                 // the same while a stage is about to start or to end
 
 __device__ __forceinline__ uint64_t lds64(uint32_t a)
 {
@@ -357,7 +358,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
     uint32_t ja = 0, jb = 0;     // joins: records of either incoming stream consumed
     uint32_t seen_new = 0;       // joins: words of the queries' bits from here on have not been touched
     uint32_t turns = 1, turns_hi = 0;        // iteration bound, in turns
-    bool any_spill = false;
+    bool any_spill = false, quick = false;
     uint64_t late_fin = 0, late_arr = 0;     // feasibility only: finish and arrival record of a query that has just left
     uint32_t miss_local = 0;
 
@@ -533,8 +534,12 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
             if (__all_sync(full, exhausted)) break;
         }
         any_spill = __any_sync(full, spill);
+        // (a stage waits for the next turn to open its first batch and to close its last one)
+        if (!JOIN) quick = __any_sync(full, (i != n_cur && !started) || (i == n_cur && bm != ~0u));
+        } else {
+            quick = false;
         }
-        const int turn_its = __any_sync(full, i - low > long_reach) ? kTurn : kLongTurn;
+        const int turn_its = quick ? kQuickTurn : __any_sync(full, i - low > long_reach) ? kTurn : kLongTurn;
 
         // The root's next records: requested two turns before their use, by all lanes of the group.
         {
