@@ -24,6 +24,9 @@ static thread_local int g_last_cuda_error = 0;
 static constexpr int kCounters = 8;
 // device and pinned block: the counters, the status word, the largest replica count of a batch
 static constexpr int64_t kSmallResults = 4096;
+static constexpr size_t kSmallConfigBytes = 65536;
+// the least candidates that are looked over for shared prefixes
+static constexpr int64_t kShareMinCandidates = 2048;
 static constexpr size_t kCounterBytes = kCounters * sizeof(unsigned long long) + 2 * sizeof(int);
 
 struct il_estimator {
@@ -80,6 +83,7 @@ struct il_estimator {
 
     // results that go to pinned memory behind the kernels of a call, so that a host entry point waits once
     void *copy_dst = nullptr; const void *copy_src = nullptr; size_t copy_bytes = 0;
+    il_stage_config *h_cfg = nullptr;                          // pinned: configurations of a small batch
     char *h_small = nullptr;                                   // pinned: 16 bytes for each of kSmallResults candidates
     char *h_out = nullptr; int64_t h_out_cap = 0;              // the same for larger batches
     il_stage_config *d_cfg = nullptr; int64_t d_cfg_cap = 0;   // staging for il_estimate
@@ -454,6 +458,17 @@ static char *host_results(il_estimator *e, int64_t n_cand)
     return e->h_out;
 }
 
+// Small batches for the lane kernel stay in pinned host memory: a lane reads its configuration once per candidate and
+// 16 bytes come back for each, which costs less across the bus than two copies and their gaps (64 candidates x 2,000
+// queries: 50 instead of 61 us around the simulation).  nullptr where the batch is larger or goes elsewhere.
+static const il_stage_config *small_configs(il_estimator *e, const il_stage_config *configs, int64_t n_cand)
+{
+    const size_t bytes = (size_t)n_cand * e->S * sizeof(il_stage_config);
+    if (!is_lane(e) || n_cand >= kShareMinCandidates || bytes > kSmallConfigBytes) return nullptr;
+    memcpy(e->h_cfg, configs, bytes);
+    return e->h_cfg;
+}
+
 // The largest replica count among host configurations, 0 if one of them is out of range.
 static int check_configs(const il_estimator *e, const il_stage_config *configs, int64_t total)
 {
@@ -706,7 +721,6 @@ static int shared_by_cover(il_estimator *e, const SharedCommon &c, char *ws, siz
 // count are put together from the nodes where its queries leave (prefix_kernel.cu).  Used when the
 // node count is at most a quarter of candidates x stages (exhaustive sweeps over per-stage choices);
 // *used tells whether the batch was evaluated here.
-constexpr int64_t kShareMinCandidates = 2048;
 constexpr int kShareMaxTop = 16384;
 
 static int estimate_shared(il_estimator *e, const il_stage_config *d_configs, int64_t n_cand, int64_t slo_us,
@@ -1106,10 +1120,11 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
     e->d_maxrep = e->d_status + 1;
     e->d_envelope = reinterpret_cast<int *>(e->d_bound + o_envelope);
     const size_t h_head = (kCounters + 2) * sizeof(unsigned long long) + envelope_max_windows() * sizeof(int);
-    IL_CUDA_E(cudaMallocHost(&e->h_counters, h_head + (size_t)kSmallResults * 16));
+    IL_CUDA_E(cudaMallocHost(&e->h_counters, h_head + (size_t)kSmallResults * 16 + kSmallConfigBytes));
     e->h_status = reinterpret_cast<int *>(e->h_counters + kCounters);
     e->h_envelope = reinterpret_cast<int *>(e->h_counters + kCounters + 2);
     e->h_small = reinterpret_cast<char *>(e->h_counters) + h_head;
+    e->h_cfg = reinterpret_cast<il_stage_config *>(e->h_small + (size_t)kSmallResults * 16);
     if (can_pack) {
         e->d_ptrace = reinterpret_cast<uint64_t *>(e->d_bound + o_ptrace);
         std::vector<uint64_t> packed((size_t)n_padded, ~0ull);
@@ -1293,7 +1308,7 @@ static int estimate_device(il_estimator *e, const il_stage_config *d_configs, in
     if (rc) return rc;
 
     cudaStream_t st = e->stream;
-    IL_CUDA(cudaEventRecord(e->events[0], st));
+    if (!is_lane(e)) IL_CUDA(cudaEventRecord(e->events[0], st));      // (before the ordering kernel)
 
     int64_t launches = e->setup_launches;
     for (int64_t ch = 0; ch < n_chunks; ch++) {
@@ -1331,12 +1346,11 @@ static int estimate_device(il_estimator *e, const il_stage_config *d_configs, in
         IL_CUDA(cudaEventRecord(e->events[4 + 3 * ch], st));
         launches++;
     }
-    IL_CUDA(cudaEventRecord(e->events[1], st));
     rc = end_call(e);
     if (rc) return rc;
 
     float ms = 0.f;
-    IL_CUDA(cudaEventElapsedTime(&ms, e->events[0], e->events[1]));
+    IL_CUDA(cudaEventElapsedTime(&ms, e->events[is_lane(e) ? 2 : 0], e->events[1 + 3 * n_chunks]));
     e->stats.total_ms = ms;
     for (int64_t ch = 0; ch < n_chunks; ch++) {
         IL_CUDA(cudaEventElapsedTime(&ms, e->events[2 + 3 * ch], e->events[3 + 3 * ch]));
@@ -1413,11 +1427,20 @@ int il_estimate(il_estimator *e, const il_stage_config *configs, int64_t n_cand,
     const int max_replicas = check_configs(e, configs, total);
     if (max_replicas < 1) return IL_ERR_BAD_CONFIG;
     IL_CUDA(cudaSetDevice(e->device));
+    char *h = host_results(e, n_cand);
+    const il_stage_config *small = small_configs(e, configs, n_cand);
+    if (small && h == e->h_small) {
+        int64_t *res = reinterpret_cast<int64_t *>(h);
+        const int rc = estimate_device(e, small, n_cand, slo_us, res, res + n_cand, max_replicas);
+        if (rc) return rc;
+        memcpy(out_p99, res, (size_t)n_cand * 8);
+        memcpy(out_miss, res + n_cand, (size_t)n_cand * 8);
+        return IL_OK;
+    }
     int rc0 = ensure_staging(e, n_cand);
     if (rc0) return rc0;
     IL_CUDA(cudaMemcpyAsync(e->d_cfg, configs, (size_t)total * sizeof(il_stage_config),
                             cudaMemcpyHostToDevice, e->stream));
-    char *h = host_results(e, n_cand);
     e->copy_dst = h; e->copy_src = e->d_out; e->copy_bytes = (size_t)n_cand * 16;
     const int rc = estimate_device(e, e->d_cfg, n_cand, slo_us, e->d_out, e->d_out + n_cand, max_replicas);
     e->copy_dst = nullptr;
@@ -1591,7 +1614,15 @@ int il_feasible(il_estimator *e, const il_stage_config *configs, int64_t n_cand,
     const int max_replicas = check_configs(e, configs, total);
     if (max_replicas < 1) return IL_ERR_BAD_CONFIG;
     IL_CUDA(cudaSetDevice(e->device));
-    int rc = ensure_staging(e, n_cand);
+    int rc = IL_OK;
+    const il_stage_config *small = e->fork ? nullptr : small_configs(e, configs, n_cand);
+    if (small) {
+        rc = feasible_device(e, small, n_cand, slo_us, reinterpret_cast<uint8_t *>(e->h_small), max_replicas, nullptr, nullptr);
+        if (rc) return rc;
+        memcpy(out_feasible, e->h_small, (size_t)n_cand);
+        return IL_OK;
+    }
+    rc = ensure_staging(e, n_cand);
     if (rc) return rc;
     IL_CUDA(cudaMemcpyAsync(e->d_cfg, configs, (size_t)total * sizeof(il_stage_config),
                             cudaMemcpyHostToDevice, e->stream));
