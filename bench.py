@@ -49,20 +49,20 @@ NCU_CAPTURES = {
     # chains of up to one warp per scheduler (workloads 1, 2): 4,096 candidates x 20,000 queries of workload 2
     "des_lane_kernel": {
         "source": "paper_1812_01776_b200/csrc/des_lane_kernel.cu",
-        "source_sha256": "ae093d540bf936352613606f82f6b10c264ff2dde1bcfa5bb1ad375320bb3c7c",
+        "source_sha256": "46a7f950bf256fd81ade833230ae768199cadba114bff277f918a1e3b338aabf",
         "dram_bytes_per_query_event": 1.84, "warp_inst_per_query_event": 4.37,
         "summary": "profiles/des_lane_kernel.md"},
     # two to three warps per scheduler (workload 4): 4,096 candidates x 20,000 queries of workload 4
     "des_lane_kernel:long": {
         "source": "paper_1812_01776_b200/csrc/des_lane_kernel.cu",
-        "source_sha256": "ae093d540bf936352613606f82f6b10c264ff2dde1bcfa5bb1ad375320bb3c7c",
+        "source_sha256": "46a7f950bf256fd81ade833230ae768199cadba114bff277f918a1e3b338aabf",
         "dram_bytes_per_query_event": 0.74, "warp_inst_per_query_event": 4.08,
         "summary": "profiles/des_lane_kernel.md"},
     # pipelines with branch points (workloads 3, 5; a lane idles while its stage has no query): 7,001 candidates x
     # 20,000 queries of workload 3
     "des_lane_kernel:tree": {
         "source": "paper_1812_01776_b200/csrc/des_lane_kernel.cu",
-        "source_sha256": "ae093d540bf936352613606f82f6b10c264ff2dde1bcfa5bb1ad375320bb3c7c",
+        "source_sha256": "46a7f950bf256fd81ade833230ae768199cadba114bff277f918a1e3b338aabf",
         "dram_bytes_per_query_event": 2.09, "warp_inst_per_query_event": 7.76,
         "summary": "profiles/des_lane_kernel.md"},
     "des_packed_kernel": {

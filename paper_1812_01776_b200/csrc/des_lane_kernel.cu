@@ -309,7 +309,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
     const uint32_t xj = is_join && lane_used ? xbw + (uint32_t)(j * L + s) * 8u : nowhere + (uint32_t)lane * 8u;
     const uint32_t xjm = is_join && lane_used ? (kX - 1) * 256u : 0u;
     const uint32_t gmask = (uint32_t)((1ull << p.lane_ring_log2) - 1ull);
-    uint32_t *spill_ring = reinterpret_cast<uint32_t *>(p.lane_ws) + ((wslot * 32 + lane) << p.lane_ring_log2);
+    uint32_t *spill_ring = reinterpret_cast<uint32_t *>(p.lane_ws) + ((wslot * (cpw * L) + lane) << p.lane_ring_log2);
     const unsigned long long n_cand = (unsigned long long)p.n_cand;
     const uint64_t slo_q = FEAS ? (uint64_t)p.slo_us << q : 0ull;   // the objective, aligned with a record's time field
     const unsigned long long limit =

@@ -160,17 +160,18 @@ int64_t cands_per_slot(const il_estimator *e, int64_t n_cand)
     return std::max<int64_t>(1, std::min<int64_t>(e->cpw, (n_cand + schedulers - 1) / schedulers));
 }
 
-size_t slot_time_bytes(const il_estimator *e)
+// Stream memory of a slot that holds cps candidates.  Lane kernel: a spill ring for every lane in use, and for joins the
+// bits of the queries of which one input has come in and the incoming streams.
+size_t slot_time_bytes(const il_estimator *e, int64_t cps)
 {
-    return is_lane(e) ? (size_t)32 * 4 << e->lane_ring_log2 : (size_t)e->slot_elems * 8;
+    return is_lane(e) ? (size_t)cps * (e->S + e->base.n_join) * 4 << e->lane_ring_log2 : (size_t)e->slot_elems * 8;
 }
-// joins on the lane kernel: per slot the bits of the queries of which one input has come in, and the incoming streams
-size_t slot_seen_bytes(const il_estimator *e) { return (size_t)e->cpw * e->base.n_join * e->base.join_seen_words * 4; }
-size_t slot_qid_bytes(const il_estimator *e)
+size_t slot_seen_bytes(const il_estimator *e, int64_t cps) { return (size_t)cps * e->base.n_join * e->base.join_seen_words * 4; }
+size_t slot_qid_bytes(const il_estimator *e, int64_t cps)
 {
-    return is_lane(e) ? slot_seen_bytes(e) + (size_t)e->cpw * e->base.join_elems * 8 : (size_t)e->slot_elems * 4;
+    return is_lane(e) ? slot_seen_bytes(e, cps) + (size_t)cps * e->base.join_elems * 8 : (size_t)e->slot_elems * 4;
 }
-size_t slot_bytes(const il_estimator *e) { return slot_time_bytes(e) + slot_qid_bytes(e); }
+size_t slot_bytes(const il_estimator *e, int64_t cps) { return slot_time_bytes(e, cps) + slot_qid_bytes(e, cps); }
 size_t cand_bytes(const il_estimator *e) { return (size_t)e->n_pad * 8 + 5; }   // slab row, order entry, overflow mark
 bool lane_fallback(const il_estimator *e) { return is_lane(e) && e->lane_wrap; }
 size_t fb_slot_bytes(const il_estimator *e) { return (size_t)e->slot_elems * 8; }
@@ -197,8 +198,8 @@ int64_t wanted_slots(const il_estimator *e, int64_t n_cand, int lane_slots)
 size_t layout(const il_estimator *e, Plan &pl)
 {
     size_t off = 0;
-    pl.off_time = off; off = align_up(off + (size_t)pl.slots * slot_time_bytes(e), 256);
-    pl.off_qid = off;  off = align_up(off + (size_t)pl.slots * slot_qid_bytes(e), 256);
+    pl.off_time = off; off = align_up(off + (size_t)pl.slots * slot_time_bytes(e, pl.cps), 256);
+    pl.off_qid = off;  off = align_up(off + (size_t)pl.slots * slot_qid_bytes(e, pl.cps), 256);
     pl.off_slab = off; off = align_up(off + (size_t)pl.chunk * e->n_pad * 8, 256);
     pl.off_order = off; off = align_up(off + (size_t)pl.chunk * 4, 256);
     pl.off_ovf = off;  off = align_up(off + (size_t)pl.chunk, 256);
@@ -216,24 +217,26 @@ int64_t fallback_slots(const il_estimator *e, size_t usable)
     return std::max<int64_t>(kWarpsPerCta, std::min<int64_t>(fit, (int64_t)e->num_sms * kWarpsPerCta));
 }
 
+size_t min_bytes(const il_estimator *e)
+{
+    Plan pl;
+    pl.cps = is_lane(e) ? e->cpw : 1;
+    pl.slots = warps_per_cta(e);
+    pl.chunk = 2 * warps_per_cta(e);
+    pl.fb_slots = lane_fallback(e) ? kWarpsPerCta : 0;
+    return layout(e, pl) + 2048;
+}
+
 size_t recommended_bytes(const il_estimator *e, int64_t n_cand)
 {
     Plan pl;
     n_cand = std::max<int64_t>(n_cand, 1);
     pl.slots = wanted_slots(e, n_cand, 16);
     const int64_t cps = cands_per_slot(e, n_cand);
+    pl.cps = cps;
     pl.chunk = std::max<int64_t>(std::min<int64_t>(n_cand, 8 * full_slots(e, 16) * cps), 2 * pl.slots * cps);
     pl.fb_slots = lane_fallback(e) ? (int64_t)e->num_sms * kWarpsPerCta : 0;
-    return layout(e, pl) + 2048;
-}
-
-size_t min_bytes(const il_estimator *e)
-{
-    Plan pl;
-    pl.slots = warps_per_cta(e);
-    pl.chunk = 2 * warps_per_cta(e);
-    pl.fb_slots = lane_fallback(e) ? kWarpsPerCta : 0;
-    return layout(e, pl) + 2048;
+    return std::max(layout(e, pl) + 2048, min_bytes(e));
 }
 
 // Splits `bytes` of workspace between warp slots and the latency slab.
@@ -243,12 +246,12 @@ bool make_plan(const il_estimator *e, size_t bytes, int64_t n_cand, Plan &pl)
     size_t usable = bytes - 1024;
     pl.fb_slots = fallback_slots(e, usable);
     if (pl.fb_slots > 0) usable -= (size_t)pl.fb_slots * fb_slot_bytes(e) + 256;
-    const size_t sb = slot_bytes(e), cb = cand_bytes(e);
     const int64_t w = warps_per_cta(e);
     const int64_t cps = cands_per_slot(e, n_cand);
+    const size_t sb = slot_bytes(e, cps), cb = cand_bytes(e);
     int64_t slots = std::min<int64_t>(wanted_slots(e, n_cand, e->lane_slots), (int64_t)(usable / (sb + 2 * cps * cb)));
-    slots = slots / w * w;
-    if (slots < w) return false;
+    slots = std::max(w, slots / w * w);
+    if ((size_t)slots * sb > usable) return false;
     pl.slots = slots;
     pl.cps = cps;
     pl.chunk = std::min<int64_t>(n_cand, (int64_t)((usable - (size_t)slots * sb) / cb));
@@ -500,10 +503,10 @@ static DesParams chunk_params(const il_estimator *e, const Plan &pl, char *ws, c
     p.lane_slots = e->lane_slots;
     p.cpw = (int32_t)pl.cps;
     if (e->join) {
-        const size_t seen = ((size_t)pl.slots * slot_seen_bytes(e) + 7) / 8 * 8;
+        const size_t seen = ((size_t)pl.slots * slot_seen_bytes(e, pl.cps) + 7) / 8 * 8;
         p.join_seen = reinterpret_cast<uint32_t *>(ws + pl.off_qid);
         p.join_ws = reinterpret_cast<uint64_t *>(ws + pl.off_qid + seen);
-        p.join_size = pl.slots * e->cpw * e->base.join_elems;
+        p.join_size = pl.slots * pl.cps * e->base.join_elems;
     }
     return p;
 }
@@ -1510,7 +1513,7 @@ static int feasible_device(il_estimator *e, const il_stage_config *d_configs, in
         }
     }
     const int64_t wpc = des_lane_warps_per_cta();
-    const size_t sb = slot_time_bytes(e);
+    const size_t sb = slot_time_bytes(e, cands_per_slot(e, n_cand));
     const size_t tail_bytes = align_up((size_t)n_cand, 256) + align_up((size_t)n_cand * 4, 256) + 1024;
     if (ws_bytes < tail_bytes + (size_t)wpc * sb) return IL_ERR_NOMEM;
     int64_t slots = std::min<int64_t>(wanted_slots(e, n_cand, e->lane_slots), (int64_t)((ws_bytes - tail_bytes) / sb)) / wpc * wpc;

@@ -73,7 +73,7 @@ struct DesParams {
     unsigned long long *counters; // [0] next candidate, [1] batches dispatched, [2] algorithmic ops
     int *status;                  // first error seen by any warp (0 = none)
     // lane-parallel kernel only (des_lane_kernel.cu)
-    uint64_t *lane_ws;            // [warp slots][32][2^lane_ring_log2] words: the lanes' spill rings
+    uint64_t *lane_ws;            // [warp slots][lanes in use][2^lane_ring_log2] words: the lanes' spill rings
     int32_t cpw;                  // candidates per warp, at most floor(32 / S)
     int32_t lane_slots;           // positions of a lane's batch ring in shared memory: 16 or 32, at least the
                                   // largest replica count among the launch's candidates
