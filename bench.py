@@ -72,7 +72,7 @@ NCU_CAPTURES = {
         "summary": "profiles/des_packed_kernel_config2.md"},
 }
 LANE_CTAS = None         # --lane-ctas: resident CTAs per SM of the lane kernel, for side measurements
-RING_LOG2 = None         # --ring-log2: ring length of the lane kernel's streams, for side measurements
+RING_LOG2 = None         # --ring-log2: length of the lane kernel's spill rings, for side measurements
 BITS_LOOKUP = False      # --bits-lookup: stages look the branch bits up instead of finding them in the records
 METRIC = "candidate_configs_per_s"
 UNIT = "candidates/s"
@@ -601,7 +601,7 @@ def main():
     ap.add_argument("--lane-ctas", type=int, default=None,
                     help="resident CTAs per SM of the lane kernel (side measurements; default 4)")
     ap.add_argument("--ring-log2", type=int, default=None,
-                    help="largest stream ring of the lane kernel, log2 records (side measurements; default 13)")
+                    help="largest spill ring of the lane kernel, log2 words (side measurements; default 13)")
     ap.add_argument("--bits-lookup", action="store_true",
                     help="lane kernel: stages look the queries' branch bits up by index instead of carrying them "
                          "in the stream records (side measurements)")

@@ -96,7 +96,7 @@ typedef struct il_estimator il_estimator;   /* opaque; owns its device copies */
  * cascade (the other queries leave there).  Two children that are not
  * alternatives -- both unconditional, or guarded by different bits -- are
  * fan-out: parallel branches.  Handles with fan-out run on the lane kernel
- * (whole streams) or the kernel with separate streams; the other kernel
+ * or the kernel with separate streams; the other kernel
  * choices, prefix sharing and the early exit of il_feasible fall back to those.
  * A stage that waits for the outputs of TWO stages (a join) is described with
  * il_join_edges and il_estimator_create_dag below.

@@ -1569,7 +1569,7 @@ static int feasible_device(il_estimator *e, const il_stage_config *d_configs, in
     rc = *e->h_status;
     const int64_t n_fb = (int64_t)e->h_counters[3];
     if (rc == IL_OK && n_fb > 0) {
-        // Rare: candidates the lane kernel gave up on (stream ring overflow).  They are evaluated in
+        // Rare: candidates the lane kernel gave up on (spill ring overflow).  They are evaluated in
         // full by the warp-per-candidate kernel; this path allocates its temporaries.
         char *tmp = nullptr;
         const size_t cfg_b = align_up((size_t)n_fb * e->S * sizeof(il_stage_config), 256);
