@@ -43,6 +43,14 @@ __device__ __forceinline__ int first_at(const int64_t *arrival, int lo, int hi, 
     return lo;
 }
 
+// The best count of a window in shared memory as it is now: the warps of the CTA raise it with atomicMax while others look.
+__device__ __forceinline__ int best_now(const int *best)
+{
+    int v;
+    asm volatile("ld.relaxed.cta.shared.s32 %0, [%1];" : "=r"(v) : "r"((unsigned)__cvta_generic_to_shared(best)) : "memory");
+    return v;
+}
+
 __global__ void __launch_bounds__(kEnvThreads) envelope_kernel(const __grid_constant__ EnvParams p)
 {
     __shared__ int end[kMaxWindows][kEnvGroups + 1];
@@ -68,8 +76,9 @@ __global__ void __launch_bounds__(kEnvThreads) envelope_kernel(const __grid_cons
     for (int k = threadIdx.x >> 5; k < W * kEnvGroups; k += kEnvThreads / 32) {
         const int w = k / kEnvGroups, g = k - w * kEnvGroups;
         const int64_t j = (int64_t)j0 + g * kEnvGroup;
-        if (j >= p.n || end[w][g + 1] - (int)j <= best[w]) continue;       // none of these 256 can be better
-        const int known = best[w];
+        // read once and shared by the warp: its lanes have to take the same way to the reduction below
+        const int known = __shfl_sync(0xffffffffu, best_now(&best[w]), 0);
+        if (j >= p.n || end[w][g + 1] - (int)j <= known) continue;       // none of these 256 can be better
         int count = 0;
 #pragma unroll
         for (int i = 0; i < kEnvGroup; i += 32) {
@@ -80,8 +89,7 @@ __global__ void __launch_bounds__(kEnvThreads) envelope_kernel(const __grid_cons
                 count = max(count, first_at(p.arrival, (int)m + known + 1, end[w][g + 1], a, p.window[w]) - (int)m);
         }
         count = __reduce_max_sync(0xffffffffu, count);
-        if (lane == 0 && count > best[w]) best[w] = max(count, atomicMax(&p.out[w], count));
-        __syncwarp();
+        if (lane == 0 && count > known) atomicMax(&best[w], max(count, atomicMax(&p.out[w], count)));
     }
 }
 

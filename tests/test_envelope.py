@@ -91,3 +91,19 @@ def test_gpu_envelope_around_group_sizes(oracle, n):
     a = w.arrival_us
     exp = [(np.searchsorted(a, a + int(win), side="left") - np.arange(n)).max() for win in wins]
     assert np.array_equal(got, exp)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [700, 4096, 9001])
+def test_gpu_envelope_where_the_best_count_keeps_rising(oracle, n):
+    """Arrivals that come closer and closer (and the same trace backwards): every group of starts beats the ones
+    before it, so the warps of a block raise the shared best counts while others read them."""
+    import paper_1812_01776_b200 as il
+    w = workloads.random_small(n, S=1, H=1, Bmax=1, n=n, C=1)
+    gaps = np.linspace(4000, 1, n).astype(np.int64)
+    wins = np.unique(np.geomspace(1, 10 ** 8, 40).astype(np.int64))
+    for step in (gaps, gaps[::-1]):
+        w.arrival_us = np.cumsum(step)
+        with il.Estimator.from_workload(w) as est:
+            got = est.traffic_envelope(wins)
+        assert np.array_equal(got, oracle.traffic_envelope(w.arrival_us, wins))
