@@ -107,7 +107,8 @@ __device__ __forceinline__ uint32_t lds32(uint32_t a)
 __device__ __forceinline__ bool before(uint64_t a, uint64_t b) { return __longlong_as_double((long long)a) < __longlong_as_double((long long)b); }
 __device__ __forceinline__ bool not_after(uint64_t a, uint64_t b) { return __longlong_as_double((long long)a) <= __longlong_as_double((long long)b); }
 
-// Words that two lanes share (stream records): each is complete in itself, so no ordering between words is needed.
+// Words that two lanes share.  Stream records, and the records in a join's windows: each is complete in itself, so no
+// ordering between words is needed.  A join's counts: stored behind the warp barrier that follows the records they cover.
 __device__ __forceinline__ uint64_t lds64_shared(uint32_t a)
 {
     uint64_t v;
@@ -195,7 +196,7 @@ __host__ __device__ inline size_t join_bytes(int cpw, int joins, int window) { r
 //       The incoming streams have no back-pressure -- either parent may have to run ahead of the other by all
 //       that the slower branch keeps in flight -- so they go to global memory whole, and the latest
 //       64 to 512 records of each to shared memory, from where the join nearly always reads them.  511 candidates
-//       of a diamond, 50,000 queries: 130 ms on the warp-per-candidate kernel, 65 ms here.
+//       of a diamond, 50,000 queries: 130 ms on the warp-per-candidate kernel, 53 ms here.
 template <bool BRANCHY, bool FEAS, bool FORK, bool JOIN>
 __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned char *smem_raw)
 {
@@ -550,11 +551,12 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
             fed = max(fed, to);
         }
 
-        // joins: a record for a join.  Records of its two streams are counted in bytes of a row, as tails are.
+        // joins: a record for a join.  Records of its two streams are counted in bytes of a row, as tails are.  The
+        // count is told to the join's lane at the top of the NEXT iteration, behind the barrier at the end of this one: whoever
+        // reads a count also sees the records it covers, in the window and in the global stream.
         auto deliver = [&](bool c, uint64_t *stream, uint32_t win, uint32_t tail, uint64_t rec) {
             stg64_if(c && IL_IN_RANGE(stream + (tail >> 8) - p.join_ws, p.join_size, p.status), stream + (tail >> 8), rec);
-            sts64_if(c, win + 8u + ((tail >> 5) & win_mask), rec);
-            sts32_if(c, win, tail + 256u);
+            sts64_shared_if(c, win + 8u + ((tail >> 5) & win_mask), rec);
         };
         // joins: one step of a join's lane takes up to two records of its two incoming streams (every query can come from
         // both sides), as long as what comes next on both sides is known.  The loads stand at the top of the
@@ -583,14 +585,17 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
         auto step = [&](auto spilling) {
             constexpr bool SPILL = decltype(spilling)::value;
             // ---- joins: what has come in, the next two records of either side, room for two
-            // (A parent may add one record to what have_a / have_b say before the barrier at the end.)
+            // (A parent may add one record to what have_a / have_b say before the barrier at the end; its place in the
+            // window is that of a record already taken, or of one that the count does not cover and whose value is not used.)
             uint32_t have_a = 0, have_b = 0, slot0 = 0, slot1 = 0;
             uint64_t va0 = 0, va1 = 0, vb0 = 0, vb1 = 0;
             bool room0 = false, room1 = false;
             if (JOIN) {
-                have_a = lds32(jw_a); have_b = lds32(jw_b);
-                va0 = lds64(jw_a + 8u + ((ja >> 5) & win_mask)); va1 = lds64(jw_a + 8u + (((ja + 256u) >> 5) & win_mask));
-                vb0 = lds64(jw_b + 8u + ((jb >> 5) & win_mask)); vb1 = lds64(jw_b + 8u + (((jb + 256u) >> 5) & win_mask));
+                sts32_shared_if(join_a && !is_join, jw_a, tail_a);
+                sts32_shared_if(join_b && !is_join, jw_b, tail_b);
+                have_a = lds32_shared(jw_a); have_b = lds32_shared(jw_b);
+                va0 = lds64_shared(jw_a + 8u + ((ja >> 5) & win_mask)); va1 = lds64_shared(jw_a + 8u + (((ja + 256u) >> 5) & win_mask));
+                vb0 = lds64_shared(jw_b + 8u + ((jb >> 5) & win_mask)); vb1 = lds64_shared(jw_b + 8u + (((jb + 256u) >> 5) & win_mask));
                 slot0 = xj | (tail_a & xjm); slot1 = xj | ((tail_a + 256u) & xjm);
                 room0 = is_join && (int)lds32_shared(slot0 + 4u) < 0;
                 room1 = (int)lds32_shared(slot1 + 4u) < 0;

@@ -99,3 +99,18 @@ def test_join_device_entry_chunks_and_static(il, oracle):
         miss = torch.full((64,), -1, dtype=torch.int64, device="cuda")
         il.il_estimate_device_static(est._h, d.data_ptr(), 64, w.slo_us, p99.data_ptr(), miss.data_ptr())
         assert np.array_equal(p99.cpu().numpy(), exp[0]) and np.array_equal(miss.cpu().numpy(), exp[1])
+
+
+@pytest.mark.parametrize("C", [1, 7, 700])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_join_level_with_its_parents(il, oracle, shape, C):
+    """Both branches as fast as each other and never busy: the join takes every record in the iteration after the one in
+    which it was delivered, so a count it read without the records it covers would show at once.  With one, a few and
+    all candidates per warp, over several lengths of the windows it reads from."""
+    w = workloads.join_small(11, n=2100, C=16, max_replicas=4, Bmax=4, shape=shape, tiny_times=True)
+    w.latency_us[:] = 1 + np.arange(w.latency_us.shape[2]) % 2
+    at = np.arange(C) % 16
+    exp = oracle.estimate_workload(w)
+    with il.Estimator.from_workload(w) as est:
+        p99, miss = est.estimate(w.configs[at], w.slo_us)
+        assert np.array_equal(p99, exp[0][at]) and np.array_equal(miss, exp[1][at])
