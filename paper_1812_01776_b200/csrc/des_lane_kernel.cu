@@ -537,6 +537,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
         any_spill = __any_sync(full, spill);
         // (a stage waits for the next turn to open its first batch and to close its last one)
         if (!JOIN) quick = __any_sync(full, (i != n_cur && !started) || (i == n_cur && bm != ~0u));
+        __syncwarp();     // a root's first position is empty before another lane of the group fills it again below
         } else {
             quick = false;
         }

@@ -49,6 +49,15 @@ def test_trace_lengths(oracle, n):
     same(w, oracle)
 
 
+@pytest.mark.parametrize("S", [1, 4, 9])
+@pytest.mark.parametrize("n", [63, 64, 65, 66, 96, 97, 127, 128, 129])
+def test_trace_lengths_around_a_root_s_stretch(oracle, n, S):
+    """Record 64 of the trace is copied to where record 0 was, in the turn in which that one opens its batch; by another
+    lane where the candidate has several."""
+    w = workloads.random_small(n + S, S=S, H=2, Bmax=8, n=n, C=700, max_replicas=3, qps=5000.0, lat_lo=1, lat_hi=3000)
+    same(w, oracle)
+
+
 @pytest.mark.parametrize("S", [1, 3])
 def test_more_candidates_than_resident_groups(oracle, S):
     w = workloads.random_small(S, S=S, H=2, Bmax=4, n=60, C=90_001, max_replicas=3)
