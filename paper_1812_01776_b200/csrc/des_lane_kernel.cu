@@ -166,7 +166,9 @@ __device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;
 // streams [kX][lane], a row of empty records (the "child" of a leaf), per warp the miss counts of the groups
 // (feasibility only), per warp the words of examined records [nq][lane], and per warp the next records of the trace
 // [kAhead][group].
-constexpr uint32_t kSmemBase = 1024;          // where a CTA's dynamic shared memory starts (checked by the kernel)
+// Where a CTA's dynamic shared memory starts with the toolkit at hand.  The host plans for it; a launch that finds it elsewhere
+// needs up to a row of batch keys more to align them and takes it from the words of examined records (more spills).
+constexpr uint32_t kSmemBase = 1024;
 __host__ __device__ inline uint32_t key_bytes(int kr) { return (uint32_t)kr * 256u; }
 constexpr uint32_t kXBytes = kX * 256u;
 __host__ __device__ inline size_t table_bytes(int rows, int Bmax) { return ((size_t)rows * (Bmax | 1) + 1) * 4; }
@@ -215,11 +217,18 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
     const int kr = p.lane_slots == 16 ? 16 : 32;      // batch ring positions of a lane
     const int S = p.S, cpw = p.cpw, rowlen = p.Bmax | 1;
     const int L = JOIN ? S + p.n_join : S;            // lanes of a candidate
+    uint32_t smem_bytes;
+    asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(smem_bytes));
+    const uint32_t smem_end = (uint32_t)__cvta_generic_to_shared(smem_raw) + smem_bytes;
+    smem_raw += p.smem_skip;
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem_raw);
-    if (sbase != kSmemBase) { atomicCAS(p.status, 0, IL_ERR_CUDA); return; }
     const uint32_t tab0 = sbase + 4u;
-    const uint32_t nq = (uint32_t)p.lane_words;       // words of examined records a lane keeps in shared memory
     const uint32_t rings = (sbase + (uint32_t)table_bytes(S * p.H, p.Bmax) + key_bytes(kr) - 1u) & ~(key_bytes(kr) - 1u);
+    // words of examined records a lane keeps in shared memory: half of what was planned where the rings start later than
+    // planned (they are at most 8 KB late, and half of the fewest words, 64 for each of 128 lanes, are 16 KB)
+    auto end_with = [&](int words) { return rings + (uint32_t)(ring_bytes(kr, words, cpw) + kTailBytes + join_bytes(cpw, p.n_join, p.join_window)); };
+    const uint32_t nq = (uint32_t)p.lane_words >> (end_with(p.lane_words) > smem_end ? 1 : 0);
+    if (end_with((int)nq) > smem_end) { atomicCAS(p.status, 0, IL_ERR_CUDA); return; }      // launched with less than planned
     const uint32_t kbw = rings + (uint32_t)wid * key_bytes(kr), kb = kbw + (uint32_t)lane * 8u;
     const uint32_t xb0 = rings + kLaneWarps * key_bytes(kr);
     const uint32_t xbw = xb0 + (uint32_t)wid * kXBytes, xb = xbw + (uint32_t)lane * 8u;

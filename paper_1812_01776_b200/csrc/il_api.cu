@@ -1219,6 +1219,11 @@ int il_set_test_knob(il_estimator *e, int knob, int64_t value)
         e->base.rec_bits = (value == 1 && e->d_ptrace_b) ? e->rec_bits : 0;
         return IL_OK;
     }
+    if (knob == IL_KNOB_SMEM_SKIP) {
+        if (value < 0 || value > 8192 || value % 16 != 0) return IL_ERR_INVALID_ARG;
+        e->base.smem_skip = (int32_t)value;
+        return IL_OK;
+    }
     if (knob == IL_KNOB_ITER_LIMIT) {
         if (value < 0) return IL_ERR_INVALID_ARG;
         e->iter_limit = (unsigned long long)value;

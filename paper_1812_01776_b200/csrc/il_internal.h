@@ -78,7 +78,8 @@ struct DesParams {
     int32_t lane_slots;           // positions of a lane's batch ring in shared memory: 16 or 32, at least the
                                   // largest replica count among the launch's candidates
     int32_t lane_ring_log2;       // a lane's spill ring in lane_ws holds 2^this words
-    int32_t lane_words;           // words of examined records a lane keeps in shared memory (a power of two)
+    int32_t lane_words;           // words of examined records a lane keeps in shared memory (a power of two, at least 64)
+    int32_t smem_skip;            // test knob: bytes left unused where shared memory starts (a multiple of 16, at most 8192)
     int32_t lane_wrap;            // the rings are shorter than the longest stream
     // lane kernel, joins: join_stage[0 .. n_join) are the stages with two incoming edges, join_no[s] their number
     int32_t n_join;

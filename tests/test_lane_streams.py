@@ -58,6 +58,28 @@ def test_trace_lengths_around_a_root_s_stretch(oracle, n, S):
     same(w, oracle)
 
 
+@pytest.mark.parametrize("skip", [16, 1024, 3072, 4080, 8192])
+@pytest.mark.parametrize("replicas", [3, 32])
+def test_shared_memory_that_starts_elsewhere(oracle, replicas, skip):
+    """The batch keys are aligned wherever shared memory starts; what that takes comes out of the words of examined records,
+    down to 32 a lane (here with more than that in flight, on a tree and with a join)."""
+    import paper_1812_01776_b200 as il
+    w = workloads.random_small(skip + replicas, S=6, H=3, Bmax=33, n=2500, C=48, max_replicas=replicas, tree=True, qps=3000.0,
+                               cv=4.0, lat_lo=500, lat_hi=90000)
+    j = workloads.join_small(replicas, n=1500, C=48, max_replicas=replicas, Bmax=8, shape="two_joins")
+    for x in (w, j):
+        exp = oracle.estimate_workload(x)
+        many = np.arange(20_000) % x.n_candidates                  # every resident CTA, and as few words as there can be
+        with il.Estimator.from_workload(x) as est:
+            est.set_test_knob(3, 2)
+            est.set_test_knob(6, skip)
+            a, b = est.estimate(x.configs[many], x.slo_us)
+            assert np.array_equal(a, exp[0][many]) and np.array_equal(b, exp[1][many])
+            assert np.array_equal(est.feasible(x.configs[many], x.slo_us), exp[0][many] <= x.slo_us)
+            with pytest.raises(Exception):
+                est.set_test_knob(6, 8)
+
+
 @pytest.mark.parametrize("S", [1, 3])
 def test_more_candidates_than_resident_groups(oracle, S):
     w = workloads.random_small(S, S=S, H=2, Bmax=4, n=60, C=90_001, max_replicas=3)
