@@ -599,7 +599,7 @@ def main():
     ap.add_argument("--no-per-workload", action="store_true",
                     help="skip the short measurements of the other workloads")
     ap.add_argument("--lane-ctas", type=int, default=None,
-                    help="resident CTAs per SM of the lane kernel (side measurements; default 4)")
+                    help="resident CTAs per SM of the lane kernel at most (side measurements; default: as many as fit)")
     ap.add_argument("--ring-log2", type=int, default=None,
                     help="largest spill ring of the lane kernel, log2 words (side measurements; default 13)")
     ap.add_argument("--bits-lookup", action="store_true",

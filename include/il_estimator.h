@@ -420,8 +420,8 @@ IL_API int il_set_variant(il_estimator *est, int variant);
  *                           preconditions hold; 2: never; 3: always, and the distinct stage runs are
  *                           simulated one by one even where a covering set of whole candidates on
  *                           the lane kernel would do.
- *   IL_KNOB_LANE_CTAS       value 0..16: resident CTAs (of four warps) per SM of the lane kernel; 0 restores
- *                           the library's choice (4).  For measurements.
+ *   IL_KNOB_LANE_CTAS       value 0..16: resident CTAs (of four warps) per SM of the lane kernel at most; 0 restores
+ *                           the library's choice, as many as fit (two or three).  For measurements.
  *   IL_KNOB_BITS_IN_RECORDS value 0 or 1: whether the lane kernel's stream records carry the queries' branch
  *                           bits (1, the default where the time range leaves room) or every stage looks
  *                           them up by query index (0).  Same results either way.

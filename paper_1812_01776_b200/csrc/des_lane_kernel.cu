@@ -883,12 +883,13 @@ size_t des_lane_smem(int table_rows, int Bmax, int ring_slots, int ring_words, i
            kSmemBase + ring_bytes(ring_slots, ring_words, cpw) + kTailBytes + join_bytes(cpw, joins, window);
 }
 
-int des_lane_max_ctas_per_sm(size_t smem)
+int des_lane_max_ctas_per_sm(size_t smem, bool joins)
 {
     int n = 0;
-    if (cudaFuncSetAttribute(des_lane_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, des_lane_kernel<true, true>, kLaneWarps * 32, smem);
+    // (all instantiations without joins are compiled for three CTAs; the one with joins takes more registers)
+    void (*kernel)(DesParams) = joins ? lanes::des_kernel : des_lane_kernel<true, true>;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kLaneWarps * 32, smem);
     return e == cudaSuccess ? n : 0;
 }
 

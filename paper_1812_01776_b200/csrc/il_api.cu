@@ -67,7 +67,7 @@ struct il_estimator {
     int ctas_lane[2] = {0, 0};         // lane kernel with 16 / 32 batch ring positions per lane: CTAs that fit an SM
     int lane_slots = 32;               // batch ring positions used by the current call
     int64_t setup_launches = 0;        // kernels a call launched before its simulation: the replica reduction, the node probe
-    int lane_ctas_knob = 0;            // test knob: resident CTAs per SM of the lane kernel (0: the library's choice)
+    int lane_ctas_knob = 0;            // test knob: resident CTAs per SM of the lane kernel at most (0: as many as fit)
     int *d_maxrep = nullptr;           // device word behind the status: largest replica count of a batch
     uint8_t *d_bits = nullptr;
     int32_t *d_lat = nullptr;
@@ -113,9 +113,6 @@ struct Plan {
 };
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
-
-// Resident CTAs (of four warps) per SM for the lane kernel: what shared memory holds, at most four.
-constexpr int kLaneCtasPerSm = 4;
 
 // Words of examined records a lane keeps in shared memory before it spills: this many where the grid needs every
 // resident CTA, more where it leaves shared memory unused.
@@ -178,8 +175,9 @@ size_t fb_slot_bytes(const il_estimator *e) { return (size_t)e->slot_elems * 8; 
 
 int lane_ctas(const il_estimator *e, int lane_slots)
 {
+    // as many (of four warps each) as registers and shared memory hold: three with few candidates per warp and small tables, two with joins
     const int fit = e->ctas_lane[lane_slots == 16 ? 0 : 1];
-    return std::max(1, std::min(fit, e->lane_ctas_knob > 0 ? e->lane_ctas_knob : kLaneCtasPerSm));
+    return e->lane_ctas_knob > 0 ? std::min(fit, e->lane_ctas_knob) : fit;
 }
 
 // Warp slots that can be resident at once; the lane kernel has more of them with 16 batch ring positions per lane.
@@ -1156,9 +1154,10 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
     e->ctas_per_sm_packed = des_packed_max_ctas_per_sm(false, e->smem);
     e->ctas_per_sm_staged = des_packed_max_ctas_per_sm(true, e->smem);
     for (int k = 0; k < 2; k++) {
-        e->ctas_lane[k] = des_lane_max_ctas_per_sm(des_lane_smem(S * H, B, k == 0 ? 16 : 32, kLaneWords, e->cpw, e->base.n_join, kJoinWindow));
+        e->ctas_lane[k] = des_lane_max_ctas_per_sm(des_lane_smem(S * H, B, k == 0 ? 16 : 32, kLaneWords, e->cpw, e->base.n_join, kJoinWindow),
+                                                   e->join);
     }
-    e->ctas_per_sm_lane = std::min(e->ctas_lane[1], kLaneCtasPerSm);
+    e->ctas_per_sm_lane = e->ctas_lane[1];
     if (e->ctas_per_sm_wide < 1 || e->ctas_per_sm_packed < 1 || e->ctas_per_sm_staged < 1 ||
         e->ctas_per_sm_lane < 1) {
         g_last_cuda_error = (int)cudaErrorLaunchOutOfResources;

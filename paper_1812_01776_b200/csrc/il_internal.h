@@ -144,7 +144,7 @@ int des_lane_warps_per_cta();
 // ring_slots: 16 or 32 batch ring positions per lane; ring_words: words of examined records (a power of two);
 // cpw candidates per warp with so many joins each, whose streams keep `window` records
 size_t des_lane_smem(int table_rows, int Bmax, int ring_slots, int ring_words, int cpw, int joins, int window);
-int des_lane_max_ctas_per_sm(size_t smem);
+int des_lane_max_ctas_per_sm(size_t smem, bool joins);     // of the instantiation for pipelines with joins, or of the others
 enum SimKernel { kSimWide = 0, kSimPacked = 1, kSimPackedStaged = 2, kSimLane = 3 };
 inline cudaError_t launch_simulation(const DesParams &p, int kernel, int grid, size_t smem,
                                      cudaStream_t stream)

@@ -101,6 +101,26 @@ def test_join_device_entry_chunks_and_static(il, oracle):
         assert np.array_equal(p99.cpu().numpy(), exp[0]) and np.array_equal(miss.cpu().numpy(), exp[1])
 
 
+def test_workspace_is_planned_for_ctas_that_can_be_resident(il, oracle):
+    """Shared memory would hold three CTAs per SM for a pipeline of 16 stages with and without a join, registers two and
+    three: no more warp slots (spill rings, incoming streams of the joins) than can be resident."""
+    from paper_1812_01776_b200 import estimator as E
+    chain = workloads.random_small(1, S=16, H=2, Bmax=8, n=900, C=12, max_replicas=4)
+    diamond = workloads.random_small(1, S=16, H=2, Bmax=8, n=900, C=12, max_replicas=4)
+    diamond.parent = np.array([-1, 0, 0, 1] + list(range(3, 15)), np.int32)
+    diamond.join = (np.array([-1, -1, -1, 2] + 12 * [-1], np.int32), np.full(16, -1, np.int8), np.zeros(16, np.uint8))
+    for w, fit in ((diamond, 2), (chain, 3)):
+        exp = oracle.estimate_workload(w)
+        with il.Estimator.from_workload(w) as est:
+            p99, miss = est.estimate(w.configs, w.slo_us)
+            assert np.array_equal(p99, exp[0]) and np.array_equal(miss, exp[1])
+            size = {}
+            for ctas in (0, fit - 1, fit, fit + 1):
+                est.set_test_knob(E.IL_KNOB_LANE_CTAS, ctas)
+                size[ctas] = E.il_workspace_bytes(est._h, 10 ** 6)
+            assert size[fit - 1] < size[fit] == size[0] == size[fit + 1]
+
+
 @pytest.mark.parametrize("C", [1, 7, 700])
 @pytest.mark.parametrize("shape", SHAPES)
 def test_join_level_with_its_parents(il, oracle, shape, C):
