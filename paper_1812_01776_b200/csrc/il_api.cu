@@ -21,12 +21,13 @@ static thread_local int g_last_cuda_error = 0;
         }                                               \
     } while (0)
 
-static constexpr int kCounters = 8;
-// device and pinned block: the counters, the status word, the largest replica count of a batch
+// pinned memory of a handle: results of so many candidates, configurations of so many bytes
 static constexpr int64_t kSmallResults = 4096;
 static constexpr size_t kSmallConfigBytes = 65536;
-// the least candidates that are looked over for shared prefixes
+// the least candidates that are looked over for shared prefixes (see looks_for_prefixes)
 static constexpr int64_t kShareMinCandidates = 2048;
+// device and pinned block: the counters, the status word, the largest replica count of a batch
+static constexpr int kCounters = 8;
 static constexpr size_t kCounterBytes = kCounters * sizeof(unsigned long long) + 2 * sizeof(int);
 
 struct il_estimator {
@@ -155,6 +156,20 @@ int64_t cands_per_slot(const il_estimator *e, int64_t n_cand)
     if (!is_lane(e)) return 1;
     const int64_t schedulers = (int64_t)e->num_sms * 4;
     return std::max<int64_t>(1, std::min<int64_t>(e->cpw, (n_cand + schedulers - 1) / schedulers));
+}
+
+// Whether a call looks its batch over for shared prefixes (3 S kernels, S table clears and a wait).  Not where every
+// candidate has a group of lanes on a scheduler's only warp: such a grid takes the time of one warp over the trace, and
+// with fewer candidates it would take the same.  Product sweeps over a tree of 8 (2,368 candidates are a wave), looked
+// over and not: 2,304 candidates, 4,000 queries 1.07 / 0.79 ms, 50,000 queries 8.76 / 8.66 ms; 8,192 candidates 1.11 /
+// 2.24 and 8.81 / 28.4 ms.  (Over a tree of 6, 2,916 candidates, 50,000 queries, it gains 3 % within a wave: 8.75 / 9.0 ms,
+// the lanes of fewer candidates diverge less.)  A Planner's calls are mostly within a wave, its questions share next to
+// nothing, and looking cost each of them 0.1 to 0.3 ms of 2.5 to 5.
+bool looks_for_prefixes(const il_estimator *e, int64_t n_cand)
+{
+    if (e->share_mode != 0) return e->share_mode != 2;
+    const int64_t wave = is_lane(e) ? (int64_t)e->num_sms * 4 * e->cpw : 0;
+    return n_cand >= kShareMinCandidates && n_cand > wave;
 }
 
 // Stream memory of a slot that holds cps candidates.  Lane kernel: a spill ring for every lane in use, and for joins the
@@ -465,7 +480,7 @@ static char *host_results(il_estimator *e, int64_t n_cand)
 static const il_stage_config *small_configs(il_estimator *e, const il_stage_config *configs, int64_t n_cand)
 {
     const size_t bytes = (size_t)n_cand * e->S * sizeof(il_stage_config);
-    if (!is_lane(e) || n_cand >= kShareMinCandidates || bytes > kSmallConfigBytes) return nullptr;
+    if (!is_lane(e) || looks_for_prefixes(e, n_cand) || bytes > kSmallConfigBytes) return nullptr;
     memcpy(e->h_cfg, configs, bytes);
     return e->h_cfg;
 }
@@ -732,8 +747,8 @@ static int estimate_shared(il_estimator *e, const il_stage_config *d_configs, in
     const int64_t n = e->n;
     const int64_t allowed = n - (99 * n + 99) / 100;           // T: queries allowed above the P99
     const int64_t top_len = allowed + 1;
-    if (e->share_mode == 2 || e->fork || !e->can_pack || e->variant != IL_VARIANT_AUTO || top_len > kShareMaxTop ||
-        n_cand >= (INT64_C(1) << 30) || (e->share_mode == 0 && n_cand < kShareMinCandidates))
+    if (!looks_for_prefixes(e, n_cand) || e->fork || !e->can_pack || e->variant != IL_VARIANT_AUTO ||
+        top_len > kShareMaxTop || n_cand >= (INT64_C(1) << 30))
         return IL_OK;
     uint32_t cap = 1024;
     while ((int64_t)cap < 2 * n_cand) cap <<= 1;
@@ -1502,7 +1517,7 @@ static int feasible_device(il_estimator *e, const il_stage_config *d_configs, in
     size_t ws_bytes = 0;
     rc = acquire_workspace(e, std::min<int64_t>(n_cand, 4096), &ws, &ws_bytes);
     if (rc) return rc;
-    if (e->share_mode == 1 || e->share_mode == 3 || (e->share_mode == 0 && n_cand >= kShareMinCandidates)) {
+    if (looks_for_prefixes(e, n_cand)) {
         // a batch full of common configuration prefixes is cheaper to evaluate node by node
         rc = ensure_staging(e, n_cand);
         if (rc) return rc;

@@ -93,6 +93,25 @@ def test_sharing_is_chosen_for_a_product_sweep(il, oracle, oracle_pool):
         assert est.stats()["stage_runs"] == w.n_candidates * w.n_stages
 
 
+@pytest.mark.parametrize("over", [0, 1])
+def test_batches_of_one_wave_are_not_looked_over(il, oracle, over):
+    """A batch that the lane kernel takes at once, with one warp per scheduler, is simulated as it is however much its
+    candidates share (three launches: clear, simulate, select); one more candidate, and the nodes are counted.  Through
+    the host entry points, whose small batches stay in pinned memory."""
+    import torch
+    w = workloads.random_small(31, S=6, H=3, Bmax=8, n=600, C=24, max_replicas=4, tree=True)
+    n = 4 * torch.cuda.get_device_properties(0).multi_processor_count * (32 // 6) + over
+    assert n >= 2048 + over
+    at = np.arange(n) % w.n_candidates
+    exp = oracle.estimate_workload(w)
+    with il.Estimator.from_workload(w) as est:
+        p99, miss = est.estimate(w.configs[at], w.slo_us)
+        st = est.stats()
+        assert np.array_equal(p99, exp[0][at]) and np.array_equal(miss, exp[1][at])
+        assert (st["stage_runs"] == n * 6 and st["kernel_launches"] == 3) if not over else st["stage_runs"] <= 24 * 6
+        assert np.array_equal(est.feasible(w.configs[at], w.slo_us), exp[0][at] <= w.slo_us)
+
+
 def test_sharing_with_latencies_above_2_32_and_one_query(il, oracle):
     w = workloads.random_small(102, S=2, H=1, Bmax=2, n=3000, C=4, max_replicas=1,
                                lat_lo=2_000_000_000, lat_hi=2_100_000_000)
