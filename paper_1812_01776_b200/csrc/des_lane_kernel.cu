@@ -50,7 +50,7 @@
 //     lie between the oldest one still needed and the one examined, the lane
 //     SPILLS: it copies the words to a ring of 2^lane_ring_log2 words of its own
 //     in global memory and reads those it has overwritten from there; looked at
-//     every eighth iteration, switched off again when the distance shrinks.  A lane
+//     once a turn (below), switched off again when the distance shrinks.  A lane
 //     whose distance outgrows that ring as well gives its candidate up (marked in
 //     the overflow array; the host's fallback evaluates it with the
 //     warp-per-candidate kernel).
@@ -59,7 +59,7 @@
 //   * The profile tables are shared by the CTA, rows padded to an odd length so
 //     that rows of different lanes start in different banks.
 //   * What happens once per candidate or rarely (its first and last batch, spills,
-//     the iteration bound, the next candidate) is looked at once a turn of 16 or
+//     the iteration bound, the next candidate) is looked at once a turn of 8, 16 or
 //     32 iterations only, behind one vote.
 //
 // Measured on B200 against the version whose streams lay in global memory (three
@@ -88,6 +88,7 @@ constexpr uint32_t kLast = 0x80000000u;       // flag of a batch's last record i
 constexpr int kAhead = 64;                    // records of the trace a root has before it: two long turns, a power of two
 constexpr int kTurn = 16, kLongTurn = 32;     // iterations between two looks at finished groups, spills, bounds
 constexpr int kQuickTurn = 8;                 // the same while a stage is about to start or to end
+constexpr uint32_t kQuickLooks = 128;         // looks at a candidate within which a stage counts as about to start
 
 __device__ __forceinline__ uint64_t lds64(uint32_t a)
 {
@@ -368,12 +369,12 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
     uint32_t ja = 0, jb = 0;     // joins: records of either incoming stream consumed
     uint32_t seen_new = 0;       // joins: words of the queries' bits from here on have not been touched
     uint32_t turns = 1, turns_hi = 0;        // iteration bound, in turns
-    bool any_spill = false, quick = false;
+    bool any_spill = false;
     uint64_t late_fin = 0, late_arr = 0;     // feasibility only: finish and arrival record of a query that has just left
     uint32_t miss_local = 0;
 
     for (;;) {
-        // ---- every kTurn-th or kLongTurn-th iteration: does a lane need more than its steps?  A stream at its start or its end, a
+        // ---- every kQuickTurn-th, kTurn-th or kLongTurn-th iteration: does a lane need more than its steps?  A stream at its start or its end, a
         // candidate that is decided, records in reach of being overwritten, the iteration bound.  (Kept short: its
         // latency is on the chain of every iteration, a kTurn-th of it.)
         if (FEAS && miss_local) { atomicAdd(missw + j, miss_local); miss_local = 0; }
@@ -392,8 +393,13 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
         copies_done();
         __syncwarp();
         turns--;
-        bool attn = !exhausted && ((is_join ? ja == join_na && jb == join_nb : i == n_cur || !started) || turns == 0u);
-        if (JOIN) attn |= !exhausted && !has;
+        // A stage whose first record is late (few queries visit it, or none until late in the trace), or whose last one has
+        // long passed, needs nothing until that record comes or the group's root is at the end of the trace.  (With a look at it
+        // in every turn, and short turns until it had started: chain of 4 whose branch is first taken 20 queries before
+        // the end of 50,000, one warp per scheduler, 11.0 ms; 8.9 now, 8.7 where half of the queries take the branch.)
+        const bool waits = i != n_cur && !started;
+        const bool starts = waits && (int)lds32_shared(xin + 4u) >= 0, closes = i == n_cur && bm != ~0u;
+        bool attn = !exhausted && (starts || closes || turns == 0u || (is_root && i == n_cur));
         attn |= i - low > reach || spill;
         if (FEAS) attn |= has && missw[j] > p.miss_allow;
         if (__any_sync(full, attn)) {
@@ -544,13 +550,12 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
             if (__all_sync(full, exhausted)) break;
         }
         any_spill = __any_sync(full, spill);
-        // (a stage waits for the next turn to open its first batch and to close its last one)
-        if (!JOIN) quick = __any_sync(full, (i != n_cur && !started) || (i == n_cur && bm != ~0u));
         __syncwarp();     // a root's first position is empty before another lane of the group fills it again below
-        } else {
-            quick = false;
         }
-        const int turn_its = quick ? kQuickTurn : __any_sync(full, i - low > long_reach) ? kTurn : kLongTurn;
+        // (A stage waits for the next turn to open its first batch and to close its last one.  One that has not started within
+        // the first kQuickLooks looks has late records: no short turns for it.)
+        const bool quick = !JOIN && ((i != n_cur && !started && (uint32_t)limit - turns < kQuickLooks) || (i == n_cur && bm != ~0u));
+        const int turn_its = (int)__reduce_min_sync(full, quick ? kQuickTurn : i - low > long_reach ? kTurn : kLongTurn);
 
         // The root's next records: requested two turns before their use, by all lanes of the group.
         {

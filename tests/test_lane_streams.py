@@ -58,6 +58,35 @@ def test_trace_lengths_around_a_root_s_stretch(oracle, n, S):
     same(w, oracle)
 
 
+def rare_branch(rows, n=20_000, C=590):
+    """A stage that only the queries in `rows` visit, one behind it, and the other way with a stage behind it."""
+    w = workloads.random_small(5, S=5, H=2, Bmax=8, n=n, C=C, max_replicas=4, tree=True, qps=300.0, lat_lo=500, lat_hi=9000)
+    w.parent = np.array([-1, 0, 0, 1, 2], np.int32)
+    w.cond_bit, w.cond_val = np.array([-1, 0, 0, -1, -1], np.int8), np.array([0, 0, 1, 0, 0], np.uint8)
+    w.branch_bits = np.zeros(n, np.uint8)
+    w.branch_bits[rows] = 1
+    return w
+
+
+@pytest.mark.parametrize("rows", [[], [0], [1999], [0, 1999], [1900, 1930], list(range(40)), list(range(1000, 2000, 400))])
+def test_rarely_taken_branches(oracle, rows):
+    same(rare_branch(rows, n=2000, C=40), oracle)
+
+
+def test_a_branch_taken_late_costs_no_short_turns():
+    """The time of a batch does not depend on where in the trace a branch is taken for the first time (while a stage waits
+    for its first record, or has seen its last one, there is nothing to look at every few iterations)."""
+    import torch
+    import paper_1812_01776_b200 as il
+    ms = {}
+    for name, rows in (("late", slice(19_980, None)), ("even", slice(0, None, 1000))):
+        w = rare_branch(rows)
+        cfg = torch.from_numpy(w.configs).cuda()
+        with il.Estimator.from_workload(w) as est:
+            ms[name] = min((est.estimate_device(cfg, w.slo_us), est.stats()["sim_ms"])[1] for _ in range(7))
+    assert ms["late"] < 1.12 * ms["even"], ms
+
+
 @pytest.mark.parametrize("skip", [16, 1024, 3072, 4080, 8192])
 @pytest.mark.parametrize("replicas", [3, 32])
 def test_shared_memory_that_starts_elsewhere(oracle, replicas, skip):
