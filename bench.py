@@ -360,7 +360,8 @@ def measure(il, torch, w, dev, stream, flush, steps, warmup, e2e_steps, variant,
     sim_s = statistics.mean(sim_ms) * 1e-3
     sel_s = statistics.mean(sel_ms) * 1e-3
     total_events = events_per_cand * n_cand
-    rec_bytes = 12 if kernel == "des_kernel" else 8  # separate time/query streams, else one 64-bit record
+    # separate time/query streams, else one 64-bit record (no workload has a join, for which the name stands for two kernels)
+    rec_bytes = 12 if kernel == "des_kernel" else 8
     slab_bytes = 8 * n * n_cand                       # written once by the simulation, read once by the select
     # the lane kernel keeps the streams between stages in shared memory; the others write and read them once
     stream_bytes = 0 if kernel == "des_lane_kernel" else (events_per_cand - n) * 2 * rec_bytes * n_cand

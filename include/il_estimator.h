@@ -189,12 +189,13 @@ typedef struct {
  * il_estimator_create for a pipeline with joins; `joins` may be NULL (then the
  * two calls are the same).  A handle with a join runs on one of the two kernels
  * that merge incoming streams, both reported as "des_kernel", whatever variant
- * is set: with IL_VARIANT_AUTO and IL_VARIANT_LANES the lane-parallel form, in
- * which a join has a lane of its own that merges the streams as they come, else
- * (or where times do not fit a record) the kernel with separate streams, which
- * builds the join's arrival stream before it simulates the stage.  Every entry
- * point works on such a handle and gives
- * the same results as on any other; il_feasible* evaluate it without early exit.
+ * is set: with IL_VARIANT_AUTO and IL_VARIANT_LANES the lane-parallel form
+ * (des_join_lane_kernel in a profile), in which a join has a lane of its own that
+ * merges the streams as they come, else (or where times do not fit a record) the
+ * kernel with separate streams (des_kernel in a profile), which builds the join's
+ * arrival stream before it simulates the stage.  Every entry point works on such a
+ * handle and gives the same results as on any other; il_feasible* evaluate it
+ * without early exit.
  * Errors: as il_estimator_create; BAD_TOPOLOGY also for a second edge outside
  * the form above or a third outgoing edge; TOO_LARGE if the streams of one
  * candidate exceed 2^31 - 1 elements.
@@ -439,8 +440,9 @@ IL_API int il_set_variant(il_estimator *est, int variant);
 IL_API int il_set_test_knob(il_estimator *est, int knob, int64_t value);
 
 /* Name of the simulation kernel the handle's next estimate call will launch
- * (the choice il_set_variant describes, resolved for the bound inputs);
- * a static string, never NULL. */
+ * (the choice il_set_variant describes, resolved for the bound inputs; one name for
+ * both kernels that serve joins, see il_estimator_create_dag); a static string,
+ * never NULL. */
 IL_API const char *il_kernel_name(const il_estimator *est);
 
 /* Counters of the last estimate call on this handle. */

@@ -832,15 +832,13 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) des_lane_kernel(const __gr
     lane_simulation<BRANCHY, FEAS, FORK, false>(p, smem_raw);
 }
 
-// Pipelines with joins: des_kernel in the lane-parallel form (des_kernel.cu holds the form for times that do not fit
-// a record).
-namespace lanes {
-__global__ void __launch_bounds__(kLaneWarps * 32) des_kernel(const __grid_constant__ DesParams p)
+// Pipelines with joins.  (il_kernel_name reports "des_kernel" for them, as for the form in des_kernel.cu that takes over
+// where times do not fit a record.)
+__global__ void __launch_bounds__(kLaneWarps * 32) des_join_lane_kernel(const __grid_constant__ DesParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     lane_simulation<true, false, true, true>(p, smem_raw);
 }
-}  // namespace lanes
 
 namespace {
 bool any_branch(const DesParams &p)
@@ -866,9 +864,9 @@ cudaError_t launch_des_lane(const DesParams &p, int grid, size_t smem, cudaStrea
 {
     if (p.n_join > 0) {
         if (p.lane_wrap || p.out_feasible) return cudaErrorInvalidValue;
-        cudaError_t e = cudaFuncSetAttribute(lanes::des_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(des_join_lane_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        lanes::des_kernel<<<grid, kLaneWarps * 32, smem, stream>>>(p);
+        des_join_lane_kernel<<<grid, kLaneWarps * 32, smem, stream>>>(p);
         return cudaGetLastError();
     }
     if (p.fork) {
@@ -892,7 +890,7 @@ int des_lane_max_ctas_per_sm(size_t smem, bool joins)
 {
     int n = 0;
     // (all instantiations without joins are compiled for three CTAs; the one with joins takes more registers)
-    void (*kernel)(DesParams) = joins ? lanes::des_kernel : des_lane_kernel<true, true>;
+    void (*kernel)(DesParams) = joins ? des_join_lane_kernel : des_lane_kernel<true, true>;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kLaneWarps * 32, smem);
     return e == cudaSuccess ? n : 0;

@@ -1250,7 +1250,7 @@ const char *il_kernel_name(const il_estimator *e)
 {
     if (!e) return "";
     switch (sim_kernel(e)) {
-    case kSimLane: return e->join ? "des_kernel" : "des_lane_kernel";      // (lanes::des_kernel)
+    case kSimLane: return e->join ? "des_kernel" : "des_lane_kernel";      // (des_join_lane_kernel)
     case kSimPacked: return "des_packed_kernel";
     case kSimPackedStaged: return "des_packed_kernel<staged>";
     default: return "des_kernel";
