@@ -31,14 +31,21 @@ struct EnvParams {
     int32_t n_windows;
     int64_t window[kMaxWindows];
     int *out;                  // [n_windows], zero on entry
+    int *status;               // checked build: where an index out of range is recorded
 };
 
+// Arrival i (checked build: recorded and 0 where there is none)
+__device__ __forceinline__ int64_t arrival_at(const EnvParams &p, int64_t i)
+{
+    return IL_IN_RANGE(i, p.n, p.status) ? __ldg(p.arrival + i) : 0;
+}
+
 // First index in [lo, hi] whose arrival is `window` or more after a (hi if there is none before it).
-__device__ __forceinline__ int first_at(const int64_t *arrival, int lo, int hi, int64_t a, int64_t window)
+__device__ __forceinline__ int first_at(const EnvParams &p, int lo, int hi, int64_t a, int64_t window)
 {
     while (lo < hi) {
         const int mid = lo + (hi - lo) / 2;
-        if (__ldg(arrival + mid) - a < window) lo = mid + 1; else hi = mid;
+        if (arrival_at(p, mid) - a < window) lo = mid + 1; else hi = mid;
     }
     return lo;
 }
@@ -64,7 +71,7 @@ __global__ void __launch_bounds__(kEnvThreads) envelope_kernel(const __grid_cons
         const int64_t j = (int64_t)j0 + g * kEnvGroup;
         int e = p.n;
         if (j < p.n) {
-            e = first_at(p.arrival, (int)j, p.n, __ldg(p.arrival + j), p.window[w]);
+            e = first_at(p, (int)j, p.n, arrival_at(p, j), p.window[w]);
             atomicMax(&best[w], e - (int)j);
         }
         end[w][g] = e;
@@ -84,9 +91,9 @@ __global__ void __launch_bounds__(kEnvThreads) envelope_kernel(const __grid_cons
         for (int i = 0; i < kEnvGroup; i += 32) {
             const int64_t m = j + i + lane;
             if (m + known >= p.n) continue;
-            const int64_t a = __ldg(p.arrival + m);
-            if (__ldg(p.arrival + m + known) - a < p.window[w])
-                count = max(count, first_at(p.arrival, (int)m + known + 1, end[w][g + 1], a, p.window[w]) - (int)m);
+            const int64_t a = arrival_at(p, m);
+            if (arrival_at(p, m + known) - a < p.window[w])
+                count = max(count, first_at(p, (int)m + known + 1, end[w][g + 1], a, p.window[w]) - (int)m);
         }
         count = __reduce_max_sync(0xffffffffu, count);
         if (lane == 0 && count > known) atomicMax(&best[w], max(count, atomicMax(&p.out[w], count)));
@@ -94,10 +101,10 @@ __global__ void __launch_bounds__(kEnvThreads) envelope_kernel(const __grid_cons
 }
 
 cudaError_t launch_envelope(const int64_t *d_arrival, int n, const int64_t *h_windows, int n_windows,
-                            int *d_out, cudaStream_t stream)
+                            int *d_out, int *d_status, cudaStream_t stream)
 {
     EnvParams p;
-    p.arrival = d_arrival; p.n = n; p.n_windows = n_windows; p.out = d_out;
+    p.arrival = d_arrival; p.n = n; p.n_windows = n_windows; p.out = d_out; p.status = d_status;
     for (int w = 0; w < n_windows; w++) p.window[w] = h_windows[w];
     const int64_t per_cta = kEnvGroups * kEnvGroup;
     envelope_kernel<<<(int)((n + per_cta - 1) / per_cta), kEnvThreads, 0, stream>>>(p);

@@ -1432,7 +1432,15 @@ int il_traffic_envelope(il_estimator *e, const int64_t *window_us, int32_t n_win
     IL_CUDA(cudaSetDevice(e->device));
     cudaStream_t st = e->stream;
     IL_CUDA(cudaMemsetAsync(e->d_envelope, 0, n_windows * sizeof(int), st));
-    IL_CUDA(launch_envelope(e->d_arrival, (int)e->n, window_us, n_windows, e->d_envelope, st));
+#ifdef IL_CHECKED
+    IL_CUDA(cudaMemsetAsync(e->d_status, 0, sizeof(int), st));
+#endif
+    IL_CUDA(launch_envelope(e->d_arrival, (int)e->n, window_us, n_windows, e->d_envelope, e->d_status, st));
+#ifdef IL_CHECKED
+    IL_CUDA(cudaMemcpyAsync(e->h_status, e->d_status, sizeof(int), cudaMemcpyDeviceToHost, st));
+    IL_CUDA(cudaStreamSynchronize(st));
+    if (*e->h_status) return *e->h_status;
+#endif
     IL_CUDA(cudaMemcpyAsync(e->h_envelope, e->d_envelope, n_windows * sizeof(int), cudaMemcpyDeviceToHost, st));
     IL_CUDA(cudaStreamSynchronize(st));
     for (int w = 0; w < n_windows; w++) out_max_count[w] = e->h_envelope[w];

@@ -243,7 +243,7 @@ cudaError_t launch_overflow_list(const uint8_t *ovf, int64_t n_cand, int32_t *or
                                  cudaStream_t stream);
 int des_max_ctas_per_sm(size_t smem);
 cudaError_t launch_envelope(const int64_t *d_arrival, int n, const int64_t *h_windows, int n_windows,
-                            int *d_out, cudaStream_t stream);
+                            int *d_out, int *d_status, cudaStream_t stream);
 int envelope_max_windows();
 cudaError_t launch_int_issue(unsigned *sink, int grid, int iters, cudaStream_t stream);
 

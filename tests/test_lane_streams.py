@@ -58,6 +58,42 @@ def test_trace_lengths_around_a_root_s_stretch(oracle, n, S):
     same(w, oracle)
 
 
+@pytest.mark.parametrize("bits_too", [False, True], ids=["query-index", "query-index-and-bits"])
+@pytest.mark.parametrize("over", [0, 1], ids=["just-below", "at-the-limit"])
+@pytest.mark.parametrize("shape", ["chain", "tree", "fan_out", "diamond", "two_joins"])
+def test_times_at_the_limit_of_a_record(oracle, shape, over, bits_too):
+    """Records are compared as doubles, so their words stay below 0x7fe0 << 48: traces whose last possible time is just below
+    what the query index (and the branch bits) leave room for, and traces one microsecond beyond."""
+    import torch
+    import paper_1812_01776_b200 as il
+    n = 1000
+    if shape in ("chain", "tree"):
+        w = workloads.random_small(3, S=5, H=2, Bmax=8, n=n, C=40, max_replicas=4, tree=shape == "tree", qps=900.0, cv=3.0,
+                                   equal_stamp_every=3)
+    elif shape == "fan_out":
+        w = workloads.fan_out_small(11, n=n, C=40, max_replicas=4, Bmax=8)
+    else:
+        w = workloads.join_small(4, n=n, C=40, max_replicas=4, Bmax=8, shape=shape)
+    guards = [w.cond_bit] + ([w.join[1]] if w.join is not None else [])
+    bits = max(int(g.max()) for g in guards) + 1
+    q = 10 + (bits if bits_too else 0)                                    # 1,000 queries: 10 bits
+    worst = n * int(w.latency_us.max(axis=(1, 2)).astype(np.int64).sum())
+    exp = oracle.estimate_workload(w)
+    _, _, lat = oracle.estimate_one(w.parent, w.cond_bit, w.cond_val, w.latency_us, w.arrival_us, w.branch_bits, w.configs[0],
+                                    w.slo_us, want_latency=True, join=w.join)
+    w.arrival_us = w.arrival_us + ((0x7fe0 << 48 >> q) - 1 + over - worst - int(w.arrival_us[-1]))
+    with il.Estimator.from_workload(w) as est:
+        if w.join is None and (not over or bits_too and bits):
+            assert est.kernel_name() == "des_lane_kernel"
+        elif shape in ("chain", "tree"):
+            assert est.kernel_name() == "des_packed_kernel"
+        a, b = est.estimate_device(torch.from_numpy(w.configs).cuda(), w.slo_us)
+        assert np.array_equal(a.cpu().numpy(), exp[0]) and np.array_equal(b.cpu().numpy(), exp[1])
+        for slo in (w.slo_us, int(np.median(exp[0])), 1 << 62):
+            assert np.array_equal(est.feasible(w.configs, slo), exp[0] <= slo)
+        assert np.array_equal(est.latencies(w.configs[0]), lat)
+
+
 def rare_branch(rows, n=20_000, C=590):
     """A stage that only the queries in `rows` visit, one behind it, and the other way with a stage behind it."""
     w = workloads.random_small(5, S=5, H=2, Bmax=8, n=n, C=C, max_replicas=4, tree=True, qps=300.0, lat_lo=500, lat_hi=9000)
