@@ -252,12 +252,14 @@ IL_API int il_estimate_device(il_estimator *est, const il_stage_config *d_config
  * "Feasible(pipeline, slo)": does the configuration meet the objective at P99?).
  *   out_feasible[c] = 1  iff  the k-th smallest latency of candidate c is <= slo_us, k = ceil(0.99 n),
  *                        equivalently iff at most n - k queries have latency > slo_us;  else 0.
- * Exactly the answer out_p99_us[c] <= slo_us of il_estimate, but cheaper to get: the lane kernel
+ * Exactly the answer out_p99_us[c] <= slo_us of il_estimate: the lane kernel
  * compares each query with the objective as it leaves the pipeline, writes no latencies and runs no
  * percentile pass, and drops a candidate as soon as more than n - k of its queries have missed the
  * objective (an overloaded candidate is decided within the first few per cent of the trace;
  * il_stats.early_exits counts them).  A feasible candidate is simulated to the end, so its answer is
- * exact too.  The warp-per-candidate kernels have no early exit: with them this call computes P99
+ * exact too.  Needs no memory per query and candidate, and is several times faster than il_estimate for a
+ * batch without feasible candidates; a batch of up to one warp per scheduler with some feasible ones takes
+ * 3 to 19 % longer than il_estimate, since the comparison is on the loop's chain.  The warp-per-candidate kernels have no early exit: with them this call computes P99
  * and compares.
  *   il_feasible         configs HOST [n][S], out_feasible HOST [n] bytes; candidates validated on the host
  *   il_feasible_device  DEVICE pointers; an invalid candidate makes the call return BAD_CONFIG

@@ -64,9 +64,9 @@
 //
 // Measured on B200 against the version whose streams lay in global memory (three
 // gathers of 8 bytes per lane and iteration through L1, 208 instructions): about
-// 120 instructions per iteration and 120 instead of 290 ns for a warp on its own;
-// 4,096 candidates x 4 stages x 50,000 queries 15.4 -> 6.7 ms, 4,096 x 10 x 10^6
-// 720 -> 367 ms.  With two or three warps per scheduler the ALU pipe (compares,
+// 120 instructions per iteration and 115 instead of 290 ns for a warp on its own;
+// 4,096 candidates x 4 stages x 50,000 queries 15.4 -> 6.3 ms, 4,096 x 10 x 10^6
+// 720 -> 330 ms.  With two or three warps per scheduler the ALU pipe (compares,
 // selects and logic, half the issue rate) is what bounds it.  What took the loop
 // from 155 to 120 ns: the trace copied ahead of its use by all lanes of a group
 // (8 instructions less, no stall on the load), the word to hand on loaded an

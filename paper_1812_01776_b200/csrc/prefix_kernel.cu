@@ -20,10 +20,13 @@
 //            records the node's configuration and parent;
 //   lookup   every candidate reads its node id back through its slot.
 //
-// The nodes are then simulated once each, level by level, by the stage loops of
-// the warp-per-candidate kernel (des_packed_kernel.cu), and a candidate's P99
-// and miss count are put together from the nodes where its queries leave the
-// pipeline (select_kernel.cu, combine step below).
+// Only the nodes that queries leave after are needed.  They are covered by a small
+// set of whole candidates of the batch (cover_* below), which the lane kernel
+// simulates like any batch; where their rows do not fit the workspace at once every
+// node is simulated by itself, level by level, by the stage loops of the
+// warp-per-candidate kernel (des_packed_kernel.cu).  A candidate's P99 and miss count
+// are put together from the nodes where its queries leave the pipeline
+// (select_kernel.cu, combine step below).
 #include "il_internal.h"
 
 #include <algorithm>
@@ -34,6 +37,7 @@ namespace {
 
 constexpr uint64_t kEmpty = ~0ull;
 
+// Hash of a key: the 64-bit finaliser of MurmurHash3 (Austin Appleby, public domain).
 __device__ __forceinline__ uint64_t mix64(uint64_t x)
 {
     x ^= x >> 33; x *= 0xff51afd7ed558ccdull;

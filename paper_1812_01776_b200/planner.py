@@ -23,11 +23,11 @@ batch of candidates:
 * which configuration an iteration of Algorithm 2 will accept can mostly be
   guessed (a downgrade to one replica at the largest batch, or what the answers of
   the previous iteration would lead to), so the questions of the iterations that
-  would follow go out with the call as long as they fit the same wave of the GPU.
-  An iteration whose questions have all been answered needs no call; a wrong guess
-  costs nothing but room in the wave.  Answers are kept for one run of the search.
-  A plan for four models took 9 to 15 dependent calls, 35 to 54 ms on a trace of
-  25,000 queries; it takes 4 to 9, 18 to 34 ms.
+  would follow go out with the call as long as there is room (CALL_ROOM below).
+  An iteration whose questions have all been answered needs no call; within a wave of
+  the GPU a wrong guess costs nothing but room in it.  Answers are kept for one run of
+  the search.  A plan for four models took 9 to 15 dependent calls, 35 to 54 ms on a
+  trace of 25,000 queries; it takes 4 to 7, 16 to 29 ms.
 
 Rules taken from the paper:
 
@@ -86,9 +86,11 @@ class Planner:
         visits       [S] queries visiting each stage (il_stage_visits); visits / visits[0] is the scale factor
         prices       [H] cost per replica-hour of each hardware type
         estimate     configs [n][S][4] uint8 -> (p99_us[n], miss[n]) for the bound trace and this objective
-        feasible     optional: configs -> bool[n], the same answer as p99_us <= slo_us but cheaper to get
-                     (Estimator.feasible drops a candidate as soon as it is decided); the search then asks
-                     only this, and `estimate` is called once, for the P99 of the final plan
+        feasible     optional: configs -> bool[n], the same answer as p99_us <= slo_us (Estimator.feasible drops
+                     a candidate as soon as it is decided and needs no memory per query; where some of a
+                     call's candidates are feasible it takes 3 to 19 % longer than `estimate` up to one wave of
+                     the GPU, see il_feasible); the search then asks only this, and `estimate` is called once,
+                     for the P99 of the final plan
         """
         self.parent = np.asarray(parent, dtype=np.int64)
         self.lat = np.asarray(latency_us, dtype=np.int64)
@@ -341,7 +343,11 @@ class Planner:
                 self._seen[(s, hw)] = ok[pos:pos + n_grid]
                 pos += n_grid
 
-    # Configurations per call: about one wave of a B200 (592 schedulers with one warp of five to eight candidates).
+    # Configurations per call.  On a B200 this is within one wave (592 schedulers with one warp of floor(32 / S)
+    # candidates) up to five models.  With more models a call asked ahead takes two or three warps on some schedulers, and
+    # fewer calls make up for it: plans on 15,000 queries with 3,200 / with room for one wave only, two traces each:
+    # 7 models 35, 40 / 39, 42 ms; 8 models 45, 41 / 42, 42; 10 models 67, 69 / 67, 69; 12 models 111, 101 / 113, 102;
+    # 16 models 191, 188 / 190, 188.
     CALL_ROOM = 3200
     MOST_AHEAD = 24         # iterations asked for ahead (a host that only builds questions is slower than the GPU)
 
