@@ -280,6 +280,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
     const uint32_t xin = from_trace ? tb : xb, xin_mask = from_trace ? kAhead - 1u : kX - 1u, xin_row = from_trace ? (uint32_t)cpw * 8u : 256u;
     // the child's stream on either side; towards the outside (or nowhere) the row of empty records
     const bool join_a = JOIN && da >= 0 && p.join_b[da >= 0 ? da : 0] >= 0, join_b = JOIN && db >= 0 && p.join_b[db >= 0 ? db : 0] >= 0;
+    const bool tells_a = join_a && lane_used && !is_join, tells_b = join_b && lane_used && !is_join;     // its records' counts
     const bool has_a = lane_used && !is_join && da >= 0 && !join_a, has_b = BRANCHY && lane_used && !is_join && db >= 0 && !join_b;
     const uint32_t xa = has_a ? xbw + (uint32_t)(j * L + da) * 8u : nowhere + (uint32_t)lane * 8u;
     const uint32_t xc = has_b ? xbw + (uint32_t)(j * L + db) * 8u : nowhere + (uint32_t)lane * 8u;
@@ -606,8 +607,8 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
             uint64_t va0 = 0, va1 = 0, vb0 = 0, vb1 = 0;
             bool room0 = false, room1 = false;
             if (JOIN) {
-                sts32_shared_if(join_a && !is_join, jw_a, tail_a);
-                sts32_shared_if(join_b && !is_join, jw_b, tail_b);
+                sts32_shared_if(tells_a, jw_a, tail_a);
+                sts32_shared_if(tells_b, jw_b, tail_b);
                 have_a = lds32_shared(jw_a); have_b = lds32_shared(jw_b);
                 va0 = lds64_shared(jw_a + 8u + ((ja >> 5) & win_mask)); va1 = lds64_shared(jw_a + 8u + (((ja + 256u) >> 5) & win_mask));
                 vb0 = lds64_shared(jw_b + 8u + ((jb >> 5) & win_mask)); vb1 = lds64_shared(jw_b + 8u + (((jb + 256u) >> 5) & win_mask));
