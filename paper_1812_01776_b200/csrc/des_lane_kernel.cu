@@ -54,26 +54,24 @@
 //     whose distance outgrows that ring as well gives its candidate up (marked in
 //     the overflow array; the host's fallback evaluates it with the
 //     warp-per-candidate kernel).
-//   * A root's records are copied to shared memory at least one turn (below)
-//     before their use (cp.async, all lanes of the group).
+//   * The records of a group's first stage (the trace, or another part's stream, see CUT below) are copied to shared
+//     memory at least one turn (below) before their use, in pairs (cp.async, all lanes of the group).
 //   * The profile tables are shared by the CTA, rows padded to an odd length so
 //     that rows of different lanes start in different banks.
 //   * What happens once per candidate or rarely (its first and last batch, spills,
-//     the iteration bound, the next candidate) is looked at once a turn of 8, 16 or
-//     32 iterations only, behind one vote.
+//     the iteration bound, the next candidate) is looked at once a turn of 8 to 30
+//     iterations only, behind one vote.
 //
-// Measured on B200 against the version whose streams lay in global memory (three
-// gathers of 8 bytes per lane and iteration through L1, 208 instructions): about
-// 120 instructions per iteration and 115 instead of 290 ns for a warp on its own;
-// 4,096 candidates x 4 stages x 50,000 queries 15.4 -> 6.3 ms, 4,096 x 10 x 10^6
-// 720 -> 330 ms.  With two or three warps per scheduler the ALU pipe (compares,
-// selects and logic, half the issue rate) is what bounds it.  What took the loop
-// from 155 to 120 ns: the trace copied ahead of its use by all lanes of a group
-// (8 instructions less, no stall on the load), the word to hand on loaded an
-// iteration early, comparisons as doubles, one counter per lane for the records
-// it passes on.
+// Measured on B200, 4,096 candidates x 4 stages x 50,000 queries and 4,096 x 10 x 10^6: streams in global memory 15.4 / 720 ms;
+// streams in shared memory, the loop in C++ 6.94 / 348 ms (123 instructions an iteration, 220 cycles for a warp on its
+// own); the loop in PTX 6.74 / 302 ms (108 instructions, 184 cycles and the turns).  What costs there is latency between
+// dependent instructions (73 of 230 cycles) and the ALU pipe (compares, selects, logic: half the issue rate).  Learned on
+// the way: a bool that lives through the loop takes one of seven predicates and costs the schedule 15 % (two of them:
+// 6.94 -> 8.14 ms), so what a lane has to remember are bits of one register; the same instructions with the loads of the next
+// iteration behind this one's stores take 7.7 ms; one branch in the loop, never taken, 50 cycles.
 #include "il_internal.h"
 
+#include <algorithm>
 #include <type_traits>
 
 namespace il {
@@ -85,8 +83,7 @@ constexpr uint64_t kInf = ~0ull;
 constexpr uint64_t kLatest = 0x7fefffffffffffffull;      // no record or key is larger
 constexpr int kX = 8;                         // records of a stream between two stages
 constexpr uint32_t kLast = 0x80000000u;       // flag of a batch's last record in that ring
-constexpr int kAhead = 64;                    // records of the trace a root has before it: two long turns, a power of two
-constexpr int kTurn = 16, kLongTurn = 32;     // iterations between two looks at finished groups, spills, bounds
+constexpr int kTurn = 16, kLongTurn = 32;     // iterations (two less) between two looks at finished groups, spills, bounds
 constexpr int kQuickTurn = 8;                 // the same while a stage is about to start or to end
 constexpr uint32_t kQuickLooks = 128;         // looks at a candidate within which a stage counts as about to start
 
@@ -105,8 +102,6 @@ __device__ __forceinline__ uint32_t lds32(uint32_t a)
 // Order of two records or keys.  Words below 0x7ff0... order the same as the doubles of their bits, and a double
 // is compared by one instruction on a pipe that is idle otherwise, where a 64-bit integer takes two on the ALU pipe
 // (5 % of a launch with three warps per scheduler).  A word with the sign or all exponent bits set compares as false.
-__device__ __forceinline__ bool before(uint64_t a, uint64_t b) { return __longlong_as_double((long long)a) < __longlong_as_double((long long)b); }
-__device__ __forceinline__ bool not_after(uint64_t a, uint64_t b) { return __longlong_as_double((long long)a) <= __longlong_as_double((long long)b); }
 
 // Words that two lanes share.  Stream records, and the records in a join's windows: each is complete in itself, so no
 // ordering between words is needed.  A join's counts: stored behind the warp barrier that follows the records they cover.
@@ -122,10 +117,6 @@ __device__ __forceinline__ uint32_t lds32_shared(uint32_t a)
     asm volatile("ld.relaxed.cta.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
     return v;
 }
-__device__ __forceinline__ void sts64_shared_if(bool c, uint32_t a, uint64_t v)
-{
-    asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p st.relaxed.cta.shared.u64 [%1], %2; }" ::"r"((uint32_t)c), "r"(a), "l"(v) : "memory");
-}
 __device__ __forceinline__ void sts32_shared_if(bool c, uint32_t a, uint32_t v)
 {
     asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p st.relaxed.cta.shared.u32 [%1], %2; }" ::"r"((uint32_t)c), "r"(a), "r"(v) : "memory");
@@ -135,14 +126,6 @@ __device__ __forceinline__ void sts32(uint32_t a, uint32_t v) { asm volatile("st
 
 // The same under a predicate: a lane's steps
 // are straight-line code (a branch costs the warp more than the few instructions it would skip).
-__device__ __forceinline__ void sts64_if(bool c, uint32_t a, uint64_t v)
-{
-    asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p st.shared.u64 [%1], %2; }" ::"r"((uint32_t)c), "r"(a), "l"(v) : "memory");
-}
-__device__ __forceinline__ void sts32_if(bool c, uint32_t a, uint32_t v)
-{
-    asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p st.shared.u32 [%1], %2; }" ::"r"((uint32_t)c), "r"(a), "r"(v) : "memory");
-}
 __device__ __forceinline__ void stg32_if(bool c, uint32_t *a, uint32_t v)
 {
     asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p st.global.u32 [%1], %2; }" ::"r"((uint32_t)c), "l"(a), "r"(v) : "memory");
@@ -151,83 +134,155 @@ __device__ __forceinline__ void ldg32_if(bool c, const uint32_t *a, uint32_t &v)
 {
     asm volatile("{ .reg .pred p; setp.ne.u32 p, %1, 0; @p ld.global.ca.u32 %0, [%2]; }" : "+r"(v) : "r"((uint32_t)c), "l"(a) : "memory");
 }
-__device__ __forceinline__ void stg64_if(bool c, uint64_t *a, uint64_t v)
+// 16 bytes from global to shared memory, asynchronously and past L1 (another SM may be writing next to them).  Each half is a
+// record that is complete before it is asked for.
+__device__ __forceinline__ void copy16(uint32_t dst, const uint64_t *src)
 {
-    asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p st.global.u64 [%1], %2; }" ::"r"((uint32_t)c), "l"(a), "l"(v) : "memory");
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
-// 8 bytes from global to shared memory, asynchronously
-__device__ __forceinline__ void copy8(uint32_t dst, const uint64_t *src)
+__device__ __forceinline__ uint64_t ldg64_shared(const uint64_t *a)
 {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+    uint64_t v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(a) : "memory");
+    return v;
+}
+// Counts of a stream's records that are there: published behind a fence that follows the records, read with acquire.
+__device__ __forceinline__ uint32_t ldg32_acquire(const uint32_t *a)
+{
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t ldg32_shared(const uint32_t *a)
+{
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void stg32_shared(uint32_t *a, uint32_t v)
+{
+    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(a), "r"(v) : "memory");
 }
 __device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Shared memory of a CTA: the tables ([S * H] rows of Bmax | 1 words, one word in front of them), then per warp
 // the batch keys [kr][lane] (aligned to their size: a ring address is (counter & mask) | base), per warp the
 // streams [kX][lane], a row of empty records (the "child" of a leaf), per warp the miss counts of the groups
-// (feasibility only), per warp the words of examined records [nq][lane], and per warp the next records of the trace
-// [kAhead][group].
+// (feasibility only), per warp the words of examined records [nq][lane], and per warp and group the next `ahead` records
+// of its arrival stream, 16 bytes apart so that groups start in different banks.
 // Where a CTA's dynamic shared memory starts with the toolkit at hand.  The host plans for it; a launch that finds it elsewhere
 // needs up to a row of batch keys more to align them and takes it from the words of examined records (more spills).
 constexpr uint32_t kSmemBase = 1024;
 __host__ __device__ inline uint32_t key_bytes(int kr) { return (uint32_t)kr * 256u; }
 constexpr uint32_t kXBytes = kX * 256u;
 __host__ __device__ inline size_t table_bytes(int rows, int Bmax) { return ((size_t)rows * (Bmax | 1) + 1) * 4; }
-__host__ __device__ inline size_t ring_bytes(int kr, int nq, int cpw)
+__host__ __device__ inline uint32_t stretch_bytes(int ahead) { return (uint32_t)ahead * 8u + 16u; }
+__host__ __device__ inline size_t ring_bytes(int kr, int nq, int stretch)
 {
-    return (size_t)kLaneWarps * (key_bytes(kr) + nq * 128u + kXBytes + (size_t)kAhead * cpw * 8);
+    return (size_t)kLaneWarps * (key_bytes(kr) + nq * 128u + kXBytes + (size_t)stretch);
 }
 constexpr size_t kTailBytes = 256 + kLaneWarps * 128;
-constexpr int kSeen = 64;                     // joins: words of the queries' bits that are kept in shared memory
-// joins: per warp and per (group, join) the counts and the windows of the two incoming streams, then the cached words
-// of the queries' bits with their numbers, then which branch bits follow both edges (256 bits)
-__host__ __device__ inline uint32_t join_lane_bytes(int window) { return 2u * (window + 1) * 8u + kSeen * 8u + 32u; }
-__host__ __device__ inline size_t join_bytes(int cpw, int joins, int window) { return (size_t)kLaneWarps * cpw * joins * join_lane_bytes(window); }
+
+// ---- Cut pipelines: who does what ---------------------------------------------------------------------------------
+// SMs set aside for root nodes, one warp per scheduler: 16 nodes a warp (up to 64 an SM), a third of the device at most.
+__host__ __device__ inline uint32_t root_sms_for(uint32_t nodes, uint32_t num_sms)
+{
+    const uint32_t want = (nodes + 4u * kRootGroups - 1u) / (4u * kRootGroups), most = num_sms / 3u > 0u ? num_sms / 3u : 1u;
+    return want < 1u ? 1u : want < most ? want : most;
+}
+
+constexpr unsigned kRoleNone = 0, kRoleRoots = 1, kRoleParts = 2;
+constexpr uint32_t kDead = 0x80000000u;       // in place of a stream's count: no more records will come, and some are missing
+
+// The first CTA on an SM gets a number; the first `root_sms` of them take root nodes and have the SM to themselves.  (Without
+// that a root shares its scheduler with one or two warps, and everything else waits for it.)  Called by one thread of a CTA.
+__device__ unsigned lane_cta_role(uint32_t *ctl, uint32_t root_sms)
+{
+    uint32_t sm;
+    asm("mov.u32 %0, %%smid;" : "=r"(sm));
+    if (sm >= kCtlSms) return atomicAdd(ctl + kCtlOrder, 1u) < root_sms ? kRoleRoots : kRoleParts;
+    if (atomicAdd(ctl + kCtlSlot + sm, 1u) == 0u) {
+        const unsigned role = atomicAdd(ctl + kCtlOrder, 1u) < root_sms ? kRoleRoots : kRoleParts;
+        atomicExch(ctl + kCtlRole + sm, role);
+        return role;
+    }
+    unsigned role = 0u;
+    for (int k = 0; k < (1 << 16) && role == 0u; k++) {       // (the other CTA is a few instructions away from telling)
+        role = atomicAdd(ctl + kCtlRole + sm, 0u);
+        if (role == 0u) __nanosleep(100);
+    }
+    return role == kRoleRoots ? kRoleNone : kRoleParts;
+}
+
+// The part a warp starts with: root nodes, or by the order in which warps start, the parts in the order of the pipeline,
+// each as many warps as the host has planned for it.  (A warp that finds no more of its part goes on with the next.)
+__device__ int lane_first_part(const LaneCut &cut, bool for_roots)
+{
+    if (for_roots) return 0;
+    uint32_t w = 0;
+    if ((threadIdx.x & 31) == 0) w = atomicAdd(cut.ctl + kCtlTicket, 1u);
+    w = __shfl_sync(0xffffffffu, w, 0);
+    const int t0 = cut.shared ? 1 : 0;
+    for (int t = t0; t < cut.n_part; t++) {
+        if (w < (uint32_t)cut.part[t].warps) return t;
+        w -= (uint32_t)cut.part[t].warps;
+    }
+    return t0 + (int)(w % (uint32_t)(cut.n_part - t0));
+}
 
 }  // namespace
 
-// BRANCHY: some stage routes by a branch bit (otherwise every stage has one way out).
 // FEAS: feasibility only (Section 4.3, "Feasible"): leaving queries are compared with the objective as
 //       they leave, nothing is written to a slab, and a candidate is dropped as soon as more queries
 //       have missed the objective than the P99 rule allows.
-// FORK: fan-out -- a query goes down every edge whose condition holds, a copy that finds none leaves, and
-//       the slab keeps per query the record of the copy that left last (only with BRANCHY, without FEAS).
-// JOIN: some stage has two incoming edges (with FORK: a query goes down both before it gets there).  A join has a
-//       lane of its own, behind the stages' lanes: it merges the two incoming streams in time order, at equal
-//       times the first parent's records first, swallows the record of an input that is not its query's last one
-//       (one bit per query and join in global memory: the other input has been seen) and feeds the stage's ring.
-//       The incoming streams have no back-pressure -- either parent may have to run ahead of the other by all
-//       that the slower branch keeps in flight -- so they go to global memory whole, and the latest
-//       64 to 512 records of each to shared memory, from where the join nearly always reads them.  511 candidates
-//       of a diamond, 50,000 queries: 130 ms on the warp-per-candidate kernel, 53 ms here.
-template <bool BRANCHY, bool FEAS, bool FORK, bool JOIN>
-__device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned char *smem_raw)
+// CUT:  pipelines with branch points.  A pipeline is cut into PARTS, chains of stages without a branch between them
+//       (LaneCut, built by the host), and a warp simulates one part of as many candidates as fit: L lanes each.  What
+//       passes from one part to the next is a stream in global memory, written once by the last lane of a part and
+//       read by the group of lanes that has the next one, which may run in any warp of the launch at the same time:
+//         * The producer publishes every few turns how many records are there (a fence, then the count); a consumer
+//           reads the count with acquire and copies records to shared memory as a root does with the trace.  A
+//           producer never waits for a consumer (streams are whole), and parts are handed out in the order of the
+//           pipeline to warps in the order in which they start, so whoever waits waits for a group that runs: every
+//           wait ends, and has a bound all the same.  A warp none of whose groups has records to examine sleeps.
+//         * Part 0 is the root stage alone, and (where no query leaves there) its groups are ROOT NODES, the distinct configurations of the root
+//           among the candidates (some hundred at most: hardware x batch x replicas), so it is simulated once per
+//           configuration and not once per candidate.  Its chain is as long as the trace and everything waits for it,
+//           so its CTAs have their SM to themselves.
+//         * A part that only leaves the pipeline (the rule) needs no memory for its stream: the records come in the
+//           region of the candidate's slab row that they go to, and no record leaves before it was examined.
+//       Against one group of lanes for the whole tree (each lane as many iterations as the root has records, whatever
+//       its branch sees, and a branch step in the loop): 7,001 candidates of a tree of 6, 199,999 queries 70.6 -> 39.8 ms;
+//       8,192, feasibility only, 100,000 queries 35.1 -> 22.2 ms; a sweep over a tree of 8 20.6 -> 16.9 ms; fan-out,
+//       2,048 candidates of 6 stages, 100,000 queries 22.7 -> 17.7 ms.  Up to a warp per scheduler the root is what
+//       takes the time (250 cycles an iteration and 40 for its turns), beyond that the ALU pipe.
+// FORK: fan-out (with CUT) -- a query goes down every edge whose condition holds, a copy that finds none leaves, and
+//       the slab keeps per query the record of the copy that left last.
+template <bool FEAS, bool CUT, bool FORK>
+__device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCut &cut, unsigned char *smem_raw)
 {
     // A stream record is (time << q) | low part; the low part is the query index, below the query's
     // branch bits when the records carry them (rb > 0: no stage then looks the bits up).  Keys of batches
     // use the same q, with the index of the batch's first arrival in the low part.
-    const int qi = p.qbits, rb = BRANCHY ? p.rec_bits : 0;
+    const int qi = p.qbits, rb = CUT ? p.rec_bits : 0;
     const int q = qi + rb;
     const uint32_t qmask = (1u << q) - 1u, imask = (1u << qi) - 1u;      // q <= 31
     const uint32_t tick = 1u << q;
-    const uint64_t *trace = rb > 0 ? p.ptrace_b : p.ptrace;
 
     const unsigned full = 0xffffffffu;
     const int wid = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int kr = p.lane_slots == 16 ? 16 : 32;      // batch ring positions of a lane
-    const int S = p.S, cpw = p.cpw, rowlen = p.Bmax | 1;
-    const int L = JOIN ? S + p.n_join : S;            // lanes of a candidate
+    const int rowlen = p.Bmax | 1;
     uint32_t smem_bytes;
     asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(smem_bytes));
     const uint32_t smem_end = (uint32_t)__cvta_generic_to_shared(smem_raw) + smem_bytes;
     smem_raw += p.smem_skip;
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem_raw);
     const uint32_t tab0 = sbase + 4u;
-    const uint32_t rings = (sbase + (uint32_t)table_bytes(S * p.H, p.Bmax) + key_bytes(kr) - 1u) & ~(key_bytes(kr) - 1u);
+    const uint32_t rings = (sbase + (uint32_t)table_bytes(p.S * p.H, p.Bmax) + key_bytes(kr) - 1u) & ~(key_bytes(kr) - 1u);
     // words of examined records a lane keeps in shared memory: half of what was planned where the rings start later than
     // planned (they are at most 8 KB late, and half of the fewest words, 64 for each of 128 lanes, are 16 KB)
-    auto end_with = [&](int words) { return rings + (uint32_t)(ring_bytes(kr, words, cpw) + kTailBytes + join_bytes(cpw, p.n_join, p.join_window)); };
+    auto end_with = [&](int words) { return rings + (uint32_t)(ring_bytes(kr, words, p.lane_stretch) + kTailBytes); };
     const uint32_t nq = (uint32_t)p.lane_words >> (end_with(p.lane_words) > smem_end ? 1 : 0);
     if (end_with((int)nq) > smem_end) { atomicCAS(p.status, 0, IL_ERR_CUDA); return; }      // launched with less than planned
     const uint32_t kbw = rings + (uint32_t)wid * key_bytes(kr), kb = kbw + (uint32_t)lane * 8u;
@@ -236,117 +291,124 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
     const uint32_t nowhere = xb0 + kLaneWarps * kXBytes;
     const uint32_t qb0 = nowhere + (uint32_t)kTailBytes;
     const uint32_t qb = qb0 + (uint32_t)wid * nq * 128u + (uint32_t)lane * 4u;
-    const uint32_t tb0 = qb0 + kLaneWarps * nq * 128u;        // per warp the next records of the trace, [kAhead][group]
+    const uint32_t tbw = qb0 + kLaneWarps * nq * 128u + (uint32_t)(wid * p.lane_stretch);     // the warp's stretches of arrival streams
+    const uint32_t ahead = (uint32_t)p.lane_ahead;
     unsigned *missw = reinterpret_cast<unsigned *>(smem_raw + (nowhere - sbase) + 256u + (uint32_t)wid * 128u);   // per group
     const uint32_t rm = (uint32_t)(kr - 1) << 8;      // ring counters epos, lpos, tpos count in bytes of a row
 
-    for (int r = threadIdx.x; r < S * p.H * p.Bmax; r += kLaneWarps * 32)
+    // Cut pipelines: a CTA that is the first on its SM may take that SM for root nodes; others that come there leave.
+    uint32_t root_warps = 1u;
+    bool for_roots = false;
+    (void)root_warps; (void)for_roots;
+    if (CUT && cut.shared) {
+        const uint32_t nodes = cut.ctl[kCtlNodes];
+        const uint32_t root_sms = root_sms_for(nodes, (uint32_t)cut.num_sms);
+        root_warps = root_sms * kLaneWarps;
+        if (threadIdx.x == 0) missw[0] = lane_cta_role(cut.ctl, root_sms);
+        __syncthreads();
+        const unsigned role = *reinterpret_cast<unsigned *>(smem_raw + (nowhere - sbase) + 256u);
+        __syncthreads();
+        if (role == kRoleNone) return;
+        for_roots = role == kRoleRoots;
+    }
+
+    for (int r = threadIdx.x; r < p.S * p.H * p.Bmax; r += kLaneWarps * 32)
         sts32(tab0 + (uint32_t)(r / p.Bmax * rowlen + r % p.Bmax) * 4u, (uint32_t)p.lat[r]);
     if (threadIdx.x < 32) sts64(nowhere + (uint32_t)lane * 8u, kInf);
     if (threadIdx.x == 0) sts32(sbase, 0u);
-    for (int k = 0; k < kX; k++) sts64(xb + (uint32_t)k * 256u, kInf);       // lanes without a stage see no record either
     __syncthreads();
 
-    const int j = lane / L, row = lane - j * L;
-    const bool lane_used = j < cpw;
-    const bool is_join = JOIN && lane_used && row >= S;      // a lane that merges the incoming streams of a join
-    const int s = JOIN && row >= S ? p.join_stage[row - S] : row;
-
-    // static facts of this lane's stage
-    int exit_off = 0;
-    for (int u = 0; u < s; u++) {
-        const int a = p.dest_a[u], b2 = p.dest_b[u];
-        int kids = 0;
-        if (a >= 0) kids += p.n_s[a];
-        if (b2 >= 0 && b2 != a) kids += p.n_s[b2];
-        exit_off += p.n_s[u] - kids;
-    }
-    const int da = FORK ? p.child_a[s] : p.dest_a[s], db = FORK ? p.child_b[s] : p.dest_b[s];
-    // (with fan-out the branch bits are needed if one of the edges is conditional)
-    const int bit = FORK ? ((p.cbit_a[s] >= 0 || p.cbit_b[s] >= 0) ? 0 : -1) : p.bit[s];
-    // Routing by the bits of a record's low part: without fan-out to side b if (bits & mask_b), with fan-out down
-    // either edge if (bits & mask) == want.
-    auto bit_at = [&](int b) { return b >= 0 ? 1u << (rb > 0 ? qi + b : b) : 0u; };      // (rb = 0: bits looked up)
-    const uint32_t mask_a = FORK && da >= 0 ? bit_at(p.cbit_a[s]) : 0u;
-    const uint32_t mask_b = FORK ? (db >= 0 ? bit_at(p.cbit_b[s]) : 0u) : bit_at(p.bit[s]);
-    const uint32_t want_a = da < 0 ? ~0u : (p.cval_a[s] ? mask_a : 0u), want_b = db < 0 ? ~0u : (p.cval_b[s] ? mask_b : 0u);
-    const uint32_t n_in = lane_used && !is_join ? (uint32_t)p.n_s[s] : 0u;
-    const unsigned group_mask = lane_used ? (((1u << L) - 1u) << (j * L)) : 0u;
-    const int root_lane = lane_used ? j * L : 0;
-    const bool is_root = row == 0;
-    // arrival stream: the lane's ring, for a root the group's stretch of the trace
-    const uint32_t tb = tb0 + (uint32_t)(wid * kAhead * cpw + (lane_used ? j : 0)) * 8u;
-    const bool from_trace = is_root && lane_used;
-    const uint32_t xin = from_trace ? tb : xb, xin_mask = from_trace ? kAhead - 1u : kX - 1u, xin_row = from_trace ? (uint32_t)cpw * 8u : 256u;
-    // the child's stream on either side; towards the outside (or nowhere) the row of empty records
-    const bool join_a = JOIN && da >= 0 && p.join_b[da >= 0 ? da : 0] >= 0, join_b = JOIN && db >= 0 && p.join_b[db >= 0 ? db : 0] >= 0;
-    const bool tells_a = join_a && lane_used && !is_join, tells_b = join_b && lane_used && !is_join;     // its records' counts
-    const bool has_a = lane_used && !is_join && da >= 0 && !join_a, has_b = BRANCHY && lane_used && !is_join && db >= 0 && !join_b;
-    const uint32_t xa = has_a ? xbw + (uint32_t)(j * L + da) * 8u : nowhere + (uint32_t)lane * 8u;
-    const uint32_t xc = has_b ? xbw + (uint32_t)(j * L + db) * 8u : nowhere + (uint32_t)lane * 8u;
-    const uint32_t xam = has_a ? (kX - 1) * 256u : 0u, xcm = has_b ? (kX - 1) * 256u : 0u;
-    const uint32_t tail_step = da >= 0 ? 256u : 8u;
-    const uint32_t leaving = (uint32_t)p.n - (uint32_t)exit_off;      // slab entries from this stage's region on
-    (void)leaving;
-
-    const int64_t wslot = (int64_t)blockIdx.x * kLaneWarps + wid;
-    // joins: where a stage's records for a join go (global stream, window and count in shared memory), and where the
-    // join's lane finds them
-    const uint32_t jbase = tb0 + (uint32_t)(kLaneWarps * kAhead * cpw) * 8u + (uint32_t)(wid * cpw * p.n_join) * join_lane_bytes(p.join_window);
-    uint64_t *jg_a = nullptr, *jg_b = nullptr;
-    uint32_t jw_a = nowhere, jw_b = nowhere, seen_cache = nowhere;      // (lanes that are no join's read there, and store nothing)
-    uint32_t *seen = nullptr;
-    (void)jbase;
-    if (JOIN && lane_used) {
-        uint64_t *streams = p.join_ws + (wslot * cpw + j) * p.join_elems;
-        auto window = [&](int t, int side) {
-            return jbase + (uint32_t)(j * p.n_join + p.join_no[t]) * join_lane_bytes(p.join_window) + (uint32_t)side * ((p.join_window + 1u) * 8u);
-        };
-        auto stream = [&](int t, int side) { return streams + (side ? p.join_lane_b[t] : p.join_lane_a[t]); };
-        if (is_join) {
-            jg_a = stream(s, 0); jw_a = window(s, 0);
-            jg_b = stream(s, 1); jw_b = window(s, 1);
-            seen_cache = jw_b + (p.join_window + 1u) * 8u;
-            seen = p.join_seen + ((wslot * cpw + j) * p.n_join + (row - S)) * p.join_seen_words;
-            for (int k = 0; k < 4; k++) sts64(seen_cache + kSeen * 8u + (uint32_t)k * 8u, p.join_both[s][k]);
-        } else {
-            if (join_a) { const int side = p.join_b[da] == s; jg_a = stream(da, side); jw_a = window(da, side); }
-            if (join_b) { const int side = p.join_b[db] == s; jg_b = stream(db, side); jw_b = window(db, side); }
-        }
-    }
-    const uint32_t join_na = is_join ? (uint32_t)p.join_na[s] << 8 : 0u, join_nb = is_join ? (uint32_t)p.join_nb[s] << 8 : 0u;
-    const uint32_t seen_mask = is_join ? kSeen - 1u : 0u, seen_both = is_join ? seen_cache + kSeen * 8u : nowhere;
-    const uint32_t win_mask = (p.join_window - 1u) * 8u, win_reach = (p.join_window - 1u) * 256u;     // (of a window's records, in bytes)
-    const bool join_always = JOIN && !p.any_bits;     // no conditional edges: every query goes down both edges into a join
-    const uint32_t xj = is_join && lane_used ? xbw + (uint32_t)(j * L + s) * 8u : nowhere + (uint32_t)lane * 8u;
-    const uint32_t xjm = is_join && lane_used ? (kX - 1) * 256u : 0u;
     const uint32_t gmask = (uint32_t)((1ull << p.lane_ring_log2) - 1ull);
-    uint32_t *spill_ring = reinterpret_cast<uint32_t *>(p.lane_ws) + ((wslot * (cpw * L) + lane) << p.lane_ring_log2);
-    const unsigned long long n_cand = (unsigned long long)p.n_cand;
+    const int64_t wslot = (int64_t)blockIdx.x * kLaneWarps + wid;
+    uint32_t *spill_ring = reinterpret_cast<uint32_t *>(p.lane_ws) + ((wslot * p.lanes_per_slot + lane) << p.lane_ring_log2);
     const uint64_t slo_q = FEAS ? (uint64_t)p.slo_us << q : 0ull;   // the objective, aligned with a record's time field
+    // (cut: a group may also wait for records while others of its warp have some)
     const unsigned long long limit =
-        (p.iter_limit ? p.iter_limit : 8ull * (unsigned)p.n * (unsigned)(S + 1) + 4096ull) / kTurn + 1ull;
+        (p.iter_limit ? p.iter_limit : (8ull * (unsigned)p.n * (unsigned)(p.S + 1) + 4096ull) * (CUT ? 4ull : 1ull)) / kTurn + 1ull;
     // a spill has to start before a record still needed is overwritten, two turns from now at the latest
     const uint32_t reach = min((uint32_t)(nq - kTurn - 2), gmask - 2u * kTurn);
     // (and no long turn may start where it would come too late)
     const uint32_t long_reach = gmask > 2u * kLongTurn && nq > kLongTurn + 2u ? min((uint32_t)(nq - kLongTurn - 2), gmask - 2u * kLongTurn) : 0u;
     unsigned long long batches = 0, alg_ops = 0, exits_seen = 0, exits_due = 0;
     unsigned early = 0;          // candidates dropped before the end of the trace (feasibility only)
+    unsigned long long naps = p.iter_limit ? p.iter_limit : cut.naps;      // bound on the sleeps of a warp
+    uint32_t quit = 0u;          // the launch has failed: nothing more is waited for
+    (void)naps; (void)quit;
+
+    int part = CUT ? lane_first_part(cut, for_roots) : 0;
+    for (int parts_left = CUT ? cut.n_part : 1; parts_left > 0; parts_left--, part = CUT && part + 1 == cut.n_part ? 0 : part + 1) {
+    const LanePart *pt = CUT ? cut.part + part : nullptr;
+    const int L = CUT ? pt->len : p.S;                // lanes of a candidate
+    const bool per_node = CUT && part == 0 && cut.shared;      // the items are root nodes, not candidates
+    const uint32_t n_items = per_node ? cut.ctl[kCtlNodes] : (uint32_t)p.n_cand;
+    const int groups = !CUT ? p.cpw : per_node ? (int)min((uint32_t)kRootGroups, (n_items + root_warps - 1u) / root_warps) : pt->groups;
+    const int j = lane / L, row = lane - j * L;
+    const bool lane_used = j < groups;
+    const int s = !CUT ? row : pt->stage[lane_used ? row : 0];
+    const bool is_first = row == 0 && lane_used, is_last = row == L - 1 && lane_used;
+
+    // static facts of this lane's stage
+    const uint32_t n_in = lane_used ? (uint32_t)p.n_s[CUT || row < p.S ? s : 0] : 0u;
+    const unsigned group_mask = lane_used ? (((L < 32 ? 1u << L : 0u) - 1u) << (j * L)) : 0u;
+    const int root_lane = lane_used ? j * L : 0;
+    // arrival stream: the lane's ring, for the first lane of a group its stretch of the trace or of another part's stream.
+    // Copies are of aligned pairs, so a stream that starts at an odd record of its row is counted from one.
+    const LaneStream *xs_in = CUT && pt->in >= 0 ? cut.stream + pt->in : nullptr;
+    const uint32_t odd = CUT && xs_in ? (uint32_t)xs_in->off & 1u : 0u;
+    const uint32_t n_first = (CUT ? (uint32_t)p.n_s[pt->stage[0]] : (uint32_t)p.n) + odd;       // where the group's stream ends
+    const uint32_t tb = tbw + (uint32_t)(lane_used ? j : 0) * stretch_bytes((int)ahead);
+    const uint32_t xin = is_first ? tb : xb, xin_mask = is_first ? ahead - 1u : kX - 1u, xin_row = is_first ? 8u : 256u;
+    // the child's stream; at the last stage the row of empty records
+    const bool has_child = lane_used && !is_last;
+    const uint32_t xa = has_child ? xbw + (uint32_t)(lane + 1) * 8u : nowhere + (uint32_t)lane * 8u;
+    const uint32_t xam = has_child ? (kX - 1) * 256u : 0u;
+    const uint32_t tail_step = has_child ? 256u : 8u;
+    const int down = has_child ? row : -1;            // (a register that the loop compares with zero: a predicate kept through it costs more)
+    // cut: the last stage's two ways out, taken by a record where (bits & mask) == want; neither: it leaves
+    const int out_kind = CUT ? pt->out_kind : FEAS ? kOutLeaf : kOutOne;
+    auto bit_at = [&](int b) { return b >= 0 ? 1u << (rb > 0 ? qi + b : b) : 0u; };      // (rb = 0: bits looked up)
+    const bool two = CUT && out_kind >= kOutTwo;
+    const uint32_t mask_a = two && is_last ? bit_at(p.cbit_a[s]) : 0u, mask_b = two && is_last && p.child_b[s] >= 0 ? bit_at(p.cbit_b[s]) : 0u;
+    const uint32_t want_a = two && is_last ? (p.cval_a[s] ? mask_a : 0u) : ~0u;
+    const uint32_t want_b = two && is_last && p.child_b[s] >= 0 ? (p.cval_b[s] ? mask_b : 0u) : ~0u;
+    const uint32_t looks_up = two && is_last && rb == 0 ? mask_a | mask_b : 0u;
+    const uint32_t room_a = CUT ? (uint32_t)(pt->out_a >= 0 ? cut.stream[pt->out_a].len : pt->n_leave) : (uint32_t)p.n;     // records its way a holds
+    const uint64_t *trace = rb > 0 ? p.ptrace_b : p.ptrace;
+    // either of two streams of the same row: the second one's tail counts from the first one's start
+    const uint32_t from_b = CUT && !FORK && out_kind == kOutTwo ? (uint32_t)(cut.stream[pt->out_b].off - cut.stream[pt->out_a].off) * 8u : 0u;
+    (void)want_a; (void)want_b; (void)looks_up; (void)from_b; (void)room_a; (void)trace;
 
     // State of the lane's candidate:
     int64_t c = 0;
-    bool has = false;            // the group holds a candidate
-    bool exhausted = !lane_used; // the group will get no further candidate
-    bool live = false, cand_bad = false, over = false;
+    uint32_t node = 0;           // cut: the candidate's root node
+    // Yes or no, in one register: kept as bools these would be predicates that live through the loop, of which there are
+    // seven in all (chain of 4, one warp per scheduler: 9.4 ms for 6.9).
+    enum : uint32_t {
+        kHas = 1,                // the group holds a candidate
+        kNoMore = 2,             // the group will get no further candidate
+        kLive = 4, kBad = 8,     // this lane's stage has records; the candidate's configuration is out of range
+        kOver = 16,              // the candidate has been given up
+        kStarted = 32,           // a first record has opened a batch
+        kSpill = 64,
+        kNobody = 128,           // cut: the stream's producer has given up
+        kDecided = 256,          // cut, feasibility only: the candidate is decided (a root node: all of its candidates are)
+        kFirst = 512, kLastStage = 1024, // first and last stage of the group (always)
+    };
+    uint32_t is = (lane_used ? 0u : (uint32_t)kNoMore) | (is_first ? (uint32_t)kFirst : 0u) | (is_last ? (uint32_t)kLastStage : 0u);
     uint32_t Rm1 = 0;            // replicas less one, in bytes of a ring row
     uint32_t kfb = nowhere, kfm = 0;         // where the first batch in use is looked up (one replica: kInf, which compares as later)
     uint32_t efull = 0;          // tpos with the batch ring full: epos + its size; epos until a first record has opened a batch
     uint32_t lfull = 0;          // tpos with every replica in use or about to be: lpos + replicas less one
-    bool started = false;        // a first record has opened a batch
     uint32_t mbm1 = 0;
     uint32_t tab = tab0;         // the lane's row of the tables
-    uint64_t *out = nullptr;     // leaving records: the stage's region of the slab row (fan-out: the row)
-    uint32_t n_left = 0;         // queries (fan-out: copies) that have left the pipeline at this lane
+    uint64_t *out = nullptr;     // records of the last stage: the stream of way a, or the stage's region of the slab row (fan-out: the row)
+    uint64_t *out_b = nullptr, *out_c = nullptr;     // two ways: the stream of way b; where records leave
+    uint32_t *count_a = nullptr, *count_b = nullptr; // the streams' published counts
+    const uint64_t *src = nullptr;           // the group's arrival stream
+    const uint32_t *src_count = nullptr;     // cut: its count
+    uint32_t avail = 0;          // records of it that are there
+    uint32_t pub_a = 0, pub_b = 0;           // tails published
+    uint32_t n_left = 0;         // two ways: queries (fan-out: copies) that have left the pipeline at this lane
     uint32_t n_cur = 0;          // records of the arrival stream; i counts those examined
     uint32_t i = 0;
     uint32_t bm = ~0u;           // size of the open batch less one (~0: none is open)
@@ -354,31 +416,48 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
     uint32_t epos = 0, lpos = 0, tpos = 0;   // batch ring: [lpos, tpos) in use by replicas, [epos, tpos) not yet handed on
     uint32_t tpos_seen = 0;      // tpos when batches were last counted
     uint32_t prev = 0;           // low part of record i - 1, with its flag
-    bool e_act = false;          // a batch is being handed on:
+    uint32_t e_on = 0;           // 1: a batch is being handed on:
     uint64_t e_key = 0;          //   its key
     uint32_t e_idx = 0;          //   the record to hand on next
-    uint32_t tail_a = 0, tail_b = 0;         // records handed to the children, in bytes of a row
+    uint32_t tail_a = 0, tail_b = 0;         // records handed on: to the child in bytes of a ring row, out in bytes
     uint32_t at1 = kb | rm, at2 = kb | (rm - 256u);          // where the last two batches of the ring are
-    uint32_t fed = 0;            // records of the trace requested for the group's root
+    uint32_t fed = 0;            // records of its stream requested for the group's first lane
     uint32_t qv = 0;             // low part of the record to hand on (where there is one)
-    bool spill = false;
     // No record before low_idx is needed any more once every batch up to low_key has been handed on (next_*: the
     // same for a later moment)
     uint32_t low = 0, next_idx = 0;
     uint64_t next_key = 0;
     unsigned nb = 0;
-    uint32_t ja = 0, jb = 0;     // joins: records of either incoming stream consumed
-    uint32_t seen_new = 0;       // joins: words of the queries' bits from here on have not been touched
     uint32_t turns = 1, turns_hi = 0;        // iteration bound, in turns
+    uint32_t look = 0;
     bool any_spill = false;
     uint64_t late_fin = 0, late_arr = 0;     // feasibility only: finish and arrival record of a query that has just left
-    uint32_t miss_local = 0;
+    uint32_t miss_local = 0, line = 0;       // (line: of the trace, the last one such a query's arrival was in)
+    (void)line; (void)node; (void)avail; (void)pub_a; (void)pub_b; (void)src_count; (void)look;
+
+    __syncwarp();
+    for (int k = 0; k < kX; k++) sts64(xb + (uint32_t)k * 256u, kInf);       // lanes without a stage see no record either
+    sts64(at1, 0ull); sts64(at2, 0ull);
+    __syncwarp();
+
+    // cut, feasibility only: misses seen by this lane are added to the candidate's; whoever passes the limit decides it
+    auto set = [&](uint32_t bit, bool yes) { is = yes ? is | bit : is & ~bit; };
+    auto count_misses = [&]() {
+        const uint32_t before = atomicAdd(cut.miss + c, miss_local);
+        if (before <= p.miss_allow && before + miss_local > p.miss_allow) {
+            p.out_feasible[c] = 0;
+            early += i < n_cur ? 1u : 0u;
+        }
+        if (before + miss_local > p.miss_allow) is |= kDecided;
+        miss_local = 0;
+    };
 
     for (;;) {
         // ---- every kQuickTurn-th, kTurn-th or kLongTurn-th iteration: does a lane need more than its steps?  A stream at its start or its end, a
         // candidate that is decided, records in reach of being overwritten, the iteration bound.  (Kept short: its
         // latency is on the chain of every iteration, a kTurn-th of it.)
-        if (FEAS && miss_local) { atomicAdd(missw + j, miss_local); miss_local = 0; }
+        if (FEAS && !CUT && miss_local) { atomicAdd(missw + j, miss_local); miss_local = 0; }
+        if (FEAS && CUT && miss_local && (look & 3u) == 0u) count_misses();
         nb += (tpos - tpos_seen) >> 8;
         tpos_seen = tpos;
         // Records before `low` are not needed any more.  Cheap and late: all batches closed when next_idx was the
@@ -387,7 +466,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
         const uint64_t fk = epos != tpos ? lds64(kb | (epos & rm)) : kInf;
         const uint64_t lk = lds64(kb | ((tpos - 256u) & rm));
         if (fk > next_key) {
-            low = e_act ? min(next_idx, e_idx) : next_idx;
+            low = e_on != 0u ? min(next_idx, e_idx) : next_idx;
             next_idx = i - (bm + 1u);
             next_key = lk;
         }
@@ -398,33 +477,34 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
         // long passed, needs nothing until that record comes or the group's root is at the end of the trace.  (With a look at it
         // in every turn, and short turns until it had started: chain of 4 whose branch is first taken 20 queries before
         // the end of 50,000, one warp per scheduler, 11.0 ms; 8.9 now, 8.7 where half of the queries take the branch.)
-        const bool waits = i != n_cur && !started;
-        const bool starts = waits && (int)lds32_shared(xin + 4u) >= 0, closes = i == n_cur && bm != ~0u;
-        bool attn = !exhausted && (starts || closes || turns == 0u || (is_root && i == n_cur));
-        attn |= i - low > reach || spill;
-        if (FEAS) attn |= has && missw[j] > p.miss_allow;
+        const bool waits = i != n_cur && !(is & kStarted);
+        const bool starts = waits && (int)lds32_shared(xin + (i & xin_mask) * xin_row + 4u) >= 0, closes = i == n_cur && bm != ~0u;
+        bool attn = !(is & kNoMore) && (starts || closes || turns == 0u || (row == 0 && i == n_cur));
+        attn |= i - low > reach || (is & kSpill);
+        if (FEAS && !CUT) attn |= (is & kHas) && missw[j] > p.miss_allow;
+        if (CUT) attn |= (is & kHas) && ((is & kNobody) || (is & kDecided) || quit);
         if (__any_sync(full, attn)) {
-        bool done = i == n_cur && bm == ~0u && epos == tpos && !e_act && !(FEAS && late_fin != 0ull);
-        if (is_join && has && !cand_bad) done = ja == join_na && jb == join_nb;
-        bool stop = FEAS && has && missw[j] > p.miss_allow;       // this lane ends its group's candidate here
-        bool give_up = false;
-        if (i - low > reach || spill) {
+        bool done = i == n_cur && bm == ~0u && epos == tpos && e_on == 0u && !(FEAS && late_fin != 0ull);
+        bool stop = FEAS && !CUT && (is & kHas) && missw[j] > p.miss_allow;       // this lane ends its group's candidate here
+        if (CUT) stop = (is & kHas) && ((is & kNobody) || (is & kDecided) || quit);
+        bool give_up = CUT && (is & kHas) && (is & kNobody) && !(is & kDecided);
+        if (i - low > reach || (is & kSpill)) {
             // the oldest record still needed, exactly
             low = i - (bm + 1u);
-            if (e_act) low = min(low, e_idx);
+            if (e_on) low = min(low, e_idx);
 #pragma unroll 1
             for (uint32_t k = epos; k != tpos; k += 256u) low = min(low, (uint32_t)lds64(kb | (k & rm)) & qmask);
             const uint32_t span = i - low;
-            if (!spill && span > (uint32_t)(nq - kTurn - 2)) {
+            if (!(is & kSpill) && span > (uint32_t)(nq - kTurn - 2)) {
 #pragma unroll 1
                 for (uint32_t k = low; k != i; k++)
                     if (IL_IN_RANGE(k & gmask, gmask + 1ull, p.status))
                         spill_ring[k & gmask] = lds32(qb + ((k & (nq - 1u)) << 7));
-                spill = true;
-            } else if (spill && span < nq / 2u) {
-                spill = false;
+                is |= kSpill;
+            } else if ((is & kSpill) && span < nq / 2u) {
+                is &= ~(uint32_t)kSpill;
             }
-            give_up = p.lane_wrap && span + 2u * kTurn > gmask;
+            give_up |= p.lane_wrap && span + 2u * kTurn > gmask;
         }
         if (turns == 0u && !done) {
             turns = ~0u;
@@ -435,29 +515,30 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
             }
         }
         stop = (__ballot_sync(full, stop) & group_mask) != 0u;                // the whole group
+        if (FEAS && CUT) set(kDecided, (__ballot_sync(full, (is & kDecided)) & group_mask) != 0u);
         if (p.lane_wrap) {
             const bool group_gives_up = (__ballot_sync(full, give_up) & group_mask) != 0u;
-            if (group_gives_up && !over) { over = true; if (has) p.ovf[c] = 1; }
+            if (group_gives_up && !(is & kOver)) { is |= kOver; if ((is & kHas) && !per_node) p.ovf[c] = 1; }
             stop |= group_gives_up;
         }
         if (stop) {
-            n_cur = i; bm = ~0u; epos = tpos; efull = tpos; e_act = false; late_fin = 0; started = false;
-            ja = join_na; jb = join_nb;
+            n_cur = i; bm = ~0u; epos = tpos; efull = tpos; e_on = 0u; late_fin = 0; is &= ~(uint32_t)kStarted;
             done = true;
         }
         // The first record of a stream opens a batch on an unused replica, and the last batch is closed by the
         // end of the stream; both once per candidate, so here and not in every iteration.
-        if (!done && !started && !is_join) {
-            const uint64_t rec = lds64_shared(xin);
+        if (!done && !(is & kStarted)) {
+            const uint32_t at = xin + (i & xin_mask) * xin_row;
+            const uint64_t rec = lds64_shared(at);
             if ((int64_t)rec >= 0) {
                 tk = rec | qmask;
-                bm = 0; i = 1;
+                bm = 0; i++;
                 prev = (uint32_t)rec & qmask;
-                sts32_shared_if(true, xin + 4u, ~0u);
-                started = true;
+                sts32_shared_if(true, at + 4u, ~0u);
+                is |= kStarted;
                 efull = epos + rm + 256u;
             }
-        } else if (!done && !is_join && i == n_cur && bm != ~0u && tpos != efull) {
+        } else if (!done && i == n_cur && bm != ~0u && tpos != efull) {
             const uint64_t key = ((tk + (uint64_t)lds32(tab + bm * 4u) * tick) & ~(uint64_t)qmask) | (i - 1u - bm);
             uint32_t pos = tpos;
             for (; pos != lpos; pos -= 256u) {
@@ -471,345 +552,812 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
             tk = kLatest;       // nothing more will be dispatched: every batch may leave
             prev |= kLast;
             sts32(qb + (((i - 1u) & (nq - 1u)) << 7), prev);
-            if (spill && IL_IN_RANGE((i - 1u) & gmask, gmask + 1ull, p.status)) spill_ring[(i - 1u) & gmask] = prev;
+            if ((is & kSpill) && IL_IN_RANGE((i - 1u) & gmask, gmask + 1ull, p.status)) spill_ring[(i - 1u) & gmask] = prev;
         }
         const unsigned dm = __ballot_sync(full, done);
-        const bool turn = !exhausted && (dm & group_mask) == group_mask;
+        const bool turn = !(is & kNoMore) && (dm & group_mask) == group_mask;
         if (__any_sync(full, turn)) {
             // wrap up the candidate the group has finished
-            if (turn && has) {
-                if (live && !over) {
+            if (turn && (is & kHas)) {
+                if (FEAS && CUT && miss_local && !stop) count_misses();
+                if ((is & kLive) && !(is & kOver) && !(CUT && quit != 0u)) {
                     batches += nb;
                     alg_ops += 3ull * n_in + (unsigned long long)nb * ((Rm1 >> 8) + mbm1 + 6u);
                 }
-                const bool decided = FEAS && missw[j] > p.miss_allow;
-                // every query of a candidate that ran to its end must have left through exactly one
-                // leaf (checked over all candidates of the warp when the kernel ends)
-                if (live && !over && !decided) exits_seen += BRANCHY ? n_left : da < 0 ? tail_a >> 3 : 0u;
-                if (is_root && !cand_bad && !over && !decided)
-                    exits_due += FORK ? (unsigned long long)p.total_leaving : (unsigned long long)(unsigned)p.n;
-                if (FEAS && is_root) {
-                    p.out_feasible[c] = over ? 2 : (decided || cand_bad ? 0 : 1);
+                const bool decided = FEAS && (CUT ? (is & kDecided) : missw[j] > p.miss_allow);
+                // every record of a group that ran to its end must have come out of its last stage, into a stream or
+                // through a leaf (checked over all groups of the warp when the kernel ends)
+                if ((is & kLive) && (is & kLastStage) && !stop && !decided) {
+                    exits_seen += (unsigned long long)(tail_a >> 3) + (two ? ((tail_b - from_b) >> 3) + n_left : 0u);
+                    exits_due += CUT ? (unsigned long long)pt->n_out : (unsigned long long)(unsigned)p.n;
+                }
+                if (FEAS && !CUT && row == 0) {
+                    p.out_feasible[c] = (is & kOver) ? 2 : (decided || (is & kBad) ? 0 : 1);
                     early += (decided && i < n_in) ? 1u : 0u;        // the root had not reached the end of the trace
                 }
+                if (CUT && (count_a || count_b)) {
+                    // all that will come, or that nothing will: then who reads the stream gives up as well
+                    __threadfence();
+                    const bool ok = !stop && !(is & kBad);
+                    if (count_a) stg32_shared(count_a, ok ? tail_a >> 3 : kDead);
+                    if (count_b) stg32_shared(count_b, ok ? (tail_b - from_b) >> 3 : kDead);
+                }
+                if (CUT && FEAS && (is & kFirst) && xs_in && xs_in->by_node && !(is & kBad)) atomicSub(cut.refs + node, 1u);
             }
             __syncwarp();
             // the group's next candidate
             unsigned long long g = 0;
-            if (turn && is_root) g = atomicAdd(&p.counters[0], 1ull);
+            if (turn && row == 0) g = CUT ? (unsigned long long)atomicAdd(cut.ctl + kCtlWork + part, 1u) : atomicAdd(&p.counters[0], 1ull);
             g = __shfl_sync(full, g, root_lane);
             il_stage_config cfg = {0, 1, 1, 0};
-            const bool got = turn && g < n_cand;
-            if (got && !is_join) cfg = p.configs[g * S + s];
-            const bool bad = got && (cfg.hw >= p.H || cfg.max_batch < 1 || cfg.max_batch > p.Bmax ||
-                                     cfg.replicas < 1 || cfg.replicas > IL_MAX_REPLICAS);
-            const bool grp_bad = (__ballot_sync(full, bad) & group_mask) != 0u;
+            const bool got = turn && g < n_items && !(CUT && quit != 0u);
+            bool bad = false;
+            if (CUT) {
+                int32_t of = 0;
+                if (got && !per_node) of = cut.root_of[g];
+                bad = of < 0;
+                if (turn) node = per_node ? (uint32_t)g : (uint32_t)max(of, 0);
+                if (got && !bad) {
+                    if (per_node) {
+                        const uint32_t w = cut.node_cfg[g];
+                        cfg.hw = (uint8_t)w; cfg.max_batch = (uint8_t)(w >> 8); cfg.replicas = (uint8_t)(w >> 16);
+                    } else {
+                        cfg = p.configs[g * p.S + s];
+                    }
+                }
+            } else {
+                if (got) cfg = p.configs[g * p.S + s];
+                bad = got && (cfg.hw >= p.H || cfg.max_batch < 1 || cfg.max_batch > p.Bmax ||
+                              cfg.replicas < 1 || cfg.replicas > IL_MAX_REPLICAS);
+                bad = (__ballot_sync(full, bad) & group_mask) != 0u;
+            }
             if (turn) {
-                has = got;
-                exhausted = !got;
-                c = (int64_t)g;      // g < n_cand whenever the group got a candidate: rows of the slab, the
-                cand_bad = grp_bad;  // overflow array and the output exist for it
-                over = false;
-                uint64_t *slab = FEAS ? nullptr : reinterpret_cast<uint64_t *>(p.slab + (got ? c : 0) * p.slab_stride);
-                if (got && cand_bad) {
-                    if (is_root) atomicCAS(p.status, 0, IL_ERR_BAD_CONFIG);
-                    if (!FEAS) for (int k = row; k < p.n; k += L) slab[k] = 0;
+                set(kHas, got);
+                set(kNoMore, !got);
+                c = (int64_t)g;      // g < n_items whenever the group got a candidate: rows of the slab, the
+                set(kBad, bad);      // overflow array and the output exist for it
+                is &= ~(uint32_t)kOver;
+                if (CUT) {
+                    auto row_at = [&](const LaneStream &x) { return x.base + (int64_t)(!got ? 0u : x.by_node ? node : (uint32_t)c) * x.stride + x.off; };
+                    auto count_at = [&](const LaneStream &x) { return x.count + (!got ? 0u : x.by_node ? node : (uint32_t)c); };
+                    uint64_t *slab = FEAS ? nullptr : reinterpret_cast<uint64_t *>(p.slab + (got && !per_node ? c : 0) * p.slab_stride);
+                    out_c = FORK || FEAS ? slab : slab + pt->leave_off;
+                    out = out_c;
+                    if (pt->out_a >= 0) { out = row_at(cut.stream[pt->out_a]); if ((is & kLastStage)) count_a = count_at(cut.stream[pt->out_a]); }
+                    if (pt->out_b >= 0) { out_b = row_at(cut.stream[pt->out_b]); if ((is & kLastStage)) count_b = count_at(cut.stream[pt->out_b]); }
+                    src = xs_in ? row_at(*xs_in) - odd : rb > 0 ? p.ptrace_b : p.ptrace;
+                    src_count = xs_in ? count_at(*xs_in) : nullptr;
+                    avail = xs_in ? odd : n_first;
+                    is &= ~(uint32_t)kNobody; is &= ~(uint32_t)kDecided; pub_a = 0; tail_b = from_b; pub_b = tail_b;
+                    if (got && (is & kBad) && !FEAS && !FORK)      // (the call fails, but the percentile pass reads the row)
+                        for (int k = row; k < pt->n_leave; k += L) out_c[k] = 0;
+                } else {
+                    uint64_t *slab = FEAS ? nullptr : reinterpret_cast<uint64_t *>(p.slab + (got ? c : 0) * p.slab_stride);
+                    if (got && (is & kBad)) {
+                        if (row == 0) atomicCAS(p.status, 0, IL_ERR_BAD_CONFIG);
+                        if (!FEAS) for (int k = row; k < p.n; k += L) slab[k] = 0;
+                    }
+                    out = slab;
+                    src = p.ptrace;
+                    avail = n_first;
                 }
-                live = got && !cand_bad && n_in > 0;
-                ja = is_join && got && !cand_bad ? 0u : join_na; jb = is_join && got && !cand_bad ? 0u : join_nb;
-                seen_new = 0u;
-                if (is_join) {
-                    sts32(jw_a, 0u); sts32(jw_b, 0u);
-                    for (int k = 0; k < kSeen; k++) sts64(seen_cache + (uint32_t)k * 8u, kInf);
-                }
+                set(kLive, got && !(is & kBad) && n_in > 0);
                 Rm1 = (cfg.replicas - 1u) << 8;
                 kfb = Rm1 != 0u ? kb : nowhere + (uint32_t)lane * 8u;
                 kfm = Rm1 != 0u ? rm : 0u;
-                started = false; efull = 0; lfull = Rm1;
+                is &= ~(uint32_t)kStarted; efull = 0; lfull = Rm1;
                 mbm1 = cfg.max_batch - 1u;
-                tab = tab0 + (uint32_t)((live ? s * p.H + cfg.hw : 0) * rowlen) * 4u;
-                out = FORK ? slab : slab + exit_off;
+                tab = tab0 + (uint32_t)(((is & kLive) ? s * p.H + cfg.hw : 0) * rowlen) * 4u;
                 n_left = 0;
-                n_cur = live ? n_in : 0u;
+                i = row == 0 ? odd : 0u;
+                n_cur = (is & kLive) ? n_in + i : i;
                 for (int k = 0; k < kX; k++) sts64(xb + (uint32_t)k * 256u, kInf);
-                if (FEAS && is_root) missw[j] = 0u;
-                i = 0; bm = ~0u; tk = 0;
+                if (FEAS && !CUT && row == 0) missw[j] = 0u;
+                bm = ~0u; tk = 0;
                 epos = 0; lpos = 0; tpos = 0; tpos_seen = 0;
                 at1 = kb | rm; at2 = kb | (rm - 256u);
                 sts64(at1, 0ull); sts64(at2, 0ull);       // (no batch before the first one)
                 prev = 0;
-                e_act = false; e_idx = 0;
-                tail_a = 0; tail_b = 0;
-                spill = false; low = 0; next_idx = 0; next_key = 0;
+                e_on = 0u; e_idx = 0;
+                tail_a = 0;
+                is &= ~(uint32_t)kSpill; low = i; next_idx = i; next_key = 0;
                 nb = 0;
                 turns = (uint32_t)limit; turns_hi = (uint32_t)(limit >> 32);
-                late_fin = 0;
-                fed = 0u;
-                if (is_root) for (int k = 0; k < kAhead; k++) sts64(tb + (uint32_t)(k * cpw) * 8u, kInf);
+                late_fin = 0; miss_local = 0;
+                fed = odd;
+                if (row == 0) for (uint32_t k = 0; k < ahead; k++) sts64(tb + k * 8u, kInf);
             }
             __syncwarp();     // the rings are empty before anybody looks
-            if (__all_sync(full, exhausted)) break;
+            if (__all_sync(full, (is & kNoMore))) break;
         }
-        any_spill = __any_sync(full, spill);
+        any_spill = __any_sync(full, (is & kSpill));
         __syncwarp();     // a root's first position is empty before another lane of the group fills it again below
         }
+
+        uint32_t at = __shfl_sync(full, i, root_lane);      // records the group's first lane has examined
+        if (CUT) {
+            // ---- the streams between the parts: what has been written is published, and what others have written is
+            // looked up, every fourth turn or when there is nothing to do
+            const bool feeds = (is & kHas) && !(is & kBad) && !(is & kNobody) && !(is & kDecided);
+            auto short_of = [&](uint32_t records) { return feeds && avail != n_first && avail - at < records; };
+            // no group has a turn's records before it: nothing is lost by waiting for the next ones
+            const bool idle = !__any_sync(full, (is & kFirst) && (is & kHas) && !short_of(kTurn));
+            look++;
+            if ((look & 3u) == 0u || idle) {
+                if (((look & 7u) == 0u || idle) && (is & kHas) && ((count_a && tail_a != pub_a) || (count_b && tail_b != pub_b))) {
+                    __threadfence();
+                    if (count_a) stg32_shared(count_a, tail_a >> 3);
+                    if (count_b) stg32_shared(count_b, (tail_b - from_b) >> 3);
+                    pub_a = tail_a; pub_b = tail_b;
+                }
+                if (__any_sync(full, short_of(2u * ahead))) {
+                    uint32_t word = 0;
+                    if ((is & kFirst) && short_of(2u * ahead)) word = ldg32_acquire(src_count);
+                    word = __shfl_sync(full, word, root_lane);
+                    if (short_of(2u * ahead)) { set(kNobody, word == kDead); avail = (is & kNobody) ? avail : max(avail, word + odd); }
+                }
+                if (FEAS && (is & kFirst) && (is & kHas)) {
+                    if (per_node) set(kDecided, ldg32_shared(cut.refs + node) == 0u);
+                    else if (!(is & kBad)) if (ldg32_shared(cut.miss + c) > p.miss_allow) is |= kDecided;
+                }
+            }
+            if (idle) {
+                if (!__any_sync(full, (is & kFirst) && (is & kHas) && !short_of(kTurn))) {
+                    __nanosleep(500);
+                    turns++;
+                    if (naps-- == 0ull) {
+                        atomicCAS(p.status, 0, IL_ERR_ITER_LIMIT);
+                        atomicOr(&p.counters[5], 1ull);
+                    }
+                    quit = __any_sync(full, *reinterpret_cast<volatile int *>(p.status) != 0) ? 1u : 0u;
+                    continue;
+                }
+            }
+        }
         // (A stage waits for the next turn to open its first batch and to close its last one.  One that has not started within
-        // the first kQuickLooks looks has late records: no short turns for it.)
-        const bool quick = !JOIN && ((i != n_cur && !started && (uint32_t)limit - turns < kQuickLooks) || (i == n_cur && bm != ~0u));
-        const int turn_its = (int)__reduce_min_sync(full, quick ? kQuickTurn : i - low > long_reach ? kTurn : kLongTurn);
+        // the first kQuickLooks looks has late records: no short turns for it.  The other lengths are two less than half of what a
+        // group has before it: one record of that is missing when the first lane is at an odd one, since copies are of pairs.)
+        const bool quick = (i != n_cur && !(is & kStarted) && (uint32_t)limit - turns < kQuickLooks) || (i == n_cur && bm != ~0u);
+        const int turn_its = (int)__reduce_min_sync(full, quick ? kQuickTurn : (i - low > long_reach || ahead < 2u * kLongTurn) ? kTurn - 2 : kLongTurn - 2);
 
-        // The root's next records: requested two turns before their use, by all lanes of the group.
+        // The group's next records: requested two turns before their use where they are there, by all lanes of the group.
         {
-            const uint32_t at = __shfl_sync(full, i, root_lane);
-            const uint32_t to = has && !cand_bad ? min(at + (uint32_t)kAhead, (uint32_t)p.n) : 0u;
+            uint32_t to = (is & kHas) && !(is & kBad) ? min(at + ahead, avail) : 0u;
+            if (to != n_first) to &= ~1u;
+            // (a stream that starts or ends within a pair)
+            if (CUT && (is & kFirst) && to > fed && (fed & 1u)) sts64(tb + (fed & (ahead - 1u)) * 8u, ldg64_shared(src + fed));
+            if ((is & kFirst) && to > fed && (to & 1u) && !((fed & 1u) && to == fed + 1u))
+                sts64(tb + ((to - 1u) & (ahead - 1u)) * 8u, ldg64_shared(src + (to - 1u)));
+            // the first lane can examine turn_its records of what has arrived before; if less has, they are waited for
+            const bool near = (is & kFirst) && (is & kHas) && to > fed && fed - at < (uint32_t)turn_its;
+            const uint32_t by = 2u * (uint32_t)L;
+            uint32_t k = ((fed + 1u) & ~1u) + 2u * (uint32_t)row;
+            auto copy_pair = [&](uint32_t at) { copy16(tb + (at & (ahead - 1u)) * 8u, src + at); };
+            if constexpr (CUT) {      // (a lane on its own copies sixteen pairs; four a round are independent)
 #pragma unroll 1
-            for (uint32_t k = fed + (uint32_t)row; k < to; k += (uint32_t)L) copy8(tb + (k & (kAhead - 1u)) * (uint32_t)cpw * 8u, trace + k);
-            fed = max(fed, to);
+                for (; k + 3u * by + 1u < to; k += 4u * by) { copy_pair(k); copy_pair(k + by); copy_pair(k + 2u * by); copy_pair(k + 3u * by); }
+            }
+#pragma unroll 1
+            for (; k + 1u < to; k += by) copy_pair(k);
+            if (to > fed) fed = to;
+            if (__any_sync(full, near)) { copies_done(); __syncwarp(); }
         }
 
-        // joins: a record for a join.  Records of its two streams are counted in bytes of a row, as tails are.  The
-        // count is told to the join's lane at the top of the NEXT iteration, behind the barrier at the end of this one: whoever
-        // reads a count also sees the records it covers, in the window and in the global stream.
-        auto deliver = [&](bool c, uint64_t *stream, uint32_t win, uint32_t tail, uint64_t rec) {
-            stg64_if(c && IL_IN_RANGE(stream + (tail >> 8) - p.join_ws, p.join_size, p.status), stream + (tail >> 8), rec);
-            sts64_shared_if(c, win + 8u + ((tail >> 5) & win_mask), rec);
-        };
-        // joins: one step of a join's lane takes up to two records of its two incoming streams (every query can come from
-        // both sides), as long as what comes next on both sides is known.  The loads stand at the top of the
-        // iteration and the rest among the stages' work, so that the two hide each other's latency: one after the other,
-        // with the second record's loads behind the first one's stores, an iteration took 0.6 us.
-        // Whether the other input of a record's query has been seen already: the queries' bits are kept in a small
-        // write-back cache; queries come in nearly in order, so a word is new when it is first needed.
-        auto new_word = [&](uint64_t &e, uint32_t w) {
-            const uint32_t old = (uint32_t)(e >> 32);
-            if (old != ~0u && IL_IN_RANGE(old, p.join_seen_words, p.status)) seen[old] = (uint32_t)e;
-            e = (uint64_t)w << 32;
-            if (w < seen_new && IL_IN_RANGE(w, p.join_seen_words, p.status)) e |= seen[w];
-#pragma unroll 1
-            for (; seen_new < w; seen_new++)         // passed over: it may come later
-                if (IL_IN_RANGE(seen_new, p.join_seen_words, p.status)) seen[seen_new] = 0u;
-            seen_new = max(seen_new, w + 1u);
-        };
-        // joins: whether the query of a record goes down both edges into the join
-        auto goes_both = [&](bool known, uint32_t low) {
-            if (join_always) return known;
-            const uint32_t qid = low & imask;
-            uint32_t bits = rb > 0 ? low >> qi : 0u;
-            if (rb == 0 && known && IL_IN_RANGE(qid, p.n, p.status)) bits = p.bits[qid];
-            return known && ((lds32(seen_both + (bits >> 5) * 4u) >> (bits & 31u)) & 1u) != 0u;
-        };
-        auto step = [&](auto spilling) {
+        // One iteration, written in PTX for the sake of its latency, which a warp on its own is bound by: a compare there takes
+        // the condition before it along (setp.and), where the compiler joins finished predicates by instructions of their own,
+        // and what the next iteration reads (its record, the room for the record in hand, the time of the open batch, the low
+        // part to hand on) is requested as soon as it is known where it lies, before this iteration's stores.
+        uint32_t xs = xin + (i & xin_mask) * xin_row, sa = xa | (tail_a & xam);
+        uint64_t rec = lds64_shared(xs);                    // record to examine
+        uint32_t rw = lds32_shared(sa + 4u);                // where the record in hand goes: empty?
+        uint32_t lat = lds32(tab + bm * 4u);                // time of the open batch
+        auto step = [&](auto spilling, auto kind) {
             constexpr bool SPILL = decltype(spilling)::value;
-            // ---- joins: what has come in, the next two records of either side, room for two
-            // (A parent may add one record to what have_a / have_b say before the barrier at the end; its place in the
-            // window is that of a record already taken, or of one that the count does not cover and whose value is not used.)
-            uint32_t have_a = 0, have_b = 0, slot0 = 0, slot1 = 0;
-            uint64_t va0 = 0, va1 = 0, vb0 = 0, vb1 = 0;
-            bool room0 = false, room1 = false;
-            if (JOIN) {
-                sts32_shared_if(tells_a, jw_a, tail_a);
-                sts32_shared_if(tells_b, jw_b, tail_b);
-                have_a = lds32_shared(jw_a); have_b = lds32_shared(jw_b);
-                va0 = lds64_shared(jw_a + 8u + ((ja >> 5) & win_mask)); va1 = lds64_shared(jw_a + 8u + (((ja + 256u) >> 5) & win_mask));
-                vb0 = lds64_shared(jw_b + 8u + ((jb >> 5) & win_mask)); vb1 = lds64_shared(jw_b + 8u + (((jb + 256u) >> 5) & win_mask));
-                slot0 = xj | (tail_a & xjm); slot1 = xj | ((tail_a + 256u) & xjm);
-                room0 = is_join && (int)lds32_shared(slot0 + 4u) < 0;
-                room1 = (int)lds32_shared(slot1 + 4u) < 0;
-            }
-            // ---- everything the iteration needs from shared memory
-            const uint32_t xs = xin + (i & xin_mask) * xin_row;
-            const uint64_t rec = lds64_shared(xs);                    // record to examine
-            const uint32_t lat = lds32(tab + bm * 4u);                // time of the open batch
-            const uint64_t kf = lds64(kfb | (lpos & kfm));            // first batch in use (one replica: kInf)
-            const uint64_t k1 = lds64(at1), k2 = lds64(at2);    // the last two batches
-            const uint64_t fkey = lds64(kb | (epos & rm));            // first batch not handed on (if there is one)
-            const uint32_t sa = xa | (tail_a & xam), sc = xc | (tail_b & xcm);
-            // where the record in hand goes, and whether there is room: towards the outside always
-            uint32_t bits = 0;
-            if (BRANCHY && rb == 0 && e_act && bit >= 0 && IL_IN_RANGE(qv & imask, p.n, p.status)) bits = p.bits[qv & imask];
-            else if (BRANCHY) bits = qv;
-            const bool to_b = BRANCHY && !FORK && (bits & mask_b) != 0u;
-            const bool go_a = FORK && (bits & mask_a) == want_a, go_b = FORK && (bits & mask_b) == want_b;
-            const uint32_t sd = to_b ? sc : sa;
-            const bool free_d = (int)lds32_shared(sd + 4u) < 0;
-            const bool free_b = FORK && (int)lds32_shared(sc + 4u) < 0;
-            const bool f_ok = epos != tpos && not_after(fkey, tk);
-
-            // ---- joins: the one or two records to take
-            uint64_t jrec0 = 0, jrec1 = 0, je0 = 0, je1 = 0;
-            uint32_t jat0 = 0, jat1 = 0;
-            bool known0 = false, known1 = false, from_a0 = false, from_a1 = false;
-            if (JOIN) {
-                const bool end_a = ja == join_na, end_b = jb == join_nb;
-                const bool far_a = is_join && !end_a && have_a - ja > win_reach, far_b = is_join && !end_b && have_b - jb > win_reach;
-                if (far_a || far_b) {
-                    // (the lines from here on are complete, so they may come through L1)
-                    if (far_a && IL_IN_RANGE(jg_a + (ja >> 8) - p.join_ws, p.join_size, p.status)) va0 = jg_a[ja >> 8];
-                    if (far_a && (ja & 0xf00u) == 0u) asm volatile("prefetch.global.L1 [%0];" ::"l"(jg_a + (ja >> 8) + 32u));
-                    if (far_b && IL_IN_RANGE(jg_b + (jb >> 8) - p.join_ws, p.join_size, p.status)) vb0 = jg_b[jb >> 8];
-                    if (far_b && (jb & 0xf00u) == 0u) asm volatile("prefetch.global.L1 [%0];" ::"l"(jg_b + (jb >> 8) + 32u));
-                }
-                known0 = room0 && (end_a || have_a != ja) && (end_b || have_b != jb) && !(end_a && end_b);
-                va0 = end_a ? kInf : va0;
-                vb0 = end_b ? kInf : vb0;
-                from_a0 = (va0 | qmask) <= (vb0 | qmask);
-                jrec0 = from_a0 ? va0 : vb0;
-                // behind it: on its side the record after it, on the other side the same one as before
-                const uint32_t ja1 = ja + (from_a0 ? 256u : 0u), jb1 = jb + (from_a0 ? 0u : 256u);
-                const bool end_a1 = ja1 == join_na, end_b1 = jb1 == join_nb;
-                known1 = known0 && room1 && !far_a && !far_b && (end_a1 || have_a != ja1) && (end_b1 || have_b != jb1) && !(end_a1 && end_b1);
-                const uint64_t va = end_a1 ? kInf : from_a0 ? va1 : va0, vb = end_b1 ? kInf : from_a0 ? vb0 : vb1;
-                from_a1 = (va | qmask) <= (vb | qmask);
-                jrec1 = from_a1 ? va : vb;
-                jat0 = seen_cache + ((((uint32_t)jrec0 & imask) >> 5) & seen_mask) * 8u;
-                jat1 = seen_cache + ((((uint32_t)jrec1 & imask) >> 5) & seen_mask) * 8u;
-                je0 = lds64(jat0);                       // number of the word << 32 | word
-                je1 = lds64(jat1);
-            }
-
-            // ---- examine record i, if it is there: it joins the open batch, or the open batch is closed and it
-            // opens the next one
-            const bool taken = (int64_t)rec >= 0 && tpos != efull;
-            const bool joins = bm < mbm1 && not_after(rec, tk);
-            const bool join = taken && joins, open = taken && !joins;
-            const uint64_t key = ((tk + (uint64_t)lat * tick) & ~(uint64_t)qmask) | (i - 1u - bm);
-            // the next batch goes to a replica never used so far (free from time 0), else to the one that is
-            // free first -- maybe the one whose batch is closed just now
-            const bool pop = tpos == lfull;
-            const uint64_t first = before(kf, key) ? kf : key;
-            // its place in the ring: behind the last one, nearly always, or just before it (a batch that finishes
-            // before one dispatched earlier); further ahead is rare enough for a loop
-            const uint32_t at0 = kb | (tpos & rm);
-            const bool overtakes = before(key, k1);
-            sts64_if(open, overtakes ? at1 : at0, key);
-            sts64_if(open && overtakes, at0, k1);
-            if (open && overtakes && before(key, k2)) {
-                uint32_t pos = tpos - 256u;
-                for (;;) {       // four at a time: the loads overlap, and most of the time one round does it
-                    const uint32_t left = pos - lpos;
-                    const uint32_t a0 = kb | (pos & rm), a1 = kb | ((pos - 256u) & rm), a2 = kb | ((pos - 512u) & rm),
-                                   a3 = kb | ((pos - 768u) & rm), a4 = kb | ((pos - 1024u) & rm);
-                    const uint64_t e1 = lds64(a1), e2 = lds64(a2), e3 = lds64(a3), e4 = lds64(a4);
-                    const bool m1 = left > 0u && e1 > key, m2 = m1 && left > 256u && e2 > key,
-                               m3 = m2 && left > 512u && e3 > key, m4 = m3 && left > 768u && e4 > key;
-                    sts64_if(m1, a0, e1); sts64_if(m2, a1, e2); sts64_if(m3, a2, e3); sts64_if(m4, a3, e4);
-                    sts64(m4 ? a4 : m3 ? a3 : m2 ? a2 : m1 ? a1 : a0, key);
-                    if (!m4) break;
-                    pos -= 1024u;
-                }
-            }
-            // dispatch time: the record's, or later the time the replica is free
-            const uint64_t start = ((pop && before(rec, first)) ? first : rec) | qmask;
-            tk = open ? start : tk;
-            tpos += open ? 256u : 0u;
-            at2 = open ? at1 : at2;
-            at1 = open ? at0 : at1;
-            lpos += (open && pop) ? 256u : 0u;
-            lfull += (open && pop) ? 256u : 0u;
-            bm += join ? 1u : 0u;
-            bm = open ? 0u : bm;
-            // the word of record i - 1 is final now: the last one of its batch or not
-            const uint32_t word = prev | (open ? kLast : 0u);
-            sts32_if(taken, qb + (((i - 1u) & (nq - 1u)) << 7), word);
-            sts32_shared_if(taken, xs + 4u, ~0u);
-            if (SPILL) {
-                stg32_if(spill && taken && IL_IN_RANGE((i - 1u) & gmask, gmask + 1ull, p.status), spill_ring + ((i - 1u) & gmask), word);
-            }
-            prev = taken ? (uint32_t)rec & qmask : prev;
-            i += taken ? 1u : 0u;
-
-            // ---- joins: the records are counted, and the last input of a query goes to the join's stage
-            if (JOIN) {
-                const uint32_t low0 = (uint32_t)jrec0 & qmask, low1 = (uint32_t)jrec1 & qmask;
-                const uint32_t w0 = (low0 & imask) >> 5, w1 = (low1 & imask) >> 5, mine0 = 1u << (low0 & 31u), mine1 = 1u << (low1 & 31u);
-                const bool both0 = goes_both(known0, low0);
-                bool both1 = goes_both(known1, low1);
-                const bool fresh = both0 && (uint32_t)(je0 >> 32) != w0;
-                if (fresh) new_word(je0, w0);
-                if (fresh || (both1 && (uint32_t)(je1 >> 32) != w1)) { known1 = false; both1 = false; }     // (next time)
-                sts64_if(both0, jat0, je0 ^ mine0);
-                if (both0 && jat0 == jat1) je1 ^= mine0;
-                sts64_if(both1, jat1, je1 ^ mine1);
-                const bool last0 = known0 && (!both0 || ((uint32_t)je0 & mine0) != 0u);
-                const bool last1 = known1 && (!both1 || ((uint32_t)je1 & mine1) != 0u);
-                sts64_shared_if(last0, slot0, jrec0);
-                sts64_shared_if(last1, last0 ? slot1 : slot0, jrec1);
-                ja += (known0 && from_a0 ? 256u : 0u) + (known1 && from_a1 ? 256u : 0u);
-                jb += (known0 && !from_a0 ? 256u : 0u) + (known1 && !from_a1 ? 256u : 0u);
-                tail_a += (last0 ? 256u : 0u) + (last1 ? 256u : 0u);
-            }
-
-            // ---- hand on
+            constexpr int OUT = decltype(kind)::value;
             if (FEAS) miss_local += (late_fin > late_arr + slo_q) ? 1u : 0u;
-            const bool last = (int)qv < 0;
-            const uint64_t e_base = e_key & ~(uint64_t)qmask;         // finish << q
-            qv &= ~kLast;
-            const uint32_t qid = BRANCHY ? qv & imask : qv;
-            bool hand;
-            if (BRANCHY) {
-                if (FORK) {
-                    hand = e_act && (!go_a || free_d) && (!go_b || free_b);
-                    sts64_shared_if(hand && go_a && !join_a, sa, e_base | qv);
-                    sts64_shared_if(hand && go_b && !join_b, sc, e_base | qv);
-                    if (JOIN) {
-                        deliver(hand && go_a && join_a, jg_a, jw_a, tail_a, e_base | qv);
-                        deliver(hand && go_b && join_b, jg_b, jw_b, tail_b, e_base | qv);
-                    }
-                    tail_a += (hand && go_a) ? 256u : 0u;
-                    tail_b += (hand && go_b) ? 256u : 0u;
-                    // this copy leaves: the query's slab entry keeps the latest of its copies
-                    if (hand && !go_a && !go_b) {
-                        if (IL_IN_RANGE(qid, p.n, p.status))
-                            atomicMax(reinterpret_cast<unsigned long long *>(out) + qid, (e_base >> rb) | qid);
-                        n_left++;
-                    }
+            [[maybe_unused]] uint32_t bits = qv;
+            if (OUT == kOutAny && looks_up != 0u && e_on != 0u && IL_IN_RANGE(qv & imask, p.n, p.status)) bits = p.bits[qv & imask];
+            [[maybe_unused]] uint32_t leaves = 0u;
+            [[maybe_unused]] const uint64_t left_rec = e_key;              // what leaves: key and low part of the record in hand
+            [[maybe_unused]] const uint32_t left_low = qv & ~kLast;
+            [[maybe_unused]] const uint32_t i_was = i, tpos_was = tpos, prev_was = prev;
+#ifdef IL_CHECKED
+            if (e_on != 0u && down < 0) {
+                bool in = IL_IN_RANGE(qv & imask, p.n, p.status);
+                if (OUT != kOutTwo && OUT != kOutAny) {
+                    in &= IL_IN_RANGE(tail_a >> 3, room_a, p.status);
                 } else {
-                    const bool leaves = to_b ? db < 0 : da < 0;
-                    hand = e_act && free_d;
-                    sts64_shared_if(hand && !leaves, sd, e_base | qv);
-                    // (slab records are plain (finish, query) records whatever the streams carry)
-                    if (!FEAS) stg64_if(hand && leaves && IL_IN_RANGE(n_left, leaving, p.status), out + n_left, (e_base >> rb) | qid);
-                    if (FEAS) {
-                        late_fin = (hand && leaves) ? e_base : 0ull;
-                        late_arr = __ldg(trace + (hand && leaves && IL_IN_RANGE(qid, p.n, p.status) ? qid : 0u));
-                    }
-                    tail_a += (hand && !to_b) ? 256u : 0u;
-                    tail_b += (hand && to_b) ? 256u : 0u;
-                    n_left += (hand && leaves) ? 1u : 0u;
+                    if ((bits & mask_a) == want_a) in &= IL_IN_RANGE(tail_a >> 3, room_a, p.status);
+                    if ((bits & mask_b) == want_b) in &= IL_IN_RANGE((tail_b - from_b) >> 3, cut.stream[pt->out_b].len, p.status);
                 }
+                if (!in) e_on = 0u;
+            }
+#endif
+            if constexpr (OUT == kOutOne) {
+                asm volatile(
+                    "{\n"
+                    ".reg .b32 i; .reg .b32 bm; .reg .b32 lpos; .reg .b32 lfull; .reg .b32 tpos; .reg .b32 at1; .reg .b32 at2;\n"
+                    ".reg .b64 tk; .reg .b32 prev; .reg .b64 rec; .reg .b32 lat; .reg .b32 xs; .reg .b32 epos; .reg .b32 efull;\n"
+                    ".reg .b32 e_on; .reg .b64 e_key; .reg .b32 e_idx; .reg .b32 qv; .reg .b32 tail_a; .reg .b32 rw; .reg .b32 sa;\n"
+                    ".reg .b32 xin; .reg .b32 xin_mask; .reg .b32 xin_row; .reg .b32 tab; .reg .b32 kfb; .reg .b32 kfm; .reg .b32 kb;\n"
+                    ".reg .b32 rm; .reg .b32 mbm1; .reg .b32 tick; .reg .b32 qmask; .reg .b32 tmask; .reg .b32 qb; .reg .b32 nqm;\n"
+                    ".reg .b32 xa; .reg .b32 xam; .reg .b32 down; .reg .b32 tail_step; .reg .b64 out;\n"
+                    "mov.b32 i, %0; mov.b32 bm, %1; mov.b32 lpos, %2; mov.b32 lfull, %3; mov.b32 tpos, %4; mov.b32 at1, %5;\n"
+                    "mov.b32 at2, %6; mov.b64 tk, %7; mov.b32 prev, %8; mov.b64 rec, %9; mov.b32 lat, %10; mov.b32 xs, %11;\n"
+                    "mov.b32 epos, %12; mov.b32 efull, %13; mov.b32 e_on, %14; mov.b64 e_key, %15; mov.b32 e_idx, %16; mov.b32 qv, %17;\n"
+                    "mov.b32 tail_a, %18; mov.b32 rw, %19; mov.b32 sa, %20; mov.b32 xin, %21; mov.b32 xin_mask, %22; mov.b32 xin_row, %23;\n"
+                    "mov.b32 tab, %24; mov.b32 kfb, %25; mov.b32 kfm, %26; mov.b32 kb, %27; mov.b32 rm, %28; mov.b32 mbm1, %29;\n"
+                    "mov.b32 tick, %30; mov.b32 qmask, %31; mov.b32 tmask, %32; mov.b32 qb, %33; mov.b32 nqm, %34; mov.b32 xa, %35;\n"
+                    "mov.b32 xam, %36; mov.b32 down, %37; mov.b32 tail_step, %38; mov.b64 out, %39;\n"
+                    ".reg .pred t, taken, open, pop, ov, dp, pz, pf, hand, hd, ho, fin, fetch;\n"
+                    ".reg .u32 at0, sd, rl, rh, kl, kh, fl, fh, word, wa, x, y, lo, hi, a, xs_was, sa_was, ta_was, pos, left, a1, a2, a3, a4;\n"
+                    ".reg .b64 kf, k1, k2, fk, key, td, r, first, v, e1, e2, e3, e4; .reg .b64 o;\n"
+                    "and.b32 a, epos, rm; or.b32 a, a, kb; ld.shared.b64 fk, [a];\n"
+                    "and.b32 a, lpos, kfm; or.b32 a, a, kfb; ld.shared.b64 kf, [a];\n"
+                    "ld.shared.b64 k1, [at1]; ld.shared.b64 k2, [at2];\n"
+                    "mov.b64 td, tk; mov.b64 {rl, rh}, rec; mov.u32 xs_was, xs; mov.u32 sa_was, sa;\n"
+                    "setp.ne.u32 t, tpos, efull; selp.b32 rh, rh, -1, t; mov.b64 r, {rl, rh};\n"
+                    "setp.ge.s32 taken, rh, 0; setp.ge.and.u32 t, bm, mbm1, taken; setp.gt.or.f64 open, r, td, t;\n"
+                    "sub.u32 y, i, bm; add.u32 y, y, -1;\n"
+                    "add.u32 wa, i, -1; and.b32 wa, wa, nqm; mad.lo.u32 wa, wa, 128, qb;\n"
+                    "@taken add.u32 i, i, 1; and.b32 xs, i, xin_mask; mad.lo.u32 xs, xs, xin_row, xin; ld.relaxed.cta.shared.b64 rec, [xs];\n"
+                    "setp.lt.s32 hand, rw, 0; setp.ne.and.u32 hand, e_on, 0, hand; setp.ge.and.s32 hd|ho, down, 0, hand; setp.lt.and.s32 fin, qv, 0, hand;\n"
+                    "and.b32 x, qv, 0x7fffffff; mov.b64 {lo, hi}, e_key; and.b32 lo, lo, tmask; or.b32 a, lo, x; mov.b64 v, {a, hi}; mov.u32 ta_was, tail_a;\n"
+                    "@hand add.u32 tail_a, tail_a, tail_step;\n"
+                    "and.b32 sa, tail_a, xam; or.b32 sa, sa, xa; ld.relaxed.cta.shared.u32 rw, [sa+4];\n"
+                    "mad.wide.u32 key, lat, tick, tk; mov.b64 {kl, kh}, key; and.b32 kl, kl, tmask; or.b32 kl, kl, y; mov.b64 key, {kl, kh};\n"
+                    "@taken add.u32 bm, bm, 1; @open mov.u32 bm, 0; mad.lo.u32 a, bm, 4, tab; ld.shared.u32 lat, [a];\n"
+                    "setp.eq.or.u32 fetch, e_on, 0, fin; setp.ne.and.u32 fetch, epos, tpos, fetch; setp.le.and.f64 fetch, fk, td, fetch;\n"
+                    "mov.b64 {fl, fh}, fk;\n"
+                    "@hand add.u32 e_idx, e_idx, 1; @fetch and.b32 e_idx, fl, qmask; and.b32 a, e_idx, nqm; mad.lo.u32 a, a, 128, qb; ld.shared.u32 qv, [a];\n"
+                    "@hd st.relaxed.cta.shared.b64 [sa_was], v;\n"
+                    "mad.wide.u32 o, ta_was, 1, out; @ho st.global.b64 [o], v;\n"
+                    "@fetch mov.b64 e_key, fk; @fin mov.u32 e_on, 0; @fetch mov.u32 e_on, 1; @fetch add.u32 epos, epos, 256; @fetch add.u32 efull, efull, 256;\n"
+                    "and.b32 at0, tpos, rm; or.b32 at0, at0, kb;\n"
+                    "setp.lt.f64 pf, kf, key; selp.b64 first, kf, key, pf;\n"
+                    "setp.eq.u32 pz, tpos, lfull; setp.lt.and.f64 pz, r, first, pz; selp.b64 first, first, r, pz;\n"
+                    "mov.b64 {fl, fh}, first; or.b32 fl, fl, qmask; mov.b64 first, {fl, fh}; selp.b64 tk, first, tk, open;\n"
+                    "setp.lt.and.f64 ov, key, k1, open; selp.u32 sd, at1, at0, ov;\n"
+                    "@open st.shared.b64 [sd], key; @ov st.shared.b64 [at0], k1;\n"
+                    "setp.lt.and.f64 dp, key, k2, ov; mov.u32 pos, tpos; mov.u32 left, lpos;\n"
+                    "setp.eq.and.u32 pop, tpos, lfull, open;\n"
+                    "mov.u32 word, prev; @open or.b32 word, word, 0x80000000; @taken st.shared.u32 [wa], word;\n"
+                    "@taken st.relaxed.cta.shared.u32 [xs_was+4], -1;\n"
+                    "@open add.u32 tpos, tpos, 256; @open mov.u32 at2, at1; @open mov.u32 at1, at0;\n"
+                    "@pop add.u32 lpos, lpos, 256; @pop add.u32 lfull, lfull, 256;\n"
+                    "@taken and.b32 prev, rl, qmask;\n"
+                    "@!dp bra PLACED;\n"
+                    "mov.u32 sd, left; sub.u32 pos, pos, 256;\n"
+                    "DEEPER:\n"
+                    "sub.u32 left, pos, sd;\n"
+                    "and.b32 at0, pos, rm; or.b32 at0, at0, kb; sub.u32 a1, pos, 256; and.b32 a1, a1, rm; or.b32 a1, a1, kb;\n"
+                    "sub.u32 a2, pos, 512; and.b32 a2, a2, rm; or.b32 a2, a2, kb; sub.u32 a3, pos, 768; and.b32 a3, a3, rm; or.b32 a3, a3, kb;\n"
+                    "sub.u32 a4, pos, 1024; and.b32 a4, a4, rm; or.b32 a4, a4, kb;\n"
+                    "ld.shared.b64 e1, [a1]; ld.shared.b64 e2, [a2]; ld.shared.b64 e3, [a3]; ld.shared.b64 e4, [a4];\n"
+                    "setp.gt.u32 t, left, 0; setp.lt.and.f64 t, key, e1, t; setp.gt.and.u32 ov, left, 256, t; setp.lt.and.f64 ov, key, e2, ov;\n"
+                    "setp.gt.and.u32 pz, left, 512, ov; setp.lt.and.f64 pz, key, e3, pz; setp.gt.and.u32 pf, left, 768, pz; setp.lt.and.f64 pf, key, e4, pf;\n"
+                    "@t st.shared.b64 [at0], e1; @ov st.shared.b64 [a1], e2; @pz st.shared.b64 [a2], e3; @pf st.shared.b64 [a3], e4;\n"
+                    "@t mov.u32 at0, a1; @ov mov.u32 at0, a2; @pz mov.u32 at0, a3; @pf mov.u32 at0, a4; st.shared.b64 [at0], key;\n"
+                    "sub.u32 pos, pos, 1024; @pf bra DEEPER;\n"
+                    "PLACED:\n"
+                    "mov.b32 %0, i; mov.b32 %1, bm; mov.b32 %2, lpos; mov.b32 %3, lfull; mov.b32 %4, tpos; mov.b32 %5, at1;\n"
+                    "mov.b32 %6, at2; mov.b64 %7, tk; mov.b32 %8, prev; mov.b64 %9, rec; mov.b32 %10, lat; mov.b32 %11, xs;\n"
+                    "mov.b32 %12, epos; mov.b32 %13, efull; mov.b32 %14, e_on; mov.b64 %15, e_key; mov.b32 %16, e_idx; mov.b32 %17, qv;\n"
+                    "mov.b32 %18, tail_a; mov.b32 %19, rw; mov.b32 %20, sa;\n"
+                    "}"
+                    : "+r"(i), "+r"(bm), "+r"(lpos), "+r"(lfull), "+r"(tpos), "+r"(at1), "+r"(at2), "+l"(tk), "+r"(prev), "+l"(rec), "+r"(lat), "+r"(xs), "+r"(epos), "+r"(efull), "+r"(e_on), "+l"(e_key), "+r"(e_idx), "+r"(qv), "+r"(tail_a), "+r"(rw), "+r"(sa)
+                    : "r"(xin), "r"(xin_mask), "r"(xin_row), "r"(tab), "r"(kfb), "r"(kfm), "r"(kb), "r"(rm), "r"(mbm1), "r"(tick), "r"(qmask), "r"(~qmask), "r"(qb), "r"(nq - 1u), "r"(xa), "r"(xam), "r"(down), "r"(tail_step), "l"(out)
+                    : "memory");
+            } else if constexpr (OUT == kOutLeaf && FEAS) {
+                // (compared with the objective in the next iteration; the arrival's line was asked for with the one before it)
+                asm volatile(
+                    "{\n"
+                    ".reg .b32 i; .reg .b32 bm; .reg .b32 lpos; .reg .b32 lfull; .reg .b32 tpos; .reg .b32 at1; .reg .b32 at2;\n"
+                    ".reg .b64 tk; .reg .b32 prev; .reg .b64 rec; .reg .b32 lat; .reg .b32 xs; .reg .b32 epos; .reg .b32 efull;\n"
+                    ".reg .b32 e_on; .reg .b64 e_key; .reg .b32 e_idx; .reg .b32 qv; .reg .b32 tail_a; .reg .b32 rw; .reg .b32 sa;\n"
+                    ".reg .b64 late_fin; .reg .b64 late_arr; .reg .b32 line; .reg .b32 xin; .reg .b32 xin_mask; .reg .b32 xin_row;\n"
+                    ".reg .b32 tab; .reg .b32 kfb; .reg .b32 kfm; .reg .b32 kb; .reg .b32 rm; .reg .b32 mbm1; .reg .b32 tick;\n"
+                    ".reg .b32 qmask; .reg .b32 tmask; .reg .b32 qb; .reg .b32 nqm; .reg .b32 xa; .reg .b32 xam; .reg .b32 down;\n"
+                    ".reg .b32 tail_step; .reg .b64 trace; .reg .b32 imask;\n"
+                    "mov.b32 i, %0; mov.b32 bm, %1; mov.b32 lpos, %2; mov.b32 lfull, %3; mov.b32 tpos, %4; mov.b32 at1, %5;\n"
+                    "mov.b32 at2, %6; mov.b64 tk, %7; mov.b32 prev, %8; mov.b64 rec, %9; mov.b32 lat, %10; mov.b32 xs, %11;\n"
+                    "mov.b32 epos, %12; mov.b32 efull, %13; mov.b32 e_on, %14; mov.b64 e_key, %15; mov.b32 e_idx, %16; mov.b32 qv, %17;\n"
+                    "mov.b32 tail_a, %18; mov.b32 rw, %19; mov.b32 sa, %20; mov.b64 late_arr, %22; mov.b32 line, %23; mov.b32 xin, %24;\n"
+                    "mov.b32 xin_mask, %25; mov.b32 xin_row, %26; mov.b32 tab, %27; mov.b32 kfb, %28; mov.b32 kfm, %29; mov.b32 kb, %30;\n"
+                    "mov.b32 rm, %31; mov.b32 mbm1, %32; mov.b32 tick, %33; mov.b32 qmask, %34; mov.b32 tmask, %35; mov.b32 qb, %36;\n"
+                    "mov.b32 nqm, %37; mov.b32 xa, %38; mov.b32 xam, %39; mov.b32 down, %40; mov.b32 tail_step, %41; mov.b64 trace, %42;\n"
+                    "mov.b32 imask, %43;\n"
+                    ".reg .pred t, taken, open, pop, ov, dp, pz, pf, hand, hd, ho, fin, fetch;\n"
+                    ".reg .u32 at0, sd, rl, rh, kl, kh, fl, fh, word, wa, x, y, lo, hi, a, xs_was, sa_was, ta_was, pos, left, a1, a2, a3, a4;\n"
+                    ".reg .b64 kf, k1, k2, fk, key, td, r, first, v, e1, e2, e3, e4; .reg .pred nl; .reg .b64 o;\n"
+                    "and.b32 a, epos, rm; or.b32 a, a, kb; ld.shared.b64 fk, [a];\n"
+                    "and.b32 a, lpos, kfm; or.b32 a, a, kfb; ld.shared.b64 kf, [a];\n"
+                    "ld.shared.b64 k1, [at1]; ld.shared.b64 k2, [at2];\n"
+                    "mov.b64 td, tk; mov.b64 {rl, rh}, rec; mov.u32 xs_was, xs; mov.u32 sa_was, sa;\n"
+                    "setp.ne.u32 t, tpos, efull; selp.b32 rh, rh, -1, t; mov.b64 r, {rl, rh};\n"
+                    "setp.ge.s32 taken, rh, 0; setp.ge.and.u32 t, bm, mbm1, taken; setp.gt.or.f64 open, r, td, t;\n"
+                    "sub.u32 y, i, bm; add.u32 y, y, -1;\n"
+                    "add.u32 wa, i, -1; and.b32 wa, wa, nqm; mad.lo.u32 wa, wa, 128, qb;\n"
+                    "@taken add.u32 i, i, 1; and.b32 xs, i, xin_mask; mad.lo.u32 xs, xs, xin_row, xin; ld.relaxed.cta.shared.b64 rec, [xs];\n"
+                    "setp.lt.s32 hand, rw, 0; setp.ne.and.u32 hand, e_on, 0, hand; setp.ge.and.s32 hd|ho, down, 0, hand; setp.lt.and.s32 fin, qv, 0, hand;\n"
+                    "and.b32 x, qv, 0x7fffffff; mov.b64 {lo, hi}, e_key; and.b32 lo, lo, tmask; or.b32 a, lo, x; mov.b64 v, {a, hi}; mov.u32 ta_was, tail_a;\n"
+                    "@hand add.u32 tail_a, tail_a, tail_step;\n"
+                    "and.b32 sa, tail_a, xam; or.b32 sa, sa, xa; ld.relaxed.cta.shared.u32 rw, [sa+4];\n"
+                    "mad.wide.u32 key, lat, tick, tk; mov.b64 {kl, kh}, key; and.b32 kl, kl, tmask; or.b32 kl, kl, y; mov.b64 key, {kl, kh};\n"
+                    "@taken add.u32 bm, bm, 1; @open mov.u32 bm, 0; mad.lo.u32 a, bm, 4, tab; ld.shared.u32 lat, [a];\n"
+                    "setp.eq.or.u32 fetch, e_on, 0, fin; setp.ne.and.u32 fetch, epos, tpos, fetch; setp.le.and.f64 fetch, fk, td, fetch;\n"
+                    "mov.b64 {fl, fh}, fk;\n"
+                    "@hand add.u32 e_idx, e_idx, 1; @fetch and.b32 e_idx, fl, qmask; and.b32 a, e_idx, nqm; mad.lo.u32 a, a, 128, qb; ld.shared.u32 qv, [a];\n"
+                    "@hd st.relaxed.cta.shared.b64 [sa_was], v;\n"
+                    "mov.b64 o, {lo, hi}; selp.b64 late_fin, o, 0, ho; and.b32 a, x, imask; mad.wide.u32 o, a, 8, trace; @ho ld.global.nc.b64 late_arr, [o];\n"
+                    "shr.u32 a, a, 4; setp.ne.and.u32 nl, a, line, ho; @nl mov.u32 line, a; @nl prefetch.global.L1 [o+128];\n"
+                    "@fetch mov.b64 e_key, fk; @fin mov.u32 e_on, 0; @fetch mov.u32 e_on, 1; @fetch add.u32 epos, epos, 256; @fetch add.u32 efull, efull, 256;\n"
+                    "and.b32 at0, tpos, rm; or.b32 at0, at0, kb;\n"
+                    "setp.lt.f64 pf, kf, key; selp.b64 first, kf, key, pf;\n"
+                    "setp.eq.u32 pz, tpos, lfull; setp.lt.and.f64 pz, r, first, pz; selp.b64 first, first, r, pz;\n"
+                    "mov.b64 {fl, fh}, first; or.b32 fl, fl, qmask; mov.b64 first, {fl, fh}; selp.b64 tk, first, tk, open;\n"
+                    "setp.lt.and.f64 ov, key, k1, open; selp.u32 sd, at1, at0, ov;\n"
+                    "@open st.shared.b64 [sd], key; @ov st.shared.b64 [at0], k1;\n"
+                    "setp.lt.and.f64 dp, key, k2, ov; mov.u32 pos, tpos; mov.u32 left, lpos;\n"
+                    "setp.eq.and.u32 pop, tpos, lfull, open;\n"
+                    "mov.u32 word, prev; @open or.b32 word, word, 0x80000000; @taken st.shared.u32 [wa], word;\n"
+                    "@taken st.relaxed.cta.shared.u32 [xs_was+4], -1;\n"
+                    "@open add.u32 tpos, tpos, 256; @open mov.u32 at2, at1; @open mov.u32 at1, at0;\n"
+                    "@pop add.u32 lpos, lpos, 256; @pop add.u32 lfull, lfull, 256;\n"
+                    "@taken and.b32 prev, rl, qmask;\n"
+                    "@!dp bra PLACED;\n"
+                    "mov.u32 sd, left; sub.u32 pos, pos, 256;\n"
+                    "DEEPER:\n"
+                    "sub.u32 left, pos, sd;\n"
+                    "and.b32 at0, pos, rm; or.b32 at0, at0, kb; sub.u32 a1, pos, 256; and.b32 a1, a1, rm; or.b32 a1, a1, kb;\n"
+                    "sub.u32 a2, pos, 512; and.b32 a2, a2, rm; or.b32 a2, a2, kb; sub.u32 a3, pos, 768; and.b32 a3, a3, rm; or.b32 a3, a3, kb;\n"
+                    "sub.u32 a4, pos, 1024; and.b32 a4, a4, rm; or.b32 a4, a4, kb;\n"
+                    "ld.shared.b64 e1, [a1]; ld.shared.b64 e2, [a2]; ld.shared.b64 e3, [a3]; ld.shared.b64 e4, [a4];\n"
+                    "setp.gt.u32 t, left, 0; setp.lt.and.f64 t, key, e1, t; setp.gt.and.u32 ov, left, 256, t; setp.lt.and.f64 ov, key, e2, ov;\n"
+                    "setp.gt.and.u32 pz, left, 512, ov; setp.lt.and.f64 pz, key, e3, pz; setp.gt.and.u32 pf, left, 768, pz; setp.lt.and.f64 pf, key, e4, pf;\n"
+                    "@t st.shared.b64 [at0], e1; @ov st.shared.b64 [a1], e2; @pz st.shared.b64 [a2], e3; @pf st.shared.b64 [a3], e4;\n"
+                    "@t mov.u32 at0, a1; @ov mov.u32 at0, a2; @pz mov.u32 at0, a3; @pf mov.u32 at0, a4; st.shared.b64 [at0], key;\n"
+                    "sub.u32 pos, pos, 1024; @pf bra DEEPER;\n"
+                    "PLACED:\n"
+                    "mov.b32 %0, i; mov.b32 %1, bm; mov.b32 %2, lpos; mov.b32 %3, lfull; mov.b32 %4, tpos; mov.b32 %5, at1;\n"
+                    "mov.b32 %6, at2; mov.b64 %7, tk; mov.b32 %8, prev; mov.b64 %9, rec; mov.b32 %10, lat; mov.b32 %11, xs;\n"
+                    "mov.b32 %12, epos; mov.b32 %13, efull; mov.b32 %14, e_on; mov.b64 %15, e_key; mov.b32 %16, e_idx; mov.b32 %17, qv;\n"
+                    "mov.b32 %18, tail_a; mov.b32 %19, rw; mov.b32 %20, sa; mov.b64 %21, late_fin; mov.b64 %22, late_arr;\n"
+                    "mov.b32 %23, line;\n"
+                    "}"
+                    : "+r"(i), "+r"(bm), "+r"(lpos), "+r"(lfull), "+r"(tpos), "+r"(at1), "+r"(at2), "+l"(tk), "+r"(prev), "+l"(rec), "+r"(lat), "+r"(xs), "+r"(epos), "+r"(efull), "+r"(e_on), "+l"(e_key), "+r"(e_idx), "+r"(qv), "+r"(tail_a), "+r"(rw), "+r"(sa), "=l"(late_fin), "+l"(late_arr), "+r"(line)
+                    : "r"(xin), "r"(xin_mask), "r"(xin_row), "r"(tab), "r"(kfb), "r"(kfm), "r"(kb), "r"(rm), "r"(mbm1), "r"(tick), "r"(qmask), "r"(~qmask), "r"(qb), "r"(nq - 1u), "r"(xa), "r"(xam), "r"(down), "r"(tail_step), "l"(trace), "r"(imask)
+                    : "memory");
+            } else if constexpr (OUT == kOutLeaf && FORK) {
+                // (the query's slab entry keeps the latest of its copies)
+                asm volatile(
+                    "{\n"
+                    ".reg .b32 i; .reg .b32 bm; .reg .b32 lpos; .reg .b32 lfull; .reg .b32 tpos; .reg .b32 at1; .reg .b32 at2;\n"
+                    ".reg .b64 tk; .reg .b32 prev; .reg .b64 rec; .reg .b32 lat; .reg .b32 xs; .reg .b32 epos; .reg .b32 efull;\n"
+                    ".reg .b32 e_on; .reg .b64 e_key; .reg .b32 e_idx; .reg .b32 qv; .reg .b32 tail_a; .reg .b32 rw; .reg .b32 sa;\n"
+                    ".reg .b32 xin; .reg .b32 xin_mask; .reg .b32 xin_row; .reg .b32 tab; .reg .b32 kfb; .reg .b32 kfm; .reg .b32 kb;\n"
+                    ".reg .b32 rm; .reg .b32 mbm1; .reg .b32 tick; .reg .b32 qmask; .reg .b32 tmask; .reg .b32 qb; .reg .b32 nqm;\n"
+                    ".reg .b32 xa; .reg .b32 xam; .reg .b32 down; .reg .b32 tail_step; .reg .b64 out; .reg .b32 imask; .reg .b32 rb;\n"
+                    "mov.b32 i, %0; mov.b32 bm, %1; mov.b32 lpos, %2; mov.b32 lfull, %3; mov.b32 tpos, %4; mov.b32 at1, %5;\n"
+                    "mov.b32 at2, %6; mov.b64 tk, %7; mov.b32 prev, %8; mov.b64 rec, %9; mov.b32 lat, %10; mov.b32 xs, %11;\n"
+                    "mov.b32 epos, %12; mov.b32 efull, %13; mov.b32 e_on, %14; mov.b64 e_key, %15; mov.b32 e_idx, %16; mov.b32 qv, %17;\n"
+                    "mov.b32 tail_a, %18; mov.b32 rw, %19; mov.b32 sa, %20; mov.b32 xin, %21; mov.b32 xin_mask, %22; mov.b32 xin_row, %23;\n"
+                    "mov.b32 tab, %24; mov.b32 kfb, %25; mov.b32 kfm, %26; mov.b32 kb, %27; mov.b32 rm, %28; mov.b32 mbm1, %29;\n"
+                    "mov.b32 tick, %30; mov.b32 qmask, %31; mov.b32 tmask, %32; mov.b32 qb, %33; mov.b32 nqm, %34; mov.b32 xa, %35;\n"
+                    "mov.b32 xam, %36; mov.b32 down, %37; mov.b32 tail_step, %38; mov.b64 out, %39; mov.b32 imask, %40; mov.b32 rb, %41;\n"
+                    ".reg .pred t, taken, open, pop, ov, dp, pz, pf, hand, hd, ho, fin, fetch;\n"
+                    ".reg .u32 at0, sd, rl, rh, kl, kh, fl, fh, word, wa, x, y, lo, hi, a, xs_was, sa_was, ta_was, pos, left, a1, a2, a3, a4;\n"
+                    ".reg .b64 kf, k1, k2, fk, key, td, r, first, v, e1, e2, e3, e4; .reg .b64 o, w;\n"
+                    "and.b32 a, epos, rm; or.b32 a, a, kb; ld.shared.b64 fk, [a];\n"
+                    "and.b32 a, lpos, kfm; or.b32 a, a, kfb; ld.shared.b64 kf, [a];\n"
+                    "ld.shared.b64 k1, [at1]; ld.shared.b64 k2, [at2];\n"
+                    "mov.b64 td, tk; mov.b64 {rl, rh}, rec; mov.u32 xs_was, xs; mov.u32 sa_was, sa;\n"
+                    "setp.ne.u32 t, tpos, efull; selp.b32 rh, rh, -1, t; mov.b64 r, {rl, rh};\n"
+                    "setp.ge.s32 taken, rh, 0; setp.ge.and.u32 t, bm, mbm1, taken; setp.gt.or.f64 open, r, td, t;\n"
+                    "sub.u32 y, i, bm; add.u32 y, y, -1;\n"
+                    "add.u32 wa, i, -1; and.b32 wa, wa, nqm; mad.lo.u32 wa, wa, 128, qb;\n"
+                    "@taken add.u32 i, i, 1; and.b32 xs, i, xin_mask; mad.lo.u32 xs, xs, xin_row, xin; ld.relaxed.cta.shared.b64 rec, [xs];\n"
+                    "setp.lt.s32 hand, rw, 0; setp.ne.and.u32 hand, e_on, 0, hand; setp.ge.and.s32 hd|ho, down, 0, hand; setp.lt.and.s32 fin, qv, 0, hand;\n"
+                    "and.b32 x, qv, 0x7fffffff; mov.b64 {lo, hi}, e_key; and.b32 lo, lo, tmask; or.b32 a, lo, x; mov.b64 v, {a, hi}; mov.u32 ta_was, tail_a;\n"
+                    "@hand add.u32 tail_a, tail_a, tail_step;\n"
+                    "and.b32 sa, tail_a, xam; or.b32 sa, sa, xa; ld.relaxed.cta.shared.u32 rw, [sa+4];\n"
+                    "mad.wide.u32 key, lat, tick, tk; mov.b64 {kl, kh}, key; and.b32 kl, kl, tmask; or.b32 kl, kl, y; mov.b64 key, {kl, kh};\n"
+                    "@taken add.u32 bm, bm, 1; @open mov.u32 bm, 0; mad.lo.u32 a, bm, 4, tab; ld.shared.u32 lat, [a];\n"
+                    "setp.eq.or.u32 fetch, e_on, 0, fin; setp.ne.and.u32 fetch, epos, tpos, fetch; setp.le.and.f64 fetch, fk, td, fetch;\n"
+                    "mov.b64 {fl, fh}, fk;\n"
+                    "@hand add.u32 e_idx, e_idx, 1; @fetch and.b32 e_idx, fl, qmask; and.b32 a, e_idx, nqm; mad.lo.u32 a, a, 128, qb; ld.shared.u32 qv, [a];\n"
+                    "@hd st.relaxed.cta.shared.b64 [sa_was], v;\n"
+                    "and.b32 a, x, imask; mad.wide.u32 o, a, 8, out;\n"
+                    "mov.b64 w, {lo, hi}; shr.u64 w, w, rb; cvt.u64.u32 v, a; or.b64 w, w, v; @ho red.relaxed.gpu.global.max.u64 [o], w;\n"
+                    "@fetch mov.b64 e_key, fk; @fin mov.u32 e_on, 0; @fetch mov.u32 e_on, 1; @fetch add.u32 epos, epos, 256; @fetch add.u32 efull, efull, 256;\n"
+                    "and.b32 at0, tpos, rm; or.b32 at0, at0, kb;\n"
+                    "setp.lt.f64 pf, kf, key; selp.b64 first, kf, key, pf;\n"
+                    "setp.eq.u32 pz, tpos, lfull; setp.lt.and.f64 pz, r, first, pz; selp.b64 first, first, r, pz;\n"
+                    "mov.b64 {fl, fh}, first; or.b32 fl, fl, qmask; mov.b64 first, {fl, fh}; selp.b64 tk, first, tk, open;\n"
+                    "setp.lt.and.f64 ov, key, k1, open; selp.u32 sd, at1, at0, ov;\n"
+                    "@open st.shared.b64 [sd], key; @ov st.shared.b64 [at0], k1;\n"
+                    "setp.lt.and.f64 dp, key, k2, ov; mov.u32 pos, tpos; mov.u32 left, lpos;\n"
+                    "setp.eq.and.u32 pop, tpos, lfull, open;\n"
+                    "mov.u32 word, prev; @open or.b32 word, word, 0x80000000; @taken st.shared.u32 [wa], word;\n"
+                    "@taken st.relaxed.cta.shared.u32 [xs_was+4], -1;\n"
+                    "@open add.u32 tpos, tpos, 256; @open mov.u32 at2, at1; @open mov.u32 at1, at0;\n"
+                    "@pop add.u32 lpos, lpos, 256; @pop add.u32 lfull, lfull, 256;\n"
+                    "@taken and.b32 prev, rl, qmask;\n"
+                    "@!dp bra PLACED;\n"
+                    "mov.u32 sd, left; sub.u32 pos, pos, 256;\n"
+                    "DEEPER:\n"
+                    "sub.u32 left, pos, sd;\n"
+                    "and.b32 at0, pos, rm; or.b32 at0, at0, kb; sub.u32 a1, pos, 256; and.b32 a1, a1, rm; or.b32 a1, a1, kb;\n"
+                    "sub.u32 a2, pos, 512; and.b32 a2, a2, rm; or.b32 a2, a2, kb; sub.u32 a3, pos, 768; and.b32 a3, a3, rm; or.b32 a3, a3, kb;\n"
+                    "sub.u32 a4, pos, 1024; and.b32 a4, a4, rm; or.b32 a4, a4, kb;\n"
+                    "ld.shared.b64 e1, [a1]; ld.shared.b64 e2, [a2]; ld.shared.b64 e3, [a3]; ld.shared.b64 e4, [a4];\n"
+                    "setp.gt.u32 t, left, 0; setp.lt.and.f64 t, key, e1, t; setp.gt.and.u32 ov, left, 256, t; setp.lt.and.f64 ov, key, e2, ov;\n"
+                    "setp.gt.and.u32 pz, left, 512, ov; setp.lt.and.f64 pz, key, e3, pz; setp.gt.and.u32 pf, left, 768, pz; setp.lt.and.f64 pf, key, e4, pf;\n"
+                    "@t st.shared.b64 [at0], e1; @ov st.shared.b64 [a1], e2; @pz st.shared.b64 [a2], e3; @pf st.shared.b64 [a3], e4;\n"
+                    "@t mov.u32 at0, a1; @ov mov.u32 at0, a2; @pz mov.u32 at0, a3; @pf mov.u32 at0, a4; st.shared.b64 [at0], key;\n"
+                    "sub.u32 pos, pos, 1024; @pf bra DEEPER;\n"
+                    "PLACED:\n"
+                    "mov.b32 %0, i; mov.b32 %1, bm; mov.b32 %2, lpos; mov.b32 %3, lfull; mov.b32 %4, tpos; mov.b32 %5, at1;\n"
+                    "mov.b32 %6, at2; mov.b64 %7, tk; mov.b32 %8, prev; mov.b64 %9, rec; mov.b32 %10, lat; mov.b32 %11, xs;\n"
+                    "mov.b32 %12, epos; mov.b32 %13, efull; mov.b32 %14, e_on; mov.b64 %15, e_key; mov.b32 %16, e_idx; mov.b32 %17, qv;\n"
+                    "mov.b32 %18, tail_a; mov.b32 %19, rw; mov.b32 %20, sa;\n"
+                    "}"
+                    : "+r"(i), "+r"(bm), "+r"(lpos), "+r"(lfull), "+r"(tpos), "+r"(at1), "+r"(at2), "+l"(tk), "+r"(prev), "+l"(rec), "+r"(lat), "+r"(xs), "+r"(epos), "+r"(efull), "+r"(e_on), "+l"(e_key), "+r"(e_idx), "+r"(qv), "+r"(tail_a), "+r"(rw), "+r"(sa)
+                    : "r"(xin), "r"(xin_mask), "r"(xin_row), "r"(tab), "r"(kfb), "r"(kfm), "r"(kb), "r"(rm), "r"(mbm1), "r"(tick), "r"(qmask), "r"(~qmask), "r"(qb), "r"(nq - 1u), "r"(xa), "r"(xam), "r"(down), "r"(tail_step), "l"(out_c), "r"(imask), "r"(rb)
+                    : "memory");
+            } else if constexpr (OUT == kOutLeaf) {
+                asm volatile(
+                    "{\n"
+                    ".reg .b32 i; .reg .b32 bm; .reg .b32 lpos; .reg .b32 lfull; .reg .b32 tpos; .reg .b32 at1; .reg .b32 at2;\n"
+                    ".reg .b64 tk; .reg .b32 prev; .reg .b64 rec; .reg .b32 lat; .reg .b32 xs; .reg .b32 epos; .reg .b32 efull;\n"
+                    ".reg .b32 e_on; .reg .b64 e_key; .reg .b32 e_idx; .reg .b32 qv; .reg .b32 tail_a; .reg .b32 rw; .reg .b32 sa;\n"
+                    ".reg .b32 xin; .reg .b32 xin_mask; .reg .b32 xin_row; .reg .b32 tab; .reg .b32 kfb; .reg .b32 kfm; .reg .b32 kb;\n"
+                    ".reg .b32 rm; .reg .b32 mbm1; .reg .b32 tick; .reg .b32 qmask; .reg .b32 tmask; .reg .b32 qb; .reg .b32 nqm;\n"
+                    ".reg .b32 xa; .reg .b32 xam; .reg .b32 down; .reg .b32 tail_step; .reg .b64 out; .reg .b32 imask; .reg .b32 rb;\n"
+                    "mov.b32 i, %0; mov.b32 bm, %1; mov.b32 lpos, %2; mov.b32 lfull, %3; mov.b32 tpos, %4; mov.b32 at1, %5;\n"
+                    "mov.b32 at2, %6; mov.b64 tk, %7; mov.b32 prev, %8; mov.b64 rec, %9; mov.b32 lat, %10; mov.b32 xs, %11;\n"
+                    "mov.b32 epos, %12; mov.b32 efull, %13; mov.b32 e_on, %14; mov.b64 e_key, %15; mov.b32 e_idx, %16; mov.b32 qv, %17;\n"
+                    "mov.b32 tail_a, %18; mov.b32 rw, %19; mov.b32 sa, %20; mov.b32 xin, %21; mov.b32 xin_mask, %22; mov.b32 xin_row, %23;\n"
+                    "mov.b32 tab, %24; mov.b32 kfb, %25; mov.b32 kfm, %26; mov.b32 kb, %27; mov.b32 rm, %28; mov.b32 mbm1, %29;\n"
+                    "mov.b32 tick, %30; mov.b32 qmask, %31; mov.b32 tmask, %32; mov.b32 qb, %33; mov.b32 nqm, %34; mov.b32 xa, %35;\n"
+                    "mov.b32 xam, %36; mov.b32 down, %37; mov.b32 tail_step, %38; mov.b64 out, %39; mov.b32 imask, %40; mov.b32 rb, %41;\n"
+                    ".reg .pred t, taken, open, pop, ov, dp, pz, pf, hand, hd, ho, fin, fetch;\n"
+                    ".reg .u32 at0, sd, rl, rh, kl, kh, fl, fh, word, wa, x, y, lo, hi, a, xs_was, sa_was, ta_was, pos, left, a1, a2, a3, a4;\n"
+                    ".reg .b64 kf, k1, k2, fk, key, td, r, first, v, e1, e2, e3, e4; .reg .b64 o, w;\n"
+                    "and.b32 a, epos, rm; or.b32 a, a, kb; ld.shared.b64 fk, [a];\n"
+                    "and.b32 a, lpos, kfm; or.b32 a, a, kfb; ld.shared.b64 kf, [a];\n"
+                    "ld.shared.b64 k1, [at1]; ld.shared.b64 k2, [at2];\n"
+                    "mov.b64 td, tk; mov.b64 {rl, rh}, rec; mov.u32 xs_was, xs; mov.u32 sa_was, sa;\n"
+                    "setp.ne.u32 t, tpos, efull; selp.b32 rh, rh, -1, t; mov.b64 r, {rl, rh};\n"
+                    "setp.ge.s32 taken, rh, 0; setp.ge.and.u32 t, bm, mbm1, taken; setp.gt.or.f64 open, r, td, t;\n"
+                    "sub.u32 y, i, bm; add.u32 y, y, -1;\n"
+                    "add.u32 wa, i, -1; and.b32 wa, wa, nqm; mad.lo.u32 wa, wa, 128, qb;\n"
+                    "@taken add.u32 i, i, 1; and.b32 xs, i, xin_mask; mad.lo.u32 xs, xs, xin_row, xin; ld.relaxed.cta.shared.b64 rec, [xs];\n"
+                    "setp.lt.s32 hand, rw, 0; setp.ne.and.u32 hand, e_on, 0, hand; setp.ge.and.s32 hd|ho, down, 0, hand; setp.lt.and.s32 fin, qv, 0, hand;\n"
+                    "and.b32 x, qv, 0x7fffffff; mov.b64 {lo, hi}, e_key; and.b32 lo, lo, tmask; or.b32 a, lo, x; mov.b64 v, {a, hi}; mov.u32 ta_was, tail_a;\n"
+                    "@hand add.u32 tail_a, tail_a, tail_step;\n"
+                    "and.b32 sa, tail_a, xam; or.b32 sa, sa, xa; ld.relaxed.cta.shared.u32 rw, [sa+4];\n"
+                    "mad.wide.u32 key, lat, tick, tk; mov.b64 {kl, kh}, key; and.b32 kl, kl, tmask; or.b32 kl, kl, y; mov.b64 key, {kl, kh};\n"
+                    "@taken add.u32 bm, bm, 1; @open mov.u32 bm, 0; mad.lo.u32 a, bm, 4, tab; ld.shared.u32 lat, [a];\n"
+                    "setp.eq.or.u32 fetch, e_on, 0, fin; setp.ne.and.u32 fetch, epos, tpos, fetch; setp.le.and.f64 fetch, fk, td, fetch;\n"
+                    "mov.b64 {fl, fh}, fk;\n"
+                    "@hand add.u32 e_idx, e_idx, 1; @fetch and.b32 e_idx, fl, qmask; and.b32 a, e_idx, nqm; mad.lo.u32 a, a, 128, qb; ld.shared.u32 qv, [a];\n"
+                    "@hd st.relaxed.cta.shared.b64 [sa_was], v;\n"
+                    "mad.wide.u32 o, ta_was, 1, out;\n"
+                    "and.b32 a, x, imask; mov.b64 w, {lo, hi}; shr.u64 w, w, rb; cvt.u64.u32 v, a; or.b64 w, w, v; @ho st.global.b64 [o], w;\n"
+                    "@fetch mov.b64 e_key, fk; @fin mov.u32 e_on, 0; @fetch mov.u32 e_on, 1; @fetch add.u32 epos, epos, 256; @fetch add.u32 efull, efull, 256;\n"
+                    "and.b32 at0, tpos, rm; or.b32 at0, at0, kb;\n"
+                    "setp.lt.f64 pf, kf, key; selp.b64 first, kf, key, pf;\n"
+                    "setp.eq.u32 pz, tpos, lfull; setp.lt.and.f64 pz, r, first, pz; selp.b64 first, first, r, pz;\n"
+                    "mov.b64 {fl, fh}, first; or.b32 fl, fl, qmask; mov.b64 first, {fl, fh}; selp.b64 tk, first, tk, open;\n"
+                    "setp.lt.and.f64 ov, key, k1, open; selp.u32 sd, at1, at0, ov;\n"
+                    "@open st.shared.b64 [sd], key; @ov st.shared.b64 [at0], k1;\n"
+                    "setp.lt.and.f64 dp, key, k2, ov; mov.u32 pos, tpos; mov.u32 left, lpos;\n"
+                    "setp.eq.and.u32 pop, tpos, lfull, open;\n"
+                    "mov.u32 word, prev; @open or.b32 word, word, 0x80000000; @taken st.shared.u32 [wa], word;\n"
+                    "@taken st.relaxed.cta.shared.u32 [xs_was+4], -1;\n"
+                    "@open add.u32 tpos, tpos, 256; @open mov.u32 at2, at1; @open mov.u32 at1, at0;\n"
+                    "@pop add.u32 lpos, lpos, 256; @pop add.u32 lfull, lfull, 256;\n"
+                    "@taken and.b32 prev, rl, qmask;\n"
+                    "@!dp bra PLACED;\n"
+                    "mov.u32 sd, left; sub.u32 pos, pos, 256;\n"
+                    "DEEPER:\n"
+                    "sub.u32 left, pos, sd;\n"
+                    "and.b32 at0, pos, rm; or.b32 at0, at0, kb; sub.u32 a1, pos, 256; and.b32 a1, a1, rm; or.b32 a1, a1, kb;\n"
+                    "sub.u32 a2, pos, 512; and.b32 a2, a2, rm; or.b32 a2, a2, kb; sub.u32 a3, pos, 768; and.b32 a3, a3, rm; or.b32 a3, a3, kb;\n"
+                    "sub.u32 a4, pos, 1024; and.b32 a4, a4, rm; or.b32 a4, a4, kb;\n"
+                    "ld.shared.b64 e1, [a1]; ld.shared.b64 e2, [a2]; ld.shared.b64 e3, [a3]; ld.shared.b64 e4, [a4];\n"
+                    "setp.gt.u32 t, left, 0; setp.lt.and.f64 t, key, e1, t; setp.gt.and.u32 ov, left, 256, t; setp.lt.and.f64 ov, key, e2, ov;\n"
+                    "setp.gt.and.u32 pz, left, 512, ov; setp.lt.and.f64 pz, key, e3, pz; setp.gt.and.u32 pf, left, 768, pz; setp.lt.and.f64 pf, key, e4, pf;\n"
+                    "@t st.shared.b64 [at0], e1; @ov st.shared.b64 [a1], e2; @pz st.shared.b64 [a2], e3; @pf st.shared.b64 [a3], e4;\n"
+                    "@t mov.u32 at0, a1; @ov mov.u32 at0, a2; @pz mov.u32 at0, a3; @pf mov.u32 at0, a4; st.shared.b64 [at0], key;\n"
+                    "sub.u32 pos, pos, 1024; @pf bra DEEPER;\n"
+                    "PLACED:\n"
+                    "mov.b32 %0, i; mov.b32 %1, bm; mov.b32 %2, lpos; mov.b32 %3, lfull; mov.b32 %4, tpos; mov.b32 %5, at1;\n"
+                    "mov.b32 %6, at2; mov.b64 %7, tk; mov.b32 %8, prev; mov.b64 %9, rec; mov.b32 %10, lat; mov.b32 %11, xs;\n"
+                    "mov.b32 %12, epos; mov.b32 %13, efull; mov.b32 %14, e_on; mov.b64 %15, e_key; mov.b32 %16, e_idx; mov.b32 %17, qv;\n"
+                    "mov.b32 %18, tail_a; mov.b32 %19, rw; mov.b32 %20, sa;\n"
+                    "}"
+                    : "+r"(i), "+r"(bm), "+r"(lpos), "+r"(lfull), "+r"(tpos), "+r"(at1), "+r"(at2), "+l"(tk), "+r"(prev), "+l"(rec), "+r"(lat), "+r"(xs), "+r"(epos), "+r"(efull), "+r"(e_on), "+l"(e_key), "+r"(e_idx), "+r"(qv), "+r"(tail_a), "+r"(rw), "+r"(sa)
+                    : "r"(xin), "r"(xin_mask), "r"(xin_row), "r"(tab), "r"(kfb), "r"(kfm), "r"(kb), "r"(rm), "r"(mbm1), "r"(tick), "r"(qmask), "r"(~qmask), "r"(qb), "r"(nq - 1u), "r"(xa), "r"(xam), "r"(down), "r"(tail_step), "l"(out), "r"(imask), "r"(rb)
+                    : "memory");
+            } else if constexpr (OUT == kOutTwo && FORK) {
+                asm volatile(
+                    "{\n"
+                    ".reg .b32 i; .reg .b32 bm; .reg .b32 lpos; .reg .b32 lfull; .reg .b32 tpos; .reg .b32 at1; .reg .b32 at2;\n"
+                    ".reg .b64 tk; .reg .b32 prev; .reg .b64 rec; .reg .b32 lat; .reg .b32 xs; .reg .b32 epos; .reg .b32 efull;\n"
+                    ".reg .b32 e_on; .reg .b64 e_key; .reg .b32 e_idx; .reg .b32 qv; .reg .b32 tail_a; .reg .b32 rw; .reg .b32 sa;\n"
+                    ".reg .b32 tail_b; .reg .b32 xin; .reg .b32 xin_mask; .reg .b32 xin_row; .reg .b32 tab; .reg .b32 kfb; .reg .b32 kfm;\n"
+                    ".reg .b32 kb; .reg .b32 rm; .reg .b32 mbm1; .reg .b32 tick; .reg .b32 qmask; .reg .b32 tmask; .reg .b32 qb;\n"
+                    ".reg .b32 nqm; .reg .b32 xa; .reg .b32 xam; .reg .b32 down; .reg .b32 mask_a; .reg .b32 mask_b; .reg .b32 want_a;\n"
+                    ".reg .b32 want_b; .reg .b64 out; .reg .b64 out_b;\n"
+                    "mov.b32 i, %0; mov.b32 bm, %1; mov.b32 lpos, %2; mov.b32 lfull, %3; mov.b32 tpos, %4; mov.b32 at1, %5;\n"
+                    "mov.b32 at2, %6; mov.b64 tk, %7; mov.b32 prev, %8; mov.b64 rec, %9; mov.b32 lat, %10; mov.b32 xs, %11;\n"
+                    "mov.b32 epos, %12; mov.b32 efull, %13; mov.b32 e_on, %14; mov.b64 e_key, %15; mov.b32 e_idx, %16; mov.b32 qv, %17;\n"
+                    "mov.b32 tail_a, %18; mov.b32 rw, %19; mov.b32 sa, %20; mov.b32 tail_b, %21; mov.b32 xin, %22; mov.b32 xin_mask, %23;\n"
+                    "mov.b32 xin_row, %24; mov.b32 tab, %25; mov.b32 kfb, %26; mov.b32 kfm, %27; mov.b32 kb, %28; mov.b32 rm, %29;\n"
+                    "mov.b32 mbm1, %30; mov.b32 tick, %31; mov.b32 qmask, %32; mov.b32 tmask, %33; mov.b32 qb, %34; mov.b32 nqm, %35;\n"
+                    "mov.b32 xa, %36; mov.b32 xam, %37; mov.b32 down, %38; mov.b32 mask_a, %39; mov.b32 mask_b, %40; mov.b32 want_a, %41;\n"
+                    "mov.b32 want_b, %42; mov.b64 out, %43; mov.b64 out_b, %44;\n"
+                    ".reg .pred t, taken, open, pop, ov, dp, pz, pf, hand, hd, ho, fin, fetch;\n"
+                    ".reg .u32 at0, sd, rl, rh, kl, kh, fl, fh, word, wa, x, y, lo, hi, a, xs_was, sa_was, ta_was, pos, left, a1, a2, a3, a4;\n"
+                    ".reg .b64 kf, k1, k2, fk, key, td, r, first, v, e1, e2, e3, e4; .reg .pred ga, gb; .reg .b64 o; .reg .u32 ma, mb;\n"
+                    "and.b32 a, epos, rm; or.b32 a, a, kb; ld.shared.b64 fk, [a];\n"
+                    "and.b32 a, lpos, kfm; or.b32 a, a, kfb; ld.shared.b64 kf, [a];\n"
+                    "ld.shared.b64 k1, [at1]; ld.shared.b64 k2, [at2];\n"
+                    "mov.b64 td, tk; mov.b64 {rl, rh}, rec; mov.u32 xs_was, xs; mov.u32 sa_was, sa;\n"
+                    "setp.ne.u32 t, tpos, efull; selp.b32 rh, rh, -1, t; mov.b64 r, {rl, rh};\n"
+                    "setp.ge.s32 taken, rh, 0; setp.ge.and.u32 t, bm, mbm1, taken; setp.gt.or.f64 open, r, td, t;\n"
+                    "sub.u32 y, i, bm; add.u32 y, y, -1;\n"
+                    "add.u32 wa, i, -1; and.b32 wa, wa, nqm; mad.lo.u32 wa, wa, 128, qb;\n"
+                    "@taken add.u32 i, i, 1; and.b32 xs, i, xin_mask; mad.lo.u32 xs, xs, xin_row, xin; ld.relaxed.cta.shared.b64 rec, [xs];\n"
+                    "setp.lt.s32 hand, rw, 0; setp.ne.and.u32 hand, e_on, 0, hand; setp.ge.and.s32 hd|ho, down, 0, hand; setp.lt.and.s32 fin, qv, 0, hand;\n"
+                    "and.b32 x, qv, 0x7fffffff; mov.b64 {lo, hi}, e_key; and.b32 lo, lo, tmask; or.b32 a, lo, x; mov.b64 v, {a, hi}; mov.u32 ta_was, tail_a;\n"
+                    "and.b32 ma, qv, mask_a; and.b32 mb, qv, mask_b;\n"
+                    "setp.eq.and.u32 ga, ma, want_a, ho; setp.eq.and.u32 gb, mb, want_b, ho;\n"
+                    "@hd add.u32 tail_a, tail_a, 256; @ga add.u32 tail_a, tail_a, 8;\n"
+                    "and.b32 sa, tail_a, xam; or.b32 sa, sa, xa; ld.relaxed.cta.shared.u32 rw, [sa+4];\n"
+                    "mad.wide.u32 key, lat, tick, tk; mov.b64 {kl, kh}, key; and.b32 kl, kl, tmask; or.b32 kl, kl, y; mov.b64 key, {kl, kh};\n"
+                    "@taken add.u32 bm, bm, 1; @open mov.u32 bm, 0; mad.lo.u32 a, bm, 4, tab; ld.shared.u32 lat, [a];\n"
+                    "setp.eq.or.u32 fetch, e_on, 0, fin; setp.ne.and.u32 fetch, epos, tpos, fetch; setp.le.and.f64 fetch, fk, td, fetch;\n"
+                    "mov.b64 {fl, fh}, fk;\n"
+                    "@hand add.u32 e_idx, e_idx, 1; @fetch and.b32 e_idx, fl, qmask; and.b32 a, e_idx, nqm; mad.lo.u32 a, a, 128, qb; ld.shared.u32 qv, [a];\n"
+                    "@hd st.relaxed.cta.shared.b64 [sa_was], v;\n"
+                    "mad.wide.u32 o, ta_was, 1, out; @ga st.global.b64 [o], v; mad.wide.u32 o, tail_b, 1, out_b; @gb st.global.b64 [o], v; @gb add.u32 tail_b, tail_b, 8;\n"
+                    "@fetch mov.b64 e_key, fk; @fin mov.u32 e_on, 0; @fetch mov.u32 e_on, 1; @fetch add.u32 epos, epos, 256; @fetch add.u32 efull, efull, 256;\n"
+                    "and.b32 at0, tpos, rm; or.b32 at0, at0, kb;\n"
+                    "setp.lt.f64 pf, kf, key; selp.b64 first, kf, key, pf;\n"
+                    "setp.eq.u32 pz, tpos, lfull; setp.lt.and.f64 pz, r, first, pz; selp.b64 first, first, r, pz;\n"
+                    "mov.b64 {fl, fh}, first; or.b32 fl, fl, qmask; mov.b64 first, {fl, fh}; selp.b64 tk, first, tk, open;\n"
+                    "setp.lt.and.f64 ov, key, k1, open; selp.u32 sd, at1, at0, ov;\n"
+                    "@open st.shared.b64 [sd], key; @ov st.shared.b64 [at0], k1;\n"
+                    "setp.lt.and.f64 dp, key, k2, ov; mov.u32 pos, tpos; mov.u32 left, lpos;\n"
+                    "setp.eq.and.u32 pop, tpos, lfull, open;\n"
+                    "mov.u32 word, prev; @open or.b32 word, word, 0x80000000; @taken st.shared.u32 [wa], word;\n"
+                    "@taken st.relaxed.cta.shared.u32 [xs_was+4], -1;\n"
+                    "@open add.u32 tpos, tpos, 256; @open mov.u32 at2, at1; @open mov.u32 at1, at0;\n"
+                    "@pop add.u32 lpos, lpos, 256; @pop add.u32 lfull, lfull, 256;\n"
+                    "@taken and.b32 prev, rl, qmask;\n"
+                    "@!dp bra PLACED;\n"
+                    "mov.u32 sd, left; sub.u32 pos, pos, 256;\n"
+                    "DEEPER:\n"
+                    "sub.u32 left, pos, sd;\n"
+                    "and.b32 at0, pos, rm; or.b32 at0, at0, kb; sub.u32 a1, pos, 256; and.b32 a1, a1, rm; or.b32 a1, a1, kb;\n"
+                    "sub.u32 a2, pos, 512; and.b32 a2, a2, rm; or.b32 a2, a2, kb; sub.u32 a3, pos, 768; and.b32 a3, a3, rm; or.b32 a3, a3, kb;\n"
+                    "sub.u32 a4, pos, 1024; and.b32 a4, a4, rm; or.b32 a4, a4, kb;\n"
+                    "ld.shared.b64 e1, [a1]; ld.shared.b64 e2, [a2]; ld.shared.b64 e3, [a3]; ld.shared.b64 e4, [a4];\n"
+                    "setp.gt.u32 t, left, 0; setp.lt.and.f64 t, key, e1, t; setp.gt.and.u32 ov, left, 256, t; setp.lt.and.f64 ov, key, e2, ov;\n"
+                    "setp.gt.and.u32 pz, left, 512, ov; setp.lt.and.f64 pz, key, e3, pz; setp.gt.and.u32 pf, left, 768, pz; setp.lt.and.f64 pf, key, e4, pf;\n"
+                    "@t st.shared.b64 [at0], e1; @ov st.shared.b64 [a1], e2; @pz st.shared.b64 [a2], e3; @pf st.shared.b64 [a3], e4;\n"
+                    "@t mov.u32 at0, a1; @ov mov.u32 at0, a2; @pz mov.u32 at0, a3; @pf mov.u32 at0, a4; st.shared.b64 [at0], key;\n"
+                    "sub.u32 pos, pos, 1024; @pf bra DEEPER;\n"
+                    "PLACED:\n"
+                    "mov.b32 %0, i; mov.b32 %1, bm; mov.b32 %2, lpos; mov.b32 %3, lfull; mov.b32 %4, tpos; mov.b32 %5, at1;\n"
+                    "mov.b32 %6, at2; mov.b64 %7, tk; mov.b32 %8, prev; mov.b64 %9, rec; mov.b32 %10, lat; mov.b32 %11, xs;\n"
+                    "mov.b32 %12, epos; mov.b32 %13, efull; mov.b32 %14, e_on; mov.b64 %15, e_key; mov.b32 %16, e_idx; mov.b32 %17, qv;\n"
+                    "mov.b32 %18, tail_a; mov.b32 %19, rw; mov.b32 %20, sa; mov.b32 %21, tail_b;\n"
+                    "}"
+                    : "+r"(i), "+r"(bm), "+r"(lpos), "+r"(lfull), "+r"(tpos), "+r"(at1), "+r"(at2), "+l"(tk), "+r"(prev), "+l"(rec), "+r"(lat), "+r"(xs), "+r"(epos), "+r"(efull), "+r"(e_on), "+l"(e_key), "+r"(e_idx), "+r"(qv), "+r"(tail_a), "+r"(rw), "+r"(sa), "+r"(tail_b)
+                    : "r"(xin), "r"(xin_mask), "r"(xin_row), "r"(tab), "r"(kfb), "r"(kfm), "r"(kb), "r"(rm), "r"(mbm1), "r"(tick), "r"(qmask), "r"(~qmask), "r"(qb), "r"(nq - 1u), "r"(xa), "r"(xam), "r"(down), "r"(mask_a), "r"(mask_b), "r"(want_a), "r"(want_b), "l"(out), "l"(out_b)
+                    : "memory");
+            } else if constexpr (OUT == kOutTwo) {
+                asm volatile(
+                    "{\n"
+                    ".reg .b32 i; .reg .b32 bm; .reg .b32 lpos; .reg .b32 lfull; .reg .b32 tpos; .reg .b32 at1; .reg .b32 at2;\n"
+                    ".reg .b64 tk; .reg .b32 prev; .reg .b64 rec; .reg .b32 lat; .reg .b32 xs; .reg .b32 epos; .reg .b32 efull;\n"
+                    ".reg .b32 e_on; .reg .b64 e_key; .reg .b32 e_idx; .reg .b32 qv; .reg .b32 tail_a; .reg .b32 rw; .reg .b32 sa;\n"
+                    ".reg .b32 tail_b; .reg .b32 xin; .reg .b32 xin_mask; .reg .b32 xin_row; .reg .b32 tab; .reg .b32 kfb; .reg .b32 kfm;\n"
+                    ".reg .b32 kb; .reg .b32 rm; .reg .b32 mbm1; .reg .b32 tick; .reg .b32 qmask; .reg .b32 tmask; .reg .b32 qb;\n"
+                    ".reg .b32 nqm; .reg .b32 xa; .reg .b32 xam; .reg .b32 down; .reg .b32 mask_a; .reg .b32 want_a; .reg .b64 out;\n"
+                    "mov.b32 i, %0; mov.b32 bm, %1; mov.b32 lpos, %2; mov.b32 lfull, %3; mov.b32 tpos, %4; mov.b32 at1, %5;\n"
+                    "mov.b32 at2, %6; mov.b64 tk, %7; mov.b32 prev, %8; mov.b64 rec, %9; mov.b32 lat, %10; mov.b32 xs, %11;\n"
+                    "mov.b32 epos, %12; mov.b32 efull, %13; mov.b32 e_on, %14; mov.b64 e_key, %15; mov.b32 e_idx, %16; mov.b32 qv, %17;\n"
+                    "mov.b32 tail_a, %18; mov.b32 rw, %19; mov.b32 sa, %20; mov.b32 tail_b, %21; mov.b32 xin, %22; mov.b32 xin_mask, %23;\n"
+                    "mov.b32 xin_row, %24; mov.b32 tab, %25; mov.b32 kfb, %26; mov.b32 kfm, %27; mov.b32 kb, %28; mov.b32 rm, %29;\n"
+                    "mov.b32 mbm1, %30; mov.b32 tick, %31; mov.b32 qmask, %32; mov.b32 tmask, %33; mov.b32 qb, %34; mov.b32 nqm, %35;\n"
+                    "mov.b32 xa, %36; mov.b32 xam, %37; mov.b32 down, %38; mov.b32 mask_a, %39; mov.b32 want_a, %40; mov.b64 out, %41;\n"
+                    ".reg .pred t, taken, open, pop, ov, dp, pz, pf, hand, hd, ho, fin, fetch;\n"
+                    ".reg .u32 at0, sd, rl, rh, kl, kh, fl, fh, word, wa, x, y, lo, hi, a, xs_was, sa_was, ta_was, pos, left, a1, a2, a3, a4;\n"
+                    ".reg .b64 kf, k1, k2, fk, key, td, r, first, v, e1, e2, e3, e4; .reg .pred ga, gb; .reg .b64 o; .reg .u32 ma, tt;\n"
+                    "and.b32 a, epos, rm; or.b32 a, a, kb; ld.shared.b64 fk, [a];\n"
+                    "and.b32 a, lpos, kfm; or.b32 a, a, kfb; ld.shared.b64 kf, [a];\n"
+                    "ld.shared.b64 k1, [at1]; ld.shared.b64 k2, [at2];\n"
+                    "mov.b64 td, tk; mov.b64 {rl, rh}, rec; mov.u32 xs_was, xs; mov.u32 sa_was, sa;\n"
+                    "setp.ne.u32 t, tpos, efull; selp.b32 rh, rh, -1, t; mov.b64 r, {rl, rh};\n"
+                    "setp.ge.s32 taken, rh, 0; setp.ge.and.u32 t, bm, mbm1, taken; setp.gt.or.f64 open, r, td, t;\n"
+                    "sub.u32 y, i, bm; add.u32 y, y, -1;\n"
+                    "add.u32 wa, i, -1; and.b32 wa, wa, nqm; mad.lo.u32 wa, wa, 128, qb;\n"
+                    "@taken add.u32 i, i, 1; and.b32 xs, i, xin_mask; mad.lo.u32 xs, xs, xin_row, xin; ld.relaxed.cta.shared.b64 rec, [xs];\n"
+                    "setp.lt.s32 hand, rw, 0; setp.ne.and.u32 hand, e_on, 0, hand; setp.ge.and.s32 hd|ho, down, 0, hand; setp.lt.and.s32 fin, qv, 0, hand;\n"
+                    "and.b32 x, qv, 0x7fffffff; mov.b64 {lo, hi}, e_key; and.b32 lo, lo, tmask; or.b32 a, lo, x; mov.b64 v, {a, hi}; mov.u32 ta_was, tail_a;\n"
+                    "and.b32 ma, qv, mask_a; setp.eq.and.u32 ga|gb, ma, want_a, ho; selp.b32 tt, tail_a, tail_b, ga;\n"
+                    "@hd add.u32 tail_a, tail_a, 256; @ga add.u32 tail_a, tail_a, 8; @gb add.u32 tail_b, tail_b, 8;\n"
+                    "and.b32 sa, tail_a, xam; or.b32 sa, sa, xa; ld.relaxed.cta.shared.u32 rw, [sa+4];\n"
+                    "mad.wide.u32 key, lat, tick, tk; mov.b64 {kl, kh}, key; and.b32 kl, kl, tmask; or.b32 kl, kl, y; mov.b64 key, {kl, kh};\n"
+                    "@taken add.u32 bm, bm, 1; @open mov.u32 bm, 0; mad.lo.u32 a, bm, 4, tab; ld.shared.u32 lat, [a];\n"
+                    "setp.eq.or.u32 fetch, e_on, 0, fin; setp.ne.and.u32 fetch, epos, tpos, fetch; setp.le.and.f64 fetch, fk, td, fetch;\n"
+                    "mov.b64 {fl, fh}, fk;\n"
+                    "@hand add.u32 e_idx, e_idx, 1; @fetch and.b32 e_idx, fl, qmask; and.b32 a, e_idx, nqm; mad.lo.u32 a, a, 128, qb; ld.shared.u32 qv, [a];\n"
+                    "@hd st.relaxed.cta.shared.b64 [sa_was], v;\n"
+                    "mad.wide.u32 o, tt, 1, out; @ho st.global.b64 [o], v;\n"
+                    "@fetch mov.b64 e_key, fk; @fin mov.u32 e_on, 0; @fetch mov.u32 e_on, 1; @fetch add.u32 epos, epos, 256; @fetch add.u32 efull, efull, 256;\n"
+                    "and.b32 at0, tpos, rm; or.b32 at0, at0, kb;\n"
+                    "setp.lt.f64 pf, kf, key; selp.b64 first, kf, key, pf;\n"
+                    "setp.eq.u32 pz, tpos, lfull; setp.lt.and.f64 pz, r, first, pz; selp.b64 first, first, r, pz;\n"
+                    "mov.b64 {fl, fh}, first; or.b32 fl, fl, qmask; mov.b64 first, {fl, fh}; selp.b64 tk, first, tk, open;\n"
+                    "setp.lt.and.f64 ov, key, k1, open; selp.u32 sd, at1, at0, ov;\n"
+                    "@open st.shared.b64 [sd], key; @ov st.shared.b64 [at0], k1;\n"
+                    "setp.lt.and.f64 dp, key, k2, ov; mov.u32 pos, tpos; mov.u32 left, lpos;\n"
+                    "setp.eq.and.u32 pop, tpos, lfull, open;\n"
+                    "mov.u32 word, prev; @open or.b32 word, word, 0x80000000; @taken st.shared.u32 [wa], word;\n"
+                    "@taken st.relaxed.cta.shared.u32 [xs_was+4], -1;\n"
+                    "@open add.u32 tpos, tpos, 256; @open mov.u32 at2, at1; @open mov.u32 at1, at0;\n"
+                    "@pop add.u32 lpos, lpos, 256; @pop add.u32 lfull, lfull, 256;\n"
+                    "@taken and.b32 prev, rl, qmask;\n"
+                    "@!dp bra PLACED;\n"
+                    "mov.u32 sd, left; sub.u32 pos, pos, 256;\n"
+                    "DEEPER:\n"
+                    "sub.u32 left, pos, sd;\n"
+                    "and.b32 at0, pos, rm; or.b32 at0, at0, kb; sub.u32 a1, pos, 256; and.b32 a1, a1, rm; or.b32 a1, a1, kb;\n"
+                    "sub.u32 a2, pos, 512; and.b32 a2, a2, rm; or.b32 a2, a2, kb; sub.u32 a3, pos, 768; and.b32 a3, a3, rm; or.b32 a3, a3, kb;\n"
+                    "sub.u32 a4, pos, 1024; and.b32 a4, a4, rm; or.b32 a4, a4, kb;\n"
+                    "ld.shared.b64 e1, [a1]; ld.shared.b64 e2, [a2]; ld.shared.b64 e3, [a3]; ld.shared.b64 e4, [a4];\n"
+                    "setp.gt.u32 t, left, 0; setp.lt.and.f64 t, key, e1, t; setp.gt.and.u32 ov, left, 256, t; setp.lt.and.f64 ov, key, e2, ov;\n"
+                    "setp.gt.and.u32 pz, left, 512, ov; setp.lt.and.f64 pz, key, e3, pz; setp.gt.and.u32 pf, left, 768, pz; setp.lt.and.f64 pf, key, e4, pf;\n"
+                    "@t st.shared.b64 [at0], e1; @ov st.shared.b64 [a1], e2; @pz st.shared.b64 [a2], e3; @pf st.shared.b64 [a3], e4;\n"
+                    "@t mov.u32 at0, a1; @ov mov.u32 at0, a2; @pz mov.u32 at0, a3; @pf mov.u32 at0, a4; st.shared.b64 [at0], key;\n"
+                    "sub.u32 pos, pos, 1024; @pf bra DEEPER;\n"
+                    "PLACED:\n"
+                    "mov.b32 %0, i; mov.b32 %1, bm; mov.b32 %2, lpos; mov.b32 %3, lfull; mov.b32 %4, tpos; mov.b32 %5, at1;\n"
+                    "mov.b32 %6, at2; mov.b64 %7, tk; mov.b32 %8, prev; mov.b64 %9, rec; mov.b32 %10, lat; mov.b32 %11, xs;\n"
+                    "mov.b32 %12, epos; mov.b32 %13, efull; mov.b32 %14, e_on; mov.b64 %15, e_key; mov.b32 %16, e_idx; mov.b32 %17, qv;\n"
+                    "mov.b32 %18, tail_a; mov.b32 %19, rw; mov.b32 %20, sa; mov.b32 %21, tail_b;\n"
+                    "}"
+                    : "+r"(i), "+r"(bm), "+r"(lpos), "+r"(lfull), "+r"(tpos), "+r"(at1), "+r"(at2), "+l"(tk), "+r"(prev), "+l"(rec), "+r"(lat), "+r"(xs), "+r"(epos), "+r"(efull), "+r"(e_on), "+l"(e_key), "+r"(e_idx), "+r"(qv), "+r"(tail_a), "+r"(rw), "+r"(sa), "+r"(tail_b)
+                    : "r"(xin), "r"(xin_mask), "r"(xin_row), "r"(tab), "r"(kfb), "r"(kfm), "r"(kb), "r"(rm), "r"(mbm1), "r"(tick), "r"(qmask), "r"(~qmask), "r"(qb), "r"(nq - 1u), "r"(xa), "r"(xam), "r"(down), "r"(mask_a), "r"(want_a), "l"(out)
+                    : "memory");
             } else {
-                hand = e_act && free_d;
-                sts64_shared_if(hand && da >= 0, sa, e_base | qv);
-                // (one counter: bytes of ring rows towards the child, of the slab on a leaf)
-                if (!FEAS) stg64_if(hand && da < 0 && IL_IN_RANGE(tail_a >> 3, leaving, p.status),
-                                    reinterpret_cast<uint64_t *>(reinterpret_cast<char *>(out) + tail_a), e_base | qv);
-                tail_a += hand ? tail_step : 0u;
-                if (FEAS) {
-                    late_fin = (hand && da < 0) ? e_base : 0ull;
-                    late_arr = __ldg(trace + (hand && da < 0 && IL_IN_RANGE(qid, p.n, p.status) ? qid : 0u));
+                asm volatile(
+                    "{\n"
+                    ".reg .b32 i; .reg .b32 bm; .reg .b32 lpos; .reg .b32 lfull; .reg .b32 tpos; .reg .b32 at1; .reg .b32 at2;\n"
+                    ".reg .b64 tk; .reg .b32 prev; .reg .b64 rec; .reg .b32 lat; .reg .b32 xs; .reg .b32 epos; .reg .b32 efull;\n"
+                    ".reg .b32 e_on; .reg .b64 e_key; .reg .b32 e_idx; .reg .b32 qv; .reg .b32 tail_a; .reg .b32 rw; .reg .b32 sa;\n"
+                    ".reg .b32 tail_b; .reg .b32 leaves; .reg .b32 xin; .reg .b32 xin_mask; .reg .b32 xin_row; .reg .b32 tab;\n"
+                    ".reg .b32 kfb; .reg .b32 kfm; .reg .b32 kb; .reg .b32 rm; .reg .b32 mbm1; .reg .b32 tick; .reg .b32 qmask;\n"
+                    ".reg .b32 tmask; .reg .b32 qb; .reg .b32 nqm; .reg .b32 xa; .reg .b32 xam; .reg .b32 down; .reg .b32 bits;\n"
+                    ".reg .b32 mask_a; .reg .b32 mask_b; .reg .b32 want_a; .reg .b32 want_b; .reg .b64 out; .reg .b64 out_b;\n"
+                    "mov.b32 i, %0; mov.b32 bm, %1; mov.b32 lpos, %2; mov.b32 lfull, %3; mov.b32 tpos, %4; mov.b32 at1, %5;\n"
+                    "mov.b32 at2, %6; mov.b64 tk, %7; mov.b32 prev, %8; mov.b64 rec, %9; mov.b32 lat, %10; mov.b32 xs, %11;\n"
+                    "mov.b32 epos, %12; mov.b32 efull, %13; mov.b32 e_on, %14; mov.b64 e_key, %15; mov.b32 e_idx, %16; mov.b32 qv, %17;\n"
+                    "mov.b32 tail_a, %18; mov.b32 rw, %19; mov.b32 sa, %20; mov.b32 tail_b, %21; mov.b32 xin, %23; mov.b32 xin_mask, %24;\n"
+                    "mov.b32 xin_row, %25; mov.b32 tab, %26; mov.b32 kfb, %27; mov.b32 kfm, %28; mov.b32 kb, %29; mov.b32 rm, %30;\n"
+                    "mov.b32 mbm1, %31; mov.b32 tick, %32; mov.b32 qmask, %33; mov.b32 tmask, %34; mov.b32 qb, %35; mov.b32 nqm, %36;\n"
+                    "mov.b32 xa, %37; mov.b32 xam, %38; mov.b32 down, %39; mov.b32 bits, %40; mov.b32 mask_a, %41; mov.b32 mask_b, %42;\n"
+                    "mov.b32 want_a, %43; mov.b32 want_b, %44; mov.b64 out, %45; mov.b64 out_b, %46;\n"
+                    ".reg .pred t, taken, open, pop, ov, dp, pz, pf, hand, hd, ho, fin, fetch;\n"
+                    ".reg .u32 at0, sd, rl, rh, kl, kh, fl, fh, word, wa, x, y, lo, hi, a, xs_was, sa_was, ta_was, pos, left, a1, a2, a3, a4;\n"
+                    ".reg .b64 kf, k1, k2, fk, key, td, r, first, v, e1, e2, e3, e4; .reg .pred ga, gb, lv; .reg .b64 o; .reg .u32 ma, mb;\n"
+                    "and.b32 a, epos, rm; or.b32 a, a, kb; ld.shared.b64 fk, [a];\n"
+                    "and.b32 a, lpos, kfm; or.b32 a, a, kfb; ld.shared.b64 kf, [a];\n"
+                    "ld.shared.b64 k1, [at1]; ld.shared.b64 k2, [at2];\n"
+                    "mov.b64 td, tk; mov.b64 {rl, rh}, rec; mov.u32 xs_was, xs; mov.u32 sa_was, sa;\n"
+                    "setp.ne.u32 t, tpos, efull; selp.b32 rh, rh, -1, t; mov.b64 r, {rl, rh};\n"
+                    "setp.ge.s32 taken, rh, 0; setp.ge.and.u32 t, bm, mbm1, taken; setp.gt.or.f64 open, r, td, t;\n"
+                    "sub.u32 y, i, bm; add.u32 y, y, -1;\n"
+                    "add.u32 wa, i, -1; and.b32 wa, wa, nqm; mad.lo.u32 wa, wa, 128, qb;\n"
+                    "@taken add.u32 i, i, 1; and.b32 xs, i, xin_mask; mad.lo.u32 xs, xs, xin_row, xin; ld.relaxed.cta.shared.b64 rec, [xs];\n"
+                    "setp.lt.s32 hand, rw, 0; setp.ne.and.u32 hand, e_on, 0, hand; setp.ge.and.s32 hd|ho, down, 0, hand; setp.lt.and.s32 fin, qv, 0, hand;\n"
+                    "and.b32 x, qv, 0x7fffffff; mov.b64 {lo, hi}, e_key; and.b32 lo, lo, tmask; or.b32 a, lo, x; mov.b64 v, {a, hi}; mov.u32 ta_was, tail_a;\n"
+                    "and.b32 ma, bits, mask_a; and.b32 mb, bits, mask_b; mov.u32 ta_was, tail_a;\n"
+                    "setp.eq.and.u32 ga|lv, ma, want_a, ho; setp.eq.and.u32 gb, mb, want_b, ho; setp.ne.and.u32 lv, mb, want_b, lv;\n"
+                    "@hd add.u32 tail_a, tail_a, 256; @ga add.u32 tail_a, tail_a, 8;\n"
+                    "and.b32 sa, tail_a, xam; or.b32 sa, sa, xa; ld.relaxed.cta.shared.u32 rw, [sa+4];\n"
+                    "mad.wide.u32 key, lat, tick, tk; mov.b64 {kl, kh}, key; and.b32 kl, kl, tmask; or.b32 kl, kl, y; mov.b64 key, {kl, kh};\n"
+                    "@taken add.u32 bm, bm, 1; @open mov.u32 bm, 0; mad.lo.u32 a, bm, 4, tab; ld.shared.u32 lat, [a];\n"
+                    "setp.eq.or.u32 fetch, e_on, 0, fin; setp.ne.and.u32 fetch, epos, tpos, fetch; setp.le.and.f64 fetch, fk, td, fetch;\n"
+                    "mov.b64 {fl, fh}, fk;\n"
+                    "@hand add.u32 e_idx, e_idx, 1; @fetch and.b32 e_idx, fl, qmask; and.b32 a, e_idx, nqm; mad.lo.u32 a, a, 128, qb; ld.shared.u32 qv, [a];\n"
+                    "@hd st.relaxed.cta.shared.b64 [sa_was], v;\n"
+                    "mad.wide.u32 o, ta_was, 1, out; @ga st.global.b64 [o], v; mad.wide.u32 o, tail_b, 1, out_b; @gb st.global.b64 [o], v;\n"
+                    "@gb add.u32 tail_b, tail_b, 8; selp.u32 leaves, 1, 0, lv;\n"
+                    "@fetch mov.b64 e_key, fk; @fin mov.u32 e_on, 0; @fetch mov.u32 e_on, 1; @fetch add.u32 epos, epos, 256; @fetch add.u32 efull, efull, 256;\n"
+                    "and.b32 at0, tpos, rm; or.b32 at0, at0, kb;\n"
+                    "setp.lt.f64 pf, kf, key; selp.b64 first, kf, key, pf;\n"
+                    "setp.eq.u32 pz, tpos, lfull; setp.lt.and.f64 pz, r, first, pz; selp.b64 first, first, r, pz;\n"
+                    "mov.b64 {fl, fh}, first; or.b32 fl, fl, qmask; mov.b64 first, {fl, fh}; selp.b64 tk, first, tk, open;\n"
+                    "setp.lt.and.f64 ov, key, k1, open; selp.u32 sd, at1, at0, ov;\n"
+                    "@open st.shared.b64 [sd], key; @ov st.shared.b64 [at0], k1;\n"
+                    "setp.lt.and.f64 dp, key, k2, ov; mov.u32 pos, tpos; mov.u32 left, lpos;\n"
+                    "setp.eq.and.u32 pop, tpos, lfull, open;\n"
+                    "mov.u32 word, prev; @open or.b32 word, word, 0x80000000; @taken st.shared.u32 [wa], word;\n"
+                    "@taken st.relaxed.cta.shared.u32 [xs_was+4], -1;\n"
+                    "@open add.u32 tpos, tpos, 256; @open mov.u32 at2, at1; @open mov.u32 at1, at0;\n"
+                    "@pop add.u32 lpos, lpos, 256; @pop add.u32 lfull, lfull, 256;\n"
+                    "@taken and.b32 prev, rl, qmask;\n"
+                    "@!dp bra PLACED;\n"
+                    "mov.u32 sd, left; sub.u32 pos, pos, 256;\n"
+                    "DEEPER:\n"
+                    "sub.u32 left, pos, sd;\n"
+                    "and.b32 at0, pos, rm; or.b32 at0, at0, kb; sub.u32 a1, pos, 256; and.b32 a1, a1, rm; or.b32 a1, a1, kb;\n"
+                    "sub.u32 a2, pos, 512; and.b32 a2, a2, rm; or.b32 a2, a2, kb; sub.u32 a3, pos, 768; and.b32 a3, a3, rm; or.b32 a3, a3, kb;\n"
+                    "sub.u32 a4, pos, 1024; and.b32 a4, a4, rm; or.b32 a4, a4, kb;\n"
+                    "ld.shared.b64 e1, [a1]; ld.shared.b64 e2, [a2]; ld.shared.b64 e3, [a3]; ld.shared.b64 e4, [a4];\n"
+                    "setp.gt.u32 t, left, 0; setp.lt.and.f64 t, key, e1, t; setp.gt.and.u32 ov, left, 256, t; setp.lt.and.f64 ov, key, e2, ov;\n"
+                    "setp.gt.and.u32 pz, left, 512, ov; setp.lt.and.f64 pz, key, e3, pz; setp.gt.and.u32 pf, left, 768, pz; setp.lt.and.f64 pf, key, e4, pf;\n"
+                    "@t st.shared.b64 [at0], e1; @ov st.shared.b64 [a1], e2; @pz st.shared.b64 [a2], e3; @pf st.shared.b64 [a3], e4;\n"
+                    "@t mov.u32 at0, a1; @ov mov.u32 at0, a2; @pz mov.u32 at0, a3; @pf mov.u32 at0, a4; st.shared.b64 [at0], key;\n"
+                    "sub.u32 pos, pos, 1024; @pf bra DEEPER;\n"
+                    "PLACED:\n"
+                    "mov.b32 %0, i; mov.b32 %1, bm; mov.b32 %2, lpos; mov.b32 %3, lfull; mov.b32 %4, tpos; mov.b32 %5, at1;\n"
+                    "mov.b32 %6, at2; mov.b64 %7, tk; mov.b32 %8, prev; mov.b64 %9, rec; mov.b32 %10, lat; mov.b32 %11, xs;\n"
+                    "mov.b32 %12, epos; mov.b32 %13, efull; mov.b32 %14, e_on; mov.b64 %15, e_key; mov.b32 %16, e_idx; mov.b32 %17, qv;\n"
+                    "mov.b32 %18, tail_a; mov.b32 %19, rw; mov.b32 %20, sa; mov.b32 %21, tail_b; mov.b32 %22, leaves;\n"
+                    "}"
+                    : "+r"(i), "+r"(bm), "+r"(lpos), "+r"(lfull), "+r"(tpos), "+r"(at1), "+r"(at2), "+l"(tk), "+r"(prev), "+l"(rec), "+r"(lat), "+r"(xs), "+r"(epos), "+r"(efull), "+r"(e_on), "+l"(e_key), "+r"(e_idx), "+r"(qv), "+r"(tail_a), "+r"(rw), "+r"(sa), "+r"(tail_b), "=r"(leaves)
+                    : "r"(xin), "r"(xin_mask), "r"(xin_row), "r"(tab), "r"(kfb), "r"(kfm), "r"(kb), "r"(rm), "r"(mbm1), "r"(tick), "r"(qmask), "r"(~qmask), "r"(qb), "r"(nq - 1u), "r"(xa), "r"(xam), "r"(down), "r"(bits), "r"(mask_a), "r"(mask_b), "r"(want_a), "r"(want_b), "l"(out), "l"(out_b)
+                    : "memory");
+                if (FEAS) late_fin = 0ull;
+                if (pt->n_leave > 0 && leaves != 0u) {
+                    // (a branch point at which some queries leave)
+                    const uint32_t qid = left_low & imask;
+                    const uint64_t fin = left_rec & ~(uint64_t)qmask;
+                    if (FEAS) {
+                        late_fin = fin;
+                        late_arr = __ldg(trace + qid);
+                    } else if (FORK) {
+                        atomicMax(reinterpret_cast<unsigned long long *>(out_c) + qid, (fin >> rb) | qid);
+                    } else if (IL_IN_RANGE(n_left, pt->n_leave, p.status)) {
+                        out_c[n_left] = (fin >> rb) | qid;
+                    }
+                    n_left++;
                 }
             }
-            // the next record to hand on: of the batch in hand, or the first one of the next batch
-            const bool goes_on = e_act && !(hand && last);
-            const bool fetch = f_ok && !goes_on;
-            e_idx += hand ? 1u : 0u;
-            e_idx = fetch ? (uint32_t)fkey & qmask : e_idx;
-            e_key = fetch ? fkey : e_key;
-            epos += fetch ? 256u : 0u;
-            efull += fetch ? 256u : 0u;
-            e_act = goes_on || fetch;
-            qv = lds32(qb + ((e_idx & (nq - 1u)) << 7));
-            // (the lane's own stores, so the words may come through L1: 32 of them with one miss)
-            if (SPILL) ldg32_if(spill && i - e_idx > nq && IL_IN_RANGE(e_idx & gmask, gmask + 1ull, p.status), spill_ring + (e_idx & gmask), qv);
-            if (JOIN) __syncwarp();      // what was delivered is there for the joins' lanes
+            if (SPILL) {
+                // (the lane's own stores, so the words may come through L1: 32 of them with one miss)
+                ldg32_if((is & kSpill) && i - e_idx > nq && IL_IN_RANGE(e_idx & gmask, gmask + 1ull, p.status), spill_ring + (e_idx & gmask), qv);
+                stg32_if((is & kSpill) && i != i_was && IL_IN_RANGE((i_was - 1u) & gmask, gmask + 1ull, p.status),
+                         spill_ring + ((i_was - 1u) & gmask), prev_was | (tpos != tpos_was ? kLast : 0u));
+            }
         };
-        if (any_spill) {
+        auto run_turn = [&](auto kind) {
+            if (any_spill) {
 #pragma unroll 1
-            for (int k = 0; k < turn_its; k++) step(std::true_type{});
-        } else {
+                for (int k = 0; k < turn_its; k++) step(std::true_type{}, kind);
+            } else {
 #pragma unroll 1
-            for (int k = 0; k < turn_its; k += 2) { step(std::false_type{}); step(std::false_type{}); }
-        }
+                for (int k = 0; k < turn_its; k += 2) { step(std::false_type{}, kind); step(std::false_type{}, kind); }
+            }
+        };
+        using One = std::integral_constant<int, kOutOne>;
+        using Leaf = std::integral_constant<int, kOutLeaf>;
+        using Two = std::integral_constant<int, kOutTwo>;
+        using Any = std::integral_constant<int, kOutAny>;
+        if (!CUT) run_turn(std::integral_constant<int, FEAS ? kOutLeaf : kOutOne>{});
+        else if (out_kind == kOutOne) run_turn(One{});
+        else if (out_kind == kOutLeaf) run_turn(Leaf{});
+        else if (out_kind == kOutTwo) run_turn(Two{});
+        else run_turn(Any{});
+    }
     }
 
     for (int o = 16; o > 0; o >>= 1) {
@@ -826,75 +1374,127 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, unsigned cha
     }
 }
 
-template <bool BRANCHY, bool FEAS, bool FORK = false>
+// Pipelines that are chains: one group of lanes per candidate.
+template <bool FEAS>
 __global__ void __launch_bounds__(kLaneWarps * 32, 3) des_lane_kernel(const __grid_constant__ DesParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    lane_simulation<BRANCHY, FEAS, FORK, false>(p, smem_raw);
+    lane_simulation<FEAS, false, false>(p, LaneCut(), smem_raw);
 }
 
-// Pipelines with joins.  (il_kernel_name reports "des_kernel" for them, as for the form in des_kernel.cu that takes over
-// where times do not fit a record.)
-__global__ void __launch_bounds__(kLaneWarps * 32) des_join_lane_kernel(const __grid_constant__ DesParams p)
+// Pipelines cut at their branch points.
+template <bool FEAS, bool FORK>
+__global__ void __launch_bounds__(kLaneWarps * 32, 2) des_part_kernel(const __grid_constant__ DesParams p, const __grid_constant__ LaneCut cut)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    lane_simulation<true, false, true, true>(p, smem_raw);
+    lane_simulation<FEAS, true, FORK>(p, cut, smem_raw);
 }
 
 namespace {
-bool any_branch(const DesParams &p)
+
+// Root nodes of a chunk: the distinct (hardware, batch, replicas) of stage 0 among its candidates, numbered, each with how
+// many groups will read its streams; every candidate's node, -1 where a configuration is out of range.  One CTA: a bit per
+// configuration in shared memory (a word per hardware and batch), a prefix sum over the words, and the numbers read back.
+constexpr int kNodeThreads = 1024;
+__global__ void __launch_bounds__(kNodeThreads) root_nodes_kernel(const RootNodeParams p)
 {
-    for (int s = 0; s < p.S; s++) if (p.bit[s] >= 0) return true;
-    return false;
+    __shared__ uint32_t seen[IL_MAX_HW * IL_MAX_BATCH], first[IL_MAX_HW * IL_MAX_BATCH], sums[32];
+    const int t = threadIdx.x, words = p.H * p.Bmax;
+    for (int w = t; w < words; w += kNodeThreads) seen[w] = 0u;
+    __syncthreads();
+    for (int64_t c = t; c < p.n_cand; c += kNodeThreads) {
+        bool ok = true;
+        for (int s = 0; s < p.S; s++) {
+            const il_stage_config k = p.configs[c * p.S + s];
+            ok &= k.hw < p.H && k.max_batch >= 1 && k.max_batch <= p.Bmax && k.replicas >= 1 && k.replicas <= IL_MAX_REPLICAS;
+        }
+        const il_stage_config k = p.configs[c * p.S];
+        if (ok) atomicOr(&seen[k.hw * p.Bmax + k.max_batch - 1], 1u << (k.replicas - 1));
+        else atomicCAS(p.status, 0, IL_ERR_BAD_CONFIG);
+        p.root_of[c] = ok ? (p.shared ? 0 : (int32_t)c) : -1;
+        if (ok && !p.shared && p.out_feasible) p.refs[c] = (uint32_t)p.readers;
+        if (p.out_feasible) { p.out_feasible[c] = ok ? 1 : 0; p.miss[c] = 0u; }
+    }
+    if (!p.shared) return;
+    __syncthreads();
+    // (IL_MAX_HW * IL_MAX_BATCH <= kNodeThreads: a word per thread)
+    const uint32_t mine = t < words ? (uint32_t)__popc(seen[t]) : 0u;
+    uint32_t upto = mine;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, upto, o);
+        if ((t & 31) >= o) upto += v;
+    }
+    if ((t & 31) == 31) sums[t >> 5] = upto;
+    __syncthreads();
+    uint32_t base = 0, all = 0;
+    for (int k = 0; k < kNodeThreads / 32; k++) { base += k < (t >> 5) ? sums[k] : 0u; all += sums[k]; }
+    if (t < words) {
+        first[t] = base + upto - mine;
+        uint32_t at = first[t];
+        for (uint32_t m = seen[t]; m != 0u; m &= m - 1u)
+            p.node_cfg[at++] = (uint32_t)(t / p.Bmax) | (uint32_t)(t % p.Bmax + 1) << 8 | (uint32_t)__ffs((int)m) << 16;
+    }
+    if (t == 0) p.ctl[kCtlNodes] = all;
+    __syncthreads();
+    for (int64_t c = t; c < p.n_cand; c += kNodeThreads) {
+        if (p.root_of[c] < 0) continue;
+        const il_stage_config k = p.configs[c * p.S];
+        const int w = k.hw * p.Bmax + k.max_batch - 1;
+        const uint32_t at = first[w] + (uint32_t)__popc(seen[w] & ((1u << (k.replicas - 1)) - 1u));
+        p.root_of[c] = (int32_t)at;
+        if (p.out_feasible) atomicAdd(p.refs + at, (uint32_t)p.readers);
+    }
 }
 
-template <bool BRANCHY, bool FEAS, bool FORK>
-cudaError_t launch_one(const DesParams &p, int grid, size_t smem, cudaStream_t stream)
+template <typename K, typename... A>
+cudaError_t launch_one(K kernel, int grid, size_t smem, cudaStream_t stream, const A &...args)
 {
-    cudaError_t e = cudaFuncSetAttribute(des_lane_kernel<BRANCHY, FEAS, FORK>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    des_lane_kernel<BRANCHY, FEAS, FORK><<<grid, kLaneWarps * 32, smem, stream>>>(p);
+    kernel<<<grid, kLaneWarps * 32, smem, stream>>>(args...);
     return cudaGetLastError();
 }
 }  // namespace
 
-// Feasibility-only when p.out_feasible is set; the fan-out instantiation when p.fork is (the host
-// never combines the two, nor fan-out with spill rings shorter than the longest stream).
-cudaError_t launch_des_lane(const DesParams &p, int grid, size_t smem, cudaStream_t stream)
+cudaError_t launch_root_nodes(const RootNodeParams &p, cudaStream_t stream)
 {
-    if (p.n_join > 0) {
-        if (p.lane_wrap || p.out_feasible) return cudaErrorInvalidValue;
-        cudaError_t e = cudaFuncSetAttribute(des_join_lane_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        des_join_lane_kernel<<<grid, kLaneWarps * 32, smem, stream>>>(p);
-        return cudaGetLastError();
-    }
+    root_nodes_kernel<<<1, kNodeThreads, 0, stream>>>(p);
+    return cudaGetLastError();
+}
+
+// Feasibility-only when p.out_feasible is set; cut: the pipeline's parts, nullptr for a chain.  (The host never combines
+// fan-out with feasibility-only, nor with spill rings shorter than the longest stream.)
+cudaError_t launch_des_lane(const DesParams &p, const LaneCut *cut, int grid, size_t smem, cudaStream_t stream)
+{
+    if (!cut)
+        return p.out_feasible ? launch_one(des_lane_kernel<true>, grid, smem, stream, p) : launch_one(des_lane_kernel<false>, grid, smem, stream, p);
     if (p.fork) {
         if (p.lane_wrap || p.out_feasible) return cudaErrorInvalidValue;
-        return launch_one<true, false, true>(p, grid, smem, stream);
+        return launch_one(des_part_kernel<false, true>, grid, smem, stream, p, *cut);
     }
-    if (any_branch(p))
-        return p.out_feasible ? launch_one<true, true, false>(p, grid, smem, stream) : launch_one<true, false, false>(p, grid, smem, stream);
-    return p.out_feasible ? launch_one<false, true, false>(p, grid, smem, stream) : launch_one<false, false, false>(p, grid, smem, stream);
+    return p.out_feasible ? launch_one(des_part_kernel<true, false>, grid, smem, stream, p, *cut)
+                          : launch_one(des_part_kernel<false, false>, grid, smem, stream, p, *cut);
 }
 
 int des_lane_warps_per_cta() { return kLaneWarps; }
+int lane_root_sms(int64_t nodes, int num_sms) { return (int)root_sms_for((uint32_t)std::min<int64_t>(nodes, 1 << 20), (uint32_t)num_sms); }
+int lane_stretch_bytes(int groups, int ahead) { return groups * (int)stretch_bytes(ahead); }
 
-size_t des_lane_smem(int table_rows, int Bmax, int ring_slots, int ring_words, int cpw, int joins, int window)
+size_t des_lane_smem(int table_rows, int Bmax, int ring_slots, int ring_words, int stretch)
 {
     return (kSmemBase + table_bytes(table_rows, Bmax) + key_bytes(ring_slots) - 1) / key_bytes(ring_slots) * key_bytes(ring_slots) -
-           kSmemBase + ring_bytes(ring_slots, ring_words, cpw) + kTailBytes + join_bytes(cpw, joins, window);
+           kSmemBase + ring_bytes(ring_slots, ring_words, stretch) + kTailBytes;
 }
 
-int des_lane_max_ctas_per_sm(size_t smem, bool joins)
+int des_lane_max_ctas_per_sm(size_t smem, bool cut)
 {
     int n = 0;
-    // (all instantiations without joins are compiled for three CTAs; the one with joins takes more registers)
-    void (*kernel)(DesParams) = joins ? des_join_lane_kernel : des_lane_kernel<true, true>;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kLaneWarps * 32, smem);
-    return e == cudaSuccess ? n : 0;
+    // (all instantiations of one kind are compiled for the same number of CTAs)
+    auto ask = [&](auto kernel) {
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) { cudaGetLastError(); return 0; }
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kLaneWarps * 32, smem) == cudaSuccess ? n : 0;
+    };
+    return cut ? ask(des_part_kernel<true, false>) : ask(des_lane_kernel<true>);
 }
 
 }  // namespace il

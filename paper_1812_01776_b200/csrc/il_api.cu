@@ -66,6 +66,15 @@ struct il_estimator {
     int32_t parent[IL_MAX_STAGES] = {};
     int cpw = 1;                       // lane kernel: candidates per warp
     int ctas_lane[2] = {0, 0};         // lane kernel with 16 / 32 batch ring positions per lane: CTAs that fit an SM
+    // lane kernel, pipelines with branch points: the parts and the streams between them (cut.n_part = 0: a chain, one group
+    // of lanes per candidate), where each stream lies, and how many records a root node and a candidate need for them
+    LaneCut cut = {};
+    int n_stream = 0;
+    enum Place : uint8_t { kAtNode, kInSlab, kExtra } stream_at[IL_MAX_STAGES] = {};
+    bool slab_streams = false;
+    int64_t node_elems = 0, extra_elems = 0;
+    int root_readers = 0;
+    int64_t leaving[IL_MAX_STAGES] = {};       // queries (fan-out: copies) that leave after a stage
     int lane_slots = 32;               // batch ring positions used by the current call
     int64_t setup_launches = 0;        // kernels a call launched before its simulation: the replica reduction, the node probe
     int lane_ctas_knob = 0;            // test knob: resident CTAs per SM of the lane kernel at most (0: as many as fit)
@@ -111,6 +120,11 @@ struct Plan {
     int64_t fb_slots = 0;    // lane kernel with wrapping rings: warp slots of the kernel that takes over
                              // the candidates given up on ring overflow
     size_t off_time = 0, off_qid = 0, off_slab = 0, off_order = 0, off_ovf = 0, off_fb = 0, total = 0;
+    bool feas = false;       // feasibility only: nothing is kept for the warp-per-candidate kernel
+    bool slab = true;        // rows of the slab are needed
+    // pipelines cut into parts: root nodes at most, control words and counts, what the host prepares, streams
+    int64_t nodes = 0;
+    size_t off_ctl = 0, ctl_bytes = 0, off_root = 0, off_node = 0, off_node_rows = 0, off_extra = 0;
 };
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -148,12 +162,13 @@ int ctas_for(const il_estimator *e)
 // warp-per-candidate kernels serve one candidate at a time from it, the lane
 // kernel cpw candidates.
 bool is_lane(const il_estimator *e) { return sim_kernel(e) == kSimLane; }
+bool is_cut(const il_estimator *e) { return is_lane(e) && e->cut.n_part > 0; }
 int warps_per_cta(const il_estimator *e) { return is_lane(e) ? des_lane_warps_per_cta() : kWarpsPerCta; }
 // A batch that leaves schedulers idle is spread over them first: a warp that has its scheduler to itself takes
 // the same time for one candidate as for cpw, and less where its lanes diverge.
 int64_t cands_per_slot(const il_estimator *e, int64_t n_cand)
 {
-    if (!is_lane(e)) return 1;
+    if (!is_lane(e) || is_cut(e)) return 1;
     const int64_t schedulers = (int64_t)e->num_sms * 4;
     return std::max<int64_t>(1, std::min<int64_t>(e->cpw, (n_cand + schedulers - 1) / schedulers));
 }
@@ -176,15 +191,94 @@ bool looks_for_prefixes(const il_estimator *e, int64_t n_cand)
 // bits of the queries of which one input has come in and the incoming streams.
 size_t slot_time_bytes(const il_estimator *e, int64_t cps)
 {
+    if (is_cut(e)) return (size_t)32 * 4 << e->lane_ring_log2;
     return is_lane(e) ? (size_t)cps * (e->S + e->base.n_join) * 4 << e->lane_ring_log2 : (size_t)e->slot_elems * 8;
 }
+// Root nodes that so many candidates can have.
+int64_t most_nodes(const il_estimator *e, int64_t n_cand)
+{
+    return e->cut.shared ? std::min<int64_t>(n_cand, (int64_t)e->H * e->Bmax * IL_MAX_REPLICAS) : n_cand;
+}
+
+// How a launch of a cut pipeline is laid out: CTAs per SM, groups per warp and warps of each part, records of its arrival
+// stream that a group keeps in shared memory.
+struct Shape {
+    int ctas = 1;
+    int64_t grid = 1;
+    int ahead = 64, stretch = 0;
+    int groups[IL_MAX_STAGES] = {}, warps[IL_MAX_STAGES] = {};
+};
+
+size_t lane_smem(const il_estimator *e, int lane_slots, int words, int stretch)
+{
+    return des_lane_smem(e->S * e->H, e->Bmax, lane_slots, words, stretch);
+}
+
+int lane_ctas(const il_estimator *e, int lane_slots);
+
+Shape cut_shape(const il_estimator *e, int64_t n_cand, int lane_slots)
+{
+    const LaneCut &cut = e->cut;
+    const int t0 = cut.shared ? 1 : 0;
+    const int64_t nodes = most_nodes(e, n_cand), root_sms = cut.shared ? lane_root_sms(nodes, e->num_sms) : 0;
+    const int64_t sms = std::max<int64_t>(1, e->num_sms - root_sms);
+    Shape sh;
+    auto warps_with = [&](int most) {
+        int64_t all = 0;
+        for (int t = t0; t < cut.n_part; t++) {
+            sh.groups[t] = std::min(most, 32 / cut.part[t].len);
+            sh.warps[t] = (int)std::min<int64_t>((n_cand + sh.groups[t] - 1) / sh.groups[t], 1 << 24);
+            all += sh.warps[t];
+        }
+        return all;
+    };
+    auto stretch_fits = [&](int ctas) {
+        int most = (int)std::min<int64_t>(kRootGroups, nodes);
+        for (int t = t0; t < cut.n_part; t++) most = std::max(most, sh.groups[t]);
+        for (sh.ahead = 64; sh.ahead >= 32; sh.ahead >>= 1) {
+            sh.stretch = lane_stretch_bytes(most, sh.ahead);
+            const size_t bytes = lane_smem(e, lane_slots, kLaneWords, sh.stretch);
+            if (bytes <= e->smem_per_cta && (bytes + 1024) * ctas <= e->smem_per_sm) return true;
+        }
+        sh.ahead = 32;
+        return false;
+    };
+    // a warp on every scheduler first, with as few groups each as that takes
+    for (int most = 1; most <= 32; most++) {
+        const int64_t need = warps_with(most);
+        if (need > sms * 4 && most < 32) continue;
+        if (need <= sms * 4 && stretch_fits(1)) {
+            sh.grid = std::min<int64_t>(e->num_sms, root_sms + (need + 3) / 4);
+            return sh;
+        }
+        break;
+    }
+    const int64_t need = warps_with(32);
+    for (sh.ctas = 1; sh.ctas < lane_ctas(e, lane_slots) && need > sms * 4 * sh.ctas; sh.ctas++) {}
+    while (!stretch_fits(sh.ctas) && sh.ctas > 1) sh.ctas--;
+    sh.grid = (int64_t)e->num_sms * sh.ctas;
+    const int64_t room = sms * 4 * sh.ctas;
+    if (need > room) {      // more than fit at once: warps by the work of the parts
+        double all = 0.0;
+        for (int t = t0; t < cut.n_part; t++) all += (double)sh.warps[t] * std::max<int64_t>(1, e->visits[cut.part[t].stage[0]]);
+        for (int t = t0; t < cut.n_part; t++)
+            sh.warps[t] = std::max(1, (int)((double)room * sh.warps[t] * std::max<int64_t>(1, e->visits[cut.part[t].stage[0]]) / all));
+    }
+    return sh;
+}
+
 size_t slot_seen_bytes(const il_estimator *e, int64_t cps) { return (size_t)cps * e->base.n_join * e->base.join_seen_words * 4; }
 size_t slot_qid_bytes(const il_estimator *e, int64_t cps)
 {
     return is_lane(e) ? slot_seen_bytes(e, cps) + (size_t)cps * e->base.join_elems * 8 : (size_t)e->slot_elems * 4;
 }
 size_t slot_bytes(const il_estimator *e, int64_t cps) { return slot_time_bytes(e, cps) + slot_qid_bytes(e, cps); }
-size_t cand_bytes(const il_estimator *e) { return (size_t)e->n_pad * 8 + 5; }   // slab row, order entry, overflow mark
+// slab row, order entry, overflow mark; cut: streams of its own, counts, root node, misses
+size_t cand_bytes(const il_estimator *e, bool slab)
+{
+    return (slab ? (size_t)e->n_pad * 8 : 0) + 5 + (is_cut(e) ? (size_t)e->extra_elems * 8 + (size_t)e->n_stream * 4 + 8 : 0);
+}
+size_t node_bytes(const il_estimator *e) { return (size_t)e->node_elems * 8 + 8; }      // a root node's streams, configuration, readers
 bool lane_fallback(const il_estimator *e) { return is_lane(e) && e->lane_wrap; }
 size_t fb_slot_bytes(const il_estimator *e) { return (size_t)e->slot_elems * 8; }
 
@@ -203,6 +297,7 @@ int64_t full_slots(const il_estimator *e, int lane_slots)
 
 int64_t wanted_slots(const il_estimator *e, int64_t n_cand, int lane_slots)
 {
+    if (is_cut(e)) return cut_shape(e, n_cand, lane_slots).grid * warps_per_cta(e);
     const int64_t w = warps_per_cta(e), cps = cands_per_slot(e, n_cand);
     const int64_t need = ((n_cand + cps - 1) / cps + w - 1) / w * w;
     return std::max<int64_t>(w, std::min(full_slots(e, lane_slots), need));
@@ -213,10 +308,19 @@ size_t layout(const il_estimator *e, Plan &pl)
     size_t off = 0;
     pl.off_time = off; off = align_up(off + (size_t)pl.slots * slot_time_bytes(e, pl.cps), 256);
     pl.off_qid = off;  off = align_up(off + (size_t)pl.slots * slot_qid_bytes(e, pl.cps), 256);
-    pl.off_slab = off; off = align_up(off + (size_t)pl.chunk * e->n_pad * 8, 256);
+    pl.off_slab = off; off = align_up(off + (pl.slab ? (size_t)pl.chunk * e->n_pad * 8 : 0), 256);
     pl.off_order = off; off = align_up(off + (size_t)pl.chunk * 4, 256);
     pl.off_ovf = off;  off = align_up(off + (size_t)pl.chunk, 256);
     pl.off_fb = off;   off = align_up(off + (size_t)pl.fb_slots * fb_slot_bytes(e), 256);
+    if (is_cut(e)) {
+        pl.nodes = most_nodes(e, pl.chunk);
+        pl.ctl_bytes = (kCtlWords + (size_t)e->n_stream * pl.chunk + pl.nodes) * 4;
+        pl.off_ctl = off;       off = align_up(off + pl.ctl_bytes, 256);
+        pl.off_root = off;      off = align_up(off + (size_t)pl.chunk * 8, 256);
+        pl.off_node = off;      off = align_up(off + (size_t)pl.nodes * 4, 256);
+        pl.off_node_rows = off; off = align_up(off + (size_t)pl.nodes * e->node_elems * 8, 256);
+        pl.off_extra = off;     off = align_up(off + (size_t)pl.chunk * e->extra_elems * 8, 256);
+    }
     pl.total = off;
     return off;
 }
@@ -247,6 +351,10 @@ size_t recommended_bytes(const il_estimator *e, int64_t n_cand)
     pl.slots = wanted_slots(e, n_cand, 16);
     const int64_t cps = cands_per_slot(e, n_cand);
     pl.cps = cps;
+    if (is_cut(e)) {
+        pl.slots = std::max(pl.slots, wanted_slots(e, n_cand, 32));
+        pl.chunk = std::max<int64_t>(2 * warps_per_cta(e), std::min<int64_t>(n_cand, 8 * full_slots(e, 16) * e->cpw));
+    } else
     pl.chunk = std::max<int64_t>(std::min<int64_t>(n_cand, 8 * full_slots(e, 16) * cps), 2 * pl.slots * cps);
     pl.fb_slots = lane_fallback(e) ? (int64_t)e->num_sms * kWarpsPerCta : 0;
     return std::max(layout(e, pl) + 2048, min_bytes(e));
@@ -255,13 +363,29 @@ size_t recommended_bytes(const il_estimator *e, int64_t n_cand)
 // Splits `bytes` of workspace between warp slots and the latency slab.
 bool make_plan(const il_estimator *e, size_t bytes, int64_t n_cand, Plan &pl)
 {
-    if (bytes < min_bytes(e)) return false;
+    if (bytes < (pl.feas ? 4096 : min_bytes(e))) return false;
     size_t usable = bytes - 1024;
-    pl.fb_slots = fallback_slots(e, usable);
+    pl.fb_slots = pl.feas ? 0 : fallback_slots(e, usable);
     if (pl.fb_slots > 0) usable -= (size_t)pl.fb_slots * fb_slot_bytes(e) + 256;
     const int64_t w = warps_per_cta(e);
     const int64_t cps = cands_per_slot(e, n_cand);
-    const size_t sb = slot_bytes(e, cps), cb = cand_bytes(e);
+    const size_t sb = slot_bytes(e, cps), cb = cand_bytes(e, pl.slab);
+    if (is_cut(e)) {
+        // any number of CTAs does (each takes whatever part is next); where not all rows fit they get half of the space at least
+        pl.cps = cps;
+        const size_t rows = (size_t)n_cand * cb + (size_t)most_nodes(e, n_cand) * node_bytes(e) + 8192;
+        const size_t for_slots = std::max(usable / 2, usable > rows ? usable - rows : 0);
+        pl.slots = std::max(w, std::min<int64_t>(wanted_slots(e, n_cand, e->lane_slots), (int64_t)(for_slots / sb)) / w * w);
+        const size_t fixed = (size_t)pl.slots * sb + kCtlWords * 4;
+        if (fixed > usable) return false;
+        const size_t rest = usable - fixed, nb = node_bytes(e);
+        const int64_t all = most_nodes(e, INT64_C(1) << 40);
+        pl.chunk = (int64_t)(rest / (cb + nb));
+        if (pl.chunk > all) pl.chunk = (int64_t)((rest - (size_t)all * nb) / cb);
+        pl.chunk = std::min(n_cand, pl.chunk);
+        while (pl.chunk > 0 && layout(e, pl) > bytes) pl.chunk -= std::max<int64_t>(1, pl.chunk / 64);
+        return pl.chunk >= 1;
+    }
     int64_t slots = std::min<int64_t>(wanted_slots(e, n_cand, e->lane_slots), (int64_t)(usable / (sb + 2 * cps * cb)));
     slots = std::max(w, slots / w * w);
     if ((size_t)slots * sb > usable) return false;
@@ -370,6 +494,63 @@ void configure_lane_rings(il_estimator *e)
     e->lane_wrap = e->lane_ring_log2 < need;
     e->base.lane_ring_log2 = e->lane_ring_log2;
     e->base.lane_wrap = e->lane_wrap ? 1 : 0;
+}
+
+// Cuts a pipeline with branch points into parts: the root stage, and chains of stages that begin behind the root or behind a
+// branch.  Part t >= 1 reads stream t - 1.  A part that nothing follows reads from the slab region that its records leave
+// to (unless the root has written them, or several parts share a row: fan-out).
+void build_parts(il_estimator *e)
+{
+    const DesParams &b = e->base;
+    const int S = e->S;
+    LaneCut &cut = e->cut;
+    auto two_ways = [&](int s) { return b.child_b[s] >= 0 || (b.child_a[s] >= 0 && b.cbit_a[s] >= 0); };
+    bool any = false;
+    for (int s = 0; s < S; s++) any |= two_ways(s);
+    if (!any || e->join) return;
+    cut.shared = e->leaving[0] == 0 ? 1 : 0;      // (records that leave there belong in every candidate's row)
+    auto even = [](int64_t v) { return (v + 1) / 2 * 2; };
+    int part_of[IL_MAX_STAGES] = {};
+    int64_t exit_off[IL_MAX_STAGES + 1] = {};
+    for (int s = 0; s < S; s++) {
+        exit_off[s + 1] = exit_off[s] + e->leaving[s];
+        const int par = e->parent[s];
+        if (s == 0 || par == 0 || two_ways(par)) part_of[s] = cut.n_part++;
+        else part_of[s] = part_of[par];
+        LanePart &pt = cut.part[part_of[s]];
+        pt.stage[pt.len++] = (int8_t)s;
+    }
+    e->n_stream = cut.n_part - 1;
+    for (int t = 0; t < cut.n_part; t++) {
+        LanePart &pt = cut.part[t];
+        const int first = pt.stage[0], end = pt.stage[pt.len - 1];
+        pt.in = (int8_t)(t - 1);
+        pt.out_a = b.child_a[end] >= 0 ? (int8_t)(part_of[b.child_a[end]] - 1) : -1;
+        pt.out_b = b.child_b[end] >= 0 ? (int8_t)(part_of[b.child_b[end]] - 1) : -1;
+        pt.out_kind = (int8_t)(two_ways(end) ? kOutTwo : pt.out_a >= 0 ? kOutOne : kOutLeaf);
+        pt.n_leave = (int32_t)e->leaving[end];
+        pt.leave_off = e->fork ? 0 : (int32_t)exit_off[end];
+        pt.n_out = e->leaving[end];
+        for (int c : {(int)b.child_a[end], (int)b.child_b[end]}) if (c >= 0) pt.n_out += e->visits[c];
+        if (t == 0) continue;
+        LaneStream &x = cut.stream[t - 1];
+        x.len = (int32_t)e->visits[first];
+        x.by_node = part_of[e->parent[first]] == 0;
+        if (x.by_node) {
+            e->stream_at[t - 1] = il_estimator::kAtNode;
+            x.off = (int32_t)e->node_elems; e->node_elems += even(x.len);
+            e->root_readers++;
+        } else if (pt.out_kind == kOutLeaf && !e->fork) {
+            e->stream_at[t - 1] = il_estimator::kInSlab;
+            x.off = pt.leave_off;
+            e->slab_streams = true;
+        } else {
+            e->stream_at[t - 1] = il_estimator::kExtra;
+            x.off = (int32_t)e->extra_elems; e->extra_elems += even(x.len);
+        }
+    }
+    e->node_elems = (e->node_elems + 31) / 32 * 32;
+    e->extra_elems = (e->extra_elems + 31) / 32 * 32;
 }
 
 void free_device(il_estimator *e)
@@ -515,6 +696,7 @@ static DesParams chunk_params(const il_estimator *e, const Plan &pl, char *ws, c
     p.iter_limit = e->iter_limit;
     p.lane_slots = e->lane_slots;
     p.cpw = (int32_t)pl.cps;
+    p.lanes_per_slot = is_cut(e) ? 32 : (int32_t)pl.cps * e->S;
     if (e->join) {
         const size_t seen = ((size_t)pl.slots * slot_seen_bytes(e, pl.cps) + 7) / 8 * 8;
         p.join_seen = reinterpret_cast<uint32_t *>(ws + pl.off_qid);
@@ -538,9 +720,15 @@ static int start_call(il_estimator *e, const il_stage_config *d_configs, int64_t
     }
     e->setup_launches = 1;
     const int64_t cps = cands_per_slot(e, n_cand), per_cta = cps * des_lane_warps_per_cta();
-    if (max_replicas > 0 || (n_cand + per_cta - 1) / per_cta <= e->num_sms) {
+    const bool one_cta = is_cut(e) ? cut_shape(e, n_cand, 32).ctas == 1 : (n_cand + per_cta - 1) / per_cta <= e->num_sms;
+    if (max_replicas > 0 && max_replicas <= 16) e->lane_slots = 16;
+    if (is_cut(e) && (max_replicas > 0 || one_cta)) {      // (the numbering of the root nodes is a launch of its own)
+        IL_CUDA(cudaMemsetAsync(e->d_counters, 0, kCounterBytes, e->stream));
+        e->setup_launches = 0;
+        return IL_OK;
+    }
+    if (max_replicas > 0 || one_cta) {
         IL_CUDA(launch_clear(e->d_counters, (int)(kCounterBytes / sizeof(unsigned long long)), e->stream));
-        if (max_replicas > 0 && max_replicas <= 16) e->lane_slots = 16;
         return IL_OK;
     }
     int *h = reinterpret_cast<int *>(e->h_counters + kCounters) + 1;
@@ -561,16 +749,86 @@ static int end_call(il_estimator *e)
     return IL_OK;
 }
 
+// Words of examined records per lane: as many as the resident CTAs leave room for.
+template <typename Fits>
+static void widen(int32_t &words, Fits fits)
+{
+    words = kLaneWordsMost;
+    while (words > kLaneWords && !fits()) words >>= 1;
+}
+
 static cudaError_t launch_lane(const il_estimator *e, DesParams p, int64_t ctas, cudaStream_t st)
 {
     const size_t per_sm = (size_t)((ctas + e->num_sms - 1) / e->num_sms);
-    p.lane_words = kLaneWordsMost;
-    p.join_window = kJoinWindowMost;
-    auto smem = [&] { return des_lane_smem(e->S * e->H, e->Bmax, e->lane_slots, p.lane_words, p.cpw, p.n_join, p.join_window); };
-    auto fits = [&] { return smem() <= e->smem_per_cta && (smem() + 1024) * per_sm <= e->smem_per_sm; };
-    while (!fits() && p.n_join > 0 && p.join_window > kJoinWindow) p.join_window >>= 1;
-    while (!fits() && p.lane_words > kLaneWords) p.lane_words >>= 1;
-    return launch_des_lane(p, (int)ctas, smem(), st);
+    auto fits = [&](size_t bytes) { return bytes <= e->smem_per_cta && (bytes + 1024) * per_sm <= e->smem_per_sm; };
+    if (e->join) {
+        p.join_window = kJoinWindowMost;
+        p.lane_words = kLaneWordsMost;
+        auto smem = [&] { return des_join_lane_smem(e->S * e->H, e->Bmax, e->lane_slots, p.lane_words, p.cpw, p.n_join, p.join_window); };
+        while (!fits(smem()) && p.join_window > kJoinWindow) p.join_window >>= 1;
+        while (!fits(smem()) && p.lane_words > kLaneWords) p.lane_words >>= 1;
+        return launch_des_join_lane(p, (int)ctas, smem(), st);
+    }
+    p.lane_ahead = 64;
+    p.lane_stretch = lane_stretch_bytes(p.cpw, p.lane_ahead);
+    widen(p.lane_words, [&] { return fits(lane_smem(e, e->lane_slots, p.lane_words, p.lane_stretch)); });
+    return launch_des_lane(p, nullptr, (int)ctas, lane_smem(e, e->lane_slots, p.lane_words, p.lane_stretch), st);
+}
+
+// A chunk of a pipeline cut into parts: control words and counts cleared, root nodes numbered, then the parts.
+static int enqueue_parts(il_estimator *e, DesParams p, const Plan &pl, char *ws, cudaStream_t st, int64_t *launches)
+{
+    const Shape sh = cut_shape(e, p.n_cand, e->lane_slots);
+    const int64_t grid = std::min<int64_t>(sh.grid, pl.slots / des_lane_warps_per_cta());
+    LaneCut cut = e->cut;
+    const bool feas = p.out_feasible != nullptr;
+    uint32_t *words = reinterpret_cast<uint32_t *>(ws + pl.off_ctl);
+    cut.num_sms = e->num_sms;
+    cut.ctl = words;
+    cut.refs = words + kCtlWords + (size_t)e->n_stream * pl.chunk;
+    int32_t *root_of = reinterpret_cast<int32_t *>(ws + pl.off_root);
+    uint32_t *node_cfg = reinterpret_cast<uint32_t *>(ws + pl.off_node);
+    cut.root_of = root_of; cut.node_cfg = node_cfg;
+    cut.miss = reinterpret_cast<uint32_t *>(root_of + pl.chunk);
+    cut.naps = 16ull * 1024 * 1024 + 64ull * (unsigned long long)e->n;
+    for (int x = 0; x < e->n_stream; x++) {
+        LaneStream &k = cut.stream[x];
+        k.count = words + kCtlWords + (size_t)x * pl.chunk;
+        switch (e->stream_at[x]) {
+        case il_estimator::kAtNode: k.base = reinterpret_cast<uint64_t *>(ws + pl.off_node_rows); k.stride = e->node_elems; break;
+        case il_estimator::kInSlab: k.base = reinterpret_cast<uint64_t *>(p.slab); k.stride = p.slab_stride; break;
+        default: k.base = reinterpret_cast<uint64_t *>(ws + pl.off_extra); k.stride = e->extra_elems; break;
+        }
+    }
+    for (int t = 0; t < cut.n_part; t++) {
+        LanePart &pt = cut.part[t];
+        pt.groups = sh.groups[t]; pt.warps = sh.warps[t];
+        // records without branch bits leave as they are
+        if (pt.out_kind == kOutLeaf && p.rec_bits == 0 && !feas && !e->fork) pt.out_kind = kOutOne;
+        // one store where the two ways are alternatives, told by a bit that the records carry, in streams of one row; two
+        // with fan-out; anything else is looked into record by record
+        const int end = pt.stage[pt.len - 1];
+        const DesParams &b = e->base;
+        const bool asks = b.cbit_a[end] >= 0 || b.cbit_b[end] >= 0;
+        if (pt.out_kind == kOutTwo && (pt.n_leave > 0 || pt.out_b < 0 || (asks && p.rec_bits == 0))) pt.out_kind = kOutAny;
+        if (pt.out_kind == kOutTwo && !e->fork &&
+            (e->stream_at[pt.out_a] != e->stream_at[pt.out_b] || cut.stream[pt.out_b].off < cut.stream[pt.out_a].off))
+            pt.out_kind = kOutAny;
+    }
+    IL_CUDA(cudaMemsetAsync(words, 0, pl.ctl_bytes, st));
+    RootNodeParams rp = {};
+    rp.configs = p.configs; rp.n_cand = p.n_cand; rp.S = e->S; rp.H = e->H; rp.Bmax = e->Bmax; rp.readers = e->root_readers; rp.shared = cut.shared;
+    rp.root_of = root_of; rp.node_cfg = node_cfg; rp.ctl = words; rp.refs = cut.refs; rp.miss = cut.miss;
+    rp.out_feasible = p.out_feasible; rp.status = p.status;
+    IL_CUDA(launch_root_nodes(rp, st));
+    p.lane_ahead = sh.ahead;
+    p.lane_stretch = sh.stretch;
+    const size_t per_sm = (size_t)((grid + e->num_sms - 1) / e->num_sms);
+    auto smem = [&] { return lane_smem(e, e->lane_slots, p.lane_words, p.lane_stretch); };
+    widen(p.lane_words, [&] { return smem() <= e->smem_per_cta && (smem() + 1024) * per_sm <= e->smem_per_sm; });
+    IL_CUDA(launch_des_lane(p, &cut, (int)grid, smem(), st));
+    *launches += 2;
+    return IL_OK;
 }
 
 // Enqueues the simulation of one chunk whose work counter is zero: the kernel the handle uses
@@ -585,9 +843,14 @@ static int enqueue_simulation(il_estimator *e, const DesParams &p, const Plan &p
     // fan-out: the lane kernel keeps per query the largest leaving record, starting from zero
     if (kernel == kSimLane && e->fork)
         IL_CUDA(cudaMemsetAsync(p.slab, 0, (size_t)p.n_cand * p.slab_stride * 8, st));
-    if (kernel == kSimLane) IL_CUDA(launch_lane(e, p, ctas, st));
-    else IL_CUDA(launch_simulation(p, kernel, (int)ctas, e->smem, st));
-    (*launches)++;
+    if (is_cut(e)) {
+        const int rc = enqueue_parts(e, p, pl, ws, st, launches);
+        if (rc) return rc;
+    } else {
+        if (kernel == kSimLane) IL_CUDA(launch_lane(e, p, ctas, st));
+        else IL_CUDA(launch_simulation(p, kernel, (int)ctas, e->smem, st));
+        (*launches)++;
+    }
     if (fb) {
         IL_CUDA(launch_overflow_list(p.ovf, p.n_cand, const_cast<int32_t *>(p.order), e->d_counters, st));
         DesParams q = p;
@@ -1030,7 +1293,7 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
                 const unsigned val = side == 0 ? bp.cval_a[s] : bp.cval_b[s];
                 taken += (bit < 0 || ((bits >> bit) & 1u) == val);
             }
-            if (taken == 0) bp.total_leaving += m;
+            if (taken == 0) { bp.total_leaving += m; e->leaving[s] += m; }
         }
     }
     e->events_per_candidate = 0;
@@ -1093,6 +1356,7 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
     }
     e->cpw = std::max(1, 32 / (S + bp.n_join));
     configure_lane_rings(e);
+    build_parts(e);
     bp.S = S; bp.H = H; bp.Bmax = B; bp.n = (int32_t)n;
     e->smem = (size_t)S * H * B * sizeof(int32_t);
 
@@ -1169,8 +1433,16 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
     e->ctas_per_sm_packed = des_packed_max_ctas_per_sm(false, e->smem);
     e->ctas_per_sm_staged = des_packed_max_ctas_per_sm(true, e->smem);
     for (int k = 0; k < 2; k++) {
-        e->ctas_lane[k] = des_lane_max_ctas_per_sm(des_lane_smem(S * H, B, k == 0 ? 16 : 32, kLaneWords, e->cpw, e->base.n_join, kJoinWindow),
-                                                   e->join);
+        const int slots = k == 0 ? 16 : 32;
+        if (e->join) {
+            e->ctas_lane[k] = des_join_lane_max_ctas_per_sm(des_join_lane_smem(S * H, B, slots, kLaneWords, e->cpw, e->base.n_join, kJoinWindow));
+        } else if (e->cut.n_part > 0) {
+            int most = 1;
+            for (int t = e->cut.shared ? 1 : 0; t < e->cut.n_part; t++) most = std::max(most, 32 / e->cut.part[t].len);
+            e->ctas_lane[k] = std::max(1, des_lane_max_ctas_per_sm(lane_smem(e, slots, kLaneWords, lane_stretch_bytes(std::max(most, kRootGroups), 32)), true));
+        } else {
+            e->ctas_lane[k] = des_lane_max_ctas_per_sm(lane_smem(e, slots, kLaneWords, lane_stretch_bytes(e->cpw, 64)), false);
+        }
     }
     e->ctas_per_sm_lane = e->ctas_lane[1];
     if (e->ctas_per_sm_wide < 1 || e->ctas_per_sm_packed < 1 || e->ctas_per_sm_staged < 1 ||
@@ -1548,35 +1820,55 @@ static int feasible_device(il_estimator *e, const il_stage_config *d_configs, in
     const size_t sb = slot_time_bytes(e, cands_per_slot(e, n_cand));
     const size_t tail_bytes = align_up((size_t)n_cand, 256) + align_up((size_t)n_cand * 4, 256) + 1024;
     if (ws_bytes < tail_bytes + (size_t)wpc * sb) return IL_ERR_NOMEM;
-    int64_t slots = std::min<int64_t>(wanted_slots(e, n_cand, e->lane_slots), (int64_t)((ws_bytes - tail_bytes) / sb)) / wpc * wpc;
-    if (slots < wpc) return IL_ERR_NOMEM;
-    const size_t off_ovf = align_up((size_t)slots * sb, 256);
+    Plan pl;
+    int64_t slots = 0;
+    if (is_cut(e)) {
+        pl.feas = true;
+        pl.slab = e->slab_streams;
+        if (!make_plan(e, ws_bytes - tail_bytes, n_cand, pl)) return IL_ERR_NOMEM;
+        slots = pl.slots;
+    } else {
+        pl.chunk = n_cand;
+        slots = std::min<int64_t>(wanted_slots(e, n_cand, e->lane_slots), (int64_t)((ws_bytes - tail_bytes) / sb)) / wpc * wpc;
+        if (slots < wpc) return IL_ERR_NOMEM;
+    }
+    const size_t off_ovf = is_cut(e) ? align_up(ws_bytes - tail_bytes, 256) : align_up((size_t)slots * sb, 256);
     const size_t off_order = off_ovf + align_up((size_t)n_cand, 256);
     rc = ensure_events(e, 4);
     if (rc) return rc;
 
-    DesParams p = e->base;
-    p.configs = d_configs;
-    p.n_cand = n_cand;
-    p.lane_ws = reinterpret_cast<uint64_t *>(ws);
-    p.ovf = reinterpret_cast<uint8_t *>(ws + off_ovf);
-    p.iter_limit = e->iter_limit;
-    p.lane_slots = e->lane_slots;
-    p.cpw = (int32_t)cands_per_slot(e, n_cand);
-    p.out_feasible = d_out_feasible;
-    // latency > objective is tested on time fields shifted by qbits: keep the objective in that range
-    // (latencies are at least 1 and every reachable time is below 2^(63 - qbits))
-    p.slo_us = std::min<int64_t>(std::max<int64_t>(slo_us, 0), INT64_C(1) << (62 - p.qbits - p.rec_bits));
-    p.miss_allow = (uint32_t)(e->n - (99 * e->n + 99) / 100);
-    if (e->lane_wrap) IL_CUDA(cudaMemsetAsync(p.ovf, 0, (size_t)n_cand, st));
-    const int64_t groups = (n_cand + p.cpw - 1) / p.cpw;
-    const int64_t ctas = std::min<int64_t>(slots / wpc, (groups + wpc - 1) / wpc);
+    const int64_t n_chunks = (n_cand + pl.chunk - 1) / pl.chunk;
+    if (e->lane_wrap) IL_CUDA(cudaMemsetAsync(ws + off_ovf, 0, (size_t)n_cand, st));
     IL_CUDA(cudaEventRecord(e->events[0], st));
-    IL_CUDA(launch_lane(e, p, ctas, st));
+    int64_t launches = 0;
+    for (int64_t lo = 0; lo < n_cand; lo += pl.chunk) {
+        DesParams p = e->base;
+        if (is_cut(e)) p = chunk_params(e, pl, ws, d_configs + lo * e->S, std::min(pl.chunk, n_cand - lo));
+        p.configs = d_configs + lo * e->S;
+        p.n_cand = std::min(pl.chunk, n_cand - lo);
+        p.lane_ws = reinterpret_cast<uint64_t *>(ws);
+        p.ovf = reinterpret_cast<uint8_t *>(ws + off_ovf) + lo;
+        p.iter_limit = e->iter_limit;
+        p.lane_slots = e->lane_slots;
+        p.cpw = (int32_t)cands_per_slot(e, n_cand);
+        p.lanes_per_slot = is_cut(e) ? 32 : p.cpw * e->S;
+        p.out_feasible = d_out_feasible + lo;
+        // latency > objective is tested on time fields shifted by qbits: keep the objective in that range
+        // (latencies are at least 1 and every reachable time is below 2^(63 - qbits))
+        p.slo_us = std::min<int64_t>(std::max<int64_t>(slo_us, 0), INT64_C(1) << (62 - p.qbits - p.rec_bits));
+        p.miss_allow = (uint32_t)(e->n - (99 * e->n + 99) / 100);
+        if (is_cut(e)) {
+            rc = enqueue_parts(e, p, pl, ws, st, &launches);
+            if (rc) return rc;
+        } else {
+            const int64_t groups = (n_cand + p.cpw - 1) / p.cpw;
+            IL_CUDA(launch_lane(e, p, std::min<int64_t>(slots / wpc, (groups + wpc - 1) / wpc), st));
+            launches++;
+        }
+    }
     IL_CUDA(cudaEventRecord(e->events[1], st));
-    int64_t launches = 1;
     if (e->lane_wrap) {
-        IL_CUDA(launch_overflow_list(p.ovf, n_cand, reinterpret_cast<int32_t *>(ws + off_order), e->d_counters, st));
+        IL_CUDA(launch_overflow_list(reinterpret_cast<uint8_t *>(ws + off_ovf), n_cand, reinterpret_cast<int32_t *>(ws + off_order), e->d_counters, st));
         launches++;
     }
     e->copy_dst = h_out; e->copy_src = d_out_feasible; e->copy_bytes = (size_t)n_cand;
@@ -1591,7 +1883,7 @@ static int feasible_device(il_estimator *e, const il_stage_config *d_configs, in
     stats.query_events = n_cand * e->events_per_candidate;
     stats.batches = (int64_t)e->h_counters[1];
     stats.algorithmic_ops = (int64_t)e->h_counters[2];
-    stats.chunks = 1;
+    stats.chunks = n_chunks;
     stats.sim_ms = ms;
     stats.total_ms = ms;
     stats.fallback_candidates = (int64_t)e->h_counters[3];

@@ -81,6 +81,9 @@ struct DesParams {
     int32_t lane_words;           // words of examined records a lane keeps in shared memory (a power of two, at least 64)
     int32_t smem_skip;            // test knob: bytes left unused where shared memory starts (a multiple of 16, at most 8192)
     int32_t lane_wrap;            // the rings are shorter than the longest stream
+    int32_t lane_ahead;           // records of its arrival stream a group has in shared memory (32 or 64)
+    int32_t lane_stretch;         // bytes of that for all groups of a warp
+    int32_t lanes_per_slot;       // spill rings of a warp slot
     // lane kernel, joins: join_stage[0 .. n_join) are the stages with two incoming edges, join_no[s] their number
     int32_t n_join;
     int8_t  join_stage[IL_MAX_STAGES], join_no[IL_MAX_STAGES];
@@ -102,6 +105,58 @@ struct DesParams {
     const unsigned long long *n_cand_dev;   // if set, the number of candidates is read from here (device
                                             // memory) instead of n_cand: the list in `order` was built on the device
 };
+
+// ---- Pipelines with branch points on the lane kernel: cut into parts (des_lane_kernel.cu) -------------------------
+// What one part passes to another: a row of records per candidate, or per root node where the root writes it, and the
+// count of those that are there.
+struct LaneStream {
+    uint64_t *base;
+    uint32_t *count;              // [rows]
+    int64_t stride;               // records from row to row
+    int32_t off, len;             // the stream's place in a row
+    int32_t by_node;
+};
+// What happens to the records of a part's last stage: all go one way (a stream, or out where records are plain anyway); all
+// leave the pipeline; either of two streams of one row, by a branch bit that the records carry; any other two ways.
+constexpr int kOutOne = 0, kOutLeaf = 1, kOutTwo = 2, kOutAny = 3;
+struct LanePart {
+    int8_t len;                   // a chain of so many stages
+    int8_t stage[IL_MAX_STAGES];
+    int8_t out_kind;
+    int8_t in, out_a, out_b;      // streams; -1: the trace, none
+    int32_t groups, warps;        // groups of lanes per warp, warps planned
+    int32_t n_leave, leave_off;   // records that leave after the last stage, and where they go in a slab row
+    int64_t n_out;                // records that come out of the last stage, all ways together
+};
+struct LaneCut {
+    int32_t n_part;               // part 0 is the root stage
+    int32_t shared;               // simulated once per distinct configuration (root node); 0: per candidate, whose number is its node's
+    int32_t num_sms;
+    LanePart part[IL_MAX_STAGES];
+    LaneStream stream[IL_MAX_STAGES];
+    uint32_t *ctl;                // control words, below; zero at launch
+    const int32_t *root_of;       // [n_cand] root node of a candidate, -1: its configuration is out of range
+    const uint32_t *node_cfg;     // hw | max batch << 8 | replicas << 16
+    uint32_t *refs;               // feasibility only: groups that will still read a node's streams
+    uint32_t *miss;               // feasibility only: [n_cand] misses so far
+    unsigned long long naps;      // bound on the sleeps of a warp
+};
+constexpr int kRootGroups = 16;   // root nodes per warp
+constexpr uint32_t kCtlNodes = 0, kCtlOrder = 1, kCtlTicket = 2, kCtlWork = 16, kCtlSms = 1024, kCtlSlot = 64,
+                   kCtlRole = kCtlSlot + kCtlSms, kCtlWords = kCtlRole + kCtlSms;
+struct RootNodeParams {
+    const il_stage_config *configs;
+    int64_t n_cand;
+    int32_t S, H, Bmax, readers;  // readers: parts that read the root's streams
+    int32_t shared;
+    int32_t *root_of;
+    uint32_t *node_cfg, *ctl, *refs, *miss;
+    uint8_t *out_feasible;        // set to 1 (0: out of range) with feasibility only, else nullptr
+    int *status;
+};
+cudaError_t launch_root_nodes(const RootNodeParams &p, cudaStream_t stream);
+int lane_root_sms(int64_t nodes, int num_sms);        // SMs set aside for so many root nodes
+int lane_stretch_bytes(int groups, int ahead);
 
 struct SelectParams {
     int64_t *slab;                // [n_cand][slab_stride]: latencies, or packed (finish, query) records
@@ -139,17 +194,20 @@ cudaError_t launch_des_packed(const DesParams &p, bool staged, int grid, size_t 
 int des_packed_max_ctas_per_sm(bool staged, size_t smem);
 int trace_tile_records();     // the packed trace is padded to a multiple of this many records
 // lane-parallel kernel: one lane per (candidate, stage); smem from des_lane_smem
-cudaError_t launch_des_lane(const DesParams &p, int grid, size_t smem, cudaStream_t stream);
+cudaError_t launch_des_lane(const DesParams &p, const LaneCut *cut, int grid, size_t smem, cudaStream_t stream);
 int des_lane_warps_per_cta();
-// ring_slots: 16 or 32 batch ring positions per lane; ring_words: words of examined records (a power of two);
-// cpw candidates per warp with so many joins each, whose streams keep `window` records
-size_t des_lane_smem(int table_rows, int Bmax, int ring_slots, int ring_words, int cpw, int joins, int window);
-int des_lane_max_ctas_per_sm(size_t smem, bool joins);     // of the instantiation for pipelines with joins, or of the others
+// ring_slots: 16 or 32 batch ring positions per lane; ring_words: words of examined records (a power of two); stretch: bytes
+// of a warp's arrival streams
+size_t des_lane_smem(int table_rows, int Bmax, int ring_slots, int ring_words, int stretch);
+int des_lane_max_ctas_per_sm(size_t smem, bool cut);
+// the same for pipelines with joins: cpw candidates per warp with so many joins each, whose streams keep `window` records
+cudaError_t launch_des_join_lane(const DesParams &p, int grid, size_t smem, cudaStream_t stream);
+size_t des_join_lane_smem(int table_rows, int Bmax, int ring_slots, int ring_words, int cpw, int joins, int window);
+int des_join_lane_max_ctas_per_sm(size_t smem);
 enum SimKernel { kSimWide = 0, kSimPacked = 1, kSimPackedStaged = 2, kSimLane = 3 };
 inline cudaError_t launch_simulation(const DesParams &p, int kernel, int grid, size_t smem,
                                      cudaStream_t stream)
 {
-    if (kernel == kSimLane) return launch_des_lane(p, grid, smem, stream);
     if (kernel == kSimWide) return launch_des(p, grid, smem, stream);
     return launch_des_packed(p, kernel == kSimPackedStaged, grid, smem, stream);
 }
