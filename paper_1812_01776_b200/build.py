@@ -9,7 +9,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libil_estimator.so")
 LIB_CHECKED = os.path.join(HERE, "libil_estimator_checked.so")     # the same sources with -DIL_CHECKED
-SOURCES = ["des_kernel.cu", "des_packed_kernel.cu", "des_lane_kernel.cu", "des_join_lane_kernel.cu", "select_kernel.cu", "order_kernel.cu", "envelope_kernel.cu", "prefix_kernel.cu", "il_api.cu", "il_static.cu"]
+SOURCES = ["des_kernel.cu", "des_packed_kernel.cu", "des_lane_kernel.cu", "select_kernel.cu", "order_kernel.cu", "envelope_kernel.cu", "prefix_kernel.cu", "il_api.cu", "il_static.cu"]
 HEADERS = [os.path.join(CSRC, "il_internal.h"), os.path.join(ROOT, "include", "il_estimator.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-shared", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden"]

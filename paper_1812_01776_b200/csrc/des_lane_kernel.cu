@@ -126,6 +126,14 @@ __device__ __forceinline__ void sts32(uint32_t a, uint32_t v) { asm volatile("st
 
 // The same under a predicate: a lane's steps
 // are straight-line code (a branch costs the warp more than the few instructions it would skip).
+__device__ __forceinline__ void sts64_if(bool c, uint32_t a, uint64_t v)
+{
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p st.shared.u64 [%1], %2; }" ::"r"((uint32_t)c), "r"(a), "l"(v) : "memory");
+}
+__device__ __forceinline__ void stg64_if(bool c, uint64_t *a, uint64_t v)
+{
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p st.global.u64 [%1], %2; }" ::"r"((uint32_t)c), "l"(a), "l"(v) : "memory");
+}
 __device__ __forceinline__ void stg32_if(bool c, uint32_t *a, uint32_t v)
 {
     asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p st.global.u32 [%1], %2; }" ::"r"((uint32_t)c), "l"(a), "r"(v) : "memory");
@@ -230,6 +238,149 @@ __device__ int lane_first_part(const LaneCut &cut, bool for_roots)
     return t0 + (int)(w % (uint32_t)(cut.n_part - t0));
 }
 
+// The merge of a join's two incoming streams, one lane per candidate: records in time order, at equal times the first
+// parent's first; a query that follows both edges passes with the later of its two records.  A record can be taken when
+// what comes next on the other side is known.  A bit per query tells whether its first record has been taken.  The bits'
+// words are in a small write-back cache in shared memory, `entries` per lane (where other parts keep words of examined
+// records); queries come in nearly in order, so a word is new when it is first needed, and one that had to make room
+// goes to global memory.  Bound by the latency of an iteration, a record each: the two heads from shared memory, their
+// order, the query's word: about 260 cycles.  511 candidates of a diamond, 50,000 queries: 53 ms with the merge in the stages'
+// loop, 14.1 as a part (29 with branches for the words, 23.3 with the words in global memory alone).
+__device__ __noinline__ void lane_merge(const DesParams &p, const LaneCut &cut, int part, uint32_t tbw, uint32_t ahead, uint32_t cache, uint32_t entries,
+                                        unsigned long long &naps, uint32_t &quit)
+{
+    const unsigned full = 0xffffffffu;
+    const LanePart &pt = cut.part[part];
+    const LaneStream &xa = cut.stream[pt.in], &xb = cut.stream[pt.in_b], &xo = cut.stream[pt.out_a];
+    const int lane = threadIdx.x & 31, s = pt.stage[0], qi = p.qbits, rb = p.rec_bits;
+    const uint32_t qmask = (1u << (qi + rb)) - 1u, imask = (1u << qi) - 1u;
+    const uint32_t window = ahead, wmask = window - 1u, its = window / 2u;
+    const uint32_t wa = tbw + (uint32_t)min(lane, pt.groups - 1) * stretch_bytes(2 * (int)ahead), wb = wa + window * 8u;
+    const uint32_t na = (uint32_t)xa.len, nb = (uint32_t)xb.len;
+    const bool always = p.any_bits == 0;        // no conditional edges: every query comes from both sides
+    // (a lane may also wait while others of its warp have records)
+    const unsigned long long limit = (p.iter_limit ? p.iter_limit : (8ull * (unsigned)p.n * (unsigned)(p.S + 1) + 4096ull) * 4ull) / its + 1ull;
+    unsigned long long spent = 0;
+    bool more = lane < pt.groups, has = false, dead = false;
+    uint32_t c = 0, ia = 0, ib = 0, fed_a = 0, fed_b = 0, have_a = 0, have_b = 0, tail = 0, pub = 0;
+    const uint64_t *src_a = nullptr, *src_b = nullptr;
+    const uint32_t *count_a = nullptr, *count_b = nullptr;
+    uint64_t *out = nullptr;
+    uint32_t *count = nullptr, *seen = nullptr;
+    uint32_t seen_new = 0;      // words from here on have not been touched
+    const uint32_t row0 = cache + (uint32_t)lane * 8u, emask = entries - 1u;
+
+    // copies what is there of a stream into its window, up to `window` records from i on
+    auto feed = [&](const uint64_t *src, uint32_t w, uint32_t i, uint32_t have, uint32_t n, uint32_t &fed) {
+        uint32_t to = min(i + window, have);
+        if (to != n) to &= ~1u;
+        if (to > fed && (to & 1u)) sts64(w + ((to - 1u) & wmask) * 8u, ldg64_shared(src + (to - 1u)));
+        for (uint32_t k = fed; k + 1u < to; k += 2u) copy16(w + (k & wmask) * 8u, src + k);
+        fed = max(fed, to);
+    };
+    for (uint32_t look = 1u;; look++) {
+        copies_done();
+        uint32_t in_a = fed_a, in_b = fed_b;             // what has arrived
+        if (has && spent++ == limit) {
+            atomicCAS(p.status, 0, IL_ERR_ITER_LIMIT);
+            atomicOr(&p.counters[5], 1ull);
+            dead = true;
+        }
+        if (has && (dead || quit != 0u || (ia == na && ib == nb))) {
+            __threadfence();
+            const bool ok = ia == na && ib == nb && !dead;
+            if (ok && tail != (uint32_t)xo.len) { atomicCAS(p.status, 0, IL_ERR_ITER_LIMIT); atomicOr(&p.counters[5], 2ull); }
+            stg32_shared(count, ok ? tail : kDead);
+            has = false;
+        }
+        if (!has && more) {
+            c = atomicAdd(cut.ctl + kCtlWork + part, 1u);
+            more = c < (uint32_t)p.n_cand && quit == 0u;
+            if (more) {
+                const int32_t of = cut.root_of[c];
+                auto row = [&](const LaneStream &x) { return x.by_node ? (uint32_t)max(of, 0) : c; };
+                has = true; dead = of < 0;
+                ia = 0; ib = 0; fed_a = 0; fed_b = 0; have_a = 0; have_b = 0; tail = 0; pub = 0;
+                in_a = 0; in_b = 0; spent = 0; seen_new = 0;
+                for (uint32_t k = 0; k < entries; k++) sts64(row0 + k * 256u, kInf);      // word number (none) << 32 | word
+                src_a = xa.base + (int64_t)row(xa) * xa.stride + xa.off; count_a = xa.count + row(xa);
+                src_b = xb.base + (int64_t)row(xb) * xb.stride + xb.off; count_b = xb.count + row(xb);
+                out = xo.base + (int64_t)row(xo) * xo.stride + xo.off; count = xo.count + row(xo);
+                seen = cut.seen + ((int64_t)c * cut.n_join + pt.join_no) * cut.seen_words;
+                if (dead) { stg32_shared(count, kDead); has = false; }
+            }
+        }
+        if (!__any_sync(full, has || more)) break;
+        auto starving = [&](uint32_t i, uint32_t have, uint32_t n) { return have != n && have - i < its; };
+        auto idle = [&]() { return !has || dead || starving(ia, have_a, na) || starving(ib, have_b, nb); };
+        const bool nothing = __all_sync(full, idle());
+        if ((look & 7u) == 0u || nothing) {
+            if (has && tail != pub) { __threadfence(); stg32_shared(count, tail); pub = tail; }
+        }
+        if ((look & 3u) == 0u || nothing) {
+            auto ask = [&](const uint32_t *from, uint32_t i, uint32_t &have, uint32_t n) {
+                if (have == n || have - i >= 2u * window) return;
+                const uint32_t w = ldg32_acquire(from);
+                dead |= w == kDead;
+                if (w != kDead) have = max(have, w);
+            };
+            if (has) { ask(count_a, ia, have_a, na); ask(count_b, ib, have_b, nb); }
+            if (nothing && __all_sync(full, idle() && !dead)) {
+                __nanosleep(500);
+                if (naps-- == 0ull) { atomicCAS(p.status, 0, IL_ERR_ITER_LIMIT); atomicOr(&p.counters[5], 1ull); }
+                quit = __any_sync(full, *reinterpret_cast<volatile int *>(p.status) != 0) ? 1u : 0u;
+                // (a side may have less than a step's records left for good while the other has ended or waits for it)
+            }
+        }
+        if (has && !dead) {
+            feed(src_a, wa, ia, have_a, na, fed_a);
+            feed(src_b, wb, ib, have_b, nb, fed_b);
+        }
+        const uint32_t la = has && !dead ? in_a : ia, lb = has && !dead ? in_b : ib;
+        uint64_t va = lds64(wa + (ia & wmask) * 8u), vb = lds64(wb + (ib & wmask) * 8u);
+        // straight-line but for words that are not simply the next ones
+        auto step = [&](auto every) {
+            const uint64_t ha = ia == na ? kInf : va, hb = ib == nb ? kInf : vb;
+            const bool from_a = (ha | qmask) <= (hb | qmask);
+            const uint64_t rec = from_a ? ha : hb;
+            const uint32_t low = (uint32_t)rec & qmask, qid = low & imask, w = qid >> 5, mine = 1u << (qid & 31u), at = row0 + (w & emask) * 256u;
+            uint64_t e = lds64(at);
+            const uint32_t known = (ia < la || ia == na) && (ib < lb || ib == nb) && (int64_t)rec >= 0 && IL_IN_RANGE(qid, p.n, p.status) ? 1u : 0u;
+            ia += from_a ? known : 0u;
+            ib += from_a ? 0u : known;
+            va = lds64(wa + (ia & wmask) * 8u);
+            vb = lds64(wb + (ib & wmask) * 8u);
+            uint32_t both = known;
+            if constexpr (!decltype(every)::value) {
+                const uint32_t bits = rb > 0 ? low >> qi : known ? p.bits[qid] : 0u;
+                both &= (uint32_t)(p.join_both[s][bits >> 6] >> (bits & 63u)) & 1u;
+            }
+            const uint32_t old = (uint32_t)(e >> 32);
+            const uint32_t other = both != 0u && old != w ? 1u : 0u;
+            stg32_if(other != 0u && old != ~0u && IL_IN_RANGE(old, cut.seen_words, p.status), seen + old, (uint32_t)e);
+            uint32_t word = other ? 0u : (uint32_t)e;
+            if (other != 0u && w != seen_new) {
+                if (w < seen_new && IL_IN_RANGE(w, cut.seen_words, p.status)) word = seen[w];
+#pragma unroll 1
+                for (; seen_new < w; seen_new++)         // passed over: it may come later
+                    if (IL_IN_RANGE(seen_new, cut.seen_words, p.status)) seen[seen_new] = 0u;
+            }
+            seen_new = other ? max(seen_new, w + 1u) : seen_new;
+            sts64_if(both != 0u, at, (uint64_t)w << 32 | (word ^ mine));
+            const uint32_t passes = both != 0u ? (word >> (qid & 31u)) & 1u : known;
+            stg64_if(passes != 0u && IL_IN_RANGE(tail, xo.len, p.status), out + tail, rec);
+            tail += passes;
+        };
+        if (always) {
+#pragma unroll 2
+            for (uint32_t k = 0; k < its; k++) step(std::true_type{});
+        } else {
+#pragma unroll 1
+            for (uint32_t k = 0; k < its; k++) step(std::false_type{});
+        }
+    }
+}
+
 }  // namespace
 
 // FEAS: feasibility only (Section 4.3, "Feasible"): leaving queries are compared with the objective as
@@ -256,7 +407,8 @@ __device__ int lane_first_part(const LaneCut &cut, bool for_roots)
 //       2,048 candidates of 6 stages, 100,000 queries 22.7 -> 17.7 ms.  Up to a warp per scheduler the root is what
 //       takes the time (250 cycles an iteration and 40 for its turns), beyond that the ALU pipe.
 // FORK: fan-out (with CUT) -- a query goes down every edge whose condition holds, a copy that finds none leaves, and
-//       the slab keeps per query the record of the copy that left last.
+//       the slab keeps per query the record of the copy that left last.  Joins: the streams of a stage's two incoming edges
+//       are merged by a part of its own (lane_merge) before the part that begins with the stage.
 template <bool FEAS, bool CUT, bool FORK>
 __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCut &cut, unsigned char *smem_raw)
 {
@@ -338,6 +490,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
     int part = CUT ? lane_first_part(cut, for_roots) : 0;
     for (int parts_left = CUT ? cut.n_part : 1; parts_left > 0; parts_left--, part = CUT && part + 1 == cut.n_part ? 0 : part + 1) {
     const LanePart *pt = CUT ? cut.part + part : nullptr;
+    if (FORK && pt->len == 0) { lane_merge(p, cut, part, tbw, ahead, qb0 + (uint32_t)wid * nq * 128u, nq / 2u, naps, quit); continue; }
     const int L = CUT ? pt->len : p.S;                // lanes of a candidate
     const bool per_node = CUT && part == 0 && cut.shared;      // the items are root nodes, not candidates
     const uint32_t n_items = per_node ? cut.ctl[kCtlNodes] : (uint32_t)p.n_cand;
@@ -497,7 +650,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
             const uint32_t span = i - low;
             if (!(is & kSpill) && span > (uint32_t)(nq - kTurn - 2)) {
 #pragma unroll 1
-                for (uint32_t k = low; k != i; k++)
+                for (uint32_t k = i - min(span, gmask + 1u); k != i; k++)
                     if (IL_IN_RANGE(k & gmask, gmask + 1ull, p.status))
                         spill_ring[k & gmask] = lds32(qb + ((k & (nq - 1u)) << 7));
                 is |= kSpill;

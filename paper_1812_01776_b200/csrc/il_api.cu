@@ -70,7 +70,7 @@ struct il_estimator {
     // of lanes per candidate), where each stream lies, and how many records a root node and a candidate need for them
     LaneCut cut = {};
     int n_stream = 0;
-    enum Place : uint8_t { kAtNode, kInSlab, kExtra } stream_at[IL_MAX_STAGES] = {};
+    enum Place : uint8_t { kAtNode, kInSlab, kExtra } stream_at[3 * IL_MAX_STAGES] = {};
     bool slab_streams = false;
     int64_t node_elems = 0, extra_elems = 0;
     int root_readers = 0;
@@ -124,7 +124,7 @@ struct Plan {
     bool slab = true;        // rows of the slab are needed
     // pipelines cut into parts: root nodes at most, control words and counts, what the host prepares, streams
     int64_t nodes = 0;
-    size_t off_ctl = 0, ctl_bytes = 0, off_root = 0, off_node = 0, off_node_rows = 0, off_extra = 0;
+    size_t off_ctl = 0, ctl_bytes = 0, off_root = 0, off_node = 0, off_node_rows = 0, off_extra = 0, off_seen = 0;
 };
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -132,8 +132,6 @@ inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 // Words of examined records a lane keeps in shared memory before it spills: this many where the grid needs every
 // resident CTA, more where it leaves shared memory unused.
 constexpr int kLaneWords = 64, kLaneWordsMost = 256;
-// Records of a join's incoming streams kept there, likewise.
-constexpr int kJoinWindow = 64, kJoinWindowMost = 512;
 
 bool use_packed(const il_estimator *e)
 {
@@ -187,12 +185,11 @@ bool looks_for_prefixes(const il_estimator *e, int64_t n_cand)
     return n_cand >= kShareMinCandidates && n_cand > wave;
 }
 
-// Stream memory of a slot that holds cps candidates.  Lane kernel: a spill ring for every lane in use, and for joins the
-// bits of the queries of which one input has come in and the incoming streams.
+// Stream memory of a slot that holds cps candidates.  Lane kernel: a spill ring for every lane in use.
 size_t slot_time_bytes(const il_estimator *e, int64_t cps)
 {
     if (is_cut(e)) return (size_t)32 * 4 << e->lane_ring_log2;
-    return is_lane(e) ? (size_t)cps * (e->S + e->base.n_join) * 4 << e->lane_ring_log2 : (size_t)e->slot_elems * 8;
+    return is_lane(e) ? (size_t)cps * e->S * 4 << e->lane_ring_log2 : (size_t)e->slot_elems * 8;
 }
 // Root nodes that so many candidates can have.
 int64_t most_nodes(const il_estimator *e, int64_t n_cand)
@@ -206,7 +203,7 @@ struct Shape {
     int ctas = 1;
     int64_t grid = 1;
     int ahead = 64, stretch = 0;
-    int groups[IL_MAX_STAGES] = {}, warps[IL_MAX_STAGES] = {};
+    int groups[2 * IL_MAX_STAGES] = {}, warps[2 * IL_MAX_STAGES] = {};
 };
 
 size_t lane_smem(const il_estimator *e, int lane_slots, int words, int stretch)
@@ -226,7 +223,7 @@ Shape cut_shape(const il_estimator *e, int64_t n_cand, int lane_slots)
     auto warps_with = [&](int most) {
         int64_t all = 0;
         for (int t = t0; t < cut.n_part; t++) {
-            sh.groups[t] = std::min(most, 32 / cut.part[t].len);
+            sh.groups[t] = std::min(most, cut.part[t].len > 0 ? 32 / cut.part[t].len : 16);      // (a merge has two stretches)
             sh.warps[t] = (int)std::min<int64_t>((n_cand + sh.groups[t] - 1) / sh.groups[t], 1 << 24);
             all += sh.warps[t];
         }
@@ -234,7 +231,7 @@ Shape cut_shape(const il_estimator *e, int64_t n_cand, int lane_slots)
     };
     auto stretch_fits = [&](int ctas) {
         int most = (int)std::min<int64_t>(kRootGroups, nodes);
-        for (int t = t0; t < cut.n_part; t++) most = std::max(most, sh.groups[t]);
+        for (int t = t0; t < cut.n_part; t++) most = std::max(most, sh.groups[t] * (cut.part[t].len > 0 ? 1 : 2));
         for (sh.ahead = 64; sh.ahead >= 32; sh.ahead >>= 1) {
             sh.stretch = lane_stretch_bytes(most, sh.ahead);
             const size_t bytes = lane_smem(e, lane_slots, kLaneWords, sh.stretch);
@@ -259,24 +256,25 @@ Shape cut_shape(const il_estimator *e, int64_t n_cand, int lane_slots)
     sh.grid = (int64_t)e->num_sms * sh.ctas;
     const int64_t room = sms * 4 * sh.ctas;
     if (need > room) {      // more than fit at once: warps by the work of the parts
+        auto work = [&](int t) {
+            const LanePart &pt = cut.part[t];
+            const int64_t records = pt.len > 0 ? e->visits[pt.stage[0]] : cut.stream[pt.in].len + (int64_t)cut.stream[pt.in_b].len;
+            return (double)sh.warps[t] * std::max<int64_t>(1, records);
+        };
         double all = 0.0;
-        for (int t = t0; t < cut.n_part; t++) all += (double)sh.warps[t] * std::max<int64_t>(1, e->visits[cut.part[t].stage[0]]);
-        for (int t = t0; t < cut.n_part; t++)
-            sh.warps[t] = std::max(1, (int)((double)room * sh.warps[t] * std::max<int64_t>(1, e->visits[cut.part[t].stage[0]]) / all));
+        for (int t = t0; t < cut.n_part; t++) all += work(t);
+        for (int t = t0; t < cut.n_part; t++) sh.warps[t] = std::max(1, (int)(room * work(t) / all));
     }
     return sh;
 }
 
-size_t slot_seen_bytes(const il_estimator *e, int64_t cps) { return (size_t)cps * e->base.n_join * e->base.join_seen_words * 4; }
-size_t slot_qid_bytes(const il_estimator *e, int64_t cps)
-{
-    return is_lane(e) ? slot_seen_bytes(e, cps) + (size_t)cps * e->base.join_elems * 8 : (size_t)e->slot_elems * 4;
-}
-size_t slot_bytes(const il_estimator *e, int64_t cps) { return slot_time_bytes(e, cps) + slot_qid_bytes(e, cps); }
-// slab row, order entry, overflow mark; cut: streams of its own, counts, root node, misses
+size_t slot_qid_bytes(const il_estimator *e) { return is_lane(e) ? 0 : (size_t)e->slot_elems * 4; }
+size_t slot_bytes(const il_estimator *e, int64_t cps) { return slot_time_bytes(e, cps) + slot_qid_bytes(e); }
+size_t seen_bytes(const il_estimator *e) { return (size_t)e->cut.n_join * e->cut.seen_words * 4; }      // of a candidate, all its joins
+// slab row, order entry, overflow mark; cut: streams of its own, joins' bits, counts, root node, misses
 size_t cand_bytes(const il_estimator *e, bool slab)
 {
-    return (slab ? (size_t)e->n_pad * 8 : 0) + 5 + (is_cut(e) ? (size_t)e->extra_elems * 8 + (size_t)e->n_stream * 4 + 8 : 0);
+    return (slab ? (size_t)e->n_pad * 8 : 0) + 5 + (is_cut(e) ? (size_t)e->extra_elems * 8 + seen_bytes(e) + (size_t)e->n_stream * 4 + 8 : 0);
 }
 size_t node_bytes(const il_estimator *e) { return (size_t)e->node_elems * 8 + 8; }      // a root node's streams, configuration, readers
 bool lane_fallback(const il_estimator *e) { return is_lane(e) && e->lane_wrap; }
@@ -307,7 +305,7 @@ size_t layout(const il_estimator *e, Plan &pl)
 {
     size_t off = 0;
     pl.off_time = off; off = align_up(off + (size_t)pl.slots * slot_time_bytes(e, pl.cps), 256);
-    pl.off_qid = off;  off = align_up(off + (size_t)pl.slots * slot_qid_bytes(e, pl.cps), 256);
+    pl.off_qid = off;  off = align_up(off + (size_t)pl.slots * slot_qid_bytes(e), 256);
     pl.off_slab = off; off = align_up(off + (pl.slab ? (size_t)pl.chunk * e->n_pad * 8 : 0), 256);
     pl.off_order = off; off = align_up(off + (size_t)pl.chunk * 4, 256);
     pl.off_ovf = off;  off = align_up(off + (size_t)pl.chunk, 256);
@@ -320,6 +318,7 @@ size_t layout(const il_estimator *e, Plan &pl)
         pl.off_node = off;      off = align_up(off + (size_t)pl.nodes * 4, 256);
         pl.off_node_rows = off; off = align_up(off + (size_t)pl.nodes * e->node_elems * 8, 256);
         pl.off_extra = off;     off = align_up(off + (size_t)pl.chunk * e->extra_elems * 8, 256);
+        pl.off_seen = off;      off = align_up(off + (size_t)pl.chunk * seen_bytes(e), 256);
     }
     pl.total = off;
     return off;
@@ -496,9 +495,9 @@ void configure_lane_rings(il_estimator *e)
     e->base.lane_wrap = e->lane_wrap ? 1 : 0;
 }
 
-// Cuts a pipeline with branch points into parts: the root stage, and chains of stages that begin behind the root or behind a
-// branch.  Part t >= 1 reads stream t - 1.  A part that nothing follows reads from the slab region that its records leave
-// to (unless the root has written them, or several parts share a row: fan-out).
+// Cuts a pipeline with branch points into parts: the root stage, and chains of stages that begin behind the root, behind a
+// branch or with a join, in front of which its two incoming streams are merged.  A part that nothing follows reads from the
+// slab region that its records leave to (unless the root has written them, or several parts share a row: fan-out).
 void build_parts(il_estimator *e)
 {
     const DesParams &b = e->base;
@@ -507,47 +506,79 @@ void build_parts(il_estimator *e)
     auto two_ways = [&](int s) { return b.child_b[s] >= 0 || (b.child_a[s] >= 0 && b.cbit_a[s] >= 0); };
     bool any = false;
     for (int s = 0; s < S; s++) any |= two_ways(s);
-    if (!any || e->join) return;
+    if (!any) return;
     cut.shared = e->leaving[0] == 0 ? 1 : 0;      // (records that leave there belong in every candidate's row)
+    cut.seen_words = (int32_t)((e->n + 31) / 32);
     auto even = [](int64_t v) { return (v + 1) / 2 * 2; };
     int part_of[IL_MAX_STAGES] = {};
     int64_t exit_off[IL_MAX_STAGES + 1] = {};
+    int8_t way[IL_MAX_STAGES][2];                 // the stream of a stage's first and second way out
+    for (int s = 0; s < S; s++) way[s][0] = way[s][1] = -1;
+    auto place = [&](int64_t len, bool from_root, bool leaves, int64_t leave_off) {
+        LaneStream &x = cut.stream[e->n_stream];
+        x.len = (int32_t)len;
+        x.by_node = from_root;
+        if (from_root) {
+            e->stream_at[e->n_stream] = il_estimator::kAtNode;
+            x.off = (int32_t)e->node_elems; e->node_elems += even(len);
+            e->root_readers++;
+        } else if (leaves && !e->fork) {
+            e->stream_at[e->n_stream] = il_estimator::kInSlab;
+            x.off = (int32_t)leave_off;
+            e->slab_streams = true;
+        } else {
+            e->stream_at[e->n_stream] = il_estimator::kExtra;
+            x.off = (int32_t)e->extra_elems; e->extra_elems += even(len);
+        }
+        return (int8_t)e->n_stream++;
+    };
+    // the stream of an edge into stage c (parents have smaller indices, so their ways are known)
+    auto edge = [&](int from, int c, int64_t len, bool leaves) {
+        const int8_t x = place(len, part_of[from] == 0, leaves, exit_off[c]);
+        way[from][b.child_a[from] == c ? 0 : 1] = x;
+        return x;
+    };
+    for (int s = 0; s < S; s++) exit_off[s + 1] = exit_off[s] + e->leaving[s];
     for (int s = 0; s < S; s++) {
-        exit_off[s + 1] = exit_off[s] + e->leaving[s];
         const int par = e->parent[s];
-        if (s == 0 || par == 0 || two_ways(par)) part_of[s] = cut.n_part++;
-        else part_of[s] = part_of[par];
-        LanePart &pt = cut.part[part_of[s]];
+        const bool join = b.join_b[s] >= 0;
+        if (s != 0 && par != 0 && !two_ways(par) && !join) {
+            LanePart &pt = cut.part[part_of[s] = part_of[par]];
+            pt.stage[pt.len++] = (int8_t)s;
+            continue;
+        }
+        int8_t in = -1;
+        // (whether nothing follows the chain that begins here)
+        int end = s;
+        while (b.child_a[end] >= 0 && !two_ways(end) && end != 0 && b.join_b[b.child_a[end]] < 0) end = b.child_a[end];
+        const bool leaves = b.child_a[end] < 0;
+        if (join) {
+            LanePart &m = cut.part[cut.n_part++];
+            m.len = 0; m.stage[0] = (int8_t)s; m.join_no = (int8_t)cut.n_join++;
+            m.in = edge(par, s, b.join_na[s], false);
+            m.in_b = edge(b.join_b[s], s, b.join_nb[s], false);
+            m.out_a = in = place(e->visits[s], false, false, 0);
+            m.out_b = -1; m.out_kind = kOutOne;
+        } else if (s != 0) {
+            in = edge(par, s, e->visits[s], leaves);
+            // (the region of the chain's last stage)
+            if (e->stream_at[in] == il_estimator::kInSlab) cut.stream[in].off = (int32_t)exit_off[end];
+        }
+        part_of[s] = cut.n_part;
+        LanePart &pt = cut.part[cut.n_part++];
+        pt.in = in;
         pt.stage[pt.len++] = (int8_t)s;
     }
-    e->n_stream = cut.n_part - 1;
     for (int t = 0; t < cut.n_part; t++) {
         LanePart &pt = cut.part[t];
-        const int first = pt.stage[0], end = pt.stage[pt.len - 1];
-        pt.in = (int8_t)(t - 1);
-        pt.out_a = b.child_a[end] >= 0 ? (int8_t)(part_of[b.child_a[end]] - 1) : -1;
-        pt.out_b = b.child_b[end] >= 0 ? (int8_t)(part_of[b.child_b[end]] - 1) : -1;
+        if (pt.len == 0) continue;
+        const int end = pt.stage[pt.len - 1];
+        pt.out_a = way[end][0]; pt.out_b = way[end][1];
         pt.out_kind = (int8_t)(two_ways(end) ? kOutTwo : pt.out_a >= 0 ? kOutOne : kOutLeaf);
         pt.n_leave = (int32_t)e->leaving[end];
         pt.leave_off = e->fork ? 0 : (int32_t)exit_off[end];
         pt.n_out = e->leaving[end];
-        for (int c : {(int)b.child_a[end], (int)b.child_b[end]}) if (c >= 0) pt.n_out += e->visits[c];
-        if (t == 0) continue;
-        LaneStream &x = cut.stream[t - 1];
-        x.len = (int32_t)e->visits[first];
-        x.by_node = part_of[e->parent[first]] == 0;
-        if (x.by_node) {
-            e->stream_at[t - 1] = il_estimator::kAtNode;
-            x.off = (int32_t)e->node_elems; e->node_elems += even(x.len);
-            e->root_readers++;
-        } else if (pt.out_kind == kOutLeaf && !e->fork) {
-            e->stream_at[t - 1] = il_estimator::kInSlab;
-            x.off = pt.leave_off;
-            e->slab_streams = true;
-        } else {
-            e->stream_at[t - 1] = il_estimator::kExtra;
-            x.off = (int32_t)e->extra_elems; e->extra_elems += even(x.len);
-        }
+        for (int x : {(int)pt.out_a, (int)pt.out_b}) if (x >= 0) pt.n_out += cut.stream[x].len;
     }
     e->node_elems = (e->node_elems + 31) / 32 * 32;
     e->extra_elems = (e->extra_elems + 31) / 32 * 32;
@@ -697,12 +728,6 @@ static DesParams chunk_params(const il_estimator *e, const Plan &pl, char *ws, c
     p.lane_slots = e->lane_slots;
     p.cpw = (int32_t)pl.cps;
     p.lanes_per_slot = is_cut(e) ? 32 : (int32_t)pl.cps * e->S;
-    if (e->join) {
-        const size_t seen = ((size_t)pl.slots * slot_seen_bytes(e, pl.cps) + 7) / 8 * 8;
-        p.join_seen = reinterpret_cast<uint32_t *>(ws + pl.off_qid);
-        p.join_ws = reinterpret_cast<uint64_t *>(ws + pl.off_qid + seen);
-        p.join_size = pl.slots * pl.cps * e->base.join_elems;
-    }
     return p;
 }
 
@@ -761,14 +786,6 @@ static cudaError_t launch_lane(const il_estimator *e, DesParams p, int64_t ctas,
 {
     const size_t per_sm = (size_t)((ctas + e->num_sms - 1) / e->num_sms);
     auto fits = [&](size_t bytes) { return bytes <= e->smem_per_cta && (bytes + 1024) * per_sm <= e->smem_per_sm; };
-    if (e->join) {
-        p.join_window = kJoinWindowMost;
-        p.lane_words = kLaneWordsMost;
-        auto smem = [&] { return des_join_lane_smem(e->S * e->H, e->Bmax, e->lane_slots, p.lane_words, p.cpw, p.n_join, p.join_window); };
-        while (!fits(smem()) && p.join_window > kJoinWindow) p.join_window >>= 1;
-        while (!fits(smem()) && p.lane_words > kLaneWords) p.lane_words >>= 1;
-        return launch_des_join_lane(p, (int)ctas, smem(), st);
-    }
     p.lane_ahead = 64;
     p.lane_stretch = lane_stretch_bytes(p.cpw, p.lane_ahead);
     widen(p.lane_words, [&] { return fits(lane_smem(e, e->lane_slots, p.lane_words, p.lane_stretch)); });
@@ -804,6 +821,7 @@ static int enqueue_parts(il_estimator *e, DesParams p, const Plan &pl, char *ws,
         LanePart &pt = cut.part[t];
         pt.groups = sh.groups[t]; pt.warps = sh.warps[t];
         // records without branch bits leave as they are
+        if (pt.len == 0) continue;
         if (pt.out_kind == kOutLeaf && p.rec_bits == 0 && !feas && !e->fork) pt.out_kind = kOutOne;
         // one store where the two ways are alternatives, told by a bit that the records carry, in streams of one row; two
         // with fan-out; anything else is looked into record by record
@@ -816,6 +834,9 @@ static int enqueue_parts(il_estimator *e, DesParams p, const Plan &pl, char *ws,
             pt.out_kind = kOutAny;
     }
     IL_CUDA(cudaMemsetAsync(words, 0, pl.ctl_bytes, st));
+    if (cut.n_join > 0) {
+        cut.seen = reinterpret_cast<uint32_t *>(ws + pl.off_seen);
+    }
     RootNodeParams rp = {};
     rp.configs = p.configs; rp.n_cand = p.n_cand; rp.S = e->S; rp.H = e->H; rp.Bmax = e->Bmax; rp.readers = e->root_readers; rp.shared = cut.shared;
     rp.root_of = root_of; rp.node_cfg = node_cfg; rp.ctl = words; rp.refs = cut.refs; rp.miss = cut.miss;
@@ -1329,19 +1350,9 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
         }
     }
     for (int s = 0; s < S; s++) bp.n_s[s] = (int32_t)e->visits[s];
-    bp.n_join = 0;
     bp.any_bits = any_cond ? 1 : 0;
-    bp.join_elems = 0;
     if (e->join) {
         // lane kernel: which queries follow both edges into a join is a function of their branch bits
-        bp.join_seen_words = (int32_t)((n + 31) / 32);
-        for (int c = 1; c < S; c++) {
-            if (bp.join_b[c] < 0) continue;
-            bp.join_no[c] = (int8_t)bp.n_join;
-            bp.join_stage[bp.n_join++] = (int8_t)c;
-            bp.join_lane_a[c] = bp.join_elems; bp.join_elems += edge_a[c];
-            bp.join_lane_b[c] = bp.join_elems; bp.join_elems += edge_b[c];
-        }
         for (unsigned bits = 0; bits < 256; bits++) {
             bool reach[IL_MAX_STAGES] = {};
             reach[0] = true;
@@ -1354,7 +1365,7 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
             }
         }
     }
-    e->cpw = std::max(1, 32 / (S + bp.n_join));
+    e->cpw = std::max(1, 32 / S);
     configure_lane_rings(e);
     build_parts(e);
     bp.S = S; bp.H = H; bp.Bmax = B; bp.n = (int32_t)n;
@@ -1434,11 +1445,9 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
     e->ctas_per_sm_staged = des_packed_max_ctas_per_sm(true, e->smem);
     for (int k = 0; k < 2; k++) {
         const int slots = k == 0 ? 16 : 32;
-        if (e->join) {
-            e->ctas_lane[k] = des_join_lane_max_ctas_per_sm(des_join_lane_smem(S * H, B, slots, kLaneWords, e->cpw, e->base.n_join, kJoinWindow));
-        } else if (e->cut.n_part > 0) {
+        if (e->cut.n_part > 0) {
             int most = 1;
-            for (int t = e->cut.shared ? 1 : 0; t < e->cut.n_part; t++) most = std::max(most, 32 / e->cut.part[t].len);
+            for (int t = e->cut.shared ? 1 : 0; t < e->cut.n_part; t++) most = std::max(most, e->cut.part[t].len > 0 ? 32 / e->cut.part[t].len : 32);
             e->ctas_lane[k] = std::max(1, des_lane_max_ctas_per_sm(lane_smem(e, slots, kLaneWords, lane_stretch_bytes(std::max(most, kRootGroups), 32)), true));
         } else {
             e->ctas_lane[k] = des_lane_max_ctas_per_sm(lane_smem(e, slots, kLaneWords, lane_stretch_bytes(e->cpw, 64)), false);
@@ -1522,7 +1531,7 @@ const char *il_kernel_name(const il_estimator *e)
 {
     if (!e) return "";
     switch (sim_kernel(e)) {
-    case kSimLane: return e->join ? "des_kernel" : "des_lane_kernel";      // (des_join_lane_kernel)
+    case kSimLane: return e->join ? "des_kernel" : "des_lane_kernel";      // (des_part_kernel where the pipeline has branch points)
     case kSimPacked: return "des_packed_kernel";
     case kSimPackedStaged: return "des_packed_kernel<staged>";
     default: return "des_kernel";

@@ -84,16 +84,8 @@ struct DesParams {
     int32_t lane_ahead;           // records of its arrival stream a group has in shared memory (32 or 64)
     int32_t lane_stretch;         // bytes of that for all groups of a warp
     int32_t lanes_per_slot;       // spill rings of a warp slot
-    // lane kernel, joins: join_stage[0 .. n_join) are the stages with two incoming edges, join_no[s] their number
-    int32_t n_join;
-    int8_t  join_stage[IL_MAX_STAGES], join_no[IL_MAX_STAGES];
+    // lane kernel, joins
     uint64_t join_both[IL_MAX_STAGES][4];    // bit b: a query with branch bits b follows both incoming edges of the stage
-    uint64_t *join_ws;            // [warp slots][cpw][join_elems] incoming streams of the joins, stage s's at
-    int64_t join_lane_a[IL_MAX_STAGES], join_lane_b[IL_MAX_STAGES];
-    int64_t join_elems, join_size;           // records per candidate; and in all of join_ws
-    uint32_t *join_seen;          // [warp slots][cpw][n_join][join_seen_words]: one input of this query has come in
-    int32_t join_seen_words;
-    int32_t join_window;          // records of an incoming stream kept in shared memory (a power of two)
     int32_t any_bits;             // some edge is conditional
     uint8_t *ovf;                 // [n_cand] set to 1 for a candidate given up on ring overflow (lane_wrap only)
     // lane kernel, feasibility only: set out_feasible to select that instantiation
@@ -120,10 +112,11 @@ struct LaneStream {
 // leave the pipeline; either of two streams of one row, by a branch bit that the records carry; any other two ways.
 constexpr int kOutOne = 0, kOutLeaf = 1, kOutTwo = 2, kOutAny = 3;
 struct LanePart {
-    int8_t len;                   // a chain of so many stages
-    int8_t stage[IL_MAX_STAGES];
+    int8_t len;                   // a chain of so many stages; 0: the merge of a join's two streams, one lane
+    int8_t stage[IL_MAX_STAGES];  // (merge: the join)
     int8_t out_kind;
-    int8_t in, out_a, out_b;      // streams; -1: the trace, none
+    int8_t in, in_b, out_a, out_b;        // streams; -1: the trace, none (in_b: merge)
+    int8_t join_no;               // merge: which row of the seen bits
     int32_t groups, warps;        // groups of lanes per warp, warps planned
     int32_t n_leave, leave_off;   // records that leave after the last stage, and where they go in a slab row
     int64_t n_out;                // records that come out of the last stage, all ways together
@@ -132,8 +125,10 @@ struct LaneCut {
     int32_t n_part;               // part 0 is the root stage
     int32_t shared;               // simulated once per distinct configuration (root node); 0: per candidate, whose number is its node's
     int32_t num_sms;
-    LanePart part[IL_MAX_STAGES];
-    LaneStream stream[IL_MAX_STAGES];
+    LanePart part[2 * IL_MAX_STAGES];
+    LaneStream stream[3 * IL_MAX_STAGES];
+    uint32_t *seen;               // [n_cand][joins][seen_words]: a bit per query of which one input has come in
+    int32_t seen_words, n_join;
     uint32_t *ctl;                // control words, below; zero at launch
     const int32_t *root_of;       // [n_cand] root node of a candidate, -1: its configuration is out of range
     const uint32_t *node_cfg;     // hw | max batch << 8 | replicas << 16
@@ -200,10 +195,6 @@ int des_lane_warps_per_cta();
 // of a warp's arrival streams
 size_t des_lane_smem(int table_rows, int Bmax, int ring_slots, int ring_words, int stretch);
 int des_lane_max_ctas_per_sm(size_t smem, bool cut);
-// the same for pipelines with joins: cpw candidates per warp with so many joins each, whose streams keep `window` records
-cudaError_t launch_des_join_lane(const DesParams &p, int grid, size_t smem, cudaStream_t stream);
-size_t des_join_lane_smem(int table_rows, int Bmax, int ring_slots, int ring_words, int cpw, int joins, int window);
-int des_join_lane_max_ctas_per_sm(size_t smem);
 enum SimKernel { kSimWide = 0, kSimPacked = 1, kSimPackedStaged = 2, kSimLane = 3 };
 inline cudaError_t launch_simulation(const DesParams &p, int kernel, int grid, size_t smem,
                                      cudaStream_t stream)

@@ -101,6 +101,23 @@ def test_small_workspace_and_bad_candidates(oracle, shape):
         assert np.array_equal(a.cpu().numpy(), exp[0])
 
 
+@pytest.mark.parametrize("n", [1, 2, 31, 33, 64, 65, 129, 1025, 2100])
+@pytest.mark.parametrize("C", [1, 40, 20_000])
+@pytest.mark.parametrize("shape", ["diamond", "guarded", "two_joins", "skip"])
+def test_merges(oracle, shape, C, n):
+    """Lengths around a merge's windows and around what it keeps of the queries' bits (1,024 at the least); one, a few and
+    several rounds of candidates per lane; one input slow, so that it falls far behind."""
+    import paper_1812_01776_b200 as il
+    w = workloads.join_small(n, n=n, C=24, max_replicas=3, Bmax=8, shape=shape)
+    w.configs[:8, 1] = (0, 1, 1, 0)
+    w.latency_us[1, 0, 0] = 9000
+    at = np.arange(C) % 24
+    exp = oracle.estimate_workload(w)
+    with il.Estimator.from_workload(w) as est:
+        a, b = est.estimate(w.configs[at], w.slo_us)
+        assert np.array_equal(a, exp[0][at]) and np.array_equal(b, exp[1][at])
+
+
 @pytest.mark.parametrize("shape", ["late_branch", "fan_out"])
 def test_iteration_bound(shape):
     import paper_1812_01776_b200 as il
