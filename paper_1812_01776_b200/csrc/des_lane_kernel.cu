@@ -650,7 +650,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
             const uint32_t span = i - low;
             if (!(is & kSpill) && span > (uint32_t)(nq - kTurn - 2)) {
 #pragma unroll 1
-                for (uint32_t k = i - min(span, gmask + 1u); k != i; k++)
+                for (uint32_t k = low; k != i; k++)
                     if (IL_IN_RANGE(k & gmask, gmask + 1ull, p.status))
                         spill_ring[k & gmask] = lds32(qb + ((k & (nq - 1u)) << 7));
                 is |= kSpill;
