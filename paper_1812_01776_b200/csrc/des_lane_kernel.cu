@@ -473,14 +473,14 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
     const uint32_t gmask = (uint32_t)((1ull << p.lane_ring_log2) - 1ull);
     const int64_t wslot = (int64_t)blockIdx.x * kLaneWarps + wid;
     uint32_t *spill_ring = reinterpret_cast<uint32_t *>(p.lane_ws) + ((wslot * p.lanes_per_slot + lane) << p.lane_ring_log2);
-    const uint64_t slo_q = FEAS ? (uint64_t)p.slo_us << q : 0ull;   // the objective, aligned with a record's time field
     // (cut: a group may also wait for records while others of its warp have some)
     const unsigned long long limit =
         (p.iter_limit ? p.iter_limit : (8ull * (unsigned)p.n * (unsigned)(p.S + 1) + 4096ull) * (CUT ? 4ull : 1ull)) / kTurn + 1ull;
     // a spill has to start before a record still needed is overwritten, two turns from now at the latest
     const uint32_t reach = min((uint32_t)(nq - kTurn - 2), gmask - 2u * kTurn);
-    // (and no long turn may start where it would come too late)
+    // (and a turn may not be so long that it would come too late)
     const uint32_t long_reach = gmask > 2u * kLongTurn && nq > kLongTurn + 2u ? min((uint32_t)(nq - kLongTurn - 2), gmask - 2u * kLongTurn) : 0u;
+    const int most_kept = (int)min(nq, gmask + 1u) - 4;
     unsigned long long batches = 0, alg_ops = 0, exits_seen = 0, exits_due = 0;
     unsigned early = 0;          // candidates dropped before the end of the trace (feasibility only)
     unsigned long long naps = p.iter_limit ? p.iter_limit : cut.naps;      // bound on the sleeps of a warp
@@ -584,15 +584,22 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
     uint32_t turns = 1, turns_hi = 0;        // iteration bound, in turns
     uint32_t look = 0;
     bool any_spill = false;
-    uint64_t late_fin = 0, late_arr = 0;     // feasibility only: finish and arrival record of a query that has just left
-    uint32_t miss_local = 0, line = 0;       // (line: of the trace, the last one such a query's arrival was in)
-    (void)line; (void)node; (void)avail; (void)pub_a; (void)pub_b; (void)src_count; (void)look;
+    // feasibility only: finish and deadline of a query that has just left, of every other iteration
+    uint64_t late_fin[2] = {0, 0}, late_arr[2] = {kLatest, kLatest};
+    uint32_t miss_local = 0;
+    (void)node; (void)avail; (void)pub_a; (void)pub_b; (void)src_count; (void)look;
 
     __syncwarp();
     for (int k = 0; k < kX; k++) sts64(xb + (uint32_t)k * 256u, kInf);       // lanes without a stage see no record either
     sts64(at1, 0ull); sts64(at2, 0ull);
     __syncwarp();
 
+    auto test_late = [&]() {
+        for (int k = 0; k < 2; k++) {
+            miss_local += late_fin[k] > late_arr[k] ? 1u : 0u;
+            late_arr[k] = kLatest;
+        }
+    };
     // cut, feasibility only: misses seen by this lane are added to the candidate's; whoever passes the limit decides it
     auto set = [&](uint32_t bit, bool yes) { is = yes ? is | bit : is & ~bit; };
     auto count_misses = [&]() {
@@ -609,6 +616,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
         // ---- every kQuickTurn-th, kTurn-th or kLongTurn-th iteration: does a lane need more than its steps?  A stream at its start or its end, a
         // candidate that is decided, records in reach of being overwritten, the iteration bound.  (Kept short: its
         // latency is on the chain of every iteration, a kTurn-th of it.)
+        if (FEAS) test_late();
         if (FEAS && !CUT && miss_local) { atomicAdd(missw + j, miss_local); miss_local = 0; }
         if (FEAS && CUT && miss_local && (look & 3u) == 0u) count_misses();
         nb += (tpos - tpos_seen) >> 8;
@@ -637,7 +645,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
         if (FEAS && !CUT) attn |= (is & kHas) && missw[j] > p.miss_allow;
         if (CUT) attn |= (is & kHas) && ((is & kNobody) || (is & kDecided) || quit);
         if (__any_sync(full, attn)) {
-        bool done = i == n_cur && bm == ~0u && epos == tpos && e_on == 0u && !(FEAS && late_fin != 0ull);
+        bool done = i == n_cur && bm == ~0u && epos == tpos && e_on == 0u;
         bool stop = FEAS && !CUT && (is & kHas) && missw[j] > p.miss_allow;       // this lane ends its group's candidate here
         if (CUT) stop = (is & kHas) && ((is & kNobody) || (is & kDecided) || quit);
         bool give_up = CUT && (is & kHas) && (is & kNobody) && !(is & kDecided);
@@ -675,7 +683,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
             stop |= group_gives_up;
         }
         if (stop) {
-            n_cur = i; bm = ~0u; epos = tpos; efull = tpos; e_on = 0u; late_fin = 0; is &= ~(uint32_t)kStarted;
+            n_cur = i; bm = ~0u; epos = tpos; efull = tpos; e_on = 0u; late_arr[0] = kLatest; late_arr[1] = kLatest; is &= ~(uint32_t)kStarted;
             done = true;
         }
         // The first record of a stream opens a batch on an unused replica, and the last batch is closed by the
@@ -816,7 +824,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
                 is &= ~(uint32_t)kSpill; low = i; next_idx = i; next_key = 0;
                 nb = 0;
                 turns = (uint32_t)limit; turns_hi = (uint32_t)(limit >> 32);
-                late_fin = 0; miss_local = 0;
+                late_arr[0] = kLatest; late_arr[1] = kLatest; miss_local = 0;
                 fed = odd;
                 if (row == 0) for (uint32_t k = 0; k < ahead; k++) sts64(tb + k * 8u, kInf);
             }
@@ -871,7 +879,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
         // the first kQuickLooks looks has late records: no short turns for it.  The other lengths are two less than half of what a
         // group has before it: one record of that is missing when the first lane is at an odd one, since copies are of pairs.)
         const bool quick = (i != n_cur && !(is & kStarted) && (uint32_t)limit - turns < kQuickLooks) || (i == n_cur && bm != ~0u);
-        const int turn_its = (int)__reduce_min_sync(full, quick ? kQuickTurn : (i - low > long_reach || ahead < 2u * kLongTurn) ? kTurn - 2 : kLongTurn - 2);
+        const int turn_its = (int)__reduce_min_sync(full, quick ? kQuickTurn : ahead < 2u * kLongTurn ? kTurn - 2 : i - low <= long_reach ? kLongTurn - 2 : CUT ? max(kTurn - 2, min(kLongTurn - 2, (most_kept - (int)(i - low)) & ~1)) : kTurn - 2);
 
         // The group's next records: requested two turns before their use where they are there, by all lanes of the group.
         {
@@ -904,10 +912,10 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
         uint64_t rec = lds64_shared(xs);                    // record to examine
         uint32_t rw = lds32_shared(sa + 4u);                // where the record in hand goes: empty?
         uint32_t lat = lds32(tab + bm * 4u);                // time of the open batch
-        auto step = [&](auto spilling, auto kind) {
+        auto step = [&](auto spilling, auto kind, auto turn_of) {
             constexpr bool SPILL = decltype(spilling)::value;
+            [[maybe_unused]] constexpr int TURN = decltype(turn_of)::value;
             constexpr int OUT = decltype(kind)::value;
-            if (FEAS) miss_local += (late_fin > late_arr + slo_q) ? 1u : 0u;
             [[maybe_unused]] uint32_t bits = qv;
             if (OUT == kOutAny && looks_up != 0u && e_on != 0u && IL_IN_RANGE(qv & imask, p.n, p.status)) bits = p.bits[qv & imask];
             [[maybe_unused]] uint32_t leaves = 0u;
@@ -1002,7 +1010,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
                     : "r"(xin), "r"(xin_mask), "r"(xin_row), "r"(tab), "r"(kfb), "r"(kfm), "r"(kb), "r"(rm), "r"(mbm1), "r"(tick), "r"(qmask), "r"(~qmask), "r"(qb), "r"(nq - 1u), "r"(xa), "r"(xam), "r"(down), "r"(tail_step), "l"(out)
                     : "memory");
             } else if constexpr (OUT == kOutLeaf && FEAS) {
-                // (compared with the objective in the next iteration; the arrival's line was asked for with the one before it)
+                // (compared with its deadline two iterations later, when that has come)
                 asm volatile(
                     "{\n"
                     ".reg .b32 i; .reg .b32 bm; .reg .b32 lpos; .reg .b32 lfull; .reg .b32 tpos; .reg .b32 at1; .reg .b32 at2;\n"
@@ -1015,7 +1023,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
                     "mov.b32 i, %0; mov.b32 bm, %1; mov.b32 lpos, %2; mov.b32 lfull, %3; mov.b32 tpos, %4; mov.b32 at1, %5;\n"
                     "mov.b32 at2, %6; mov.b64 tk, %7; mov.b32 prev, %8; mov.b64 rec, %9; mov.b32 lat, %10; mov.b32 xs, %11;\n"
                     "mov.b32 epos, %12; mov.b32 efull, %13; mov.b32 e_on, %14; mov.b64 e_key, %15; mov.b32 e_idx, %16; mov.b32 qv, %17;\n"
-                    "mov.b32 tail_a, %18; mov.b32 rw, %19; mov.b32 sa, %20; mov.b64 late_arr, %22; mov.b32 line, %23; mov.b32 xin, %24;\n"
+                    "mov.b32 tail_a, %18; mov.b32 rw, %19; mov.b32 sa, %20; mov.b64 late_arr, %22; mov.b64 late_fin, %21; .reg .b32 nobody; mov.b32 nobody, %44; mov.b32 line, %23; mov.b32 xin, %24;\n"
                     "mov.b32 xin_mask, %25; mov.b32 xin_row, %26; mov.b32 tab, %27; mov.b32 kfb, %28; mov.b32 kfm, %29; mov.b32 kb, %30;\n"
                     "mov.b32 rm, %31; mov.b32 mbm1, %32; mov.b32 tick, %33; mov.b32 qmask, %34; mov.b32 tmask, %35; mov.b32 qb, %36;\n"
                     "mov.b32 nqm, %37; mov.b32 xa, %38; mov.b32 xam, %39; mov.b32 down, %40; mov.b32 tail_step, %41; mov.b64 trace, %42;\n"
@@ -1042,8 +1050,8 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
                     "mov.b64 {fl, fh}, fk;\n"
                     "@hand add.u32 e_idx, e_idx, 1; @fetch and.b32 e_idx, fl, qmask; and.b32 a, e_idx, nqm; mad.lo.u32 a, a, 128, qb; ld.shared.u32 qv, [a];\n"
                     "@hd st.relaxed.cta.shared.b64 [sa_was], v;\n"
-                    "mov.b64 o, {lo, hi}; selp.b64 late_fin, o, 0, ho; and.b32 a, x, imask; mad.wide.u32 o, a, 8, trace; @ho ld.global.nc.b64 late_arr, [o];\n"
-                    "shr.u32 a, a, 4; setp.ne.and.u32 nl, a, line, ho; @nl mov.u32 line, a; @nl prefetch.global.L1 [o+128];\n"
+                    "setp.gt.f64 nl, late_fin, late_arr; @nl add.u32 line, line, 1; mov.b64 late_fin, {lo, hi};\n"
+                    "and.b32 a, x, imask; selp.b32 a, a, nobody, ho; mad.wide.u32 o, a, 8, trace; ld.global.nc.b64 late_arr, [o];\n"
                     "@fetch mov.b64 e_key, fk; @fin mov.u32 e_on, 0; @fetch mov.u32 e_on, 1; @fetch add.u32 epos, epos, 256; @fetch add.u32 efull, efull, 256;\n"
                     "and.b32 at0, tpos, rm; or.b32 at0, at0, kb;\n"
                     "setp.lt.f64 pf, kf, key; selp.b64 first, kf, key, pf;\n"
@@ -1058,7 +1066,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
                     "@open add.u32 tpos, tpos, 256; @open mov.u32 at2, at1; @open mov.u32 at1, at0;\n"
                     "@pop add.u32 lpos, lpos, 256; @pop add.u32 lfull, lfull, 256;\n"
                     "@taken and.b32 prev, rl, qmask;\n"
-                    "@!dp bra PLACED;\n"
+                    "vote.sync.any.pred pf, dp, 0xffffffff; @!pf bra.uni PLACED;\n"
                     "mov.u32 sd, left; sub.u32 pos, pos, 256;\n"
                     "DEEPER:\n"
                     "sub.u32 left, pos, sd;\n"
@@ -1066,11 +1074,11 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
                     "sub.u32 a2, pos, 512; and.b32 a2, a2, rm; or.b32 a2, a2, kb; sub.u32 a3, pos, 768; and.b32 a3, a3, rm; or.b32 a3, a3, kb;\n"
                     "sub.u32 a4, pos, 1024; and.b32 a4, a4, rm; or.b32 a4, a4, kb;\n"
                     "ld.shared.b64 e1, [a1]; ld.shared.b64 e2, [a2]; ld.shared.b64 e3, [a3]; ld.shared.b64 e4, [a4];\n"
-                    "setp.gt.u32 t, left, 0; setp.lt.and.f64 t, key, e1, t; setp.gt.and.u32 ov, left, 256, t; setp.lt.and.f64 ov, key, e2, ov;\n"
+                    "setp.gt.and.u32 t, left, 0, dp; setp.lt.and.f64 t, key, e1, t; setp.gt.and.u32 ov, left, 256, t; setp.lt.and.f64 ov, key, e2, ov;\n"
                     "setp.gt.and.u32 pz, left, 512, ov; setp.lt.and.f64 pz, key, e3, pz; setp.gt.and.u32 pf, left, 768, pz; setp.lt.and.f64 pf, key, e4, pf;\n"
                     "@t st.shared.b64 [at0], e1; @ov st.shared.b64 [a1], e2; @pz st.shared.b64 [a2], e3; @pf st.shared.b64 [a3], e4;\n"
-                    "@t mov.u32 at0, a1; @ov mov.u32 at0, a2; @pz mov.u32 at0, a3; @pf mov.u32 at0, a4; st.shared.b64 [at0], key;\n"
-                    "sub.u32 pos, pos, 1024; @pf bra DEEPER;\n"
+                    "@t mov.u32 at0, a1; @ov mov.u32 at0, a2; @pz mov.u32 at0, a3; @pf mov.u32 at0, a4; @dp st.shared.b64 [at0], key;\n"
+                    "sub.u32 pos, pos, 1024; setp.ne.and.u32 dp, pos, 1, pf; vote.sync.any.pred pf, dp, 0xffffffff; @pf bra.uni DEEPER;\n"
                     "PLACED:\n"
                     "mov.b32 %0, i; mov.b32 %1, bm; mov.b32 %2, lpos; mov.b32 %3, lfull; mov.b32 %4, tpos; mov.b32 %5, at1;\n"
                     "mov.b32 %6, at2; mov.b64 %7, tk; mov.b32 %8, prev; mov.b64 %9, rec; mov.b32 %10, lat; mov.b32 %11, xs;\n"
@@ -1078,8 +1086,8 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
                     "mov.b32 %18, tail_a; mov.b32 %19, rw; mov.b32 %20, sa; mov.b64 %21, late_fin; mov.b64 %22, late_arr;\n"
                     "mov.b32 %23, line;\n"
                     "}"
-                    : "+r"(i), "+r"(bm), "+r"(lpos), "+r"(lfull), "+r"(tpos), "+r"(at1), "+r"(at2), "+l"(tk), "+r"(prev), "+l"(rec), "+r"(lat), "+r"(xs), "+r"(epos), "+r"(efull), "+r"(e_on), "+l"(e_key), "+r"(e_idx), "+r"(qv), "+r"(tail_a), "+r"(rw), "+r"(sa), "=l"(late_fin), "+l"(late_arr), "+r"(line)
-                    : "r"(xin), "r"(xin_mask), "r"(xin_row), "r"(tab), "r"(kfb), "r"(kfm), "r"(kb), "r"(rm), "r"(mbm1), "r"(tick), "r"(qmask), "r"(~qmask), "r"(qb), "r"(nq - 1u), "r"(xa), "r"(xam), "r"(down), "r"(tail_step), "l"(trace), "r"(imask)
+                    : "+r"(i), "+r"(bm), "+r"(lpos), "+r"(lfull), "+r"(tpos), "+r"(at1), "+r"(at2), "+l"(tk), "+r"(prev), "+l"(rec), "+r"(lat), "+r"(xs), "+r"(epos), "+r"(efull), "+r"(e_on), "+l"(e_key), "+r"(e_idx), "+r"(qv), "+r"(tail_a), "+r"(rw), "+r"(sa), "+l"(late_fin[TURN]), "+l"(late_arr[TURN]), "+r"(miss_local)
+                    : "r"(xin), "r"(xin_mask), "r"(xin_row), "r"(tab), "r"(kfb), "r"(kfm), "r"(kb), "r"(rm), "r"(mbm1), "r"(tick), "r"(qmask), "r"(~qmask), "r"(qb), "r"(nq - 1u), "r"(xa), "r"(xam), "r"(down), "r"(tail_step), "l"(p.deadline), "r"(imask), "r"((uint32_t)p.n)
                     : "memory");
             } else if constexpr (OUT == kOutLeaf && FORK) {
                 // (the query's slab entry keeps the latest of its copies)
@@ -1136,7 +1144,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
                     "@open add.u32 tpos, tpos, 256; @open mov.u32 at2, at1; @open mov.u32 at1, at0;\n"
                     "@pop add.u32 lpos, lpos, 256; @pop add.u32 lfull, lfull, 256;\n"
                     "@taken and.b32 prev, rl, qmask;\n"
-                    "@!dp bra PLACED;\n"
+                    "vote.sync.any.pred pf, dp, 0xffffffff; @!pf bra.uni PLACED;\n"
                     "mov.u32 sd, left; sub.u32 pos, pos, 256;\n"
                     "DEEPER:\n"
                     "sub.u32 left, pos, sd;\n"
@@ -1144,11 +1152,11 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
                     "sub.u32 a2, pos, 512; and.b32 a2, a2, rm; or.b32 a2, a2, kb; sub.u32 a3, pos, 768; and.b32 a3, a3, rm; or.b32 a3, a3, kb;\n"
                     "sub.u32 a4, pos, 1024; and.b32 a4, a4, rm; or.b32 a4, a4, kb;\n"
                     "ld.shared.b64 e1, [a1]; ld.shared.b64 e2, [a2]; ld.shared.b64 e3, [a3]; ld.shared.b64 e4, [a4];\n"
-                    "setp.gt.u32 t, left, 0; setp.lt.and.f64 t, key, e1, t; setp.gt.and.u32 ov, left, 256, t; setp.lt.and.f64 ov, key, e2, ov;\n"
+                    "setp.gt.and.u32 t, left, 0, dp; setp.lt.and.f64 t, key, e1, t; setp.gt.and.u32 ov, left, 256, t; setp.lt.and.f64 ov, key, e2, ov;\n"
                     "setp.gt.and.u32 pz, left, 512, ov; setp.lt.and.f64 pz, key, e3, pz; setp.gt.and.u32 pf, left, 768, pz; setp.lt.and.f64 pf, key, e4, pf;\n"
                     "@t st.shared.b64 [at0], e1; @ov st.shared.b64 [a1], e2; @pz st.shared.b64 [a2], e3; @pf st.shared.b64 [a3], e4;\n"
-                    "@t mov.u32 at0, a1; @ov mov.u32 at0, a2; @pz mov.u32 at0, a3; @pf mov.u32 at0, a4; st.shared.b64 [at0], key;\n"
-                    "sub.u32 pos, pos, 1024; @pf bra DEEPER;\n"
+                    "@t mov.u32 at0, a1; @ov mov.u32 at0, a2; @pz mov.u32 at0, a3; @pf mov.u32 at0, a4; @dp st.shared.b64 [at0], key;\n"
+                    "sub.u32 pos, pos, 1024; setp.ne.and.u32 dp, pos, 1, pf; vote.sync.any.pred pf, dp, 0xffffffff; @pf bra.uni DEEPER;\n"
                     "PLACED:\n"
                     "mov.b32 %0, i; mov.b32 %1, bm; mov.b32 %2, lpos; mov.b32 %3, lfull; mov.b32 %4, tpos; mov.b32 %5, at1;\n"
                     "mov.b32 %6, at2; mov.b64 %7, tk; mov.b32 %8, prev; mov.b64 %9, rec; mov.b32 %10, lat; mov.b32 %11, xs;\n"
@@ -1291,7 +1299,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
                     "@open add.u32 tpos, tpos, 256; @open mov.u32 at2, at1; @open mov.u32 at1, at0;\n"
                     "@pop add.u32 lpos, lpos, 256; @pop add.u32 lfull, lfull, 256;\n"
                     "@taken and.b32 prev, rl, qmask;\n"
-                    "@!dp bra PLACED;\n"
+                    "vote.sync.any.pred pf, dp, 0xffffffff; @!pf bra.uni PLACED;\n"
                     "mov.u32 sd, left; sub.u32 pos, pos, 256;\n"
                     "DEEPER:\n"
                     "sub.u32 left, pos, sd;\n"
@@ -1299,11 +1307,11 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
                     "sub.u32 a2, pos, 512; and.b32 a2, a2, rm; or.b32 a2, a2, kb; sub.u32 a3, pos, 768; and.b32 a3, a3, rm; or.b32 a3, a3, kb;\n"
                     "sub.u32 a4, pos, 1024; and.b32 a4, a4, rm; or.b32 a4, a4, kb;\n"
                     "ld.shared.b64 e1, [a1]; ld.shared.b64 e2, [a2]; ld.shared.b64 e3, [a3]; ld.shared.b64 e4, [a4];\n"
-                    "setp.gt.u32 t, left, 0; setp.lt.and.f64 t, key, e1, t; setp.gt.and.u32 ov, left, 256, t; setp.lt.and.f64 ov, key, e2, ov;\n"
+                    "setp.gt.and.u32 t, left, 0, dp; setp.lt.and.f64 t, key, e1, t; setp.gt.and.u32 ov, left, 256, t; setp.lt.and.f64 ov, key, e2, ov;\n"
                     "setp.gt.and.u32 pz, left, 512, ov; setp.lt.and.f64 pz, key, e3, pz; setp.gt.and.u32 pf, left, 768, pz; setp.lt.and.f64 pf, key, e4, pf;\n"
                     "@t st.shared.b64 [at0], e1; @ov st.shared.b64 [a1], e2; @pz st.shared.b64 [a2], e3; @pf st.shared.b64 [a3], e4;\n"
-                    "@t mov.u32 at0, a1; @ov mov.u32 at0, a2; @pz mov.u32 at0, a3; @pf mov.u32 at0, a4; st.shared.b64 [at0], key;\n"
-                    "sub.u32 pos, pos, 1024; @pf bra DEEPER;\n"
+                    "@t mov.u32 at0, a1; @ov mov.u32 at0, a2; @pz mov.u32 at0, a3; @pf mov.u32 at0, a4; @dp st.shared.b64 [at0], key;\n"
+                    "sub.u32 pos, pos, 1024; setp.ne.and.u32 dp, pos, 1, pf; vote.sync.any.pred pf, dp, 0xffffffff; @pf bra.uni DEEPER;\n"
                     "PLACED:\n"
                     "mov.b32 %0, i; mov.b32 %1, bm; mov.b32 %2, lpos; mov.b32 %3, lfull; mov.b32 %4, tpos; mov.b32 %5, at1;\n"
                     "mov.b32 %6, at2; mov.b64 %7, tk; mov.b32 %8, prev; mov.b64 %9, rec; mov.b32 %10, lat; mov.b32 %11, xs;\n"
@@ -1469,14 +1477,14 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
                     : "+r"(i), "+r"(bm), "+r"(lpos), "+r"(lfull), "+r"(tpos), "+r"(at1), "+r"(at2), "+l"(tk), "+r"(prev), "+l"(rec), "+r"(lat), "+r"(xs), "+r"(epos), "+r"(efull), "+r"(e_on), "+l"(e_key), "+r"(e_idx), "+r"(qv), "+r"(tail_a), "+r"(rw), "+r"(sa), "+r"(tail_b), "=r"(leaves)
                     : "r"(xin), "r"(xin_mask), "r"(xin_row), "r"(tab), "r"(kfb), "r"(kfm), "r"(kb), "r"(rm), "r"(mbm1), "r"(tick), "r"(qmask), "r"(~qmask), "r"(qb), "r"(nq - 1u), "r"(xa), "r"(xam), "r"(down), "r"(bits), "r"(mask_a), "r"(mask_b), "r"(want_a), "r"(want_b), "l"(out), "l"(out_b)
                     : "memory");
-                if (FEAS) late_fin = 0ull;
+                if (FEAS) test_late();
                 if (pt->n_leave > 0 && leaves != 0u) {
                     // (a branch point at which some queries leave)
                     const uint32_t qid = left_low & imask;
                     const uint64_t fin = left_rec & ~(uint64_t)qmask;
                     if (FEAS) {
-                        late_fin = fin;
-                        late_arr = __ldg(trace + qid);
+                        late_fin[0] = fin;
+                        late_arr[0] = __ldg(p.deadline + qid);
                     } else if (FORK) {
                         atomicMax(reinterpret_cast<unsigned long long *>(out_c) + qid, (fin >> rb) | qid);
                     } else if (IL_IN_RANGE(n_left, pt->n_leave, p.status)) {
@@ -1495,10 +1503,10 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
         auto run_turn = [&](auto kind) {
             if (any_spill) {
 #pragma unroll 1
-                for (int k = 0; k < turn_its; k++) step(std::true_type{}, kind);
+                for (int k = 0; k < turn_its; k++) step(std::true_type{}, kind, std::integral_constant<int, 0>{});
             } else {
 #pragma unroll 1
-                for (int k = 0; k < turn_its; k += 2) { step(std::false_type{}, kind); step(std::false_type{}, kind); }
+                for (int k = 0; k < turn_its; k += 2) { step(std::false_type{}, kind, std::integral_constant<int, 0>{}); step(std::false_type{}, kind, std::integral_constant<int, 1>{}); }
             }
         };
         using One = std::integral_constant<int, kOutOne>;
@@ -1544,6 +1552,14 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) des_part_kernel(const __gr
 }
 
 namespace {
+
+// Feasibility only: per query the latest record time at which it still meets the objective, compared as records are;
+// behind the last one, for lanes that have nothing to compare, a time that none exceeds.
+__global__ void __launch_bounds__(256) deadline_kernel(const uint64_t *trace, int n, uint64_t slo, uint32_t qmask, uint64_t *out)
+{
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= n; i += gridDim.x * blockDim.x)
+        out[i] = i < n ? min((unsigned long long)((trace[i] | qmask) + slo), (unsigned long long)kLatest) : kLatest;
+}
 
 // Root nodes of a chunk: the distinct (hardware, batch, replicas) of stage 0 among its candidates, numbered, each with how
 // many groups will read its streams; every candidate's node, -1 where a configuration is out of range.  One CTA: a bit per
@@ -1608,6 +1624,13 @@ cudaError_t launch_one(K kernel, int grid, size_t smem, cudaStream_t stream, con
     return cudaGetLastError();
 }
 }  // namespace
+
+cudaError_t launch_deadlines(const DesParams &p, uint64_t *out, cudaStream_t stream)
+{
+    const int q = p.qbits + p.rec_bits, grid = std::min((p.n + 256) / 256, 592);
+    deadline_kernel<<<grid, 256, 0, stream>>>(p.rec_bits > 0 ? p.ptrace_b : p.ptrace, p.n, (uint64_t)p.slo_us << q, (uint32_t)((1ull << q) - 1ull), out);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_root_nodes(const RootNodeParams &p, cudaStream_t stream)
 {

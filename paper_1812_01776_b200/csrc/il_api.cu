@@ -50,6 +50,7 @@ struct il_estimator {
     char *d_bound = nullptr;           // the allocation that holds the bound inputs and the counters (pointers below)
     int64_t *d_arrival = nullptr;
     uint64_t *d_ptrace = nullptr;      // packed root stream
+    uint64_t *d_deadline = nullptr;    // feasibility only: the current objective's deadlines
     uint64_t *d_ptrace_b = nullptr;    // the same with the branch bits inside each record (lane kernel)
     int rec_bits = 0;                  // branch bits a record of d_ptrace_b carries (0: there is none)
     bool can_pack = false;             // every reachable time fits a packed record
@@ -1401,9 +1402,11 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
     auto place = [&](size_t bytes) { const size_t at = size; size = align_up(size + bytes, 256); return at; };
     const size_t o_arrival = place((size_t)n * 8), o_bits = place((size_t)n), o_ptrace = place((size_t)n_padded * 8);
     const size_t o_ptrace_b = place(with_bits_inside ? (size_t)n_padded * 8 : 0), o_lat = place(e->smem);
+    const size_t o_deadline = place(can_pack ? (size_t)(n + 1) * 8 : 0);
     const size_t o_counters = place(kCounterBytes), o_envelope = place(envelope_max_windows() * sizeof(int));
     IL_CUDA_E(cudaMalloc(&e->d_bound, size));
     e->d_arrival = reinterpret_cast<int64_t *>(e->d_bound + o_arrival);
+    if (can_pack) e->d_deadline = reinterpret_cast<uint64_t *>(e->d_bound + o_deadline);
     e->d_bits = reinterpret_cast<uint8_t *>(e->d_bound + o_bits);
     e->d_lat = reinterpret_cast<int32_t *>(e->d_bound + o_lat);
     e->d_counters = reinterpret_cast<unsigned long long *>(e->d_bound + o_counters);
@@ -1866,6 +1869,8 @@ static int feasible_device(il_estimator *e, const il_stage_config *d_configs, in
         // (latencies are at least 1 and every reachable time is below 2^(63 - qbits))
         p.slo_us = std::min<int64_t>(std::max<int64_t>(slo_us, 0), INT64_C(1) << (62 - p.qbits - p.rec_bits));
         p.miss_allow = (uint32_t)(e->n - (99 * e->n + 99) / 100);
+        p.deadline = e->d_deadline;
+        if (lo == 0) { IL_CUDA(launch_deadlines(p, e->d_deadline, st)); launches++; }
         if (is_cut(e)) {
             rc = enqueue_parts(e, p, pl, ws, st, &launches);
             if (rc) return rc;

@@ -91,6 +91,7 @@ struct DesParams {
     // lane kernel, feasibility only: set out_feasible to select that instantiation
     uint8_t *out_feasible;        // [n_cand] 1: P99 <= slo_us, 0: not, 2: given up on ring overflow (see ovf)
     int64_t slo_us;               // the objective, clamped by the host to 0 .. 2^(62 - qbits)
+    const uint64_t *deadline;     // [n + 1] (launch_deadlines)
     uint32_t miss_allow;          // n - ceil(0.99 n): a candidate with more misses than this is infeasible
     // all simulation kernels
     unsigned long long iter_limit;   // iteration bound of a device loop; 0 = the bound the loop derives itself
@@ -150,6 +151,7 @@ struct RootNodeParams {
     int *status;
 };
 cudaError_t launch_root_nodes(const RootNodeParams &p, cudaStream_t stream);
+cudaError_t launch_deadlines(const DesParams &p, uint64_t *out, cudaStream_t stream);      // feasibility only, before the lane kernel
 int lane_root_sms(int64_t nodes, int num_sms);        // SMs set aside for so many root nodes
 int lane_stretch_bytes(int groups, int ahead);
 
