@@ -989,7 +989,7 @@ static int shared_by_cover(il_estimator *e, const SharedCommon &c, char *ws, siz
     IL_CUDA(cudaEventRecord(e->events[1], st));
 
     CombineParams cp = {};
-    cp.n_cand = n_cand; cp.node_of = c.node_of; cp.top_len = (int32_t)c.top_len; cp.allowed = c.allowed;
+    cp.n_cand = n_cand; cp.node_of = c.node_of; cp.top_len = (int32_t)c.top_len;
     cp.out_p99 = c.d_out_p99; cp.out_miss = c.d_out_miss;
     int64_t region = 0;
     for (int s = 0; s < S; s++) {
@@ -1140,7 +1140,7 @@ static int estimate_shared(il_estimator *e, const il_stage_config *d_configs, in
     }
     IL_CUDA(cudaEventRecord(e->events[1], st));
     CombineParams cp = {};
-    cp.n_cand = n_cand; cp.node_of = node_of; cp.top_len = (int32_t)top_len; cp.allowed = allowed;
+    cp.n_cand = n_cand; cp.node_of = node_of; cp.top_len = (int32_t)top_len;
     cp.out_p99 = d_out_p99; cp.out_miss = d_out_miss;
     for (int s = 0; s < S; s++) {
         if (leaving[s] <= 0) continue;

@@ -249,6 +249,7 @@ struct NodeTopParams {
     int64_t *top;                 // [n_nodes][top_len] descending, zero-filled beyond the node's count
     int64_t *miss;                // [n_nodes]
     int64_t n_nodes;
+    int32_t one_pass;             // (set by the launch)
 };
 cudaError_t launch_node_top(const NodeTopParams &p, cudaStream_t stream);
 size_t node_top_smem(int top_len);
@@ -260,7 +261,6 @@ struct CombineParams {
     const int64_t *top[IL_MAX_STAGES];
     const int64_t *miss[IL_MAX_STAGES];
     int32_t top_len;
-    int64_t allowed;              // T = n - k
     int64_t *out_p99, *out_miss;
 };
 cudaError_t launch_prefix_combine(const CombineParams &p, cudaStream_t stream);

@@ -304,7 +304,9 @@ select_kernel(const __grid_constant__ SelectParams p)
 // being the number of queries allowed above it, so no node ever contributes more than its own T + 1
 // largest: they are kept, in descending order, for the combine step (prefix_kernel.cu), together with
 // the node's miss count.  One CTA per node: records -> latencies (in place), radix select of the
-// (T + 1)-th largest, collection of everything above it into shared memory, bitonic sort.
+// (T + 1)-th largest, collection of everything above it into shared memory, bitonic sort.  Where a row is several times as
+// long as the list a sample of it tells what to collect, and one pass that changes nothing does (2,816 rows of 10,500 to 35,000
+// records: 1.2 ms with lists of 1,001).
 __global__ void __launch_bounds__(kSelectThreads)
 node_top_kernel(const __grid_constant__ NodeTopParams p)
 {
@@ -313,16 +315,95 @@ node_top_kernel(const __grid_constant__ NodeTopParams p)
     __shared__ unsigned hist[256];
     __shared__ unsigned long long s_prefix, s_or;
     __shared__ unsigned s_rank, s_miss, s_fill;
+    __shared__ SelectShared sh;
 
     int pow2 = 1;
     while (pow2 < p.top_len) pow2 <<= 1;
     const uint64_t qmask = (1ull << p.qbits) - 1ull;
+    // bitonic sort of s_top[0 .. size), descending
+    auto sort = [&](int size) {
+        for (int k = 2; k <= size; k <<= 1) {
+            for (int j = k >> 1; j > 0; j >>= 1) {
+                for (int i = threadIdx.x; i < size; i += kSelectThreads) {
+                    const int partner = i ^ j;
+                    if (partner > i) {
+                        const int64_t a = s_top[i], b = s_top[partner];
+                        const bool desc = (i & k) == 0;
+                        if (desc ? a < b : a > b) { s_top[i] = b; s_top[partner] = a; }
+                    }
+                }
+                __syncthreads();
+            }
+        }
+    };
+    unsigned *bins = reinterpret_cast<unsigned *>(s_top + 2 * pow2);      // (one pass only)
     for (int64_t node = blockIdx.x; node < p.n_nodes; node += gridDim.x) {
         int64_t *lat = reinterpret_cast<int64_t *>(p.records + (p.row_of ? (int64_t)p.row_of[node] : node) * p.stride + p.offset);
         if (threadIdx.x == 0) { s_or = 0; s_miss = 0; s_fill = 0; s_prefix = 0; }
         __syncthreads();
         unsigned miss = 0;
         unsigned long long my_or = 0;
+        if (p.one_pass) {
+            // A sample (whole sectors, a sixteenth of the records) tells which latency somewhat more than top_len records reach;
+            // the pass that counts the misses collects those, and where at least top_len and at most twice the sort's
+            // size come together, the sort is all that is left.
+            for (int i = threadIdx.x; i < kSelBins; i += kSelectThreads) bins[i] = 0u;
+            __syncthreads();
+            for (int j = threadIdx.x; 64 * (j / 4) + 4 <= p.len; j += kSelectThreads) {
+                const uint64_t rec = (uint64_t)__ldg(lat + 64 * (j / 4) + j % 4);
+                atomicAdd(&bins[first_bin((rec >> p.qbits) - (uint64_t)__ldg(p.arrival + (rec & qmask)))], 1u);
+            }
+            __syncthreads();
+            const unsigned sampled = 4u * (unsigned)((p.len - 4) / 64 + 1);
+            const unsigned upper = min(sampled - 1u, (unsigned)((1.35 * p.top_len + 64.0) * sampled / p.len));
+            find_rank<kSelBins / kSelectThreads>(bins, sampled - upper, sh);
+            const int64_t from = sh.bin < 256u ? (int64_t)sh.bin : (int64_t)(sh.bin - ((sh.bin >> 7) - 1u) * 128u) << ((sh.bin >> 7) - 1u);
+            constexpr int kAhead = 4;
+            uint64_t next[kAhead];
+            auto request = [&](int base) {
+#pragma unroll
+                for (int u = 0; u < kAhead; u++) {
+                    const int i = base + u * kSelectThreads + (int)threadIdx.x;
+                    next[u] = i < p.len ? (uint64_t)__ldg(lat + i) : 0ull;
+                }
+            };
+            request(0);
+            for (int base = 0; base < p.len; base += kAhead * kSelectThreads) {
+                uint64_t rec[kAhead];
+#pragma unroll
+                for (int u = 0; u < kAhead; u++) rec[u] = next[u];
+                request(base + kAhead * kSelectThreads);
+#pragma unroll
+                for (int u = 0; u < kAhead; u++) {
+                    if (base + u * kSelectThreads + (int)threadIdx.x >= p.len) continue;
+                    const int64_t l = (int64_t)(rec[u] >> p.qbits) - __ldg(p.arrival + (rec[u] & qmask));
+                    miss += l > p.slo_us;
+                    if (l >= from) {
+                        const unsigned pos = atomicAdd(&s_fill, 1u);
+                        if (pos < 2u * (unsigned)pow2) s_top[pos] = l;
+                    }
+                }
+            }
+            for (int o = 16; o > 0; o >>= 1) miss += __shfl_xor_sync(0xffffffffu, miss, o);
+            if ((threadIdx.x & 31) == 0 && miss) atomicAdd(&s_miss, miss);
+            __syncthreads();
+            const int got = (int)s_fill;
+            if (got >= p.top_len && got <= 2 * pow2) {
+                const int size = got <= pow2 ? pow2 : 2 * pow2;
+                for (int i = got + (int)threadIdx.x; i < size; i += kSelectThreads) s_top[i] = 0;
+                __syncthreads();
+                sort(size);
+                int64_t *out = p.top + node * p.top_len;
+                for (int i = threadIdx.x; i < p.top_len; i += kSelectThreads) out[i] = s_top[i];
+                if (threadIdx.x == 0) p.miss[node] = (int64_t)s_miss;
+                __syncthreads();
+                continue;
+            }
+            __syncthreads();
+            if (threadIdx.x == 0) { s_miss = 0; s_fill = 0; }
+            miss = 0;
+            __syncthreads();
+        }
         for (int i = threadIdx.x; i < p.len; i += kSelectThreads) {
             const uint64_t rec = (uint64_t)lat[i];
             const int64_t l = (int64_t)(rec >> p.qbits) - p.arrival[rec & qmask];
@@ -376,20 +457,7 @@ node_top_kernel(const __grid_constant__ NodeTopParams p)
         const int keep = p.len > p.top_len ? p.top_len : got;
         for (int i = got + (int)threadIdx.x; i < pow2; i += kSelectThreads) s_top[i] = i < keep ? threshold : 0;
         __syncthreads();
-        // bitonic sort, descending
-        for (int k = 2; k <= pow2; k <<= 1) {
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                for (int i = threadIdx.x; i < pow2; i += kSelectThreads) {
-                    const int partner = i ^ j;
-                    if (partner > i) {
-                        const int64_t a = s_top[i], b = s_top[partner];
-                        const bool desc = (i & k) == 0;
-                        if (desc ? a < b : a > b) { s_top[i] = b; s_top[partner] = a; }
-                    }
-                }
-                __syncthreads();
-            }
-        }
+        sort(pow2);
         int64_t *out = p.top + node * p.top_len;
         for (int i = threadIdx.x; i < p.top_len; i += kSelectThreads) out[i] = s_top[i];
         if (threadIdx.x == 0) p.miss[node] = (int64_t)s_miss;
@@ -404,9 +472,13 @@ size_t node_top_smem(int top_len)
     return pow2 * sizeof(int64_t);
 }
 
-cudaError_t launch_node_top(const NodeTopParams &p, cudaStream_t stream)
+cudaError_t launch_node_top(const NodeTopParams &q, cudaStream_t stream)
 {
-    const size_t smem = node_top_smem(p.top_len);
+    NodeTopParams p = q;
+    size_t smem = node_top_smem(p.top_len);
+    // in one pass where a row is several times what is kept of it, and both the longer list and the sample's bins fit
+    p.one_pass = p.len >= kSelOnePass / 4 && p.len >= 4 * p.top_len && smem <= 32768;
+    if (p.one_pass) smem = 2 * smem + kSelBins * sizeof(unsigned);
     cudaError_t e = cudaFuncSetAttribute(node_top_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int grid = (int)(p.n_nodes < 148 * 8 ? p.n_nodes : 148 * 8);

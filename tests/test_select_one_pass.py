@@ -51,3 +51,32 @@ def test_percentile_of_long_rows(case, n):
         for slo in (int(np.median(want)), p99, 0):
             a, b = est.estimate(w.configs, slo)
             assert a[0] == p99 and b[0] == int((want > slo).sum()), (slo, a, b, p99)
+
+
+@pytest.mark.parametrize("n", [4095, 4096, 4099, 12_000])
+@pytest.mark.parametrize("case", ["ordinary", "one_value", "few_late"])
+@pytest.mark.parametrize("tree", [False, True])
+def test_largest_latencies_of_shared_nodes(oracle, tree, case, n):
+    """The same for the lists of the largest latencies per node that a shared batch is put together from: ordinary rows, rows
+    of one value (everything reaches what the sample says) and rows whose late queries the sample does not see."""
+    import workloads
+    import paper_1812_01776_b200 as il
+    w = workloads.random_small(n, S=4 if tree else 2, H=2, Bmax=4, n=n, C=40, max_replicas=6, tree=False, qps=300.0, cv=3.0, lat_lo=1,
+                               lat_hi=9000)
+    if tree:
+        w.parent, w.cond_bit = np.array([-1, 0, 0, 2], np.int32), np.array([-1, 0, 0, 1], np.int8)
+        w.cond_val = np.array([0, 0, 1, 0], np.uint8)
+        w.branch_bits = np.random.default_rng(n).integers(0, 4, n).astype(np.uint8)
+    if case != "ordinary":
+        w.latency_us[:] = 100
+        w.arrival_us = np.arange(n, dtype=np.int64) * 1000
+        w.configs[:, :, 2] = 1
+        if case == "few_late":
+            late = np.nonzero((np.arange(n) % 64 == 40) & (np.arange(n) // 64 % 2 == 0))[0]
+            w.arrival_us[late] = w.arrival_us[late - 1]
+            w.configs[:, :, 1] = 1
+    exp = oracle.estimate_workload(w)
+    with il.Estimator.from_workload(w) as est:
+        est.set_test_knob(3, 1)
+        a, b = est.estimate(w.configs, w.slo_us)
+        assert np.array_equal(a, exp[0]) and np.array_equal(b, exp[1])
