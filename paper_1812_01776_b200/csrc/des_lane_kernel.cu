@@ -59,7 +59,7 @@
 //   * The profile tables are shared by the CTA, rows padded to an odd length so
 //     that rows of different lanes start in different banks.
 //   * What happens once per candidate or rarely (its first and last batch, spills,
-//     the iteration bound, the next candidate) is looked at once a turn of 8 to 30
+//     the iteration bound, the next candidate) is looked at once a turn of 8 to 62
 //     iterations only, behind one vote.
 //
 // Measured on B200, 4,096 candidates x 4 stages x 50,000 queries and 4,096 x 10 x 10^6: streams in global memory 15.4 / 720 ms;
@@ -83,7 +83,8 @@ constexpr uint64_t kInf = ~0ull;
 constexpr uint64_t kLatest = 0x7fefffffffffffffull;      // no record or key is larger
 constexpr int kX = 8;                         // records of a stream between two stages
 constexpr uint32_t kLast = 0x80000000u;       // flag of a batch's last record in that ring
-constexpr int kTurn = 16, kLongTurn = 32;     // iterations (two less) between two looks at finished groups, spills, bounds
+constexpr int kTurn = 16;                     // iterations (two less) between two looks at finished groups, spills, bounds, where a lane
+                                              // keeps much; else half of what a group has before it
 constexpr int kQuickTurn = 8;                 // the same while a stage is about to start or to end
 constexpr uint32_t kQuickLooks = 128;         // looks at a candidate within which a stage counts as about to start
 
@@ -479,8 +480,13 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
     // a spill has to start before a record still needed is overwritten, two turns from now at the latest
     const uint32_t reach = min((uint32_t)(nq - kTurn - 2), gmask - 2u * kTurn);
     // (and a turn may not be so long that it would come too late)
-    const uint32_t long_reach = gmask > 2u * kLongTurn && nq > kLongTurn + 2u ? min((uint32_t)(nq - kLongTurn - 2), gmask - 2u * kLongTurn) : 0u;
+    // (kept from the compiler, which schedules the loop of chains by 5 % worse when it knows where this comes from)
+    uint32_t half = ahead / 2u;
+    asm volatile("" : "+r"(half));
+    const uint32_t long_reach = gmask > 2u * half && nq > half + 2u ? min((uint32_t)(nq - half - 2), gmask - 2u * half) : 0u;
     const int most_kept = (int)min(nq, gmask + 1u) - 4;
+    const uint32_t poll = ahead > 64u ? 1u : 3u;       // cut: looks between two at the streams, less one
+    (void)poll;
     unsigned long long batches = 0, alg_ops = 0, exits_seen = 0, exits_due = 0;
     unsigned early = 0;          // candidates dropped before the end of the trace (feasibility only)
     unsigned long long naps = p.iter_limit ? p.iter_limit : cut.naps;      // bound on the sleeps of a warp
@@ -613,7 +619,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
     };
 
     for (;;) {
-        // ---- every kQuickTurn-th, kTurn-th or kLongTurn-th iteration: does a lane need more than its steps?  A stream at its start or its end, a
+        // ---- every turn of 8 to 62 iterations: does a lane need more than its steps?  A stream at its start or its end, a
         // candidate that is decided, records in reach of being overwritten, the iteration bound.  (Kept short: its
         // latency is on the chain of every iteration, a kTurn-th of it.)
         if (FEAS) test_late();
@@ -844,8 +850,8 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
             // no group has a turn's records before it: nothing is lost by waiting for the next ones
             const bool idle = !__any_sync(full, (is & kFirst) && (is & kHas) && !short_of(kTurn));
             look++;
-            if ((look & 3u) == 0u || idle) {
-                if (((look & 7u) == 0u || idle) && (is & kHas) && ((count_a && tail_a != pub_a) || (count_b && tail_b != pub_b))) {
+            if ((look & poll) == 0u || idle) {
+                if (((look & (2u * poll + 1u)) == 0u || idle) && (is & kHas) && ((count_a && tail_a != pub_a) || (count_b && tail_b != pub_b))) {
                     __threadfence();
                     if (count_a) stg32_shared(count_a, tail_a >> 3);
                     if (count_b) stg32_shared(count_b, (tail_b - from_b) >> 3);
@@ -879,7 +885,8 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
         // the first kQuickLooks looks has late records: no short turns for it.  The other lengths are two less than half of what a
         // group has before it: one record of that is missing when the first lane is at an odd one, since copies are of pairs.)
         const bool quick = (i != n_cur && !(is & kStarted) && (uint32_t)limit - turns < kQuickLooks) || (i == n_cur && bm != ~0u);
-        const int turn_its = (int)__reduce_min_sync(full, quick ? kQuickTurn : ahead < 2u * kLongTurn ? kTurn - 2 : i - low <= long_reach ? kLongTurn - 2 : CUT ? max(kTurn - 2, min(kLongTurn - 2, (most_kept - (int)(i - low)) & ~1)) : kTurn - 2);
+        const int turn_its = (int)__reduce_min_sync(full, quick ? kQuickTurn : i - low <= long_reach ? (int)half - 2 :
+                                                    CUT ? max(kTurn - 2, min((int)half - 2, (most_kept - (int)(i - low)) & ~1)) : kTurn - 2);
 
         // The group's next records: requested two turns before their use where they are there, by all lanes of the group.
         {

@@ -133,6 +133,10 @@ inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 // Words of examined records a lane keeps in shared memory before it spills: this many where the grid needs every
 // resident CTA, more where it leaves shared memory unused.
 constexpr int kLaneWords = 64, kLaneWordsMost = 256;
+// Traces from here on have 128 records of an arrival stream before a group instead of 64, and so turns twice as long, where a CTA
+// has its SM to itself (4,096 candidates of a chain of 4, 50,000 queries 6.36 for 6.50 ms; 64 of a chain of 2, 2,000 queries 308
+// for 297 us: the end of a stream is noticed once a turn).
+constexpr int64_t kLongTurnsFrom = 16384;
 
 bool use_packed(const il_estimator *e)
 {
@@ -233,9 +237,9 @@ Shape cut_shape(const il_estimator *e, int64_t n_cand, int lane_slots)
     auto stretch_fits = [&](int ctas) {
         int most = (int)std::min<int64_t>(kRootGroups, nodes);
         for (int t = t0; t < cut.n_part; t++) most = std::max(most, sh.groups[t] * (cut.part[t].len > 0 ? 1 : 2));
-        for (sh.ahead = 64; sh.ahead >= 32; sh.ahead >>= 1) {
+        for (sh.ahead = ctas == 1 && e->n >= kLongTurnsFrom ? 128 : 64; sh.ahead >= 32; sh.ahead >>= 1) {
             sh.stretch = lane_stretch_bytes(most, sh.ahead);
-            const size_t bytes = lane_smem(e, lane_slots, kLaneWords, sh.stretch);
+            const size_t bytes = lane_smem(e, lane_slots, sh.ahead > 64 ? 2 * kLaneWords : kLaneWords, sh.stretch);
             if (bytes <= e->smem_per_cta && (bytes + 1024) * ctas <= e->smem_per_sm) return true;
         }
         sh.ahead = 32;
@@ -787,7 +791,7 @@ static cudaError_t launch_lane(const il_estimator *e, DesParams p, int64_t ctas,
 {
     const size_t per_sm = (size_t)((ctas + e->num_sms - 1) / e->num_sms);
     auto fits = [&](size_t bytes) { return bytes <= e->smem_per_cta && (bytes + 1024) * per_sm <= e->smem_per_sm; };
-    p.lane_ahead = 64;
+    p.lane_ahead = per_sm == 1 && e->n >= kLongTurnsFrom && fits(lane_smem(e, e->lane_slots, 2 * kLaneWords, lane_stretch_bytes(p.cpw, 128))) ? 128 : 64;
     p.lane_stretch = lane_stretch_bytes(p.cpw, p.lane_ahead);
     widen(p.lane_words, [&] { return fits(lane_smem(e, e->lane_slots, p.lane_words, p.lane_stretch)); });
     return launch_des_lane(p, nullptr, (int)ctas, lane_smem(e, e->lane_slots, p.lane_words, p.lane_stretch), st);
