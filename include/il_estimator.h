@@ -190,8 +190,8 @@ typedef struct {
  * two calls are the same).  A handle with a join runs on one of the two kernels
  * that merge incoming streams, both reported as "des_kernel", whatever variant
  * is set: with IL_VARIANT_AUTO and IL_VARIANT_LANES the lane-parallel form
- * (des_join_lane_kernel in a profile), in which a join has a lane of its own that
- * merges the streams as they come, else (or where times do not fit a record) the
+ * (des_part_kernel in a profile), in which a join is a merge of its two streams
+ * as they come, else (or where times do not fit a record) the
  * kernel with separate streams (des_kernel in a profile), which builds the join's
  * arrival stream before it simulates the stage.  Every entry point works on such a
  * handle and gives the same results as on any other; il_feasible* evaluate it
@@ -257,9 +257,9 @@ IL_API int il_estimate_device(il_estimator *est, const il_stage_config *d_config
  * percentile pass, and drops a candidate as soon as more than n - k of its queries have missed the
  * objective (an overloaded candidate is decided within the first few per cent of the trace;
  * il_stats.early_exits counts them).  A feasible candidate is simulated to the end, so its answer is
- * exact too.  Needs no memory per query and candidate, and is several times faster than il_estimate for a
- * batch without feasible candidates; a batch of up to one warp per scheduler with some feasible ones takes
- * 3 to 19 % longer than il_estimate, since the comparison is on the loop's chain.  The warp-per-candidate kernels have no early exit: with them this call computes P99
+ * exact too.  Needs no memory per query and candidate except on pipelines with branches below branches, and is several
+ * times faster than il_estimate for a batch without feasible candidates; a batch of up to one warp per scheduler with
+ * some feasible ones takes up to 20 % longer, since the comparison is on the loop's chain.  The warp-per-candidate kernels have no early exit: with them this call computes P99
  * and compares.
  *   il_feasible         configs HOST [n][S], out_feasible HOST [n] bytes; candidates validated on the host
  *   il_feasible_device  DEVICE pointers; an invalid candidate makes the call return BAD_CONFIG

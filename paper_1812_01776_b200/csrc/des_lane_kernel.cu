@@ -861,6 +861,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
                     uint32_t word = 0;
                     if ((is & kFirst) && short_of(2u * ahead)) word = ldg32_acquire(src_count);
                     word = __shfl_sync(full, word, root_lane);
+                    __syncwarp();     // (what the first lane has acquired, the others of its group copy)
                     if (short_of(2u * ahead)) { set(kNobody, word == kDead); avail = (is & kNobody) ? avail : max(avail, word + odd); }
                 }
                 if (FEAS && (is & kFirst) && (is & kHas)) {

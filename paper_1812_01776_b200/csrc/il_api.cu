@@ -525,15 +525,15 @@ void build_parts(il_estimator *e)
         x.by_node = from_root;
         if (from_root) {
             e->stream_at[e->n_stream] = il_estimator::kAtNode;
-            x.off = (int32_t)e->node_elems; e->node_elems += even(len);
+            x.off = e->node_elems; e->node_elems += even(len);
             e->root_readers++;
         } else if (leaves && !e->fork) {
             e->stream_at[e->n_stream] = il_estimator::kInSlab;
-            x.off = (int32_t)leave_off;
+            x.off = leave_off;
             e->slab_streams = true;
         } else {
             e->stream_at[e->n_stream] = il_estimator::kExtra;
-            x.off = (int32_t)e->extra_elems; e->extra_elems += even(len);
+            x.off = e->extra_elems; e->extra_elems += even(len);
         }
         return (int8_t)e->n_stream++;
     };
@@ -567,7 +567,7 @@ void build_parts(il_estimator *e)
         } else if (s != 0) {
             in = edge(par, s, e->visits[s], leaves);
             // (the region of the chain's last stage)
-            if (e->stream_at[in] == il_estimator::kInSlab) cut.stream[in].off = (int32_t)exit_off[end];
+            if (e->stream_at[in] == il_estimator::kInSlab) cut.stream[in].off = exit_off[end];
         }
         part_of[s] = cut.n_part;
         LanePart &pt = cut.part[cut.n_part++];

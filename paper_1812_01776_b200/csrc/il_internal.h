@@ -106,7 +106,8 @@ struct LaneStream {
     uint64_t *base;
     uint32_t *count;              // [rows]
     int64_t stride;               // records from row to row
-    int32_t off, len;             // the stream's place in a row
+    int64_t off;                  // the stream's place in a row
+    int32_t len;
     int32_t by_node;
 };
 // What happens to the records of a part's last stage: all go one way (a stream, or out where records are plain anyway); all
