@@ -64,7 +64,8 @@
 //
 // Measured on B200, 4,096 candidates x 4 stages x 50,000 queries and 4,096 x 10 x 10^6: streams in global memory 15.4 / 720 ms;
 // streams in shared memory, the loop in C++ 6.94 / 348 ms (123 instructions an iteration, 220 cycles for a warp on its
-// own); the loop in PTX 6.74 / 302 ms (108 instructions, 184 cycles and the turns).  What costs there is latency between
+// own); the loop in PTX and twice as long turns where a CTA
+// has its SM to itself 6.37 / 302 ms (108 instructions, 184 cycles and the turns).  What costs there is latency between
 // dependent instructions (73 of 230 cycles) and the ALU pipe (compares, selects, logic: half the issue rate).  Learned on
 // the way: a bool that lives through the loop takes one of seven predicates and costs the schedule 15 % (two of them:
 // 6.94 -> 8.14 ms), so what a lane has to remember are bits of one register; the same instructions with the loads of the next
@@ -246,7 +247,7 @@ __device__ int lane_first_part(const LaneCut &cut, bool for_roots)
 // records); queries come in nearly in order, so a word is new when it is first needed, and one that had to make room
 // goes to global memory.  Bound by the latency of an iteration, a record each: the two heads from shared memory, their
 // order, the query's word: about 260 cycles.  511 candidates of a diamond, 50,000 queries: 53 ms with the merge in the stages'
-// loop, 14.1 as a part (29 with branches for the words, 23.3 with the words in global memory alone).
+// loop, 13.1 as a part (29 with branches for the words, 23.3 with the words in global memory alone).
 __device__ __noinline__ void lane_merge(const DesParams &p, const LaneCut &cut, int part, uint32_t tbw, uint32_t ahead, uint32_t cache, uint32_t entries,
                                         unsigned long long &naps, uint32_t &quit)
 {
@@ -403,10 +404,10 @@ __device__ __noinline__ void lane_merge(const DesParams &p, const LaneCut &cut, 
 //         * A part that only leaves the pipeline (the rule) needs no memory for its stream: the records come in the
 //           region of the candidate's slab row that they go to, and no record leaves before it was examined.
 //       Against one group of lanes for the whole tree (each lane as many iterations as the root has records, whatever
-//       its branch sees, and a branch step in the loop): 7,001 candidates of a tree of 6, 199,999 queries 70.6 -> 39.8 ms;
-//       8,192, feasibility only, 100,000 queries 35.1 -> 22.2 ms; a sweep over a tree of 8 20.6 -> 16.9 ms; fan-out,
-//       2,048 candidates of 6 stages, 100,000 queries 22.7 -> 17.7 ms.  Up to a warp per scheduler the root is what
-//       takes the time (250 cycles an iteration and 40 for its turns), beyond that the ALU pipe.
+//       its branch sees, and a branch step in the loop): 7,001 candidates of a tree of 6, 199,999 queries 66 -> 34 ms;
+//       8,192, feasibility only, 100,000 queries 35.1 -> 19.5 ms; the covering candidates of a sweep over a tree of 8 17.4 -> 14.6
+//       ms; fan-out, 2,048 candidates of 6 stages, 100,000 queries 21.7 -> 15.7 ms.  Up to a warp per scheduler the root is
+//       what takes the time (240 cycles an iteration and 30 for its turns), beyond that the ALU pipe.
 // FORK: fan-out (with CUT) -- a query goes down every edge whose condition holds, a copy that finds none leaves, and
 //       the slab keeps per query the record of the copy that left last.  Joins: the streams of a stage's two incoming edges
 //       are merged by a part of its own (lane_merge) before the part that begins with the stage.
@@ -844,7 +845,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
         uint32_t at = __shfl_sync(full, i, root_lane);      // records the group's first lane has examined
         if (CUT) {
             // ---- the streams between the parts: what has been written is published, and what others have written is
-            // looked up, every fourth turn or when there is nothing to do
+            // looked up, every fourth (second where turns are long) turn or when there is nothing to do
             const bool feeds = (is & kHas) && !(is & kBad) && !(is & kNobody) && !(is & kDecided);
             auto short_of = [&](uint32_t records) { return feeds && avail != n_first && avail - at < records; };
             // no group has a turn's records before it: nothing is lost by waiting for the next ones

@@ -169,9 +169,12 @@ bool is_cut(const il_estimator *e) { return is_lane(e) && e->cut.n_part > 0; }
 int warps_per_cta(const il_estimator *e) { return is_lane(e) ? des_lane_warps_per_cta() : kWarpsPerCta; }
 // A batch that leaves schedulers idle is spread over them first: a warp that has its scheduler to itself takes
 // the same time for one candidate as for cpw, and less where its lanes diverge.
+// (Pipelines cut into parts: lanes in use of a slot instead.)
+int64_t cut_lanes(const il_estimator *e, int64_t n_cand);
 int64_t cands_per_slot(const il_estimator *e, int64_t n_cand)
 {
-    if (!is_lane(e) || is_cut(e)) return 1;
+    if (is_cut(e)) return cut_lanes(e, n_cand);
+    if (!is_lane(e)) return 1;
     const int64_t schedulers = (int64_t)e->num_sms * 4;
     return std::max<int64_t>(1, std::min<int64_t>(e->cpw, (n_cand + schedulers - 1) / schedulers));
 }
@@ -193,7 +196,7 @@ bool looks_for_prefixes(const il_estimator *e, int64_t n_cand)
 // Stream memory of a slot that holds cps candidates.  Lane kernel: a spill ring for every lane in use.
 size_t slot_time_bytes(const il_estimator *e, int64_t cps)
 {
-    if (is_cut(e)) return (size_t)32 * 4 << e->lane_ring_log2;
+    if (is_cut(e)) return (size_t)cps * 4 << e->lane_ring_log2;
     return is_lane(e) ? (size_t)cps * e->S * 4 << e->lane_ring_log2 : (size_t)e->slot_elems * 8;
 }
 // Root nodes that so many candidates can have.
@@ -273,6 +276,15 @@ Shape cut_shape(const il_estimator *e, int64_t n_cand, int lane_slots)
     return sh;
 }
 
+// The most lanes that a warp of a launch over so many candidates (or fewer) uses: a spill ring for each.
+int64_t cut_lanes(const il_estimator *e, int64_t n_cand)
+{
+    const Shape sh = cut_shape(e, n_cand, e->lane_slots);
+    int64_t most = e->cut.shared ? std::min<int64_t>(kRootGroups, (most_nodes(e, n_cand) + 3) / 4) : 1;
+    for (int t = e->cut.shared ? 1 : 0; t < e->cut.n_part; t++) most = std::max<int64_t>(most, (int64_t)sh.groups[t] * e->cut.part[t].len);
+    return most;
+}
+
 size_t slot_qid_bytes(const il_estimator *e) { return is_lane(e) ? 0 : (size_t)e->slot_elems * 4; }
 size_t slot_bytes(const il_estimator *e, int64_t cps) { return slot_time_bytes(e, cps) + slot_qid_bytes(e); }
 size_t seen_bytes(const il_estimator *e) { return (size_t)e->cut.n_join * e->cut.seen_words * 4; }      // of a candidate, all its joins
@@ -341,7 +353,7 @@ int64_t fallback_slots(const il_estimator *e, size_t usable)
 size_t min_bytes(const il_estimator *e)
 {
     Plan pl;
-    pl.cps = is_lane(e) ? e->cpw : 1;
+    pl.cps = is_cut(e) ? 32 : is_lane(e) ? e->cpw : 1;
     pl.slots = warps_per_cta(e);
     pl.chunk = 2 * warps_per_cta(e);
     pl.fb_slots = lane_fallback(e) ? kWarpsPerCta : 0;
@@ -357,7 +369,9 @@ size_t recommended_bytes(const il_estimator *e, int64_t n_cand)
     pl.cps = cps;
     if (is_cut(e)) {
         pl.slots = std::max(pl.slots, wanted_slots(e, n_cand, 32));
-        pl.chunk = std::max<int64_t>(2 * warps_per_cta(e), std::min<int64_t>(n_cand, 8 * full_slots(e, 16) * e->cpw));
+        if (wanted_slots(e, n_cand, 16) != wanted_slots(e, n_cand, 32)) pl.cps = 32;
+        // (and some rows more, in which a small batch that shares prefixes keeps its nodes)
+        pl.chunk = 64 + std::max<int64_t>(2 * warps_per_cta(e), std::min<int64_t>(n_cand, 8 * full_slots(e, 16) * e->cpw));
     } else
     pl.chunk = std::max<int64_t>(std::min<int64_t>(n_cand, 8 * full_slots(e, 16) * cps), 2 * pl.slots * cps);
     pl.fb_slots = lane_fallback(e) ? (int64_t)e->num_sms * kWarpsPerCta : 0;
@@ -732,7 +746,7 @@ static DesParams chunk_params(const il_estimator *e, const Plan &pl, char *ws, c
     p.iter_limit = e->iter_limit;
     p.lane_slots = e->lane_slots;
     p.cpw = (int32_t)pl.cps;
-    p.lanes_per_slot = is_cut(e) ? 32 : (int32_t)pl.cps * e->S;
+    p.lanes_per_slot = is_cut(e) ? (int32_t)pl.cps : (int32_t)pl.cps * e->S;
     return p;
 }
 
@@ -1810,7 +1824,7 @@ static int feasible_device(il_estimator *e, const il_stage_config *d_configs, in
     // decided.  What that gives depends on the batch (50,000 queries, chain of 4 / tree of 6, il_estimate in brackets):
     // nothing feasible, one warp per scheduler 1.4 / 1.1 ms (7.1 / 9.4), three 1.7 / 1.5 ms (16.7 / 18.8); everything or
     // one in six feasible, one warp per scheduler 7.2 / 9.6 ms (6.9 / 9.3), where a warp ends with its last feasible
-    // candidate and an iteration takes 146 instead of 115 ns; the same with two and three warps 10.3 to 16.9 / 12.5 to
+    // candidate and an iteration takes 140 instead of 113 ns; the same with two and three warps 10.3 to 16.9 / 12.5 to
     // 17.4 ms (10.6 to 16.7 / 13 to 18.7).  It is also the way that needs no memory per candidate, so it is the only one.
     int rc = start_call(e, d_configs, n_cand, max_replicas);
     if (rc) return rc;
@@ -1867,7 +1881,7 @@ static int feasible_device(il_estimator *e, const il_stage_config *d_configs, in
         p.iter_limit = e->iter_limit;
         p.lane_slots = e->lane_slots;
         p.cpw = (int32_t)cands_per_slot(e, n_cand);
-        p.lanes_per_slot = is_cut(e) ? 32 : p.cpw * e->S;
+        p.lanes_per_slot = is_cut(e) ? (int32_t)pl.cps : p.cpw * e->S;
         p.out_feasible = d_out_feasible + lo;
         // latency > objective is tested on time fields shifted by qbits: keep the objective in that range
         // (latencies are at least 1 and every reachable time is below 2^(63 - qbits))
