@@ -1820,12 +1820,11 @@ static int feasible_device(il_estimator *e, const il_stage_config *d_configs, in
         return IL_OK;
     }
 
-    // Lane kernel: no slab and no percentile pass, so the whole batch is one chunk, and a candidate ends as soon as it is
-    // decided.  What that gives depends on the batch (50,000 queries, chain of 4 / tree of 6, il_estimate in brackets):
-    // nothing feasible, one warp per scheduler 1.4 / 1.1 ms (7.1 / 9.4), three 1.7 / 1.5 ms (16.7 / 18.8); everything or
-    // one in six feasible, one warp per scheduler 7.2 / 9.6 ms (6.9 / 9.3), where a warp ends with its last feasible
-    // candidate and an iteration takes 140 instead of 113 ns; the same with two and three warps 10.3 to 16.9 / 12.5 to
-    // 17.4 ms (10.6 to 16.7 / 13 to 18.7).  It is also the way that needs no memory per candidate, so it is the only one.
+    // Lane kernel: no percentile pass, and a candidate ends as soon as it is decided.  What that gives depends on the batch (50,000
+    // queries, chain of 4 / tree of 6, 2,048 and 6,000 candidates): nothing feasible 0.11 and 0.17 / 0.20 and 0.21 ms;
+    // everything or a part feasible 6.8 and 9.9 / 6.4 and 7.9 ms, where a warp ends with its last feasible candidate and an
+    // iteration takes 140 instead of 113 ns.  It is also the way that needs no memory per candidate (but for streams where
+    // branches lie below branches, which may make several chunks of the batch), so it is the only one.
     int rc = start_call(e, d_configs, n_cand, max_replicas);
     if (rc) return rc;
     char *ws = nullptr;
