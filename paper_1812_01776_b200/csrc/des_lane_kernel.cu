@@ -655,7 +655,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
         bool done = i == n_cur && bm == ~0u && epos == tpos && e_on == 0u;
         bool stop = FEAS && !CUT && (is & kHas) && missw[j] > p.miss_allow;       // this lane ends its group's candidate here
         if (CUT) stop = (is & kHas) && ((is & kNobody) || (is & kDecided) || quit);
-        bool give_up = CUT && (is & kHas) && (is & kNobody) && !(is & kDecided);
+        bool give_up = false;
         if (i - low > reach || (is & kSpill)) {
             // the oldest record still needed, exactly
             low = i - (bm + 1u);
@@ -684,6 +684,8 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
         }
         stop = (__ballot_sync(full, stop) & group_mask) != 0u;                // the whole group
         if (FEAS && CUT) set(kDecided, (__ballot_sync(full, (is & kDecided)) & group_mask) != 0u);
+        // (behind the vote: a producer also ends early because the candidate is decided, which the first lane alone has looked up)
+        if (CUT) give_up = (give_up || ((is & kHas) && (is & kNobody))) && !(is & kDecided);
         if (p.lane_wrap) {
             const bool group_gives_up = (__ballot_sync(full, give_up) & group_mask) != 0u;
             if (group_gives_up && !(is & kOver)) { is |= kOver; if ((is & kHas) && !per_node) p.ovf[c] = 1; }

@@ -108,3 +108,30 @@ def test_feasible_full_size_samples(il, oracle_on, cid):
     assert np.array_equal(got, want), np.nonzero(got != want)[0][:8]
     if cid == 2:
         assert st["early_exits"] > 0.5 * (~got).sum()
+
+
+@pytest.mark.parametrize("n,C", [(9000, 300), (20000, 120)])
+def test_decided_candidates_are_not_evaluated_again(il, oracle_pool, n, C):
+    """A tree with branches below branches and a chain of two stages behind one of them, streams longer than a spill ring
+    (so that lanes can give candidates up at all), half of the batch infeasible: a candidate that is decided ends in
+    every part, also in those whose stream then never comes to its end, and none of them is handed to the
+    warp-per-candidate kernel.  (Where a lane has to give up for want of room the estimate gives up as well: none here.)"""
+    import oracle
+    import torch
+    w = workloads.make(5, n_queries=n, n_candidates=C)
+    exp_p99, _ = oracle.estimate_many_parallel(w.parent, w.cond_bit, w.cond_val, w.latency_us, w.arrival_us, w.branch_bits,
+                                               w.configs, w.slo_us, pool=oracle_pool)
+    at = np.arange(8 * C) % C
+    d = torch.from_numpy(np.ascontiguousarray(w.configs[at])).cuda()
+    with il.Estimator.from_workload(w) as est:
+        est.set_test_knob(3, 2)
+        est.estimate_device(d, w.slo_us)
+        assert est.stats()["fallback_candidates"] == 0
+        given_up = early = 0
+        for slo in sorted({int(x) for x in np.quantile(exp_p99, np.linspace(0.02, 0.9, 23))}):
+            got = est.feasible_device(d, slo).cpu().numpy().astype(bool)
+            st = est.stats()
+            assert np.array_equal(got, exp_p99[at] <= slo)
+            given_up += st["fallback_candidates"]
+            early += st["early_exits"]
+        assert early > 0 and given_up == 0, (early, given_up)
