@@ -1629,8 +1629,6 @@ __global__ void __launch_bounds__(kNodeThreads) root_nodes_kernel(const RootNode
 template <typename K, typename... A>
 cudaError_t launch_one(K kernel, int grid, size_t smem, cudaStream_t stream, const A &...args)
 {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     kernel<<<grid, kLaneWarps * 32, smem, stream>>>(args...);
     return cudaGetLastError();
 }
@@ -1673,15 +1671,22 @@ size_t des_lane_smem(int table_rows, int Bmax, int ring_slots, int ring_words, i
            kSmemBase + ring_bytes(ring_slots, ring_words, stretch) + kTailBytes;
 }
 
-int des_lane_max_ctas_per_sm(size_t smem, bool cut)
+int des_lane_max_ctas_per_sm(size_t smem, bool cut, bool fork)
 {
+    // (all instantiations of one kind are compiled for the same number of CTAs; the last one of those that a handle can launch answers)
     int n = 0;
-    // (all instantiations of one kind are compiled for the same number of CTAs)
-    auto ask = [&](auto kernel) {
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) { cudaGetLastError(); return 0; }
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kLaneWarps * 32, smem) == cudaSuccess ? n : 0;
+    auto ask = [&](auto... kernels) {
+        cudaError_t e = cudaSuccess;
+        auto one = [&](auto kernel) {
+            if (e == cudaSuccess) e = allow_all_smem(kernel);
+            if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kLaneWarps * 32, smem);
+        };
+        (one(kernels), ...);
+        if (e != cudaSuccess) { cudaGetLastError(); n = 0; }
+        return n;
     };
-    return cut ? ask(des_part_kernel<true, false>) : ask(des_lane_kernel<true>);
+    if (!cut) return ask(des_lane_kernel<false>, des_lane_kernel<true>);
+    return fork ? ask(des_part_kernel<false, true>) : ask(des_part_kernel<false, false>, des_part_kernel<true, false>);
 }
 
 }  // namespace il

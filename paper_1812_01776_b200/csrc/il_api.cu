@@ -1469,12 +1469,13 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
         if (e->cut.n_part > 0) {
             int most = 1;
             for (int t = e->cut.shared ? 1 : 0; t < e->cut.n_part; t++) most = std::max(most, e->cut.part[t].len > 0 ? 32 / e->cut.part[t].len : 32);
-            e->ctas_lane[k] = std::max(1, des_lane_max_ctas_per_sm(lane_smem(e, slots, kLaneWords, lane_stretch_bytes(std::max(most, kRootGroups), 32)), true));
+            e->ctas_lane[k] = std::max(1, des_lane_max_ctas_per_sm(lane_smem(e, slots, kLaneWords, lane_stretch_bytes(std::max(most, kRootGroups), 32)), true, e->fork));
         } else {
-            e->ctas_lane[k] = des_lane_max_ctas_per_sm(lane_smem(e, slots, kLaneWords, lane_stretch_bytes(e->cpw, 64)), false);
+            e->ctas_lane[k] = des_lane_max_ctas_per_sm(lane_smem(e, slots, kLaneWords, lane_stretch_bytes(e->cpw, 64)), false, e->fork);
         }
     }
     e->ctas_per_sm_lane = e->ctas_lane[1];
+    if (cudaError_t ce = prepare_node_top(); ce != cudaSuccess) { g_last_cuda_error = (int)ce; return fail(IL_ERR_CUDA); }
     if (e->ctas_per_sm_wide < 1 || e->ctas_per_sm_packed < 1 || e->ctas_per_sm_staged < 1 ||
         e->ctas_per_sm_lane < 1) {
         g_last_cuda_error = (int)cudaErrorLaunchOutOfResources;

@@ -170,6 +170,21 @@ struct SelectParams {
     int64_t *out_miss;
 };
 
+// A kernel's limit of dynamic shared memory belongs to the function and not to a launch: handles on other threads share it.
+// So it is raised to what the device can give, the same for every handle, where a handle is created, and no launch touches it.
+template <typename K>
+inline cudaError_t allow_all_smem(K kernel)
+{
+    int dev = 0, most = 0;
+    cudaFuncAttributes a;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, kernel);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)a.sharedSizeBytes);
+    return e;
+}
+
 // Read-only view of what a handle has bound, for translation units that do not
 // see the handle's definition.
 struct BoundView {
@@ -197,7 +212,8 @@ int des_lane_warps_per_cta();
 // ring_slots: 16 or 32 batch ring positions per lane; ring_words: words of examined records (a power of two); stretch: bytes
 // of a warp's arrival streams
 size_t des_lane_smem(int table_rows, int Bmax, int ring_slots, int ring_words, int stretch);
-int des_lane_max_ctas_per_sm(size_t smem, bool cut);
+// (the three that ask for resident CTAs also prepare their kernels for launches: allow_all_smem)
+int des_lane_max_ctas_per_sm(size_t smem, bool cut, bool fork);
 enum SimKernel { kSimWide = 0, kSimPacked = 1, kSimPackedStaged = 2, kSimLane = 3 };
 inline cudaError_t launch_simulation(const DesParams &p, int kernel, int grid, size_t smem,
                                      cudaStream_t stream)
@@ -253,6 +269,7 @@ struct NodeTopParams {
     int32_t one_pass;             // (set by the launch)
 };
 cudaError_t launch_node_top(const NodeTopParams &p, cudaStream_t stream);
+cudaError_t prepare_node_top();      // once per handle, before the first launch
 size_t node_top_smem(int top_len);
 struct CombineParams {
     int64_t n_cand;
