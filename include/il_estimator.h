@@ -431,6 +431,8 @@ IL_API int il_set_variant(il_estimator *est, int variant);
  *                           them up by query index (0).  Same results either way.
  *   IL_KNOB_SMEM_SKIP       value 0..8192, a multiple of 16: the lane kernel leaves so many bytes unused where its
  *                           shared memory starts, as if that began elsewhere.  Same results.
+ *   IL_KNOB_LANE_SMS        value 0..1024: the lane kernel's CTAs tell only so many SMs apart (0: all), as if a kernel of
+ *                           somebody else's held the others and CTA after CTA came to the same few.  Same results.
  * Set a knob before il_workspace_bytes / il_set_workspace: sizes depend on the ring length.
  */
 #define IL_KNOB_LANE_RING_LOG2 1
@@ -439,6 +441,7 @@ IL_API int il_set_variant(il_estimator *est, int variant);
 #define IL_KNOB_LANE_CTAS 4
 #define IL_KNOB_BITS_IN_RECORDS 5
 #define IL_KNOB_SMEM_SKIP 6
+#define IL_KNOB_LANE_SMS 7
 IL_API int il_set_test_knob(il_estimator *est, int knob, int64_t value);
 
 /* Name of the simulation kernel the handle's next estimate call will launch

@@ -78,6 +78,7 @@ struct il_estimator {
     int64_t leaving[IL_MAX_STAGES] = {};       // queries (fan-out: copies) that leave after a stage
     int lane_slots = 32;               // batch ring positions used by the current call
     int64_t setup_launches = 0;        // kernels a call launched before its simulation: the replica reduction, the node probe
+    int lane_sms_knob = 0;             // test knob: SMs that the lane kernel's CTAs tell apart (0: all)
     int lane_ctas_knob = 0;            // test knob: resident CTAs per SM of the lane kernel at most (0: as many as fit)
     int *d_maxrep = nullptr;           // device word behind the status: largest replica count of a batch
     uint8_t *d_bits = nullptr;
@@ -820,6 +821,7 @@ static int enqueue_parts(il_estimator *e, DesParams p, const Plan &pl, char *ws,
     const bool feas = p.out_feasible != nullptr;
     uint32_t *words = reinterpret_cast<uint32_t *>(ws + pl.off_ctl);
     cut.num_sms = e->num_sms;
+    cut.sms_seen = e->lane_sms_knob;
     cut.ctl = words;
     cut.refs = words + kCtlWords + (size_t)e->n_stream * pl.chunk;
     int32_t *root_of = reinterpret_cast<int32_t *>(ws + pl.off_root);
@@ -1529,6 +1531,11 @@ int il_set_test_knob(il_estimator *e, int knob, int64_t value)
     if (knob == IL_KNOB_LANE_CTAS) {
         if (value < 0 || value > 16) return IL_ERR_INVALID_ARG;
         e->lane_ctas_knob = (int)value;
+        return IL_OK;
+    }
+    if (knob == IL_KNOB_LANE_SMS) {
+        if (value < 0 || value > 1024) return IL_ERR_INVALID_ARG;
+        e->lane_sms_knob = (int)value;
         return IL_OK;
     }
     if (knob == IL_KNOB_BITS_IN_RECORDS) {

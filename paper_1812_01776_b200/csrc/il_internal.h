@@ -127,6 +127,7 @@ struct LaneCut {
     int32_t n_part;               // part 0 is the root stage
     int32_t shared;               // simulated once per distinct configuration (root node); 0: per candidate, whose number is its node's
     int32_t num_sms;
+    int32_t sms_seen;             // test knob: SM numbers count modulo this (0: as they are)
     LanePart part[2 * IL_MAX_STAGES];
     LaneStream stream[3 * IL_MAX_STAGES];
     uint32_t *seen;               // [n_cand][joins][seen_words]: a bit per query of which one input has come in
@@ -139,7 +140,7 @@ struct LaneCut {
     unsigned long long naps;      // bound on the sleeps of a warp
 };
 constexpr int kRootGroups = 16;   // root nodes per warp
-constexpr uint32_t kCtlNodes = 0, kCtlOrder = 1, kCtlTicket = 2, kCtlWork = 16, kCtlSms = 1024, kCtlSlot = 64,
+constexpr uint32_t kCtlNodes = 0, kCtlOrder = 1, kCtlTicket = 2, kCtlLeft = 3, kCtlWork = 16, kCtlSms = 1024, kCtlSlot = 64,
                    kCtlRole = kCtlSlot + kCtlSms, kCtlWords = kCtlRole + kCtlSms;
 struct RootNodeParams {
     const il_stage_config *configs;

@@ -130,3 +130,27 @@ def test_iteration_bound(shape):
         assert ei.value.code == E.IL_ERR_ITER_LIMIT
         est.set_test_knob(2, 0)
         assert (est.estimate(w.configs, w.slo_us)[0] > 0).all()
+
+
+@pytest.mark.parametrize("C,sms", [(300, 1), (4096, 1), (4096, 2), (4096, 40)])
+def test_ctas_that_come_to_few_sms_still_work(oracle, C, sms):
+    """The first CTA on an SM may take it for root nodes, and others that come there leave.  Where the rest of the device is
+    taken by somebody else's kernel all CTAs come to the same few SMs; all but the planned ones must work all the same,
+    or the first few do everything (which takes some forty times as long)."""
+    import torch
+    import paper_1812_01776_b200 as il
+    w = workloads.make(3, n_queries=3000, n_candidates=400)
+    exp = oracle.estimate_workload(w)
+    at = np.arange(C) % 400
+    d = torch.from_numpy(np.ascontiguousarray(w.configs[at])).cuda()
+    ms = {}
+    with il.Estimator.from_workload(w) as est:
+        for seen in (0, sms):
+            est.set_test_knob(7, seen)
+            for _ in range(4):
+                p99, miss = est.estimate_device(d, w.slo_us)
+                assert np.array_equal(p99.cpu().numpy(), exp[0][at]) and np.array_equal(miss.cpu().numpy(), exp[1][at])
+                ms[seen] = min(ms.get(seen, 1e9), est.stats()["sim_ms"])
+            assert np.array_equal(est.feasible(w.configs[at], w.slo_us), exp[0][at] <= w.slo_us)
+    print(f"{C} candidates, {sms} SMs: {ms[0]:.2f} / {ms[sms]:.2f} ms")
+    assert ms[sms] < 4.0 * ms[0] + 0.5, ms
