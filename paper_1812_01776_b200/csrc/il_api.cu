@@ -851,7 +851,8 @@ static int enqueue_parts(il_estimator *e, DesParams p, const Plan &pl, char *ws,
         const bool asks = b.cbit_a[end] >= 0 || b.cbit_b[end] >= 0;
         if (pt.out_kind == kOutTwo && (pt.n_leave > 0 || pt.out_b < 0 || (asks && p.rec_bits == 0))) pt.out_kind = kOutAny;
         if (pt.out_kind == kOutTwo && !e->fork &&
-            (e->stream_at[pt.out_a] != e->stream_at[pt.out_b] || cut.stream[pt.out_b].off < cut.stream[pt.out_a].off))
+            (e->stream_at[pt.out_a] != e->stream_at[pt.out_b] ||
+             !one_row_counts(cut.stream[pt.out_a].off, cut.stream[pt.out_b].off, cut.stream[pt.out_b].len)))
             pt.out_kind = kOutAny;
     }
     IL_CUDA(cudaMemsetAsync(words, 0, pl.ctl_bytes, st));

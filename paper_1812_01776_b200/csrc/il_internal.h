@@ -113,6 +113,12 @@ struct LaneStream {
 // What happens to the records of a part's last stage: all go one way (a stream, or out where records are plain anyway); all
 // leave the pipeline; either of two streams of one row, by a branch bit that the records carry; any other two ways.
 constexpr int kOutOne = 0, kOutLeaf = 1, kOutTwo = 2, kOutAny = 3;
+// Whether the tails of two streams of a row can be counted from the first one's start: a lane keeps them as bytes in 32 bits.  (A
+// stream has fewer than 2^29 records, but in a deep tree the streams between the two may hold several times as many.)
+constexpr bool one_row_counts(int64_t off_a, int64_t off_b, int64_t len_b)
+{
+    return off_b >= off_a && off_b - off_a + len_b < (INT64_C(1) << 29);
+}
 struct LanePart {
     int8_t len;                   // a chain of so many stages; 0: the merge of a join's two streams, one lane
     int8_t stage[IL_MAX_STAGES];  // (merge: the join)
