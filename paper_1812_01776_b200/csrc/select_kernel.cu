@@ -346,11 +346,12 @@ node_top_kernel(const __grid_constant__ NodeTopParams p)
         if (p.one_pass) {
             // A sample (whole sectors, a sixteenth of the records) tells which latency somewhat more than top_len records reach;
             // the pass that counts the misses collects those, and where at least top_len and at most twice the sort's
-            // size come together, the sort is all that is left.
+            // size come together, the sort is all that is left.  (Plain loads: where that fails the row is rewritten below, in
+            // this kernel, and what a kernel writes must not be read through the read-only path.)
             for (int i = threadIdx.x; i < kSelBins; i += kSelectThreads) bins[i] = 0u;
             __syncthreads();
             for (int j = threadIdx.x; 64 * (j / 4) + 4 <= p.len; j += kSelectThreads) {
-                const uint64_t rec = (uint64_t)__ldg(lat + 64 * (j / 4) + j % 4);
+                const uint64_t rec = (uint64_t)lat[64 * (j / 4) + j % 4];
                 atomicAdd(&bins[first_bin((rec >> p.qbits) - (uint64_t)__ldg(p.arrival + (rec & qmask)))], 1u);
             }
             __syncthreads();
@@ -364,7 +365,7 @@ node_top_kernel(const __grid_constant__ NodeTopParams p)
 #pragma unroll
                 for (int u = 0; u < kAhead; u++) {
                     const int i = base + u * kSelectThreads + (int)threadIdx.x;
-                    next[u] = i < p.len ? (uint64_t)__ldg(lat + i) : 0ull;
+                    next[u] = i < p.len ? (uint64_t)lat[i] : 0ull;
                 }
             };
             request(0);

@@ -37,3 +37,13 @@ def test_tails_of_two_streams_of_a_row(tmp_path):
                            str(src), "-o", str(exe), "-L" + os.path.join(cuda, "lib64"), "-lcudart"])
     run = subprocess.run([str(exe)], capture_output=True, text=True)
     assert run.returncode == 0, run.stdout
+
+
+def test_rows_that_a_kernel_rewrites_are_read_by_plain_loads():
+    """node_top_kernel turns a row's records into latencies in place where its one-pass form does not hold: no access to the row
+    may take the read-only path (__ldg, ld.global.nc, a pointer said to be const and restrict)."""
+    text = open(os.path.join(ROOT, "paper_1812_01776_b200", "csrc", "select_kernel.cu")).read()
+    kernel = text[text.index("node_top_kernel(const __grid_constant__"):text.index("size_t node_top_smem")]
+    assert "lat[i] = l;" in kernel                                       # it does rewrite the row
+    for way in ("__ldg(lat", "__ldg(p.records", "ld.global.nc", "__restrict__"):
+        assert way not in kernel, way
