@@ -1838,7 +1838,9 @@ static int feasible_device(il_estimator *e, const il_stage_config *d_configs, in
     if (rc) return rc;
     char *ws = nullptr;
     size_t ws_bytes = 0;
-    rc = acquire_workspace(e, std::min<int64_t>(n_cand, 4096), &ws, &ws_bytes);
+    // (rows for all candidates where parts keep streams per candidate; else spill rings for a few thousand are all that is needed)
+    const bool rows = is_cut(e) && (e->slab_streams || e->extra_elems > 0);
+    rc = acquire_workspace(e, rows ? n_cand : std::min<int64_t>(n_cand, 4096), &ws, &ws_bytes);
     if (rc) return rc;
     if (looks_for_prefixes(e, n_cand)) {
         // a batch full of common configuration prefixes is cheaper to evaluate node by node

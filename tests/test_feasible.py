@@ -135,3 +135,20 @@ def test_decided_candidates_are_not_evaluated_again(il, oracle_pool, n, C):
             given_up += st["fallback_candidates"]
             early += st["early_exits"]
         assert early > 0 and given_up == 0, (early, given_up)
+
+
+@pytest.mark.parametrize("C", [8192, 12001])
+def test_own_workspace_holds_the_rows_of_nested_branches(il, oracle, C):
+    """Pipelines with branches below branches keep streams per candidate in feasibility-only mode too.  The workspace that the
+    library allocates for a call holds them for the whole batch, as it does for an estimate: each further chunk would
+    cost the root's chain once more."""
+    w = workloads.make(5, n_queries=20_000, n_candidates=40)
+    exp_p99, _ = oracle.estimate_workload(w)
+    at = np.arange(C) % 40
+    cfg, slo = np.ascontiguousarray(w.configs[at]), int(np.median(exp_p99))
+    with il.Estimator.from_workload(w) as est:
+        est.set_test_knob(3, 2)
+        assert np.array_equal(est.feasible(cfg, slo), exp_p99[at] <= slo)
+        assert est.stats()["chunks"] == 1
+        p99, _ = est.estimate(cfg, slo)
+        assert np.array_equal(p99, exp_p99[at]) and est.stats()["chunks"] == 1
