@@ -233,9 +233,9 @@ IL_API int il_estimate(il_estimator *est, const il_stage_config *configs, int64_
  * Shared prefixes.  The completion stream of a stage depends only on the
  * configurations of the stages on its path from the root, so candidates that
  * agree there need that part simulated once.  With the default kernel choice
- * (IL_VARIANT_AUTO), a batch of at least 2,048 candidates and more than the
+ * (IL_VARIANT_AUTO), a batch of at least 2,048 candidates that is larger than the
  * lane kernel takes at once with one warp per scheduler (592 x floor(32 / S)
- * on a B200), n - ceil(0.99 n) < 16,384 and enough workspace, the call first builds the set of distinct (stage,
+ * on a B200) or would take several chunks, n - ceil(0.99 n) < 16,384 and enough workspace, the call first builds the set of distinct (stage,
  * configuration, parent) nodes on the device; if there are at most a quarter as
  * many nodes as candidates x stages (an exhaustive sweep over per-stage choices,
  * not a uniform random draw) it simulates the nodes instead of the candidates --

@@ -180,17 +180,20 @@ int64_t cands_per_slot(const il_estimator *e, int64_t n_cand)
     return std::max<int64_t>(1, std::min<int64_t>(e->cpw, (n_cand + schedulers - 1) / schedulers));
 }
 
-// Whether a call looks its batch over for shared prefixes (3 S kernels, S table clears and a wait).  Not where every
-// candidate has a group of lanes on a scheduler's only warp: such a grid takes the time of one warp over the trace, and
-// with fewer candidates it would take the same.  Product sweeps over a tree of 8 (2,368 candidates are a wave), looked
-// over and not: 2,304 candidates, 4,000 queries 1.07 / 0.79 ms, 50,000 queries 8.76 / 8.66 ms; 8,192 candidates 1.11 /
-// 2.24 and 8.81 / 28.4 ms.  (Over a tree of 6, 2,916 candidates, 50,000 queries, it gains 3 % within a wave: 8.75 / 9.0 ms,
-// the lanes of fewer candidates diverge less.)  A Planner's calls are mostly within a wave, its questions share next to
-// nothing, and looking cost each of them 0.1 to 0.3 ms of 2.5 to 5.
-bool looks_for_prefixes(const il_estimator *e, int64_t n_cand)
+// Whether a call looks its batch over for shared prefixes (3 S kernels, S table clears and a wait).  Not where a warp per
+// scheduler takes all candidates (floor(32 / S) each; pipelines cut into parts: somewhat more) in one chunk: such a grid takes
+// the time of one warp over the trace, and with fewer candidates it would take the same.  Product sweeps, looked over and not, 4,000 /
+// 50,000 queries, in ms: a tree of 8 (line at 2,368 candidates) with 2,304 candidates 1.00 / 6.95 and 0.74 / 7.16, with 4,608
+// 1.00 / 6.94 and 1.19 / 12.2; a tree of 6 (line at 2,960) with 2,304 candidates 0.85 / 6.79 and 0.70 / 6.74, with 8,192 1.20 / 10.6
+// and 1.23 / 12.5, with 16,384 0.90 / 6.9 and 1.66 / 18.2.  Between 2,960 and 6,000 candidates that tree of 6 loses (3,456:
+// 1.19 / 10.6 and 0.78 / 7.4): its rows have few distinct latencies, which the lists of the largest take several passes
+// over; other sweeps gain there.  A Planner's calls are mostly below the line, its questions share next to nothing, and looking
+// cost each of them 0.1 to 0.5 ms.  chunked: the batch would take several chunks, each of which costs the chain of one warp, where a
+// covering set may fit one.  2,304 candidates of that tree of 8, 50,000 queries, in room for 600 rows (six chunks): 50.2 ms, looked over 6.9.
+bool looks_for_prefixes(const il_estimator *e, int64_t n_cand, bool chunked)
 {
     if (e->share_mode != 0) return e->share_mode != 2;
-    const int64_t wave = is_lane(e) ? (int64_t)e->num_sms * 4 * e->cpw : 0;
+    const int64_t wave = is_lane(e) && !chunked ? (int64_t)e->num_sms * 4 * e->cpw : 0;
     return n_cand >= kShareMinCandidates && n_cand > wave;
 }
 
@@ -712,7 +715,7 @@ static char *host_results(il_estimator *e, int64_t n_cand)
 static const il_stage_config *small_configs(il_estimator *e, const il_stage_config *configs, int64_t n_cand)
 {
     const size_t bytes = (size_t)n_cand * e->S * sizeof(il_stage_config);
-    if (!is_lane(e) || looks_for_prefixes(e, n_cand) || bytes > kSmallConfigBytes) return nullptr;
+    if (!is_lane(e) || looks_for_prefixes(e, n_cand, false) || bytes > kSmallConfigBytes) return nullptr;
     memcpy(e->h_cfg, configs, bytes);
     return e->h_cfg;
 }
@@ -1041,20 +1044,21 @@ static int shared_by_cover(il_estimator *e, const SharedCommon &c, char *ws, siz
 // completion stream at the end of that path; the batch is turned into the set of distinct (stage,
 // configuration, parent node) nodes, every node is simulated once, and each candidate's P99 and miss
 // count are put together from the nodes where its queries leave (prefix_kernel.cu).  Used when the
-// node count is at most a quarter of candidates x stages (exhaustive sweeps over per-stage choices);
+// node count is at most a quarter of candidates x stages (exhaustive sweeps over per-stage choices); chunked: the whole
+// batch would not fit one chunk otherwise;
 // *used tells whether the batch was evaluated here.
 constexpr int kShareMaxTop = 16384;
 
 static int estimate_shared(il_estimator *e, const il_stage_config *d_configs, int64_t n_cand, int64_t slo_us,
-                           int64_t *d_out_p99, int64_t *d_out_miss, char *ws, size_t ws_bytes, bool *used)
+                           int64_t *d_out_p99, int64_t *d_out_miss, char *ws, size_t ws_bytes, bool chunked, bool *used)
 {
     *used = false;
     const int S = e->S;
     const int64_t n = e->n;
     const int64_t allowed = n - (99 * n + 99) / 100;           // T: queries allowed above the P99
     const int64_t top_len = allowed + 1;
-    if (!looks_for_prefixes(e, n_cand) || e->fork || !e->can_pack || e->variant != IL_VARIANT_AUTO ||
-        top_len > kShareMaxTop || n_cand >= (INT64_C(1) << 30))
+    if (e->fork || !e->can_pack || e->variant != IL_VARIANT_AUTO || top_len > kShareMaxTop || n_cand >= (INT64_C(1) << 30) ||
+        !looks_for_prefixes(e, n_cand, chunked))
         return IL_OK;
     uint32_t cap = 1024;
     while ((int64_t)cap < 2 * n_cand) cap <<= 1;
@@ -1630,11 +1634,12 @@ static int estimate_device(il_estimator *e, const il_stage_config *d_configs, in
     size_t ws_bytes = 0;
     int wrc = acquire_workspace(e, n_cand, &ws, &ws_bytes);
     if (wrc) return wrc;
-    bool shared = false;
-    int src = estimate_shared(e, d_configs, n_cand, slo_us, d_out_p99, d_out_miss, ws, ws_bytes, &shared);
-    if (shared || src) return src;
     Plan pl;
-    if (!make_plan(e, ws_bytes, n_cand, pl)) return IL_ERR_NOMEM;
+    const bool planned = make_plan(e, ws_bytes, n_cand, pl);
+    bool shared = false;
+    int src = estimate_shared(e, d_configs, n_cand, slo_us, d_out_p99, d_out_miss, ws, ws_bytes, planned && pl.chunk < n_cand, &shared);
+    if (shared || src) return src;
+    if (!planned) return IL_ERR_NOMEM;
 
     const int64_t n_chunks = (n_cand + pl.chunk - 1) / pl.chunk;
     int rc = ensure_events(e, (size_t)(2 + 3 * n_chunks));
@@ -1842,12 +1847,29 @@ static int feasible_device(il_estimator *e, const il_stage_config *d_configs, in
     const bool rows = is_cut(e) && (e->slab_streams || e->extra_elems > 0);
     rc = acquire_workspace(e, rows ? n_cand : std::min<int64_t>(n_cand, 4096), &ws, &ws_bytes);
     if (rc) return rc;
-    if (looks_for_prefixes(e, n_cand)) {
+    const int64_t wpc = des_lane_warps_per_cta();
+    const size_t sb = slot_time_bytes(e, cands_per_slot(e, n_cand));
+    const size_t tail_bytes = align_up((size_t)n_cand, 256) + align_up((size_t)n_cand * 4, 256) + 1024;
+    Plan pl;
+    int64_t slots = 0;
+    bool planned = ws_bytes >= tail_bytes + (size_t)wpc * sb;
+    if (planned && is_cut(e)) {
+        pl.feas = true;
+        pl.slab = e->slab_streams;
+        planned = make_plan(e, ws_bytes - tail_bytes, n_cand, pl);
+        slots = pl.slots;
+    } else if (planned) {
+        pl.chunk = n_cand;
+        slots = std::min<int64_t>(wanted_slots(e, n_cand, e->lane_slots), (int64_t)((ws_bytes - tail_bytes) / sb)) / wpc * wpc;
+        planned = slots >= wpc;
+    }
+    const bool chunked = planned && pl.chunk < n_cand;
+    if (looks_for_prefixes(e, n_cand, chunked)) {
         // a batch full of common configuration prefixes is cheaper to evaluate node by node
         rc = ensure_staging(e, n_cand);
         if (rc) return rc;
         bool shared = false;
-        rc = estimate_shared(e, d_configs, n_cand, slo_us, e->d_out, e->d_out + e->d_out_cap, ws, ws_bytes, &shared);
+        rc = estimate_shared(e, d_configs, n_cand, slo_us, e->d_out, e->d_out + e->d_out_cap, ws, ws_bytes, chunked, &shared);
         if (rc) return rc;
         if (shared) {
             IL_CUDA(launch_feasible_from_p99(e->d_out, nullptr, n_cand, slo_us, d_out_feasible, st));
@@ -1856,22 +1878,7 @@ static int feasible_device(il_estimator *e, const il_stage_config *d_configs, in
             return IL_OK;
         }
     }
-    const int64_t wpc = des_lane_warps_per_cta();
-    const size_t sb = slot_time_bytes(e, cands_per_slot(e, n_cand));
-    const size_t tail_bytes = align_up((size_t)n_cand, 256) + align_up((size_t)n_cand * 4, 256) + 1024;
-    if (ws_bytes < tail_bytes + (size_t)wpc * sb) return IL_ERR_NOMEM;
-    Plan pl;
-    int64_t slots = 0;
-    if (is_cut(e)) {
-        pl.feas = true;
-        pl.slab = e->slab_streams;
-        if (!make_plan(e, ws_bytes - tail_bytes, n_cand, pl)) return IL_ERR_NOMEM;
-        slots = pl.slots;
-    } else {
-        pl.chunk = n_cand;
-        slots = std::min<int64_t>(wanted_slots(e, n_cand, e->lane_slots), (int64_t)((ws_bytes - tail_bytes) / sb)) / wpc * wpc;
-        if (slots < wpc) return IL_ERR_NOMEM;
-    }
+    if (!planned) return IL_ERR_NOMEM;
     const size_t off_ovf = is_cut(e) ? align_up(ws_bytes - tail_bytes, 256) : align_up((size_t)slots * sb, 256);
     const size_t off_order = off_ovf + align_up((size_t)n_cand, 256);
     rc = ensure_events(e, 4);

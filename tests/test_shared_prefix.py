@@ -112,6 +112,31 @@ def test_batches_of_one_wave_are_not_looked_over(il, oracle, over):
         assert np.array_equal(est.feasible(w.configs[at], w.slo_us), exp[0][at] <= w.slo_us)
 
 
+@pytest.mark.parametrize("call", ["estimate", "feasible"])
+def test_batches_of_one_wave_that_take_several_chunks_are_looked_over(il, oracle, call):
+    """With room for all rows a product sweep within one wave is simulated as it is; where the workspace makes several chunks
+    of it, each of which costs the chain of a warp over the trace, its covering set is simulated in one."""
+    import torch
+    w = workloads.make(5, n_queries=3000, n_candidates=8)
+    w.configs = product_configs(np.random.default_rng(5), 8, 4, 64, 16, [4, 4, 2, 2, 2, 2, 3, 3])
+    n, some = len(w.configs), np.arange(0, len(w.configs), 37)
+    assert 2048 <= n <= 592 * 4
+    exp = oracle.estimate_many(w.parent, w.cond_bit, w.cond_val, w.latency_us, w.arrival_us, w.branch_bits, w.configs[some], w.slo_us)
+    d = torch.from_numpy(w.configs).cuda()
+    with il.Estimator.from_workload(w) as est:
+        full = est.reserve_workspace(n)
+        for room in (full, il.il_workspace_min_bytes(est._h) + 700 * 3008 * 8 * 2):
+            est._ws = None
+            est.reserve_workspace(n, max_bytes=room)
+            if call == "estimate":
+                p99, miss = est.estimate_device(d, w.slo_us)
+                assert np.array_equal(p99.cpu().numpy()[some], exp[0]) and np.array_equal(miss.cpu().numpy()[some], exp[1])
+            else:
+                assert np.array_equal(est.feasible_device(d, w.slo_us).cpu().numpy()[some], exp[0] <= w.slo_us)
+            st = est.stats()
+            assert st["chunks"] == 1 and (st["stage_runs"] == n * 8 if room == full else st["stage_runs"] * 4 <= n * 8), st
+
+
 def test_sharing_with_latencies_above_2_32_and_one_query(il, oracle):
     w = workloads.random_small(102, S=2, H=1, Bmax=2, n=3000, C=4, max_replicas=1,
                                lat_lo=2_000_000_000, lat_hi=2_100_000_000)
