@@ -389,6 +389,103 @@ __device__ __noinline__ void lane_merge(const DesParams &p, const LaneCut &cut, 
     }
 }
 
+// ---- One iteration of a lane, in PTX ------------------------------------------------------------------------------
+// Why PTX: a warp that has its scheduler to itself is bound by the iteration's latency.  A compare here takes the condition
+// before it along (setp.and), where the compiler joins finished predicates by instructions of their own, and what the next
+// iteration reads (its record, the room for the record in hand, the time of the open batch, the low part to hand on) is requested as soon as
+// it is known where it lies, before this iteration's stores.
+// The seven forms of the iteration (lane_simulation: step) are one text.  A form gives what is its own: more operands, more
+// registers, how the tails of its ways out move, the way out itself, how the deeper insertion is reached, what more it hands back.
+// Operands by number: 0 to 20 the state that all forms have, then what state a form adds, the inputs that all have, a form's.
+#define IL_LOAD(type, name, number) ".reg ." #type " " #name "; mov." #type " " #name ", %" #number ";\n"
+#define IL_STORE(type, name, number) "mov." #type " %" #number ", " #name ";\n"
+#define IL_STEP_STATE(X) \
+    X(b32, i, 0) X(b32, bm, 1) X(b32, lpos, 2) X(b32, lfull, 3) X(b32, tpos, 4) X(b32, at1, 5) X(b32, at2, 6) X(b64, tk, 7) \
+    X(b32, prev, 8) X(b64, rec, 9) X(b32, lat, 10) X(b32, xs, 11) X(b32, epos, 12) X(b32, efull, 13) X(b32, e_on, 14) \
+    X(b64, e_key, 15) X(b32, e_idx, 16) X(b32, qv, 17) X(b32, tail_a, 18) X(b32, rw, 19) X(b32, sa, 20)
+#define IL_STATE_OPERANDS \
+    "+r"(i), "+r"(bm), "+r"(lpos), "+r"(lfull), "+r"(tpos), "+r"(at1), "+r"(at2), "+l"(tk), "+r"(prev), "+l"(rec), "+r"(lat), \
+    "+r"(xs), "+r"(epos), "+r"(efull), "+r"(e_on), "+l"(e_key), "+r"(e_idx), "+r"(qv), "+r"(tail_a), "+r"(rw), "+r"(sa)
+#define IL_STEP_INPUTS(n0, n1, n2, n3, n4, n5, n6, n7, n8, n9, n10, n11, n12, n13, n14, n15, n16) \
+    IL_LOAD(b32, xin, n0) IL_LOAD(b32, xin_mask, n1) IL_LOAD(b32, xin_row, n2) IL_LOAD(b32, tab, n3) IL_LOAD(b32, kfb, n4) \
+    IL_LOAD(b32, kfm, n5) IL_LOAD(b32, kb, n6) IL_LOAD(b32, rm, n7) IL_LOAD(b32, mbm1, n8) IL_LOAD(b32, tick, n9) \
+    IL_LOAD(b32, qmask, n10) IL_LOAD(b32, tmask, n11) IL_LOAD(b32, qb, n12) IL_LOAD(b32, nqm, n13) IL_LOAD(b32, xa, n14) \
+    IL_LOAD(b32, xam, n15) IL_LOAD(b32, down, n16)
+#define IL_INPUT_OPERANDS \
+    "r"(xin), "r"(xin_mask), "r"(xin_row), "r"(tab), "r"(kfb), "r"(kfm), "r"(kb), "r"(rm), "r"(mbm1), "r"(tick), "r"(qmask), \
+    "r"(~qmask), "r"(qb), "r"(nq - 1u), "r"(xa), "r"(xam), "r"(down)
+// The record to examine: joins the open batch, or closes it and opens the next.  The record in hand: handed on where there is room.
+#define IL_EXAMINE \
+    "and.b32 a, epos, rm; or.b32 a, a, kb; ld.shared.b64 fk, [a];\n" \
+    "and.b32 a, lpos, kfm; or.b32 a, a, kfb; ld.shared.b64 kf, [a];\n" \
+    "ld.shared.b64 k1, [at1]; ld.shared.b64 k2, [at2];\n" \
+    "mov.b64 td, tk; mov.b64 {rl, rh}, rec; mov.u32 xs_was, xs; mov.u32 sa_was, sa;\n" \
+    "setp.ne.u32 t, tpos, efull; selp.b32 rh, rh, -1, t; mov.b64 r, {rl, rh};\n" \
+    "setp.ge.s32 taken, rh, 0; setp.ge.and.u32 t, bm, mbm1, taken; setp.gt.or.f64 open, r, td, t;\n" \
+    "sub.u32 y, i, bm; add.u32 y, y, -1;\n" \
+    "add.u32 wa, i, -1; and.b32 wa, wa, nqm; mad.lo.u32 wa, wa, 128, qb;\n" \
+    "@taken add.u32 i, i, 1; and.b32 xs, i, xin_mask; mad.lo.u32 xs, xs, xin_row, xin; ld.relaxed.cta.shared.b64 rec, [xs];\n" \
+    "setp.lt.s32 hand, rw, 0; setp.ne.and.u32 hand, e_on, 0, hand; setp.ge.and.s32 hd|ho, down, 0, hand; setp.lt.and.s32 fin, qv, 0, hand;\n" \
+    "and.b32 x, qv, 0x7fffffff; mov.b64 {lo, hi}, e_key; and.b32 lo, lo, tmask; or.b32 a, lo, x; mov.b64 v, {a, hi}; mov.u32 ta_was, tail_a;\n"
+// (the tails have moved) what the next iteration needs of the child's stream and of the tables; the next batch to hand on, if it may
+// leave; a record for the child.
+#define IL_FETCH \
+    "and.b32 sa, tail_a, xam; or.b32 sa, sa, xa; ld.relaxed.cta.shared.u32 rw, [sa+4];\n" \
+    "mad.wide.u32 key, lat, tick, tk; mov.b64 {kl, kh}, key; and.b32 kl, kl, tmask; or.b32 kl, kl, y; mov.b64 key, {kl, kh};\n" \
+    "@taken add.u32 bm, bm, 1; @open mov.u32 bm, 0; mad.lo.u32 a, bm, 4, tab; ld.shared.u32 lat, [a];\n" \
+    "setp.eq.or.u32 fetch, e_on, 0, fin; setp.ne.and.u32 fetch, epos, tpos, fetch; setp.le.and.f64 fetch, fk, td, fetch;\n" \
+    "mov.b64 {fl, fh}, fk;\n" \
+    "@hand add.u32 e_idx, e_idx, 1; @fetch and.b32 e_idx, fl, qmask; and.b32 a, e_idx, nqm; mad.lo.u32 a, a, 128, qb; ld.shared.u32 qv, [a];\n" \
+    "@hd st.relaxed.cta.shared.b64 [sa_was], v;\n"
+// The closed batch goes behind the last one of the ring or just before it; the replica that is free first; the record's low part
+// to the ring of examined records, its position in the stream emptied; counters.
+#define IL_INSERT \
+    "@fetch mov.b64 e_key, fk; @fin mov.u32 e_on, 0; @fetch mov.u32 e_on, 1; @fetch add.u32 epos, epos, 256; @fetch add.u32 efull, efull, 256;\n" \
+    "and.b32 at0, tpos, rm; or.b32 at0, at0, kb;\n" \
+    "setp.lt.f64 pf, kf, key; selp.b64 first, kf, key, pf;\n" \
+    "setp.eq.u32 pz, tpos, lfull; setp.lt.and.f64 pz, r, first, pz; selp.b64 first, first, r, pz;\n" \
+    "mov.b64 {fl, fh}, first; or.b32 fl, fl, qmask; mov.b64 first, {fl, fh}; selp.b64 tk, first, tk, open;\n" \
+    "setp.lt.and.f64 ov, key, k1, open; selp.u32 sd, at1, at0, ov;\n" \
+    "@open st.shared.b64 [sd], key; @ov st.shared.b64 [at0], k1;\n" \
+    "setp.lt.and.f64 dp, key, k2, ov; mov.u32 pos, tpos; mov.u32 left, lpos;\n" \
+    "setp.eq.and.u32 pop, tpos, lfull, open;\n" \
+    "mov.u32 word, prev; @open or.b32 word, word, 0x80000000; @taken st.shared.u32 [wa], word;\n" \
+    "@taken st.relaxed.cta.shared.u32 [xs_was+4], -1;\n" \
+    "@open add.u32 tpos, tpos, 256; @open mov.u32 at2, at1; @open mov.u32 at1, at0;\n" \
+    "@pop add.u32 lpos, lpos, 256; @pop add.u32 lfull, lfull, 256;\n" \
+    "@taken and.b32 prev, rl, qmask;\n"
+// A batch that goes further back, past the batches that finish later: four a round.  Each lane by itself, or (WARP) all lanes behind
+// a vote: chains of 4 take 6.7 ms with the one and 7.3 with the other, but feasibility only takes 20.2 with the vote for 21.3
+// and fan-out 17.6 for 17.9.
+#define IL_DEEPER(SKIP, FIRST, WHO, AGAIN) \
+    SKIP "\n" \
+    "mov.u32 sd, left; sub.u32 pos, pos, 256;\n" \
+    "DEEPER:\n" \
+    "sub.u32 left, pos, sd;\n" \
+    "and.b32 at0, pos, rm; or.b32 at0, at0, kb; sub.u32 a1, pos, 256; and.b32 a1, a1, rm; or.b32 a1, a1, kb;\n" \
+    "sub.u32 a2, pos, 512; and.b32 a2, a2, rm; or.b32 a2, a2, kb; sub.u32 a3, pos, 768; and.b32 a3, a3, rm; or.b32 a3, a3, kb;\n" \
+    "sub.u32 a4, pos, 1024; and.b32 a4, a4, rm; or.b32 a4, a4, kb;\n" \
+    "ld.shared.b64 e1, [a1]; ld.shared.b64 e2, [a2]; ld.shared.b64 e3, [a3]; ld.shared.b64 e4, [a4];\n" \
+    FIRST " setp.lt.and.f64 t, key, e1, t; setp.gt.and.u32 ov, left, 256, t; setp.lt.and.f64 ov, key, e2, ov;\n" \
+    "setp.gt.and.u32 pz, left, 512, ov; setp.lt.and.f64 pz, key, e3, pz; setp.gt.and.u32 pf, left, 768, pz; setp.lt.and.f64 pf, key, e4, pf;\n" \
+    "@t st.shared.b64 [at0], e1; @ov st.shared.b64 [a1], e2; @pz st.shared.b64 [a2], e3; @pf st.shared.b64 [a3], e4;\n" \
+    "@t mov.u32 at0, a1; @ov mov.u32 at0, a2; @pz mov.u32 at0, a3; @pf mov.u32 at0, a4; " WHO "st.shared.b64 [at0], key;\n" \
+    "sub.u32 pos, pos, 1024; " AGAIN "\n" \
+    "PLACED:\n"
+#define IL_DEEPER_LANE IL_DEEPER("@!dp bra PLACED;", "setp.gt.u32 t, left, 0;", "", "@pf bra DEEPER;")
+#define IL_DEEPER_WARP \
+    IL_DEEPER("vote.sync.any.pred pf, dp, 0xffffffff; @!pf bra.uni PLACED;", "setp.gt.and.u32 t, left, 0, dp;", "@dp ", \
+              "setp.ne.and.u32 dp, pos, 1, pf; vote.sync.any.pred pf, dp, 0xffffffff; @pf bra.uni DEEPER;")
+#define IL_STEP(MORE_STATE, INPUTS, REGISTERS, TAILS, OUT, DEEPER, MORE_BACK) \
+    "{\n" IL_STEP_STATE(IL_LOAD) MORE_STATE INPUTS \
+    ".reg .pred t, taken, open, pop, ov, dp, pz, pf, hand, hd, ho, fin, fetch;\n" \
+    ".reg .u32 at0, sd, rl, rh, kl, kh, fl, fh, word, wa, x, y, lo, hi, a, xs_was, sa_was, ta_was, pos, left, a1, a2, a3, a4;\n" \
+    ".reg .b64 kf, k1, k2, fk, key, td, r, first, v, e1, e2, e3, e4;\n" REGISTERS \
+    IL_EXAMINE TAILS IL_FETCH OUT IL_INSERT DEEPER IL_STEP_STATE(IL_STORE) MORE_BACK "}"
+// One way out: its tail; the record as it leaves the pipeline, without branch bits.
+#define IL_ONE_TAIL "@hand add.u32 tail_a, tail_a, tail_step;\n"
+#define IL_PLAIN_RECORD "mov.b64 w, {lo, hi}; shr.u64 w, w, rb; cvt.u64.u32 v, a; or.b64 w, w, v; "
+
 }  // namespace
 
 // FEAS: feasibility only (Section 4.3, "Feasible"): leaving queries are compared with the objective as
@@ -921,10 +1018,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
             if (__any_sync(full, near)) { copies_done(); __syncwarp(); }
         }
 
-        // One iteration, written in PTX for the sake of its latency, which a warp on its own is bound by: a compare there takes
-        // the condition before it along (setp.and), where the compiler joins finished predicates by instructions of their own,
-        // and what the next iteration reads (its record, the room for the record in hand, the time of the open batch, the low
-        // part to hand on) is requested as soon as it is known where it lies, before this iteration's stores.
+        // One iteration (IL_STEP), in the form that the way out of the group's last stage asks for.
         uint32_t xs = xin + (i & xin_mask) * xin_row, sa = xa | (tail_a & xam);
         uint64_t rec = lds64_shared(xs);                    // record to examine
         uint32_t rw = lds32_shared(sa + 4u);                // where the record in hand goes: empty?
@@ -952,548 +1046,85 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
             }
 #endif
             if constexpr (OUT == kOutOne) {
-                asm volatile(
-                    "{\n"
-                    ".reg .b32 i; .reg .b32 bm; .reg .b32 lpos; .reg .b32 lfull; .reg .b32 tpos; .reg .b32 at1; .reg .b32 at2;\n"
-                    ".reg .b64 tk; .reg .b32 prev; .reg .b64 rec; .reg .b32 lat; .reg .b32 xs; .reg .b32 epos; .reg .b32 efull;\n"
-                    ".reg .b32 e_on; .reg .b64 e_key; .reg .b32 e_idx; .reg .b32 qv; .reg .b32 tail_a; .reg .b32 rw; .reg .b32 sa;\n"
-                    ".reg .b32 xin; .reg .b32 xin_mask; .reg .b32 xin_row; .reg .b32 tab; .reg .b32 kfb; .reg .b32 kfm; .reg .b32 kb;\n"
-                    ".reg .b32 rm; .reg .b32 mbm1; .reg .b32 tick; .reg .b32 qmask; .reg .b32 tmask; .reg .b32 qb; .reg .b32 nqm;\n"
-                    ".reg .b32 xa; .reg .b32 xam; .reg .b32 down; .reg .b32 tail_step; .reg .b64 out;\n"
-                    "mov.b32 i, %0; mov.b32 bm, %1; mov.b32 lpos, %2; mov.b32 lfull, %3; mov.b32 tpos, %4; mov.b32 at1, %5;\n"
-                    "mov.b32 at2, %6; mov.b64 tk, %7; mov.b32 prev, %8; mov.b64 rec, %9; mov.b32 lat, %10; mov.b32 xs, %11;\n"
-                    "mov.b32 epos, %12; mov.b32 efull, %13; mov.b32 e_on, %14; mov.b64 e_key, %15; mov.b32 e_idx, %16; mov.b32 qv, %17;\n"
-                    "mov.b32 tail_a, %18; mov.b32 rw, %19; mov.b32 sa, %20; mov.b32 xin, %21; mov.b32 xin_mask, %22; mov.b32 xin_row, %23;\n"
-                    "mov.b32 tab, %24; mov.b32 kfb, %25; mov.b32 kfm, %26; mov.b32 kb, %27; mov.b32 rm, %28; mov.b32 mbm1, %29;\n"
-                    "mov.b32 tick, %30; mov.b32 qmask, %31; mov.b32 tmask, %32; mov.b32 qb, %33; mov.b32 nqm, %34; mov.b32 xa, %35;\n"
-                    "mov.b32 xam, %36; mov.b32 down, %37; mov.b32 tail_step, %38; mov.b64 out, %39;\n"
-                    ".reg .pred t, taken, open, pop, ov, dp, pz, pf, hand, hd, ho, fin, fetch;\n"
-                    ".reg .u32 at0, sd, rl, rh, kl, kh, fl, fh, word, wa, x, y, lo, hi, a, xs_was, sa_was, ta_was, pos, left, a1, a2, a3, a4;\n"
-                    ".reg .b64 kf, k1, k2, fk, key, td, r, first, v, e1, e2, e3, e4; .reg .b64 o;\n"
-                    "and.b32 a, epos, rm; or.b32 a, a, kb; ld.shared.b64 fk, [a];\n"
-                    "and.b32 a, lpos, kfm; or.b32 a, a, kfb; ld.shared.b64 kf, [a];\n"
-                    "ld.shared.b64 k1, [at1]; ld.shared.b64 k2, [at2];\n"
-                    "mov.b64 td, tk; mov.b64 {rl, rh}, rec; mov.u32 xs_was, xs; mov.u32 sa_was, sa;\n"
-                    "setp.ne.u32 t, tpos, efull; selp.b32 rh, rh, -1, t; mov.b64 r, {rl, rh};\n"
-                    "setp.ge.s32 taken, rh, 0; setp.ge.and.u32 t, bm, mbm1, taken; setp.gt.or.f64 open, r, td, t;\n"
-                    "sub.u32 y, i, bm; add.u32 y, y, -1;\n"
-                    "add.u32 wa, i, -1; and.b32 wa, wa, nqm; mad.lo.u32 wa, wa, 128, qb;\n"
-                    "@taken add.u32 i, i, 1; and.b32 xs, i, xin_mask; mad.lo.u32 xs, xs, xin_row, xin; ld.relaxed.cta.shared.b64 rec, [xs];\n"
-                    "setp.lt.s32 hand, rw, 0; setp.ne.and.u32 hand, e_on, 0, hand; setp.ge.and.s32 hd|ho, down, 0, hand; setp.lt.and.s32 fin, qv, 0, hand;\n"
-                    "and.b32 x, qv, 0x7fffffff; mov.b64 {lo, hi}, e_key; and.b32 lo, lo, tmask; or.b32 a, lo, x; mov.b64 v, {a, hi}; mov.u32 ta_was, tail_a;\n"
-                    "@hand add.u32 tail_a, tail_a, tail_step;\n"
-                    "and.b32 sa, tail_a, xam; or.b32 sa, sa, xa; ld.relaxed.cta.shared.u32 rw, [sa+4];\n"
-                    "mad.wide.u32 key, lat, tick, tk; mov.b64 {kl, kh}, key; and.b32 kl, kl, tmask; or.b32 kl, kl, y; mov.b64 key, {kl, kh};\n"
-                    "@taken add.u32 bm, bm, 1; @open mov.u32 bm, 0; mad.lo.u32 a, bm, 4, tab; ld.shared.u32 lat, [a];\n"
-                    "setp.eq.or.u32 fetch, e_on, 0, fin; setp.ne.and.u32 fetch, epos, tpos, fetch; setp.le.and.f64 fetch, fk, td, fetch;\n"
-                    "mov.b64 {fl, fh}, fk;\n"
-                    "@hand add.u32 e_idx, e_idx, 1; @fetch and.b32 e_idx, fl, qmask; and.b32 a, e_idx, nqm; mad.lo.u32 a, a, 128, qb; ld.shared.u32 qv, [a];\n"
-                    "@hd st.relaxed.cta.shared.b64 [sa_was], v;\n"
-                    "mad.wide.u32 o, ta_was, 1, out; @ho st.global.b64 [o], v;\n"
-                    "@fetch mov.b64 e_key, fk; @fin mov.u32 e_on, 0; @fetch mov.u32 e_on, 1; @fetch add.u32 epos, epos, 256; @fetch add.u32 efull, efull, 256;\n"
-                    "and.b32 at0, tpos, rm; or.b32 at0, at0, kb;\n"
-                    "setp.lt.f64 pf, kf, key; selp.b64 first, kf, key, pf;\n"
-                    "setp.eq.u32 pz, tpos, lfull; setp.lt.and.f64 pz, r, first, pz; selp.b64 first, first, r, pz;\n"
-                    "mov.b64 {fl, fh}, first; or.b32 fl, fl, qmask; mov.b64 first, {fl, fh}; selp.b64 tk, first, tk, open;\n"
-                    "setp.lt.and.f64 ov, key, k1, open; selp.u32 sd, at1, at0, ov;\n"
-                    "@open st.shared.b64 [sd], key; @ov st.shared.b64 [at0], k1;\n"
-                    "setp.lt.and.f64 dp, key, k2, ov; mov.u32 pos, tpos; mov.u32 left, lpos;\n"
-                    "setp.eq.and.u32 pop, tpos, lfull, open;\n"
-                    "mov.u32 word, prev; @open or.b32 word, word, 0x80000000; @taken st.shared.u32 [wa], word;\n"
-                    "@taken st.relaxed.cta.shared.u32 [xs_was+4], -1;\n"
-                    "@open add.u32 tpos, tpos, 256; @open mov.u32 at2, at1; @open mov.u32 at1, at0;\n"
-                    "@pop add.u32 lpos, lpos, 256; @pop add.u32 lfull, lfull, 256;\n"
-                    "@taken and.b32 prev, rl, qmask;\n"
-                    "@!dp bra PLACED;\n"
-                    "mov.u32 sd, left; sub.u32 pos, pos, 256;\n"
-                    "DEEPER:\n"
-                    "sub.u32 left, pos, sd;\n"
-                    "and.b32 at0, pos, rm; or.b32 at0, at0, kb; sub.u32 a1, pos, 256; and.b32 a1, a1, rm; or.b32 a1, a1, kb;\n"
-                    "sub.u32 a2, pos, 512; and.b32 a2, a2, rm; or.b32 a2, a2, kb; sub.u32 a3, pos, 768; and.b32 a3, a3, rm; or.b32 a3, a3, kb;\n"
-                    "sub.u32 a4, pos, 1024; and.b32 a4, a4, rm; or.b32 a4, a4, kb;\n"
-                    "ld.shared.b64 e1, [a1]; ld.shared.b64 e2, [a2]; ld.shared.b64 e3, [a3]; ld.shared.b64 e4, [a4];\n"
-                    "setp.gt.u32 t, left, 0; setp.lt.and.f64 t, key, e1, t; setp.gt.and.u32 ov, left, 256, t; setp.lt.and.f64 ov, key, e2, ov;\n"
-                    "setp.gt.and.u32 pz, left, 512, ov; setp.lt.and.f64 pz, key, e3, pz; setp.gt.and.u32 pf, left, 768, pz; setp.lt.and.f64 pf, key, e4, pf;\n"
-                    "@t st.shared.b64 [at0], e1; @ov st.shared.b64 [a1], e2; @pz st.shared.b64 [a2], e3; @pf st.shared.b64 [a3], e4;\n"
-                    "@t mov.u32 at0, a1; @ov mov.u32 at0, a2; @pz mov.u32 at0, a3; @pf mov.u32 at0, a4; st.shared.b64 [at0], key;\n"
-                    "sub.u32 pos, pos, 1024; @pf bra DEEPER;\n"
-                    "PLACED:\n"
-                    "mov.b32 %0, i; mov.b32 %1, bm; mov.b32 %2, lpos; mov.b32 %3, lfull; mov.b32 %4, tpos; mov.b32 %5, at1;\n"
-                    "mov.b32 %6, at2; mov.b64 %7, tk; mov.b32 %8, prev; mov.b64 %9, rec; mov.b32 %10, lat; mov.b32 %11, xs;\n"
-                    "mov.b32 %12, epos; mov.b32 %13, efull; mov.b32 %14, e_on; mov.b64 %15, e_key; mov.b32 %16, e_idx; mov.b32 %17, qv;\n"
-                    "mov.b32 %18, tail_a; mov.b32 %19, rw; mov.b32 %20, sa;\n"
-                    "}"
-                    : "+r"(i), "+r"(bm), "+r"(lpos), "+r"(lfull), "+r"(tpos), "+r"(at1), "+r"(at2), "+l"(tk), "+r"(prev), "+l"(rec), "+r"(lat), "+r"(xs), "+r"(epos), "+r"(efull), "+r"(e_on), "+l"(e_key), "+r"(e_idx), "+r"(qv), "+r"(tail_a), "+r"(rw), "+r"(sa)
-                    : "r"(xin), "r"(xin_mask), "r"(xin_row), "r"(tab), "r"(kfb), "r"(kfm), "r"(kb), "r"(rm), "r"(mbm1), "r"(tick), "r"(qmask), "r"(~qmask), "r"(qb), "r"(nq - 1u), "r"(xa), "r"(xam), "r"(down), "r"(tail_step), "l"(out)
-                    : "memory");
+                asm volatile(IL_STEP("", IL_STEP_INPUTS(21, 22, 23, 24, 25, 26, 27, 28, 29, 30, 31, 32, 33, 34, 35, 36, 37) IL_LOAD(b32, tail_step, 38) IL_LOAD(b64, out, 39),
+                                     ".reg .b64 o;\n", IL_ONE_TAIL,
+                                     "mad.wide.u32 o, ta_was, 1, out; @ho st.global.b64 [o], v;\n",
+                                     IL_DEEPER_LANE, "")
+                             : IL_STATE_OPERANDS
+                             : IL_INPUT_OPERANDS, "r"(tail_step), "l"(out)
+                             : "memory");
             } else if constexpr (OUT == kOutLeaf && FEAS) {
                 // (compared with its deadline two iterations later, when that has come)
-                asm volatile(
-                    "{\n"
-                    ".reg .b32 i; .reg .b32 bm; .reg .b32 lpos; .reg .b32 lfull; .reg .b32 tpos; .reg .b32 at1; .reg .b32 at2;\n"
-                    ".reg .b64 tk; .reg .b32 prev; .reg .b64 rec; .reg .b32 lat; .reg .b32 xs; .reg .b32 epos; .reg .b32 efull;\n"
-                    ".reg .b32 e_on; .reg .b64 e_key; .reg .b32 e_idx; .reg .b32 qv; .reg .b32 tail_a; .reg .b32 rw; .reg .b32 sa;\n"
-                    ".reg .b64 late_fin; .reg .b64 late_arr; .reg .b32 line; .reg .b32 xin; .reg .b32 xin_mask; .reg .b32 xin_row;\n"
-                    ".reg .b32 tab; .reg .b32 kfb; .reg .b32 kfm; .reg .b32 kb; .reg .b32 rm; .reg .b32 mbm1; .reg .b32 tick;\n"
-                    ".reg .b32 qmask; .reg .b32 tmask; .reg .b32 qb; .reg .b32 nqm; .reg .b32 xa; .reg .b32 xam; .reg .b32 down;\n"
-                    ".reg .b32 tail_step; .reg .b64 trace; .reg .b32 imask;\n"
-                    "mov.b32 i, %0; mov.b32 bm, %1; mov.b32 lpos, %2; mov.b32 lfull, %3; mov.b32 tpos, %4; mov.b32 at1, %5;\n"
-                    "mov.b32 at2, %6; mov.b64 tk, %7; mov.b32 prev, %8; mov.b64 rec, %9; mov.b32 lat, %10; mov.b32 xs, %11;\n"
-                    "mov.b32 epos, %12; mov.b32 efull, %13; mov.b32 e_on, %14; mov.b64 e_key, %15; mov.b32 e_idx, %16; mov.b32 qv, %17;\n"
-                    "mov.b32 tail_a, %18; mov.b32 rw, %19; mov.b32 sa, %20; mov.b64 late_arr, %22; mov.b64 late_fin, %21; .reg .b32 nobody; mov.b32 nobody, %44; mov.b32 line, %23; mov.b32 xin, %24;\n"
-                    "mov.b32 xin_mask, %25; mov.b32 xin_row, %26; mov.b32 tab, %27; mov.b32 kfb, %28; mov.b32 kfm, %29; mov.b32 kb, %30;\n"
-                    "mov.b32 rm, %31; mov.b32 mbm1, %32; mov.b32 tick, %33; mov.b32 qmask, %34; mov.b32 tmask, %35; mov.b32 qb, %36;\n"
-                    "mov.b32 nqm, %37; mov.b32 xa, %38; mov.b32 xam, %39; mov.b32 down, %40; mov.b32 tail_step, %41; mov.b64 trace, %42;\n"
-                    "mov.b32 imask, %43;\n"
-                    ".reg .pred t, taken, open, pop, ov, dp, pz, pf, hand, hd, ho, fin, fetch;\n"
-                    ".reg .u32 at0, sd, rl, rh, kl, kh, fl, fh, word, wa, x, y, lo, hi, a, xs_was, sa_was, ta_was, pos, left, a1, a2, a3, a4;\n"
-                    ".reg .b64 kf, k1, k2, fk, key, td, r, first, v, e1, e2, e3, e4; .reg .pred nl; .reg .b64 o;\n"
-                    "and.b32 a, epos, rm; or.b32 a, a, kb; ld.shared.b64 fk, [a];\n"
-                    "and.b32 a, lpos, kfm; or.b32 a, a, kfb; ld.shared.b64 kf, [a];\n"
-                    "ld.shared.b64 k1, [at1]; ld.shared.b64 k2, [at2];\n"
-                    "mov.b64 td, tk; mov.b64 {rl, rh}, rec; mov.u32 xs_was, xs; mov.u32 sa_was, sa;\n"
-                    "setp.ne.u32 t, tpos, efull; selp.b32 rh, rh, -1, t; mov.b64 r, {rl, rh};\n"
-                    "setp.ge.s32 taken, rh, 0; setp.ge.and.u32 t, bm, mbm1, taken; setp.gt.or.f64 open, r, td, t;\n"
-                    "sub.u32 y, i, bm; add.u32 y, y, -1;\n"
-                    "add.u32 wa, i, -1; and.b32 wa, wa, nqm; mad.lo.u32 wa, wa, 128, qb;\n"
-                    "@taken add.u32 i, i, 1; and.b32 xs, i, xin_mask; mad.lo.u32 xs, xs, xin_row, xin; ld.relaxed.cta.shared.b64 rec, [xs];\n"
-                    "setp.lt.s32 hand, rw, 0; setp.ne.and.u32 hand, e_on, 0, hand; setp.ge.and.s32 hd|ho, down, 0, hand; setp.lt.and.s32 fin, qv, 0, hand;\n"
-                    "and.b32 x, qv, 0x7fffffff; mov.b64 {lo, hi}, e_key; and.b32 lo, lo, tmask; or.b32 a, lo, x; mov.b64 v, {a, hi}; mov.u32 ta_was, tail_a;\n"
-                    "@hand add.u32 tail_a, tail_a, tail_step;\n"
-                    "and.b32 sa, tail_a, xam; or.b32 sa, sa, xa; ld.relaxed.cta.shared.u32 rw, [sa+4];\n"
-                    "mad.wide.u32 key, lat, tick, tk; mov.b64 {kl, kh}, key; and.b32 kl, kl, tmask; or.b32 kl, kl, y; mov.b64 key, {kl, kh};\n"
-                    "@taken add.u32 bm, bm, 1; @open mov.u32 bm, 0; mad.lo.u32 a, bm, 4, tab; ld.shared.u32 lat, [a];\n"
-                    "setp.eq.or.u32 fetch, e_on, 0, fin; setp.ne.and.u32 fetch, epos, tpos, fetch; setp.le.and.f64 fetch, fk, td, fetch;\n"
-                    "mov.b64 {fl, fh}, fk;\n"
-                    "@hand add.u32 e_idx, e_idx, 1; @fetch and.b32 e_idx, fl, qmask; and.b32 a, e_idx, nqm; mad.lo.u32 a, a, 128, qb; ld.shared.u32 qv, [a];\n"
-                    "@hd st.relaxed.cta.shared.b64 [sa_was], v;\n"
-                    "setp.gt.f64 nl, late_fin, late_arr; @nl add.u32 line, line, 1; mov.b64 late_fin, {lo, hi};\n"
-                    "and.b32 a, x, imask; selp.b32 a, a, nobody, ho; mad.wide.u32 o, a, 8, trace; ld.global.nc.b64 late_arr, [o];\n"
-                    "@fetch mov.b64 e_key, fk; @fin mov.u32 e_on, 0; @fetch mov.u32 e_on, 1; @fetch add.u32 epos, epos, 256; @fetch add.u32 efull, efull, 256;\n"
-                    "and.b32 at0, tpos, rm; or.b32 at0, at0, kb;\n"
-                    "setp.lt.f64 pf, kf, key; selp.b64 first, kf, key, pf;\n"
-                    "setp.eq.u32 pz, tpos, lfull; setp.lt.and.f64 pz, r, first, pz; selp.b64 first, first, r, pz;\n"
-                    "mov.b64 {fl, fh}, first; or.b32 fl, fl, qmask; mov.b64 first, {fl, fh}; selp.b64 tk, first, tk, open;\n"
-                    "setp.lt.and.f64 ov, key, k1, open; selp.u32 sd, at1, at0, ov;\n"
-                    "@open st.shared.b64 [sd], key; @ov st.shared.b64 [at0], k1;\n"
-                    "setp.lt.and.f64 dp, key, k2, ov; mov.u32 pos, tpos; mov.u32 left, lpos;\n"
-                    "setp.eq.and.u32 pop, tpos, lfull, open;\n"
-                    "mov.u32 word, prev; @open or.b32 word, word, 0x80000000; @taken st.shared.u32 [wa], word;\n"
-                    "@taken st.relaxed.cta.shared.u32 [xs_was+4], -1;\n"
-                    "@open add.u32 tpos, tpos, 256; @open mov.u32 at2, at1; @open mov.u32 at1, at0;\n"
-                    "@pop add.u32 lpos, lpos, 256; @pop add.u32 lfull, lfull, 256;\n"
-                    "@taken and.b32 prev, rl, qmask;\n"
-                    "vote.sync.any.pred pf, dp, 0xffffffff; @!pf bra.uni PLACED;\n"
-                    "mov.u32 sd, left; sub.u32 pos, pos, 256;\n"
-                    "DEEPER:\n"
-                    "sub.u32 left, pos, sd;\n"
-                    "and.b32 at0, pos, rm; or.b32 at0, at0, kb; sub.u32 a1, pos, 256; and.b32 a1, a1, rm; or.b32 a1, a1, kb;\n"
-                    "sub.u32 a2, pos, 512; and.b32 a2, a2, rm; or.b32 a2, a2, kb; sub.u32 a3, pos, 768; and.b32 a3, a3, rm; or.b32 a3, a3, kb;\n"
-                    "sub.u32 a4, pos, 1024; and.b32 a4, a4, rm; or.b32 a4, a4, kb;\n"
-                    "ld.shared.b64 e1, [a1]; ld.shared.b64 e2, [a2]; ld.shared.b64 e3, [a3]; ld.shared.b64 e4, [a4];\n"
-                    "setp.gt.and.u32 t, left, 0, dp; setp.lt.and.f64 t, key, e1, t; setp.gt.and.u32 ov, left, 256, t; setp.lt.and.f64 ov, key, e2, ov;\n"
-                    "setp.gt.and.u32 pz, left, 512, ov; setp.lt.and.f64 pz, key, e3, pz; setp.gt.and.u32 pf, left, 768, pz; setp.lt.and.f64 pf, key, e4, pf;\n"
-                    "@t st.shared.b64 [at0], e1; @ov st.shared.b64 [a1], e2; @pz st.shared.b64 [a2], e3; @pf st.shared.b64 [a3], e4;\n"
-                    "@t mov.u32 at0, a1; @ov mov.u32 at0, a2; @pz mov.u32 at0, a3; @pf mov.u32 at0, a4; @dp st.shared.b64 [at0], key;\n"
-                    "sub.u32 pos, pos, 1024; setp.ne.and.u32 dp, pos, 1, pf; vote.sync.any.pred pf, dp, 0xffffffff; @pf bra.uni DEEPER;\n"
-                    "PLACED:\n"
-                    "mov.b32 %0, i; mov.b32 %1, bm; mov.b32 %2, lpos; mov.b32 %3, lfull; mov.b32 %4, tpos; mov.b32 %5, at1;\n"
-                    "mov.b32 %6, at2; mov.b64 %7, tk; mov.b32 %8, prev; mov.b64 %9, rec; mov.b32 %10, lat; mov.b32 %11, xs;\n"
-                    "mov.b32 %12, epos; mov.b32 %13, efull; mov.b32 %14, e_on; mov.b64 %15, e_key; mov.b32 %16, e_idx; mov.b32 %17, qv;\n"
-                    "mov.b32 %18, tail_a; mov.b32 %19, rw; mov.b32 %20, sa; mov.b64 %21, late_fin; mov.b64 %22, late_arr;\n"
-                    "mov.b32 %23, line;\n"
-                    "}"
-                    : "+r"(i), "+r"(bm), "+r"(lpos), "+r"(lfull), "+r"(tpos), "+r"(at1), "+r"(at2), "+l"(tk), "+r"(prev), "+l"(rec), "+r"(lat), "+r"(xs), "+r"(epos), "+r"(efull), "+r"(e_on), "+l"(e_key), "+r"(e_idx), "+r"(qv), "+r"(tail_a), "+r"(rw), "+r"(sa), "+l"(late_fin[TURN]), "+l"(late_arr[TURN]), "+r"(miss_local)
-                    : "r"(xin), "r"(xin_mask), "r"(xin_row), "r"(tab), "r"(kfb), "r"(kfm), "r"(kb), "r"(rm), "r"(mbm1), "r"(tick), "r"(qmask), "r"(~qmask), "r"(qb), "r"(nq - 1u), "r"(xa), "r"(xam), "r"(down), "r"(tail_step), "l"(p.deadline), "r"(imask), "r"((uint32_t)p.n)
-                    : "memory");
+                asm volatile(IL_STEP(IL_LOAD(b64, late_arr, 22) IL_LOAD(b64, late_fin, 21) IL_LOAD(b32, nobody, 44) IL_LOAD(b32, line, 23),
+                                     IL_STEP_INPUTS(24, 25, 26, 27, 28, 29, 30, 31, 32, 33, 34, 35, 36, 37, 38, 39, 40) IL_LOAD(b32, tail_step, 41) IL_LOAD(b64, trace, 42)
+                                     IL_LOAD(b32, imask, 43),
+                                     ".reg .pred nl; .reg .b64 o;\n", IL_ONE_TAIL,
+                                     "setp.gt.f64 nl, late_fin, late_arr; @nl add.u32 line, line, 1; mov.b64 late_fin, {lo, hi};\n"
+                                     "and.b32 a, x, imask; selp.b32 a, a, nobody, ho; mad.wide.u32 o, a, 8, trace; ld.global.nc.b64 late_arr, [o];\n",
+                                     IL_DEEPER_WARP, IL_STORE(b64, late_fin, 21) IL_STORE(b64, late_arr, 22) IL_STORE(b32, line, 23))
+                             : IL_STATE_OPERANDS, "+l"(late_fin[TURN]), "+l"(late_arr[TURN]), "+r"(miss_local)
+                             : IL_INPUT_OPERANDS, "r"(tail_step), "l"(p.deadline), "r"(imask), "r"((uint32_t)p.n)
+                             : "memory");
             } else if constexpr (OUT == kOutLeaf && FORK) {
-                // (the query's slab entry keeps the latest of its copies)
-                asm volatile(
-                    "{\n"
-                    ".reg .b32 i; .reg .b32 bm; .reg .b32 lpos; .reg .b32 lfull; .reg .b32 tpos; .reg .b32 at1; .reg .b32 at2;\n"
-                    ".reg .b64 tk; .reg .b32 prev; .reg .b64 rec; .reg .b32 lat; .reg .b32 xs; .reg .b32 epos; .reg .b32 efull;\n"
-                    ".reg .b32 e_on; .reg .b64 e_key; .reg .b32 e_idx; .reg .b32 qv; .reg .b32 tail_a; .reg .b32 rw; .reg .b32 sa;\n"
-                    ".reg .b32 xin; .reg .b32 xin_mask; .reg .b32 xin_row; .reg .b32 tab; .reg .b32 kfb; .reg .b32 kfm; .reg .b32 kb;\n"
-                    ".reg .b32 rm; .reg .b32 mbm1; .reg .b32 tick; .reg .b32 qmask; .reg .b32 tmask; .reg .b32 qb; .reg .b32 nqm;\n"
-                    ".reg .b32 xa; .reg .b32 xam; .reg .b32 down; .reg .b32 tail_step; .reg .b64 out; .reg .b32 imask; .reg .b32 rb;\n"
-                    "mov.b32 i, %0; mov.b32 bm, %1; mov.b32 lpos, %2; mov.b32 lfull, %3; mov.b32 tpos, %4; mov.b32 at1, %5;\n"
-                    "mov.b32 at2, %6; mov.b64 tk, %7; mov.b32 prev, %8; mov.b64 rec, %9; mov.b32 lat, %10; mov.b32 xs, %11;\n"
-                    "mov.b32 epos, %12; mov.b32 efull, %13; mov.b32 e_on, %14; mov.b64 e_key, %15; mov.b32 e_idx, %16; mov.b32 qv, %17;\n"
-                    "mov.b32 tail_a, %18; mov.b32 rw, %19; mov.b32 sa, %20; mov.b32 xin, %21; mov.b32 xin_mask, %22; mov.b32 xin_row, %23;\n"
-                    "mov.b32 tab, %24; mov.b32 kfb, %25; mov.b32 kfm, %26; mov.b32 kb, %27; mov.b32 rm, %28; mov.b32 mbm1, %29;\n"
-                    "mov.b32 tick, %30; mov.b32 qmask, %31; mov.b32 tmask, %32; mov.b32 qb, %33; mov.b32 nqm, %34; mov.b32 xa, %35;\n"
-                    "mov.b32 xam, %36; mov.b32 down, %37; mov.b32 tail_step, %38; mov.b64 out, %39; mov.b32 imask, %40; mov.b32 rb, %41;\n"
-                    ".reg .pred t, taken, open, pop, ov, dp, pz, pf, hand, hd, ho, fin, fetch;\n"
-                    ".reg .u32 at0, sd, rl, rh, kl, kh, fl, fh, word, wa, x, y, lo, hi, a, xs_was, sa_was, ta_was, pos, left, a1, a2, a3, a4;\n"
-                    ".reg .b64 kf, k1, k2, fk, key, td, r, first, v, e1, e2, e3, e4; .reg .b64 o, w;\n"
-                    "and.b32 a, epos, rm; or.b32 a, a, kb; ld.shared.b64 fk, [a];\n"
-                    "and.b32 a, lpos, kfm; or.b32 a, a, kfb; ld.shared.b64 kf, [a];\n"
-                    "ld.shared.b64 k1, [at1]; ld.shared.b64 k2, [at2];\n"
-                    "mov.b64 td, tk; mov.b64 {rl, rh}, rec; mov.u32 xs_was, xs; mov.u32 sa_was, sa;\n"
-                    "setp.ne.u32 t, tpos, efull; selp.b32 rh, rh, -1, t; mov.b64 r, {rl, rh};\n"
-                    "setp.ge.s32 taken, rh, 0; setp.ge.and.u32 t, bm, mbm1, taken; setp.gt.or.f64 open, r, td, t;\n"
-                    "sub.u32 y, i, bm; add.u32 y, y, -1;\n"
-                    "add.u32 wa, i, -1; and.b32 wa, wa, nqm; mad.lo.u32 wa, wa, 128, qb;\n"
-                    "@taken add.u32 i, i, 1; and.b32 xs, i, xin_mask; mad.lo.u32 xs, xs, xin_row, xin; ld.relaxed.cta.shared.b64 rec, [xs];\n"
-                    "setp.lt.s32 hand, rw, 0; setp.ne.and.u32 hand, e_on, 0, hand; setp.ge.and.s32 hd|ho, down, 0, hand; setp.lt.and.s32 fin, qv, 0, hand;\n"
-                    "and.b32 x, qv, 0x7fffffff; mov.b64 {lo, hi}, e_key; and.b32 lo, lo, tmask; or.b32 a, lo, x; mov.b64 v, {a, hi}; mov.u32 ta_was, tail_a;\n"
-                    "@hand add.u32 tail_a, tail_a, tail_step;\n"
-                    "and.b32 sa, tail_a, xam; or.b32 sa, sa, xa; ld.relaxed.cta.shared.u32 rw, [sa+4];\n"
-                    "mad.wide.u32 key, lat, tick, tk; mov.b64 {kl, kh}, key; and.b32 kl, kl, tmask; or.b32 kl, kl, y; mov.b64 key, {kl, kh};\n"
-                    "@taken add.u32 bm, bm, 1; @open mov.u32 bm, 0; mad.lo.u32 a, bm, 4, tab; ld.shared.u32 lat, [a];\n"
-                    "setp.eq.or.u32 fetch, e_on, 0, fin; setp.ne.and.u32 fetch, epos, tpos, fetch; setp.le.and.f64 fetch, fk, td, fetch;\n"
-                    "mov.b64 {fl, fh}, fk;\n"
-                    "@hand add.u32 e_idx, e_idx, 1; @fetch and.b32 e_idx, fl, qmask; and.b32 a, e_idx, nqm; mad.lo.u32 a, a, 128, qb; ld.shared.u32 qv, [a];\n"
-                    "@hd st.relaxed.cta.shared.b64 [sa_was], v;\n"
-                    "and.b32 a, x, imask; mad.wide.u32 o, a, 8, out;\n"
-                    "mov.b64 w, {lo, hi}; shr.u64 w, w, rb; cvt.u64.u32 v, a; or.b64 w, w, v; @ho red.relaxed.gpu.global.max.u64 [o], w;\n"
-                    "@fetch mov.b64 e_key, fk; @fin mov.u32 e_on, 0; @fetch mov.u32 e_on, 1; @fetch add.u32 epos, epos, 256; @fetch add.u32 efull, efull, 256;\n"
-                    "and.b32 at0, tpos, rm; or.b32 at0, at0, kb;\n"
-                    "setp.lt.f64 pf, kf, key; selp.b64 first, kf, key, pf;\n"
-                    "setp.eq.u32 pz, tpos, lfull; setp.lt.and.f64 pz, r, first, pz; selp.b64 first, first, r, pz;\n"
-                    "mov.b64 {fl, fh}, first; or.b32 fl, fl, qmask; mov.b64 first, {fl, fh}; selp.b64 tk, first, tk, open;\n"
-                    "setp.lt.and.f64 ov, key, k1, open; selp.u32 sd, at1, at0, ov;\n"
-                    "@open st.shared.b64 [sd], key; @ov st.shared.b64 [at0], k1;\n"
-                    "setp.lt.and.f64 dp, key, k2, ov; mov.u32 pos, tpos; mov.u32 left, lpos;\n"
-                    "setp.eq.and.u32 pop, tpos, lfull, open;\n"
-                    "mov.u32 word, prev; @open or.b32 word, word, 0x80000000; @taken st.shared.u32 [wa], word;\n"
-                    "@taken st.relaxed.cta.shared.u32 [xs_was+4], -1;\n"
-                    "@open add.u32 tpos, tpos, 256; @open mov.u32 at2, at1; @open mov.u32 at1, at0;\n"
-                    "@pop add.u32 lpos, lpos, 256; @pop add.u32 lfull, lfull, 256;\n"
-                    "@taken and.b32 prev, rl, qmask;\n"
-                    "vote.sync.any.pred pf, dp, 0xffffffff; @!pf bra.uni PLACED;\n"
-                    "mov.u32 sd, left; sub.u32 pos, pos, 256;\n"
-                    "DEEPER:\n"
-                    "sub.u32 left, pos, sd;\n"
-                    "and.b32 at0, pos, rm; or.b32 at0, at0, kb; sub.u32 a1, pos, 256; and.b32 a1, a1, rm; or.b32 a1, a1, kb;\n"
-                    "sub.u32 a2, pos, 512; and.b32 a2, a2, rm; or.b32 a2, a2, kb; sub.u32 a3, pos, 768; and.b32 a3, a3, rm; or.b32 a3, a3, kb;\n"
-                    "sub.u32 a4, pos, 1024; and.b32 a4, a4, rm; or.b32 a4, a4, kb;\n"
-                    "ld.shared.b64 e1, [a1]; ld.shared.b64 e2, [a2]; ld.shared.b64 e3, [a3]; ld.shared.b64 e4, [a4];\n"
-                    "setp.gt.and.u32 t, left, 0, dp; setp.lt.and.f64 t, key, e1, t; setp.gt.and.u32 ov, left, 256, t; setp.lt.and.f64 ov, key, e2, ov;\n"
-                    "setp.gt.and.u32 pz, left, 512, ov; setp.lt.and.f64 pz, key, e3, pz; setp.gt.and.u32 pf, left, 768, pz; setp.lt.and.f64 pf, key, e4, pf;\n"
-                    "@t st.shared.b64 [at0], e1; @ov st.shared.b64 [a1], e2; @pz st.shared.b64 [a2], e3; @pf st.shared.b64 [a3], e4;\n"
-                    "@t mov.u32 at0, a1; @ov mov.u32 at0, a2; @pz mov.u32 at0, a3; @pf mov.u32 at0, a4; @dp st.shared.b64 [at0], key;\n"
-                    "sub.u32 pos, pos, 1024; setp.ne.and.u32 dp, pos, 1, pf; vote.sync.any.pred pf, dp, 0xffffffff; @pf bra.uni DEEPER;\n"
-                    "PLACED:\n"
-                    "mov.b32 %0, i; mov.b32 %1, bm; mov.b32 %2, lpos; mov.b32 %3, lfull; mov.b32 %4, tpos; mov.b32 %5, at1;\n"
-                    "mov.b32 %6, at2; mov.b64 %7, tk; mov.b32 %8, prev; mov.b64 %9, rec; mov.b32 %10, lat; mov.b32 %11, xs;\n"
-                    "mov.b32 %12, epos; mov.b32 %13, efull; mov.b32 %14, e_on; mov.b64 %15, e_key; mov.b32 %16, e_idx; mov.b32 %17, qv;\n"
-                    "mov.b32 %18, tail_a; mov.b32 %19, rw; mov.b32 %20, sa;\n"
-                    "}"
-                    : "+r"(i), "+r"(bm), "+r"(lpos), "+r"(lfull), "+r"(tpos), "+r"(at1), "+r"(at2), "+l"(tk), "+r"(prev), "+l"(rec), "+r"(lat), "+r"(xs), "+r"(epos), "+r"(efull), "+r"(e_on), "+l"(e_key), "+r"(e_idx), "+r"(qv), "+r"(tail_a), "+r"(rw), "+r"(sa)
-                    : "r"(xin), "r"(xin_mask), "r"(xin_row), "r"(tab), "r"(kfb), "r"(kfm), "r"(kb), "r"(rm), "r"(mbm1), "r"(tick), "r"(qmask), "r"(~qmask), "r"(qb), "r"(nq - 1u), "r"(xa), "r"(xam), "r"(down), "r"(tail_step), "l"(out_c), "r"(imask), "r"(rb)
-                    : "memory");
+                // (several copies of a query may leave: the slab keeps the last one's record)
+                asm volatile(IL_STEP("", IL_STEP_INPUTS(21, 22, 23, 24, 25, 26, 27, 28, 29, 30, 31, 32, 33, 34, 35, 36, 37) IL_LOAD(b32, tail_step, 38) IL_LOAD(b64, out, 39)
+                                     IL_LOAD(b32, imask, 40) IL_LOAD(b32, rb, 41),
+                                     ".reg .b64 o, w;\n", IL_ONE_TAIL,
+                                     "and.b32 a, x, imask; mad.wide.u32 o, a, 8, out;\n" IL_PLAIN_RECORD "@ho red.relaxed.gpu.global.max.u64 [o], w;\n",
+                                     IL_DEEPER_WARP, "")
+                             : IL_STATE_OPERANDS
+                             : IL_INPUT_OPERANDS, "r"(tail_step), "l"(out_c), "r"(imask), "r"(rb)
+                             : "memory");
             } else if constexpr (OUT == kOutLeaf) {
-                asm volatile(
-                    "{\n"
-                    ".reg .b32 i; .reg .b32 bm; .reg .b32 lpos; .reg .b32 lfull; .reg .b32 tpos; .reg .b32 at1; .reg .b32 at2;\n"
-                    ".reg .b64 tk; .reg .b32 prev; .reg .b64 rec; .reg .b32 lat; .reg .b32 xs; .reg .b32 epos; .reg .b32 efull;\n"
-                    ".reg .b32 e_on; .reg .b64 e_key; .reg .b32 e_idx; .reg .b32 qv; .reg .b32 tail_a; .reg .b32 rw; .reg .b32 sa;\n"
-                    ".reg .b32 xin; .reg .b32 xin_mask; .reg .b32 xin_row; .reg .b32 tab; .reg .b32 kfb; .reg .b32 kfm; .reg .b32 kb;\n"
-                    ".reg .b32 rm; .reg .b32 mbm1; .reg .b32 tick; .reg .b32 qmask; .reg .b32 tmask; .reg .b32 qb; .reg .b32 nqm;\n"
-                    ".reg .b32 xa; .reg .b32 xam; .reg .b32 down; .reg .b32 tail_step; .reg .b64 out; .reg .b32 imask; .reg .b32 rb;\n"
-                    "mov.b32 i, %0; mov.b32 bm, %1; mov.b32 lpos, %2; mov.b32 lfull, %3; mov.b32 tpos, %4; mov.b32 at1, %5;\n"
-                    "mov.b32 at2, %6; mov.b64 tk, %7; mov.b32 prev, %8; mov.b64 rec, %9; mov.b32 lat, %10; mov.b32 xs, %11;\n"
-                    "mov.b32 epos, %12; mov.b32 efull, %13; mov.b32 e_on, %14; mov.b64 e_key, %15; mov.b32 e_idx, %16; mov.b32 qv, %17;\n"
-                    "mov.b32 tail_a, %18; mov.b32 rw, %19; mov.b32 sa, %20; mov.b32 xin, %21; mov.b32 xin_mask, %22; mov.b32 xin_row, %23;\n"
-                    "mov.b32 tab, %24; mov.b32 kfb, %25; mov.b32 kfm, %26; mov.b32 kb, %27; mov.b32 rm, %28; mov.b32 mbm1, %29;\n"
-                    "mov.b32 tick, %30; mov.b32 qmask, %31; mov.b32 tmask, %32; mov.b32 qb, %33; mov.b32 nqm, %34; mov.b32 xa, %35;\n"
-                    "mov.b32 xam, %36; mov.b32 down, %37; mov.b32 tail_step, %38; mov.b64 out, %39; mov.b32 imask, %40; mov.b32 rb, %41;\n"
-                    ".reg .pred t, taken, open, pop, ov, dp, pz, pf, hand, hd, ho, fin, fetch;\n"
-                    ".reg .u32 at0, sd, rl, rh, kl, kh, fl, fh, word, wa, x, y, lo, hi, a, xs_was, sa_was, ta_was, pos, left, a1, a2, a3, a4;\n"
-                    ".reg .b64 kf, k1, k2, fk, key, td, r, first, v, e1, e2, e3, e4; .reg .b64 o, w;\n"
-                    "and.b32 a, epos, rm; or.b32 a, a, kb; ld.shared.b64 fk, [a];\n"
-                    "and.b32 a, lpos, kfm; or.b32 a, a, kfb; ld.shared.b64 kf, [a];\n"
-                    "ld.shared.b64 k1, [at1]; ld.shared.b64 k2, [at2];\n"
-                    "mov.b64 td, tk; mov.b64 {rl, rh}, rec; mov.u32 xs_was, xs; mov.u32 sa_was, sa;\n"
-                    "setp.ne.u32 t, tpos, efull; selp.b32 rh, rh, -1, t; mov.b64 r, {rl, rh};\n"
-                    "setp.ge.s32 taken, rh, 0; setp.ge.and.u32 t, bm, mbm1, taken; setp.gt.or.f64 open, r, td, t;\n"
-                    "sub.u32 y, i, bm; add.u32 y, y, -1;\n"
-                    "add.u32 wa, i, -1; and.b32 wa, wa, nqm; mad.lo.u32 wa, wa, 128, qb;\n"
-                    "@taken add.u32 i, i, 1; and.b32 xs, i, xin_mask; mad.lo.u32 xs, xs, xin_row, xin; ld.relaxed.cta.shared.b64 rec, [xs];\n"
-                    "setp.lt.s32 hand, rw, 0; setp.ne.and.u32 hand, e_on, 0, hand; setp.ge.and.s32 hd|ho, down, 0, hand; setp.lt.and.s32 fin, qv, 0, hand;\n"
-                    "and.b32 x, qv, 0x7fffffff; mov.b64 {lo, hi}, e_key; and.b32 lo, lo, tmask; or.b32 a, lo, x; mov.b64 v, {a, hi}; mov.u32 ta_was, tail_a;\n"
-                    "@hand add.u32 tail_a, tail_a, tail_step;\n"
-                    "and.b32 sa, tail_a, xam; or.b32 sa, sa, xa; ld.relaxed.cta.shared.u32 rw, [sa+4];\n"
-                    "mad.wide.u32 key, lat, tick, tk; mov.b64 {kl, kh}, key; and.b32 kl, kl, tmask; or.b32 kl, kl, y; mov.b64 key, {kl, kh};\n"
-                    "@taken add.u32 bm, bm, 1; @open mov.u32 bm, 0; mad.lo.u32 a, bm, 4, tab; ld.shared.u32 lat, [a];\n"
-                    "setp.eq.or.u32 fetch, e_on, 0, fin; setp.ne.and.u32 fetch, epos, tpos, fetch; setp.le.and.f64 fetch, fk, td, fetch;\n"
-                    "mov.b64 {fl, fh}, fk;\n"
-                    "@hand add.u32 e_idx, e_idx, 1; @fetch and.b32 e_idx, fl, qmask; and.b32 a, e_idx, nqm; mad.lo.u32 a, a, 128, qb; ld.shared.u32 qv, [a];\n"
-                    "@hd st.relaxed.cta.shared.b64 [sa_was], v;\n"
-                    "mad.wide.u32 o, ta_was, 1, out;\n"
-                    "and.b32 a, x, imask; mov.b64 w, {lo, hi}; shr.u64 w, w, rb; cvt.u64.u32 v, a; or.b64 w, w, v; @ho st.global.b64 [o], w;\n"
-                    "@fetch mov.b64 e_key, fk; @fin mov.u32 e_on, 0; @fetch mov.u32 e_on, 1; @fetch add.u32 epos, epos, 256; @fetch add.u32 efull, efull, 256;\n"
-                    "and.b32 at0, tpos, rm; or.b32 at0, at0, kb;\n"
-                    "setp.lt.f64 pf, kf, key; selp.b64 first, kf, key, pf;\n"
-                    "setp.eq.u32 pz, tpos, lfull; setp.lt.and.f64 pz, r, first, pz; selp.b64 first, first, r, pz;\n"
-                    "mov.b64 {fl, fh}, first; or.b32 fl, fl, qmask; mov.b64 first, {fl, fh}; selp.b64 tk, first, tk, open;\n"
-                    "setp.lt.and.f64 ov, key, k1, open; selp.u32 sd, at1, at0, ov;\n"
-                    "@open st.shared.b64 [sd], key; @ov st.shared.b64 [at0], k1;\n"
-                    "setp.lt.and.f64 dp, key, k2, ov; mov.u32 pos, tpos; mov.u32 left, lpos;\n"
-                    "setp.eq.and.u32 pop, tpos, lfull, open;\n"
-                    "mov.u32 word, prev; @open or.b32 word, word, 0x80000000; @taken st.shared.u32 [wa], word;\n"
-                    "@taken st.relaxed.cta.shared.u32 [xs_was+4], -1;\n"
-                    "@open add.u32 tpos, tpos, 256; @open mov.u32 at2, at1; @open mov.u32 at1, at0;\n"
-                    "@pop add.u32 lpos, lpos, 256; @pop add.u32 lfull, lfull, 256;\n"
-                    "@taken and.b32 prev, rl, qmask;\n"
-                    "@!dp bra PLACED;\n"
-                    "mov.u32 sd, left; sub.u32 pos, pos, 256;\n"
-                    "DEEPER:\n"
-                    "sub.u32 left, pos, sd;\n"
-                    "and.b32 at0, pos, rm; or.b32 at0, at0, kb; sub.u32 a1, pos, 256; and.b32 a1, a1, rm; or.b32 a1, a1, kb;\n"
-                    "sub.u32 a2, pos, 512; and.b32 a2, a2, rm; or.b32 a2, a2, kb; sub.u32 a3, pos, 768; and.b32 a3, a3, rm; or.b32 a3, a3, kb;\n"
-                    "sub.u32 a4, pos, 1024; and.b32 a4, a4, rm; or.b32 a4, a4, kb;\n"
-                    "ld.shared.b64 e1, [a1]; ld.shared.b64 e2, [a2]; ld.shared.b64 e3, [a3]; ld.shared.b64 e4, [a4];\n"
-                    "setp.gt.u32 t, left, 0; setp.lt.and.f64 t, key, e1, t; setp.gt.and.u32 ov, left, 256, t; setp.lt.and.f64 ov, key, e2, ov;\n"
-                    "setp.gt.and.u32 pz, left, 512, ov; setp.lt.and.f64 pz, key, e3, pz; setp.gt.and.u32 pf, left, 768, pz; setp.lt.and.f64 pf, key, e4, pf;\n"
-                    "@t st.shared.b64 [at0], e1; @ov st.shared.b64 [a1], e2; @pz st.shared.b64 [a2], e3; @pf st.shared.b64 [a3], e4;\n"
-                    "@t mov.u32 at0, a1; @ov mov.u32 at0, a2; @pz mov.u32 at0, a3; @pf mov.u32 at0, a4; st.shared.b64 [at0], key;\n"
-                    "sub.u32 pos, pos, 1024; @pf bra DEEPER;\n"
-                    "PLACED:\n"
-                    "mov.b32 %0, i; mov.b32 %1, bm; mov.b32 %2, lpos; mov.b32 %3, lfull; mov.b32 %4, tpos; mov.b32 %5, at1;\n"
-                    "mov.b32 %6, at2; mov.b64 %7, tk; mov.b32 %8, prev; mov.b64 %9, rec; mov.b32 %10, lat; mov.b32 %11, xs;\n"
-                    "mov.b32 %12, epos; mov.b32 %13, efull; mov.b32 %14, e_on; mov.b64 %15, e_key; mov.b32 %16, e_idx; mov.b32 %17, qv;\n"
-                    "mov.b32 %18, tail_a; mov.b32 %19, rw; mov.b32 %20, sa;\n"
-                    "}"
-                    : "+r"(i), "+r"(bm), "+r"(lpos), "+r"(lfull), "+r"(tpos), "+r"(at1), "+r"(at2), "+l"(tk), "+r"(prev), "+l"(rec), "+r"(lat), "+r"(xs), "+r"(epos), "+r"(efull), "+r"(e_on), "+l"(e_key), "+r"(e_idx), "+r"(qv), "+r"(tail_a), "+r"(rw), "+r"(sa)
-                    : "r"(xin), "r"(xin_mask), "r"(xin_row), "r"(tab), "r"(kfb), "r"(kfm), "r"(kb), "r"(rm), "r"(mbm1), "r"(tick), "r"(qmask), "r"(~qmask), "r"(qb), "r"(nq - 1u), "r"(xa), "r"(xam), "r"(down), "r"(tail_step), "l"(out), "r"(imask), "r"(rb)
-                    : "memory");
+                asm volatile(IL_STEP("", IL_STEP_INPUTS(21, 22, 23, 24, 25, 26, 27, 28, 29, 30, 31, 32, 33, 34, 35, 36, 37) IL_LOAD(b32, tail_step, 38) IL_LOAD(b64, out, 39)
+                                     IL_LOAD(b32, imask, 40) IL_LOAD(b32, rb, 41),
+                                     ".reg .b64 o, w;\n", IL_ONE_TAIL,
+                                     "mad.wide.u32 o, ta_was, 1, out;\n" "and.b32 a, x, imask; " IL_PLAIN_RECORD "@ho st.global.b64 [o], w;\n",
+                                     IL_DEEPER_LANE, "")
+                             : IL_STATE_OPERANDS
+                             : IL_INPUT_OPERANDS, "r"(tail_step), "l"(out), "r"(imask), "r"(rb)
+                             : "memory");
             } else if constexpr (OUT == kOutTwo && FORK) {
-                asm volatile(
-                    "{\n"
-                    ".reg .b32 i; .reg .b32 bm; .reg .b32 lpos; .reg .b32 lfull; .reg .b32 tpos; .reg .b32 at1; .reg .b32 at2;\n"
-                    ".reg .b64 tk; .reg .b32 prev; .reg .b64 rec; .reg .b32 lat; .reg .b32 xs; .reg .b32 epos; .reg .b32 efull;\n"
-                    ".reg .b32 e_on; .reg .b64 e_key; .reg .b32 e_idx; .reg .b32 qv; .reg .b32 tail_a; .reg .b32 rw; .reg .b32 sa;\n"
-                    ".reg .b32 tail_b; .reg .b32 xin; .reg .b32 xin_mask; .reg .b32 xin_row; .reg .b32 tab; .reg .b32 kfb; .reg .b32 kfm;\n"
-                    ".reg .b32 kb; .reg .b32 rm; .reg .b32 mbm1; .reg .b32 tick; .reg .b32 qmask; .reg .b32 tmask; .reg .b32 qb;\n"
-                    ".reg .b32 nqm; .reg .b32 xa; .reg .b32 xam; .reg .b32 down; .reg .b32 mask_a; .reg .b32 mask_b; .reg .b32 want_a;\n"
-                    ".reg .b32 want_b; .reg .b64 out; .reg .b64 out_b;\n"
-                    "mov.b32 i, %0; mov.b32 bm, %1; mov.b32 lpos, %2; mov.b32 lfull, %3; mov.b32 tpos, %4; mov.b32 at1, %5;\n"
-                    "mov.b32 at2, %6; mov.b64 tk, %7; mov.b32 prev, %8; mov.b64 rec, %9; mov.b32 lat, %10; mov.b32 xs, %11;\n"
-                    "mov.b32 epos, %12; mov.b32 efull, %13; mov.b32 e_on, %14; mov.b64 e_key, %15; mov.b32 e_idx, %16; mov.b32 qv, %17;\n"
-                    "mov.b32 tail_a, %18; mov.b32 rw, %19; mov.b32 sa, %20; mov.b32 tail_b, %21; mov.b32 xin, %22; mov.b32 xin_mask, %23;\n"
-                    "mov.b32 xin_row, %24; mov.b32 tab, %25; mov.b32 kfb, %26; mov.b32 kfm, %27; mov.b32 kb, %28; mov.b32 rm, %29;\n"
-                    "mov.b32 mbm1, %30; mov.b32 tick, %31; mov.b32 qmask, %32; mov.b32 tmask, %33; mov.b32 qb, %34; mov.b32 nqm, %35;\n"
-                    "mov.b32 xa, %36; mov.b32 xam, %37; mov.b32 down, %38; mov.b32 mask_a, %39; mov.b32 mask_b, %40; mov.b32 want_a, %41;\n"
-                    "mov.b32 want_b, %42; mov.b64 out, %43; mov.b64 out_b, %44;\n"
-                    ".reg .pred t, taken, open, pop, ov, dp, pz, pf, hand, hd, ho, fin, fetch;\n"
-                    ".reg .u32 at0, sd, rl, rh, kl, kh, fl, fh, word, wa, x, y, lo, hi, a, xs_was, sa_was, ta_was, pos, left, a1, a2, a3, a4;\n"
-                    ".reg .b64 kf, k1, k2, fk, key, td, r, first, v, e1, e2, e3, e4; .reg .pred ga, gb; .reg .b64 o; .reg .u32 ma, mb;\n"
-                    "and.b32 a, epos, rm; or.b32 a, a, kb; ld.shared.b64 fk, [a];\n"
-                    "and.b32 a, lpos, kfm; or.b32 a, a, kfb; ld.shared.b64 kf, [a];\n"
-                    "ld.shared.b64 k1, [at1]; ld.shared.b64 k2, [at2];\n"
-                    "mov.b64 td, tk; mov.b64 {rl, rh}, rec; mov.u32 xs_was, xs; mov.u32 sa_was, sa;\n"
-                    "setp.ne.u32 t, tpos, efull; selp.b32 rh, rh, -1, t; mov.b64 r, {rl, rh};\n"
-                    "setp.ge.s32 taken, rh, 0; setp.ge.and.u32 t, bm, mbm1, taken; setp.gt.or.f64 open, r, td, t;\n"
-                    "sub.u32 y, i, bm; add.u32 y, y, -1;\n"
-                    "add.u32 wa, i, -1; and.b32 wa, wa, nqm; mad.lo.u32 wa, wa, 128, qb;\n"
-                    "@taken add.u32 i, i, 1; and.b32 xs, i, xin_mask; mad.lo.u32 xs, xs, xin_row, xin; ld.relaxed.cta.shared.b64 rec, [xs];\n"
-                    "setp.lt.s32 hand, rw, 0; setp.ne.and.u32 hand, e_on, 0, hand; setp.ge.and.s32 hd|ho, down, 0, hand; setp.lt.and.s32 fin, qv, 0, hand;\n"
-                    "and.b32 x, qv, 0x7fffffff; mov.b64 {lo, hi}, e_key; and.b32 lo, lo, tmask; or.b32 a, lo, x; mov.b64 v, {a, hi}; mov.u32 ta_was, tail_a;\n"
-                    "and.b32 ma, qv, mask_a; and.b32 mb, qv, mask_b;\n"
-                    "setp.eq.and.u32 ga, ma, want_a, ho; setp.eq.and.u32 gb, mb, want_b, ho;\n"
-                    "@hd add.u32 tail_a, tail_a, 256; @ga add.u32 tail_a, tail_a, 8;\n"
-                    "and.b32 sa, tail_a, xam; or.b32 sa, sa, xa; ld.relaxed.cta.shared.u32 rw, [sa+4];\n"
-                    "mad.wide.u32 key, lat, tick, tk; mov.b64 {kl, kh}, key; and.b32 kl, kl, tmask; or.b32 kl, kl, y; mov.b64 key, {kl, kh};\n"
-                    "@taken add.u32 bm, bm, 1; @open mov.u32 bm, 0; mad.lo.u32 a, bm, 4, tab; ld.shared.u32 lat, [a];\n"
-                    "setp.eq.or.u32 fetch, e_on, 0, fin; setp.ne.and.u32 fetch, epos, tpos, fetch; setp.le.and.f64 fetch, fk, td, fetch;\n"
-                    "mov.b64 {fl, fh}, fk;\n"
-                    "@hand add.u32 e_idx, e_idx, 1; @fetch and.b32 e_idx, fl, qmask; and.b32 a, e_idx, nqm; mad.lo.u32 a, a, 128, qb; ld.shared.u32 qv, [a];\n"
-                    "@hd st.relaxed.cta.shared.b64 [sa_was], v;\n"
-                    "mad.wide.u32 o, ta_was, 1, out; @ga st.global.b64 [o], v; mad.wide.u32 o, tail_b, 1, out_b; @gb st.global.b64 [o], v; @gb add.u32 tail_b, tail_b, 8;\n"
-                    "@fetch mov.b64 e_key, fk; @fin mov.u32 e_on, 0; @fetch mov.u32 e_on, 1; @fetch add.u32 epos, epos, 256; @fetch add.u32 efull, efull, 256;\n"
-                    "and.b32 at0, tpos, rm; or.b32 at0, at0, kb;\n"
-                    "setp.lt.f64 pf, kf, key; selp.b64 first, kf, key, pf;\n"
-                    "setp.eq.u32 pz, tpos, lfull; setp.lt.and.f64 pz, r, first, pz; selp.b64 first, first, r, pz;\n"
-                    "mov.b64 {fl, fh}, first; or.b32 fl, fl, qmask; mov.b64 first, {fl, fh}; selp.b64 tk, first, tk, open;\n"
-                    "setp.lt.and.f64 ov, key, k1, open; selp.u32 sd, at1, at0, ov;\n"
-                    "@open st.shared.b64 [sd], key; @ov st.shared.b64 [at0], k1;\n"
-                    "setp.lt.and.f64 dp, key, k2, ov; mov.u32 pos, tpos; mov.u32 left, lpos;\n"
-                    "setp.eq.and.u32 pop, tpos, lfull, open;\n"
-                    "mov.u32 word, prev; @open or.b32 word, word, 0x80000000; @taken st.shared.u32 [wa], word;\n"
-                    "@taken st.relaxed.cta.shared.u32 [xs_was+4], -1;\n"
-                    "@open add.u32 tpos, tpos, 256; @open mov.u32 at2, at1; @open mov.u32 at1, at0;\n"
-                    "@pop add.u32 lpos, lpos, 256; @pop add.u32 lfull, lfull, 256;\n"
-                    "@taken and.b32 prev, rl, qmask;\n"
-                    "vote.sync.any.pred pf, dp, 0xffffffff; @!pf bra.uni PLACED;\n"
-                    "mov.u32 sd, left; sub.u32 pos, pos, 256;\n"
-                    "DEEPER:\n"
-                    "sub.u32 left, pos, sd;\n"
-                    "and.b32 at0, pos, rm; or.b32 at0, at0, kb; sub.u32 a1, pos, 256; and.b32 a1, a1, rm; or.b32 a1, a1, kb;\n"
-                    "sub.u32 a2, pos, 512; and.b32 a2, a2, rm; or.b32 a2, a2, kb; sub.u32 a3, pos, 768; and.b32 a3, a3, rm; or.b32 a3, a3, kb;\n"
-                    "sub.u32 a4, pos, 1024; and.b32 a4, a4, rm; or.b32 a4, a4, kb;\n"
-                    "ld.shared.b64 e1, [a1]; ld.shared.b64 e2, [a2]; ld.shared.b64 e3, [a3]; ld.shared.b64 e4, [a4];\n"
-                    "setp.gt.and.u32 t, left, 0, dp; setp.lt.and.f64 t, key, e1, t; setp.gt.and.u32 ov, left, 256, t; setp.lt.and.f64 ov, key, e2, ov;\n"
-                    "setp.gt.and.u32 pz, left, 512, ov; setp.lt.and.f64 pz, key, e3, pz; setp.gt.and.u32 pf, left, 768, pz; setp.lt.and.f64 pf, key, e4, pf;\n"
-                    "@t st.shared.b64 [at0], e1; @ov st.shared.b64 [a1], e2; @pz st.shared.b64 [a2], e3; @pf st.shared.b64 [a3], e4;\n"
-                    "@t mov.u32 at0, a1; @ov mov.u32 at0, a2; @pz mov.u32 at0, a3; @pf mov.u32 at0, a4; @dp st.shared.b64 [at0], key;\n"
-                    "sub.u32 pos, pos, 1024; setp.ne.and.u32 dp, pos, 1, pf; vote.sync.any.pred pf, dp, 0xffffffff; @pf bra.uni DEEPER;\n"
-                    "PLACED:\n"
-                    "mov.b32 %0, i; mov.b32 %1, bm; mov.b32 %2, lpos; mov.b32 %3, lfull; mov.b32 %4, tpos; mov.b32 %5, at1;\n"
-                    "mov.b32 %6, at2; mov.b64 %7, tk; mov.b32 %8, prev; mov.b64 %9, rec; mov.b32 %10, lat; mov.b32 %11, xs;\n"
-                    "mov.b32 %12, epos; mov.b32 %13, efull; mov.b32 %14, e_on; mov.b64 %15, e_key; mov.b32 %16, e_idx; mov.b32 %17, qv;\n"
-                    "mov.b32 %18, tail_a; mov.b32 %19, rw; mov.b32 %20, sa; mov.b32 %21, tail_b;\n"
-                    "}"
-                    : "+r"(i), "+r"(bm), "+r"(lpos), "+r"(lfull), "+r"(tpos), "+r"(at1), "+r"(at2), "+l"(tk), "+r"(prev), "+l"(rec), "+r"(lat), "+r"(xs), "+r"(epos), "+r"(efull), "+r"(e_on), "+l"(e_key), "+r"(e_idx), "+r"(qv), "+r"(tail_a), "+r"(rw), "+r"(sa), "+r"(tail_b)
-                    : "r"(xin), "r"(xin_mask), "r"(xin_row), "r"(tab), "r"(kfb), "r"(kfm), "r"(kb), "r"(rm), "r"(mbm1), "r"(tick), "r"(qmask), "r"(~qmask), "r"(qb), "r"(nq - 1u), "r"(xa), "r"(xam), "r"(down), "r"(mask_a), "r"(mask_b), "r"(want_a), "r"(want_b), "l"(out), "l"(out_b)
-                    : "memory");
+                // (a record goes down every way whose condition holds)
+                asm volatile(IL_STEP(IL_LOAD(b32, tail_b, 21),
+                                     IL_STEP_INPUTS(22, 23, 24, 25, 26, 27, 28, 29, 30, 31, 32, 33, 34, 35, 36, 37, 38) IL_LOAD(b32, mask_a, 39) IL_LOAD(b32, mask_b, 40)
+                                     IL_LOAD(b32, want_a, 41) IL_LOAD(b32, want_b, 42) IL_LOAD(b64, out, 43) IL_LOAD(b64, out_b, 44),
+                                     ".reg .pred ga, gb; .reg .b64 o; .reg .u32 ma, mb;\n",
+                                     "and.b32 ma, qv, mask_a; and.b32 mb, qv, mask_b;\n"
+                                     "setp.eq.and.u32 ga, ma, want_a, ho; setp.eq.and.u32 gb, mb, want_b, ho;\n"
+                                     "@hd add.u32 tail_a, tail_a, 256; @ga add.u32 tail_a, tail_a, 8;\n",
+                                     "mad.wide.u32 o, ta_was, 1, out; @ga st.global.b64 [o], v; mad.wide.u32 o, tail_b, 1, out_b; @gb st.global.b64 [o], v; @gb add.u32 tail_b, tail_b, 8;\n",
+                                     IL_DEEPER_WARP, IL_STORE(b32, tail_b, 21))
+                             : IL_STATE_OPERANDS, "+r"(tail_b)
+                             : IL_INPUT_OPERANDS, "r"(mask_a), "r"(mask_b), "r"(want_a), "r"(want_b), "l"(out), "l"(out_b)
+                             : "memory");
             } else if constexpr (OUT == kOutTwo) {
-                asm volatile(
-                    "{\n"
-                    ".reg .b32 i; .reg .b32 bm; .reg .b32 lpos; .reg .b32 lfull; .reg .b32 tpos; .reg .b32 at1; .reg .b32 at2;\n"
-                    ".reg .b64 tk; .reg .b32 prev; .reg .b64 rec; .reg .b32 lat; .reg .b32 xs; .reg .b32 epos; .reg .b32 efull;\n"
-                    ".reg .b32 e_on; .reg .b64 e_key; .reg .b32 e_idx; .reg .b32 qv; .reg .b32 tail_a; .reg .b32 rw; .reg .b32 sa;\n"
-                    ".reg .b32 tail_b; .reg .b32 xin; .reg .b32 xin_mask; .reg .b32 xin_row; .reg .b32 tab; .reg .b32 kfb; .reg .b32 kfm;\n"
-                    ".reg .b32 kb; .reg .b32 rm; .reg .b32 mbm1; .reg .b32 tick; .reg .b32 qmask; .reg .b32 tmask; .reg .b32 qb;\n"
-                    ".reg .b32 nqm; .reg .b32 xa; .reg .b32 xam; .reg .b32 down; .reg .b32 mask_a; .reg .b32 want_a; .reg .b64 out;\n"
-                    "mov.b32 i, %0; mov.b32 bm, %1; mov.b32 lpos, %2; mov.b32 lfull, %3; mov.b32 tpos, %4; mov.b32 at1, %5;\n"
-                    "mov.b32 at2, %6; mov.b64 tk, %7; mov.b32 prev, %8; mov.b64 rec, %9; mov.b32 lat, %10; mov.b32 xs, %11;\n"
-                    "mov.b32 epos, %12; mov.b32 efull, %13; mov.b32 e_on, %14; mov.b64 e_key, %15; mov.b32 e_idx, %16; mov.b32 qv, %17;\n"
-                    "mov.b32 tail_a, %18; mov.b32 rw, %19; mov.b32 sa, %20; mov.b32 tail_b, %21; mov.b32 xin, %22; mov.b32 xin_mask, %23;\n"
-                    "mov.b32 xin_row, %24; mov.b32 tab, %25; mov.b32 kfb, %26; mov.b32 kfm, %27; mov.b32 kb, %28; mov.b32 rm, %29;\n"
-                    "mov.b32 mbm1, %30; mov.b32 tick, %31; mov.b32 qmask, %32; mov.b32 tmask, %33; mov.b32 qb, %34; mov.b32 nqm, %35;\n"
-                    "mov.b32 xa, %36; mov.b32 xam, %37; mov.b32 down, %38; mov.b32 mask_a, %39; mov.b32 want_a, %40; mov.b64 out, %41;\n"
-                    ".reg .pred t, taken, open, pop, ov, dp, pz, pf, hand, hd, ho, fin, fetch;\n"
-                    ".reg .u32 at0, sd, rl, rh, kl, kh, fl, fh, word, wa, x, y, lo, hi, a, xs_was, sa_was, ta_was, pos, left, a1, a2, a3, a4;\n"
-                    ".reg .b64 kf, k1, k2, fk, key, td, r, first, v, e1, e2, e3, e4; .reg .pred ga, gb; .reg .b64 o; .reg .u32 ma, tt;\n"
-                    "and.b32 a, epos, rm; or.b32 a, a, kb; ld.shared.b64 fk, [a];\n"
-                    "and.b32 a, lpos, kfm; or.b32 a, a, kfb; ld.shared.b64 kf, [a];\n"
-                    "ld.shared.b64 k1, [at1]; ld.shared.b64 k2, [at2];\n"
-                    "mov.b64 td, tk; mov.b64 {rl, rh}, rec; mov.u32 xs_was, xs; mov.u32 sa_was, sa;\n"
-                    "setp.ne.u32 t, tpos, efull; selp.b32 rh, rh, -1, t; mov.b64 r, {rl, rh};\n"
-                    "setp.ge.s32 taken, rh, 0; setp.ge.and.u32 t, bm, mbm1, taken; setp.gt.or.f64 open, r, td, t;\n"
-                    "sub.u32 y, i, bm; add.u32 y, y, -1;\n"
-                    "add.u32 wa, i, -1; and.b32 wa, wa, nqm; mad.lo.u32 wa, wa, 128, qb;\n"
-                    "@taken add.u32 i, i, 1; and.b32 xs, i, xin_mask; mad.lo.u32 xs, xs, xin_row, xin; ld.relaxed.cta.shared.b64 rec, [xs];\n"
-                    "setp.lt.s32 hand, rw, 0; setp.ne.and.u32 hand, e_on, 0, hand; setp.ge.and.s32 hd|ho, down, 0, hand; setp.lt.and.s32 fin, qv, 0, hand;\n"
-                    "and.b32 x, qv, 0x7fffffff; mov.b64 {lo, hi}, e_key; and.b32 lo, lo, tmask; or.b32 a, lo, x; mov.b64 v, {a, hi}; mov.u32 ta_was, tail_a;\n"
-                    "and.b32 ma, qv, mask_a; setp.eq.and.u32 ga|gb, ma, want_a, ho; selp.b32 tt, tail_a, tail_b, ga;\n"
-                    "@hd add.u32 tail_a, tail_a, 256; @ga add.u32 tail_a, tail_a, 8; @gb add.u32 tail_b, tail_b, 8;\n"
-                    "and.b32 sa, tail_a, xam; or.b32 sa, sa, xa; ld.relaxed.cta.shared.u32 rw, [sa+4];\n"
-                    "mad.wide.u32 key, lat, tick, tk; mov.b64 {kl, kh}, key; and.b32 kl, kl, tmask; or.b32 kl, kl, y; mov.b64 key, {kl, kh};\n"
-                    "@taken add.u32 bm, bm, 1; @open mov.u32 bm, 0; mad.lo.u32 a, bm, 4, tab; ld.shared.u32 lat, [a];\n"
-                    "setp.eq.or.u32 fetch, e_on, 0, fin; setp.ne.and.u32 fetch, epos, tpos, fetch; setp.le.and.f64 fetch, fk, td, fetch;\n"
-                    "mov.b64 {fl, fh}, fk;\n"
-                    "@hand add.u32 e_idx, e_idx, 1; @fetch and.b32 e_idx, fl, qmask; and.b32 a, e_idx, nqm; mad.lo.u32 a, a, 128, qb; ld.shared.u32 qv, [a];\n"
-                    "@hd st.relaxed.cta.shared.b64 [sa_was], v;\n"
-                    "mad.wide.u32 o, tt, 1, out; @ho st.global.b64 [o], v;\n"
-                    "@fetch mov.b64 e_key, fk; @fin mov.u32 e_on, 0; @fetch mov.u32 e_on, 1; @fetch add.u32 epos, epos, 256; @fetch add.u32 efull, efull, 256;\n"
-                    "and.b32 at0, tpos, rm; or.b32 at0, at0, kb;\n"
-                    "setp.lt.f64 pf, kf, key; selp.b64 first, kf, key, pf;\n"
-                    "setp.eq.u32 pz, tpos, lfull; setp.lt.and.f64 pz, r, first, pz; selp.b64 first, first, r, pz;\n"
-                    "mov.b64 {fl, fh}, first; or.b32 fl, fl, qmask; mov.b64 first, {fl, fh}; selp.b64 tk, first, tk, open;\n"
-                    "setp.lt.and.f64 ov, key, k1, open; selp.u32 sd, at1, at0, ov;\n"
-                    "@open st.shared.b64 [sd], key; @ov st.shared.b64 [at0], k1;\n"
-                    "setp.lt.and.f64 dp, key, k2, ov; mov.u32 pos, tpos; mov.u32 left, lpos;\n"
-                    "setp.eq.and.u32 pop, tpos, lfull, open;\n"
-                    "mov.u32 word, prev; @open or.b32 word, word, 0x80000000; @taken st.shared.u32 [wa], word;\n"
-                    "@taken st.relaxed.cta.shared.u32 [xs_was+4], -1;\n"
-                    "@open add.u32 tpos, tpos, 256; @open mov.u32 at2, at1; @open mov.u32 at1, at0;\n"
-                    "@pop add.u32 lpos, lpos, 256; @pop add.u32 lfull, lfull, 256;\n"
-                    "@taken and.b32 prev, rl, qmask;\n"
-                    "@!dp bra PLACED;\n"
-                    "mov.u32 sd, left; sub.u32 pos, pos, 256;\n"
-                    "DEEPER:\n"
-                    "sub.u32 left, pos, sd;\n"
-                    "and.b32 at0, pos, rm; or.b32 at0, at0, kb; sub.u32 a1, pos, 256; and.b32 a1, a1, rm; or.b32 a1, a1, kb;\n"
-                    "sub.u32 a2, pos, 512; and.b32 a2, a2, rm; or.b32 a2, a2, kb; sub.u32 a3, pos, 768; and.b32 a3, a3, rm; or.b32 a3, a3, kb;\n"
-                    "sub.u32 a4, pos, 1024; and.b32 a4, a4, rm; or.b32 a4, a4, kb;\n"
-                    "ld.shared.b64 e1, [a1]; ld.shared.b64 e2, [a2]; ld.shared.b64 e3, [a3]; ld.shared.b64 e4, [a4];\n"
-                    "setp.gt.u32 t, left, 0; setp.lt.and.f64 t, key, e1, t; setp.gt.and.u32 ov, left, 256, t; setp.lt.and.f64 ov, key, e2, ov;\n"
-                    "setp.gt.and.u32 pz, left, 512, ov; setp.lt.and.f64 pz, key, e3, pz; setp.gt.and.u32 pf, left, 768, pz; setp.lt.and.f64 pf, key, e4, pf;\n"
-                    "@t st.shared.b64 [at0], e1; @ov st.shared.b64 [a1], e2; @pz st.shared.b64 [a2], e3; @pf st.shared.b64 [a3], e4;\n"
-                    "@t mov.u32 at0, a1; @ov mov.u32 at0, a2; @pz mov.u32 at0, a3; @pf mov.u32 at0, a4; st.shared.b64 [at0], key;\n"
-                    "sub.u32 pos, pos, 1024; @pf bra DEEPER;\n"
-                    "PLACED:\n"
-                    "mov.b32 %0, i; mov.b32 %1, bm; mov.b32 %2, lpos; mov.b32 %3, lfull; mov.b32 %4, tpos; mov.b32 %5, at1;\n"
-                    "mov.b32 %6, at2; mov.b64 %7, tk; mov.b32 %8, prev; mov.b64 %9, rec; mov.b32 %10, lat; mov.b32 %11, xs;\n"
-                    "mov.b32 %12, epos; mov.b32 %13, efull; mov.b32 %14, e_on; mov.b64 %15, e_key; mov.b32 %16, e_idx; mov.b32 %17, qv;\n"
-                    "mov.b32 %18, tail_a; mov.b32 %19, rw; mov.b32 %20, sa; mov.b32 %21, tail_b;\n"
-                    "}"
-                    : "+r"(i), "+r"(bm), "+r"(lpos), "+r"(lfull), "+r"(tpos), "+r"(at1), "+r"(at2), "+l"(tk), "+r"(prev), "+l"(rec), "+r"(lat), "+r"(xs), "+r"(epos), "+r"(efull), "+r"(e_on), "+l"(e_key), "+r"(e_idx), "+r"(qv), "+r"(tail_a), "+r"(rw), "+r"(sa), "+r"(tail_b)
-                    : "r"(xin), "r"(xin_mask), "r"(xin_row), "r"(tab), "r"(kfb), "r"(kfm), "r"(kb), "r"(rm), "r"(mbm1), "r"(tick), "r"(qmask), "r"(~qmask), "r"(qb), "r"(nq - 1u), "r"(xa), "r"(xam), "r"(down), "r"(mask_a), "r"(want_a), "l"(out)
-                    : "memory");
+                // (either way: one store; way b's tail counts from where way a's stream starts)
+                asm volatile(IL_STEP(IL_LOAD(b32, tail_b, 21),
+                                     IL_STEP_INPUTS(22, 23, 24, 25, 26, 27, 28, 29, 30, 31, 32, 33, 34, 35, 36, 37, 38) IL_LOAD(b32, mask_a, 39) IL_LOAD(b32, want_a, 40)
+                                     IL_LOAD(b64, out, 41),
+                                     ".reg .pred ga, gb; .reg .b64 o; .reg .u32 ma, tt;\n",
+                                     "and.b32 ma, qv, mask_a; setp.eq.and.u32 ga|gb, ma, want_a, ho; selp.b32 tt, tail_a, tail_b, ga;\n"
+                                     "@hd add.u32 tail_a, tail_a, 256; @ga add.u32 tail_a, tail_a, 8; @gb add.u32 tail_b, tail_b, 8;\n",
+                                     "mad.wide.u32 o, tt, 1, out; @ho st.global.b64 [o], v;\n",
+                                     IL_DEEPER_LANE, IL_STORE(b32, tail_b, 21))
+                             : IL_STATE_OPERANDS, "+r"(tail_b)
+                             : IL_INPUT_OPERANDS, "r"(mask_a), "r"(want_a), "l"(out)
+                             : "memory");
             } else {
-                asm volatile(
-                    "{\n"
-                    ".reg .b32 i; .reg .b32 bm; .reg .b32 lpos; .reg .b32 lfull; .reg .b32 tpos; .reg .b32 at1; .reg .b32 at2;\n"
-                    ".reg .b64 tk; .reg .b32 prev; .reg .b64 rec; .reg .b32 lat; .reg .b32 xs; .reg .b32 epos; .reg .b32 efull;\n"
-                    ".reg .b32 e_on; .reg .b64 e_key; .reg .b32 e_idx; .reg .b32 qv; .reg .b32 tail_a; .reg .b32 rw; .reg .b32 sa;\n"
-                    ".reg .b32 tail_b; .reg .b32 leaves; .reg .b32 xin; .reg .b32 xin_mask; .reg .b32 xin_row; .reg .b32 tab;\n"
-                    ".reg .b32 kfb; .reg .b32 kfm; .reg .b32 kb; .reg .b32 rm; .reg .b32 mbm1; .reg .b32 tick; .reg .b32 qmask;\n"
-                    ".reg .b32 tmask; .reg .b32 qb; .reg .b32 nqm; .reg .b32 xa; .reg .b32 xam; .reg .b32 down; .reg .b32 bits;\n"
-                    ".reg .b32 mask_a; .reg .b32 mask_b; .reg .b32 want_a; .reg .b32 want_b; .reg .b64 out; .reg .b64 out_b;\n"
-                    "mov.b32 i, %0; mov.b32 bm, %1; mov.b32 lpos, %2; mov.b32 lfull, %3; mov.b32 tpos, %4; mov.b32 at1, %5;\n"
-                    "mov.b32 at2, %6; mov.b64 tk, %7; mov.b32 prev, %8; mov.b64 rec, %9; mov.b32 lat, %10; mov.b32 xs, %11;\n"
-                    "mov.b32 epos, %12; mov.b32 efull, %13; mov.b32 e_on, %14; mov.b64 e_key, %15; mov.b32 e_idx, %16; mov.b32 qv, %17;\n"
-                    "mov.b32 tail_a, %18; mov.b32 rw, %19; mov.b32 sa, %20; mov.b32 tail_b, %21; mov.b32 xin, %23; mov.b32 xin_mask, %24;\n"
-                    "mov.b32 xin_row, %25; mov.b32 tab, %26; mov.b32 kfb, %27; mov.b32 kfm, %28; mov.b32 kb, %29; mov.b32 rm, %30;\n"
-                    "mov.b32 mbm1, %31; mov.b32 tick, %32; mov.b32 qmask, %33; mov.b32 tmask, %34; mov.b32 qb, %35; mov.b32 nqm, %36;\n"
-                    "mov.b32 xa, %37; mov.b32 xam, %38; mov.b32 down, %39; mov.b32 bits, %40; mov.b32 mask_a, %41; mov.b32 mask_b, %42;\n"
-                    "mov.b32 want_a, %43; mov.b32 want_b, %44; mov.b64 out, %45; mov.b64 out_b, %46;\n"
-                    ".reg .pred t, taken, open, pop, ov, dp, pz, pf, hand, hd, ho, fin, fetch;\n"
-                    ".reg .u32 at0, sd, rl, rh, kl, kh, fl, fh, word, wa, x, y, lo, hi, a, xs_was, sa_was, ta_was, pos, left, a1, a2, a3, a4;\n"
-                    ".reg .b64 kf, k1, k2, fk, key, td, r, first, v, e1, e2, e3, e4; .reg .pred ga, gb, lv; .reg .b64 o; .reg .u32 ma, mb;\n"
-                    "and.b32 a, epos, rm; or.b32 a, a, kb; ld.shared.b64 fk, [a];\n"
-                    "and.b32 a, lpos, kfm; or.b32 a, a, kfb; ld.shared.b64 kf, [a];\n"
-                    "ld.shared.b64 k1, [at1]; ld.shared.b64 k2, [at2];\n"
-                    "mov.b64 td, tk; mov.b64 {rl, rh}, rec; mov.u32 xs_was, xs; mov.u32 sa_was, sa;\n"
-                    "setp.ne.u32 t, tpos, efull; selp.b32 rh, rh, -1, t; mov.b64 r, {rl, rh};\n"
-                    "setp.ge.s32 taken, rh, 0; setp.ge.and.u32 t, bm, mbm1, taken; setp.gt.or.f64 open, r, td, t;\n"
-                    "sub.u32 y, i, bm; add.u32 y, y, -1;\n"
-                    "add.u32 wa, i, -1; and.b32 wa, wa, nqm; mad.lo.u32 wa, wa, 128, qb;\n"
-                    "@taken add.u32 i, i, 1; and.b32 xs, i, xin_mask; mad.lo.u32 xs, xs, xin_row, xin; ld.relaxed.cta.shared.b64 rec, [xs];\n"
-                    "setp.lt.s32 hand, rw, 0; setp.ne.and.u32 hand, e_on, 0, hand; setp.ge.and.s32 hd|ho, down, 0, hand; setp.lt.and.s32 fin, qv, 0, hand;\n"
-                    "and.b32 x, qv, 0x7fffffff; mov.b64 {lo, hi}, e_key; and.b32 lo, lo, tmask; or.b32 a, lo, x; mov.b64 v, {a, hi}; mov.u32 ta_was, tail_a;\n"
-                    "and.b32 ma, bits, mask_a; and.b32 mb, bits, mask_b; mov.u32 ta_was, tail_a;\n"
-                    "setp.eq.and.u32 ga|lv, ma, want_a, ho; setp.eq.and.u32 gb, mb, want_b, ho; setp.ne.and.u32 lv, mb, want_b, lv;\n"
-                    "@hd add.u32 tail_a, tail_a, 256; @ga add.u32 tail_a, tail_a, 8;\n"
-                    "and.b32 sa, tail_a, xam; or.b32 sa, sa, xa; ld.relaxed.cta.shared.u32 rw, [sa+4];\n"
-                    "mad.wide.u32 key, lat, tick, tk; mov.b64 {kl, kh}, key; and.b32 kl, kl, tmask; or.b32 kl, kl, y; mov.b64 key, {kl, kh};\n"
-                    "@taken add.u32 bm, bm, 1; @open mov.u32 bm, 0; mad.lo.u32 a, bm, 4, tab; ld.shared.u32 lat, [a];\n"
-                    "setp.eq.or.u32 fetch, e_on, 0, fin; setp.ne.and.u32 fetch, epos, tpos, fetch; setp.le.and.f64 fetch, fk, td, fetch;\n"
-                    "mov.b64 {fl, fh}, fk;\n"
-                    "@hand add.u32 e_idx, e_idx, 1; @fetch and.b32 e_idx, fl, qmask; and.b32 a, e_idx, nqm; mad.lo.u32 a, a, 128, qb; ld.shared.u32 qv, [a];\n"
-                    "@hd st.relaxed.cta.shared.b64 [sa_was], v;\n"
-                    "mad.wide.u32 o, ta_was, 1, out; @ga st.global.b64 [o], v; mad.wide.u32 o, tail_b, 1, out_b; @gb st.global.b64 [o], v;\n"
-                    "@gb add.u32 tail_b, tail_b, 8; selp.u32 leaves, 1, 0, lv;\n"
-                    "@fetch mov.b64 e_key, fk; @fin mov.u32 e_on, 0; @fetch mov.u32 e_on, 1; @fetch add.u32 epos, epos, 256; @fetch add.u32 efull, efull, 256;\n"
-                    "and.b32 at0, tpos, rm; or.b32 at0, at0, kb;\n"
-                    "setp.lt.f64 pf, kf, key; selp.b64 first, kf, key, pf;\n"
-                    "setp.eq.u32 pz, tpos, lfull; setp.lt.and.f64 pz, r, first, pz; selp.b64 first, first, r, pz;\n"
-                    "mov.b64 {fl, fh}, first; or.b32 fl, fl, qmask; mov.b64 first, {fl, fh}; selp.b64 tk, first, tk, open;\n"
-                    "setp.lt.and.f64 ov, key, k1, open; selp.u32 sd, at1, at0, ov;\n"
-                    "@open st.shared.b64 [sd], key; @ov st.shared.b64 [at0], k1;\n"
-                    "setp.lt.and.f64 dp, key, k2, ov; mov.u32 pos, tpos; mov.u32 left, lpos;\n"
-                    "setp.eq.and.u32 pop, tpos, lfull, open;\n"
-                    "mov.u32 word, prev; @open or.b32 word, word, 0x80000000; @taken st.shared.u32 [wa], word;\n"
-                    "@taken st.relaxed.cta.shared.u32 [xs_was+4], -1;\n"
-                    "@open add.u32 tpos, tpos, 256; @open mov.u32 at2, at1; @open mov.u32 at1, at0;\n"
-                    "@pop add.u32 lpos, lpos, 256; @pop add.u32 lfull, lfull, 256;\n"
-                    "@taken and.b32 prev, rl, qmask;\n"
-                    "@!dp bra PLACED;\n"
-                    "mov.u32 sd, left; sub.u32 pos, pos, 256;\n"
-                    "DEEPER:\n"
-                    "sub.u32 left, pos, sd;\n"
-                    "and.b32 at0, pos, rm; or.b32 at0, at0, kb; sub.u32 a1, pos, 256; and.b32 a1, a1, rm; or.b32 a1, a1, kb;\n"
-                    "sub.u32 a2, pos, 512; and.b32 a2, a2, rm; or.b32 a2, a2, kb; sub.u32 a3, pos, 768; and.b32 a3, a3, rm; or.b32 a3, a3, kb;\n"
-                    "sub.u32 a4, pos, 1024; and.b32 a4, a4, rm; or.b32 a4, a4, kb;\n"
-                    "ld.shared.b64 e1, [a1]; ld.shared.b64 e2, [a2]; ld.shared.b64 e3, [a3]; ld.shared.b64 e4, [a4];\n"
-                    "setp.gt.u32 t, left, 0; setp.lt.and.f64 t, key, e1, t; setp.gt.and.u32 ov, left, 256, t; setp.lt.and.f64 ov, key, e2, ov;\n"
-                    "setp.gt.and.u32 pz, left, 512, ov; setp.lt.and.f64 pz, key, e3, pz; setp.gt.and.u32 pf, left, 768, pz; setp.lt.and.f64 pf, key, e4, pf;\n"
-                    "@t st.shared.b64 [at0], e1; @ov st.shared.b64 [a1], e2; @pz st.shared.b64 [a2], e3; @pf st.shared.b64 [a3], e4;\n"
-                    "@t mov.u32 at0, a1; @ov mov.u32 at0, a2; @pz mov.u32 at0, a3; @pf mov.u32 at0, a4; st.shared.b64 [at0], key;\n"
-                    "sub.u32 pos, pos, 1024; @pf bra DEEPER;\n"
-                    "PLACED:\n"
-                    "mov.b32 %0, i; mov.b32 %1, bm; mov.b32 %2, lpos; mov.b32 %3, lfull; mov.b32 %4, tpos; mov.b32 %5, at1;\n"
-                    "mov.b32 %6, at2; mov.b64 %7, tk; mov.b32 %8, prev; mov.b64 %9, rec; mov.b32 %10, lat; mov.b32 %11, xs;\n"
-                    "mov.b32 %12, epos; mov.b32 %13, efull; mov.b32 %14, e_on; mov.b64 %15, e_key; mov.b32 %16, e_idx; mov.b32 %17, qv;\n"
-                    "mov.b32 %18, tail_a; mov.b32 %19, rw; mov.b32 %20, sa; mov.b32 %21, tail_b; mov.b32 %22, leaves;\n"
-                    "}"
-                    : "+r"(i), "+r"(bm), "+r"(lpos), "+r"(lfull), "+r"(tpos), "+r"(at1), "+r"(at2), "+l"(tk), "+r"(prev), "+l"(rec), "+r"(lat), "+r"(xs), "+r"(epos), "+r"(efull), "+r"(e_on), "+l"(e_key), "+r"(e_idx), "+r"(qv), "+r"(tail_a), "+r"(rw), "+r"(sa), "+r"(tail_b), "=r"(leaves)
-                    : "r"(xin), "r"(xin_mask), "r"(xin_row), "r"(tab), "r"(kfb), "r"(kfm), "r"(kb), "r"(rm), "r"(mbm1), "r"(tick), "r"(qmask), "r"(~qmask), "r"(qb), "r"(nq - 1u), "r"(xa), "r"(xam), "r"(down), "r"(bits), "r"(mask_a), "r"(mask_b), "r"(want_a), "r"(want_b), "l"(out), "l"(out_b)
-                    : "memory");
+                asm volatile(IL_STEP(IL_LOAD(b32, tail_b, 21) ".reg .b32 leaves;\n",
+                                     IL_STEP_INPUTS(23, 24, 25, 26, 27, 28, 29, 30, 31, 32, 33, 34, 35, 36, 37, 38, 39) IL_LOAD(b32, bits, 40) IL_LOAD(b32, mask_a, 41)
+                                     IL_LOAD(b32, mask_b, 42) IL_LOAD(b32, want_a, 43) IL_LOAD(b32, want_b, 44) IL_LOAD(b64, out, 45) IL_LOAD(b64, out_b, 46),
+                                     ".reg .pred ga, gb, lv; .reg .b64 o; .reg .u32 ma, mb;\n",
+                                     "and.b32 ma, bits, mask_a; and.b32 mb, bits, mask_b;\n"
+                                     "setp.eq.and.u32 ga|lv, ma, want_a, ho; setp.eq.and.u32 gb, mb, want_b, ho; setp.ne.and.u32 lv, mb, want_b, lv;\n"
+                                     "@hd add.u32 tail_a, tail_a, 256; @ga add.u32 tail_a, tail_a, 8;\n",
+                                     "mad.wide.u32 o, ta_was, 1, out; @ga st.global.b64 [o], v; mad.wide.u32 o, tail_b, 1, out_b; @gb st.global.b64 [o], v;\n"
+                                     "@gb add.u32 tail_b, tail_b, 8; selp.u32 leaves, 1, 0, lv;\n",
+                                     IL_DEEPER_LANE, IL_STORE(b32, tail_b, 21) IL_STORE(b32, leaves, 22))
+                             : IL_STATE_OPERANDS, "+r"(tail_b), "=r"(leaves)
+                             : IL_INPUT_OPERANDS, "r"(bits), "r"(mask_a), "r"(mask_b), "r"(want_a), "r"(want_b), "l"(out), "l"(out_b)
+                             : "memory");
                 if (FEAS) test_late();
                 if (pt->n_leave > 0 && leaves != 0u) {
                     // (a branch point at which some queries leave)
