@@ -346,6 +346,8 @@ des_kernel(const __grid_constant__ DesParams p)
 
 cudaError_t launch_des(const DesParams &p, int grid, size_t smem, cudaStream_t stream)
 {
+    cudaError_t e = allow_smem(des_kernel, kLargestTables);
+    if (e != cudaSuccess) return e;
     des_kernel<<<grid, kWarpsPerCta * 32, smem, stream>>>(p);
     return cudaGetLastError();
 }
@@ -353,7 +355,7 @@ cudaError_t launch_des(const DesParams &p, int grid, size_t smem, cudaStream_t s
 int des_max_ctas_per_sm(size_t smem)
 {
     int n = 0;
-    if (allow_all_smem(des_kernel) != cudaSuccess) return 0;
+    if (allow_smem(des_kernel, kLargestTables) != cudaSuccess) return 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, des_kernel, kWarpsPerCta * 32, smem) != cudaSuccess)
         return 0;
     return n;

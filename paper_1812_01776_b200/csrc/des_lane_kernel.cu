@@ -1264,8 +1264,10 @@ __global__ void __launch_bounds__(kNodeThreads) root_nodes_kernel(const RootNode
 }
 
 template <typename K, typename... A>
-cudaError_t launch_one(K kernel, int grid, size_t smem, cudaStream_t stream, const A &...args)
+cudaError_t launch_one(K kernel, int grid, size_t smem, size_t smem_most, cudaStream_t stream, const A &...args)
 {
+    cudaError_t e = allow_smem(kernel, smem_most);      // (these kernels have no static shared memory)
+    if (e != cudaSuccess) return e;
     kernel<<<grid, kLaneWarps * 32, smem, stream>>>(args...);
     return cudaGetLastError();
 }
@@ -1286,16 +1288,16 @@ cudaError_t launch_root_nodes(const RootNodeParams &p, cudaStream_t stream)
 
 // Feasibility-only when p.out_feasible is set; cut: the pipeline's parts, nullptr for a chain.  (The host never combines
 // fan-out with feasibility-only, nor with spill rings shorter than the longest stream.)
-cudaError_t launch_des_lane(const DesParams &p, const LaneCut *cut, int grid, size_t smem, cudaStream_t stream)
+cudaError_t launch_des_lane(const DesParams &p, const LaneCut *cut, int grid, size_t smem, size_t smem_most, cudaStream_t stream)
 {
     if (!cut)
-        return p.out_feasible ? launch_one(des_lane_kernel<true>, grid, smem, stream, p) : launch_one(des_lane_kernel<false>, grid, smem, stream, p);
+        return p.out_feasible ? launch_one(des_lane_kernel<true>, grid, smem, smem_most, stream, p) : launch_one(des_lane_kernel<false>, grid, smem, smem_most, stream, p);
     if (p.fork) {
         if (p.lane_wrap || p.out_feasible) return cudaErrorInvalidValue;
-        return launch_one(des_part_kernel<false, true>, grid, smem, stream, p, *cut);
+        return launch_one(des_part_kernel<false, true>, grid, smem, smem_most, stream, p, *cut);
     }
-    return p.out_feasible ? launch_one(des_part_kernel<true, false>, grid, smem, stream, p, *cut)
-                          : launch_one(des_part_kernel<false, false>, grid, smem, stream, p, *cut);
+    return p.out_feasible ? launch_one(des_part_kernel<true, false>, grid, smem, smem_most, stream, p, *cut)
+                          : launch_one(des_part_kernel<false, false>, grid, smem, smem_most, stream, p, *cut);
 }
 
 int des_lane_warps_per_cta() { return kLaneWarps; }
@@ -1308,22 +1310,15 @@ size_t des_lane_smem(int table_rows, int Bmax, int ring_slots, int ring_words, i
            kSmemBase + ring_bytes(ring_slots, ring_words, stretch) + kTailBytes;
 }
 
-int des_lane_max_ctas_per_sm(size_t smem, bool cut, bool fork)
+int des_lane_max_ctas_per_sm(size_t smem, size_t smem_most, bool cut)
 {
-    // (all instantiations of one kind are compiled for the same number of CTAs; the last one of those that a handle can launch answers)
     int n = 0;
-    auto ask = [&](auto... kernels) {
-        cudaError_t e = cudaSuccess;
-        auto one = [&](auto kernel) {
-            if (e == cudaSuccess) e = allow_all_smem(kernel);
-            if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kLaneWarps * 32, smem);
-        };
-        (one(kernels), ...);
-        if (e != cudaSuccess) { cudaGetLastError(); n = 0; }
-        return n;
+    // (all instantiations of one kind are compiled for the same number of CTAs)
+    auto ask = [&](auto kernel) {
+        if (allow_smem(kernel, smem_most) != cudaSuccess) { cudaGetLastError(); return 0; }
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kLaneWarps * 32, smem) == cudaSuccess ? n : 0;
     };
-    if (!cut) return ask(des_lane_kernel<false>, des_lane_kernel<true>);
-    return fork ? ask(des_part_kernel<false, true>) : ask(des_part_kernel<false, false>, des_part_kernel<true, false>);
+    return cut ? ask(des_part_kernel<true, false>) : ask(des_lane_kernel<true>);
 }
 
 }  // namespace il

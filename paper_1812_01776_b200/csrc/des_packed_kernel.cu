@@ -1050,8 +1050,19 @@ cudaError_t launch_node_stage(const NodeStageParams &p, int grid, cudaStream_t s
     return cudaGetLastError();
 }
 
+namespace {
+// Static plus dynamic shared memory passes 48 KB for the largest table shapes the interface takes
+// (16 stages x 8 hardware types x 64 batch sizes = 32 KB of tables): opt in before every use.
+cudaError_t packed_opt_in(bool staged)
+{
+    return staged ? allow_smem(des_packed_kernel<true>, kLargestTables) : allow_smem(des_packed_kernel<false>, kLargestTables);
+}
+}  // namespace
+
 cudaError_t launch_des_packed(const DesParams &p, bool staged, int grid, size_t smem, cudaStream_t stream)
 {
+    cudaError_t e = packed_opt_in(staged);
+    if (e != cudaSuccess) return e;
     if (staged) des_packed_kernel<true><<<grid, kWarpsPerCta * 32, smem, stream>>>(p);
     else des_packed_kernel<false><<<grid, kWarpsPerCta * 32, smem, stream>>>(p);
     return cudaGetLastError();
@@ -1060,9 +1071,7 @@ cudaError_t launch_des_packed(const DesParams &p, bool staged, int grid, size_t 
 int des_packed_max_ctas_per_sm(bool staged, size_t smem)
 {
     int n = 0;
-    // static plus dynamic shared memory passes 48 KB for the largest table shapes the interface takes
-    // (16 stages x 8 hardware types x 64 batch sizes = 32 KB of tables)
-    if ((staged ? allow_all_smem(des_packed_kernel<true>) : allow_all_smem(des_packed_kernel<false>)) != cudaSuccess) return 0;
+    if (packed_opt_in(staged) != cudaSuccess) return 0;
     cudaError_t e = staged
         ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, des_packed_kernel<true>, kWarpsPerCta * 32, smem)
         : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, des_packed_kernel<false>, kWarpsPerCta * 32, smem);

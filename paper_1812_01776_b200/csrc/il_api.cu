@@ -812,7 +812,7 @@ static cudaError_t launch_lane(const il_estimator *e, DesParams p, int64_t ctas,
     p.lane_ahead = per_sm == 1 && e->n >= kLongTurnsFrom && fits(lane_smem(e, e->lane_slots, 2 * kLaneWords, lane_stretch_bytes(p.cpw, 128))) ? 128 : 64;
     p.lane_stretch = lane_stretch_bytes(p.cpw, p.lane_ahead);
     widen(p.lane_words, [&] { return fits(lane_smem(e, e->lane_slots, p.lane_words, p.lane_stretch)); });
-    return launch_des_lane(p, nullptr, (int)ctas, lane_smem(e, e->lane_slots, p.lane_words, p.lane_stretch), st);
+    return launch_des_lane(p, nullptr, (int)ctas, lane_smem(e, e->lane_slots, p.lane_words, p.lane_stretch), e->smem_per_cta, st);
 }
 
 // A chunk of a pipeline cut into parts: control words and counts cleared, root nodes numbered, then the parts.
@@ -872,7 +872,7 @@ static int enqueue_parts(il_estimator *e, DesParams p, const Plan &pl, char *ws,
     const size_t per_sm = (size_t)((grid + e->num_sms - 1) / e->num_sms);
     auto smem = [&] { return lane_smem(e, e->lane_slots, p.lane_words, p.lane_stretch); };
     widen(p.lane_words, [&] { return smem() <= e->smem_per_cta && (smem() + 1024) * per_sm <= e->smem_per_sm; });
-    IL_CUDA(launch_des_lane(p, &cut, (int)grid, smem(), st));
+    IL_CUDA(launch_des_lane(p, &cut, (int)grid, smem(), e->smem_per_cta, st));
     *launches += 2;
     return IL_OK;
 }
@@ -1047,8 +1047,6 @@ static int shared_by_cover(il_estimator *e, const SharedCommon &c, char *ws, siz
 // node count is at most a quarter of candidates x stages (exhaustive sweeps over per-stage choices); chunked: the whole
 // batch would not fit one chunk otherwise;
 // *used tells whether the batch was evaluated here.
-constexpr int kShareMaxTop = 16384;
-
 static int estimate_shared(il_estimator *e, const il_stage_config *d_configs, int64_t n_cand, int64_t slo_us,
                            int64_t *d_out_p99, int64_t *d_out_miss, char *ws, size_t ws_bytes, bool chunked, bool *used)
 {
@@ -1476,13 +1474,12 @@ int il_estimator_create_dag(const il_profiles *pr, const il_join_edges *jn, cons
         if (e->cut.n_part > 0) {
             int most = 1;
             for (int t = e->cut.shared ? 1 : 0; t < e->cut.n_part; t++) most = std::max(most, e->cut.part[t].len > 0 ? 32 / e->cut.part[t].len : 32);
-            e->ctas_lane[k] = std::max(1, des_lane_max_ctas_per_sm(lane_smem(e, slots, kLaneWords, lane_stretch_bytes(std::max(most, kRootGroups), 32)), true, e->fork));
+            e->ctas_lane[k] = std::max(1, des_lane_max_ctas_per_sm(lane_smem(e, slots, kLaneWords, lane_stretch_bytes(std::max(most, kRootGroups), 32)), e->smem_per_cta, true));
         } else {
-            e->ctas_lane[k] = des_lane_max_ctas_per_sm(lane_smem(e, slots, kLaneWords, lane_stretch_bytes(e->cpw, 64)), false, e->fork);
+            e->ctas_lane[k] = des_lane_max_ctas_per_sm(lane_smem(e, slots, kLaneWords, lane_stretch_bytes(e->cpw, 64)), e->smem_per_cta, false);
         }
     }
     e->ctas_per_sm_lane = e->ctas_lane[1];
-    if (cudaError_t ce = prepare_node_top(); ce != cudaSuccess) { g_last_cuda_error = (int)ce; return fail(IL_ERR_CUDA); }
     if (e->ctas_per_sm_wide < 1 || e->ctas_per_sm_packed < 1 || e->ctas_per_sm_staged < 1 ||
         e->ctas_per_sm_lane < 1) {
         g_last_cuda_error = (int)cudaErrorLaunchOutOfResources;

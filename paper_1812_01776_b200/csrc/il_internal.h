@@ -177,20 +177,15 @@ struct SelectParams {
     int64_t *out_miss;
 };
 
-// A kernel's limit of dynamic shared memory belongs to the function and not to a launch: handles on other threads share it.
-// So it is raised to what the device can give, the same for every handle, where a handle is created, and no launch touches it.
+// A kernel's limit of dynamic shared memory belongs to the function and not to a launch: handles on other threads share it.  So
+// it is only ever set to one value per kernel, that of the largest launch there can be, whatever the launch at hand needs.
 template <typename K>
-inline cudaError_t allow_all_smem(K kernel)
+inline cudaError_t allow_smem(K kernel, size_t largest)
 {
-    int dev = 0, most = 0;
-    cudaFuncAttributes a;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, kernel);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)a.sharedSizeBytes);
-    return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)largest);
 }
+constexpr size_t kLargestTables = (size_t)IL_MAX_STAGES * IL_MAX_HW * IL_MAX_BATCH * sizeof(int32_t);
+constexpr int kShareMaxTop = 16384;      // shared prefixes: latencies kept per node at most (a power of two)
 
 // Read-only view of what a handle has bound, for translation units that do not
 // see the handle's definition.
@@ -214,13 +209,13 @@ cudaError_t launch_des_packed(const DesParams &p, bool staged, int grid, size_t 
 int des_packed_max_ctas_per_sm(bool staged, size_t smem);
 int trace_tile_records();     // the packed trace is padded to a multiple of this many records
 // lane-parallel kernel: one lane per (candidate, stage); smem from des_lane_smem
-cudaError_t launch_des_lane(const DesParams &p, const LaneCut *cut, int grid, size_t smem, cudaStream_t stream);
+// smem_most: what the device gives a CTA
+cudaError_t launch_des_lane(const DesParams &p, const LaneCut *cut, int grid, size_t smem, size_t smem_most, cudaStream_t stream);
 int des_lane_warps_per_cta();
 // ring_slots: 16 or 32 batch ring positions per lane; ring_words: words of examined records (a power of two); stretch: bytes
 // of a warp's arrival streams
 size_t des_lane_smem(int table_rows, int Bmax, int ring_slots, int ring_words, int stretch);
-// (the three that ask for resident CTAs also prepare their kernels for launches: allow_all_smem)
-int des_lane_max_ctas_per_sm(size_t smem, bool cut, bool fork);
+int des_lane_max_ctas_per_sm(size_t smem, size_t smem_most, bool cut);
 enum SimKernel { kSimWide = 0, kSimPacked = 1, kSimPackedStaged = 2, kSimLane = 3 };
 inline cudaError_t launch_simulation(const DesParams &p, int kernel, int grid, size_t smem,
                                      cudaStream_t stream)
@@ -276,7 +271,6 @@ struct NodeTopParams {
     int32_t one_pass;             // (set by the launch)
 };
 cudaError_t launch_node_top(const NodeTopParams &p, cudaStream_t stream);
-cudaError_t prepare_node_top();      // once per handle, before the first launch
 size_t node_top_smem(int top_len);
 struct CombineParams {
     int64_t n_cand;

@@ -473,8 +473,6 @@ size_t node_top_smem(int top_len)
     return pow2 * sizeof(int64_t);
 }
 
-cudaError_t prepare_node_top() { return allow_all_smem(node_top_kernel); }
-
 cudaError_t launch_node_top(const NodeTopParams &q, cudaStream_t stream)
 {
     NodeTopParams p = q;
@@ -482,6 +480,8 @@ cudaError_t launch_node_top(const NodeTopParams &q, cudaStream_t stream)
     // in one pass where a row is several times what is kept of it, and both the longer list and the sample's bins fit
     p.one_pass = p.len >= kSelOnePass / 4 && p.len >= 4 * p.top_len && smem <= 32768;
     if (p.one_pass) smem = 2 * smem + kSelBins * sizeof(unsigned);
+    cudaError_t e = allow_smem(node_top_kernel, kShareMaxTop * sizeof(int64_t));     // (more than in one pass: 96 KB)
+    if (e != cudaSuccess) return e;
     const int grid = (int)(p.n_nodes < 148 * 8 ? p.n_nodes : 148 * 8);
     node_top_kernel<<<grid, kSelectThreads, smem, stream>>>(p);
     return cudaGetLastError();
