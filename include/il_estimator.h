@@ -258,8 +258,8 @@ IL_API int il_estimate_device(il_estimator *est, const il_stage_config *d_config
  * objective (an overloaded candidate is decided within the first few per cent of the trace;
  * il_stats.early_exits counts them).  A feasible candidate is simulated to the end, so its answer is
  * exact too.  Needs no memory per query and candidate except on pipelines with branches below branches, and is several
- * times faster than il_estimate for a batch without feasible candidates; a batch of up to one warp per scheduler with
- * some feasible ones takes up to 20 % longer, since the comparison is on the loop's chain.  The warp-per-candidate kernels have no early exit: with them this call computes P99
+ * times faster than il_estimate for a batch without feasible candidates; on a chain, a batch of up to one warp per scheduler
+ * with some feasible ones takes 15 to 25 % longer, since the comparison is on the loop's chain.  The warp-per-candidate kernels have no early exit: with them this call computes P99
  * and compares.
  *   il_feasible         configs HOST [n][S], out_feasible HOST [n] bytes; candidates validated on the host
  *   il_feasible_device  DEVICE pointers; an invalid candidate makes the call return BAD_CONFIG
@@ -352,7 +352,15 @@ IL_API int il_set_stream(il_estimator *est, void *cuda_stream);
 /*
  * Scratch memory.  The simulation keeps, per resident warp, the streams of
  * (time, query) pairs that flow between stages, and per candidate of a chunk
- * its n latencies for the percentile kernel.
+ * its n latencies for the percentile kernel.  The lane kernel keeps spill rings
+ * per warp instead, and on pipelines with branch points streams in memory: per
+ * distinct configuration of the root those that the root writes; per candidate,
+ * with fan-out, joins or where a part that more parts follow reads from
+ * another than the root, 8 bytes for each record of the other streams (fan-out over six stages
+ * 1.5 n records, a diamond 3 n and a bit per query, on top of the n latencies);
+ * and with branches below branches the n latencies in feasibility-only mode too.
+ * A batch for which that does not fit takes several chunks, each of which costs
+ * the time of one warp over the trace.
  *   il_workspace_bytes  size that lets a call of n_candidates run at full
  *                       occupancy (for large n_candidates: the size beyond
  *                       which more memory no longer helps)

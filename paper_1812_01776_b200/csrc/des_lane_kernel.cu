@@ -62,10 +62,10 @@
 //     the iteration bound, the next candidate) is looked at once a turn of 8 to 62
 //     iterations only, behind one vote.
 //
-// Measured on B200, 4,096 candidates x 4 stages x 50,000 queries and 4,096 x 10 x 10^6: streams in global memory 15.4 / 720 ms;
-// streams in shared memory, the loop in C++ 6.94 / 348 ms (123 instructions an iteration, 220 cycles for a warp on its
-// own); the loop in PTX and twice as long turns where a CTA
-// has its SM to itself 6.37 / 302 ms (108 instructions, 184 cycles and the turns).  What costs there is latency between
+// Measured on B200, 4,096 candidates x 4 stages x 50,000 queries and 4,096 x 10 x 10^6, whole calls: streams in global memory
+// 15.4 / 720 ms; streams in shared memory, the loop in C++ 6.97 / 346 ms (123 instructions an iteration, 220 cycles for a warp on
+// its own); the loop in PTX and twice as long turns where a CTA has its SM to itself 6.3 / 300 to 329 ms, within the noise of
+// the other on the second (108 instructions, 184 cycles and the turns).  What costs there is latency between
 // dependent instructions (73 of 230 cycles) and the ALU pipe (compares, selects, logic: half the issue rate).  Learned on
 // the way: a bool that lives through the loop takes one of seven predicates and costs the schedule 15 % (two of them:
 // 6.94 -> 8.14 ms), so what a lane has to remember are bits of one register; the same instructions with the loads of the next
@@ -101,10 +101,6 @@ __device__ __forceinline__ uint32_t lds32(uint32_t a)
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
     return v;
 }
-// Order of two records or keys.  Words below 0x7ff0... order the same as the doubles of their bits, and a double
-// is compared by one instruction on a pipe that is idle otherwise, where a 64-bit integer takes two on the ALU pipe
-// (5 % of a launch with three warps per scheduler).  A word with the sign or all exponent bits set compares as false.
-
 // Words that two lanes share.  Stream records, and the records in a join's windows: each is complete in itself, so no
 // ordering between words is needed.  A join's counts: stored behind the warp barrier that follows the records they cover.
 __device__ __forceinline__ uint64_t lds64_shared(uint32_t a)
@@ -394,6 +390,9 @@ __device__ __noinline__ void lane_merge(const DesParams &p, const LaneCut &cut, 
 // before it along (setp.and), where the compiler joins finished predicates by instructions of their own, and what the next
 // iteration reads (its record, the room for the record in hand, the time of the open batch, the low part to hand on) is requested as soon as
 // it is known where it lies, before this iteration's stores.
+// Records and keys are compared as doubles: words below 0x7ff0... order the same as the doubles of their bits, and a double takes one
+// instruction on a pipe that is idle otherwise, where a 64-bit integer takes two on the ALU pipe (5 % of a launch with
+// three warps per scheduler).  A word with the sign or all exponent bits set compares as false.
 // The seven forms of the iteration (lane_simulation: step) are one text.  A form gives what is its own: more operands, more
 // registers, how the tails of its ways out move, the way out itself, how the deeper insertion is reached, what more it hands back.
 // Operands by number: 0 to 20 the state that all forms have, then what state a form adds, the inputs that all have, a form's.
@@ -455,8 +454,8 @@ __device__ __noinline__ void lane_merge(const DesParams &p, const LaneCut &cut, 
     "@pop add.u32 lpos, lpos, 256; @pop add.u32 lfull, lfull, 256;\n" \
     "@taken and.b32 prev, rl, qmask;\n"
 // A batch that goes further back, past the batches that finish later: four a round.  Each lane by itself, or (WARP) all lanes behind
-// a vote: chains of 4 take 6.7 ms with the one and 7.3 with the other, but feasibility only takes 20.2 with the vote for 21.3
-// and fan-out 17.6 for 17.9.
+// a vote: a chain of 4 takes 6.7 ms without it and 7.3 with it, but a tree of 6 feasibility only 21.3 and 20.2, and fan-out
+// 17.9 and 17.6 (taken while the loop was written; a chain feasibility only has not been timed without the vote).
 #define IL_DEEPER(SKIP, FIRST, WHO, AGAIN) \
     SKIP "\n" \
     "mov.u32 sd, left; sub.u32 pos, pos, 256;\n" \
@@ -507,10 +506,10 @@ __device__ __noinline__ void lane_merge(const DesParams &p, const LaneCut &cut, 
 //         * A part that only leaves the pipeline (the rule) needs no memory for its stream: the records come in the
 //           region of the candidate's slab row that they go to, and no record leaves before it was examined.
 //       Against one group of lanes for the whole tree (each lane as many iterations as the root has records, whatever
-//       its branch sees, and a branch step in the loop): 7,001 candidates of a tree of 6, 199,999 queries 66 -> 34 ms;
-//       8,192, feasibility only, 100,000 queries 35.1 -> 19.5 ms; the covering candidates of a sweep over a tree of 8 17.4 -> 14.6
+//       its branch sees, and a branch step in the loop): 7,001 candidates of a tree of 6, 199,999 queries 66 -> 33 ms;
+//       8,192, feasibility only, 100,000 queries 34.9 -> 19.4 ms; the covering candidates of a sweep over a tree of 8 17.4 -> 14.5
 //       ms; fan-out, 2,048 candidates of 6 stages, 100,000 queries 21.7 -> 15.7 ms.  Up to a warp per scheduler the root is
-//       what takes the time (240 cycles an iteration and 30 for its turns), beyond that the ALU pipe.
+//       what takes the time (250 to 265 cycles an iteration with its turns), beyond that the ALU pipe.
 // FORK: fan-out (with CUT) -- a query goes down every edge whose condition holds, a copy that finds none leaves, and
 //       the slab keeps per query the record of the copy that left last.  Joins: the streams of a stage's two incoming edges
 //       are merged by a part of its own (lane_merge) before the part that begins with the stage.
@@ -553,7 +552,7 @@ __device__ __forceinline__ void lane_simulation(const DesParams &p, const LaneCu
     unsigned *missw = reinterpret_cast<unsigned *>(smem_raw + (nowhere - sbase) + 256u + (uint32_t)wid * 128u);   // per group
     const uint32_t rm = (uint32_t)(kr - 1) << 8;      // ring counters epos, lpos, tpos count in bytes of a row
 
-    // Cut pipelines: a CTA that is the first on its SM may take that SM for root nodes; others that come there leave.
+    // Cut pipelines: a CTA that is the first on its SM may take that SM for root nodes; as many others that come there as are planned leave.
     uint32_t root_warps = 1u;
     bool for_roots = false;
     (void)root_warps; (void)for_roots;

@@ -1832,10 +1832,11 @@ static int feasible_device(il_estimator *e, const il_stage_config *d_configs, in
     }
 
     // Lane kernel: no percentile pass, and a candidate ends as soon as it is decided.  What that gives depends on the batch (50,000
-    // queries, chain of 4 / tree of 6, 2,048 and 6,000 candidates): nothing feasible 0.11 and 0.17 / 0.20 and 0.21 ms;
-    // everything or a part feasible 6.8 and 9.9 / 6.4 and 7.9 ms, where a warp ends with its last feasible candidate and an
-    // iteration takes 140 instead of 113 ns.  It is also the way that needs no memory per candidate (but for streams where
-    // branches lie below branches, which may make several chunks of the batch), so it is the only one.
+    // queries, a chain of 4 with 2,048 and 16,384 candidates / a tree of 6 with 2,048 and 6,000): nothing feasible 0.16 and 0.38 / 0.25
+    // and 0.26 ms; everything or a part feasible 6.8 and 18.9 / 6.4 and 7.3 ms (the estimate 5.9 and 18.5 / 6.8 and 7.8), where a warp
+    // ends with its last feasible candidate and an iteration of a chain takes 131 to 140 instead of 106 to 113 ns.  It is also the
+    // way that needs no memory per candidate (but for streams where branches lie below branches, which may make several chunks
+    // of the batch), so it is the only one.
     int rc = start_call(e, d_configs, n_cand, max_replicas);
     if (rc) return rc;
     char *ws = nullptr;

@@ -81,7 +81,7 @@ struct DesParams {
     int32_t lane_words;           // words of examined records a lane keeps in shared memory (a power of two, at least 64)
     int32_t smem_skip;            // test knob: bytes left unused where shared memory starts (a multiple of 16, at most 8192)
     int32_t lane_wrap;            // the rings are shorter than the longest stream
-    int32_t lane_ahead;           // records of its arrival stream a group has in shared memory (32 or 64)
+    int32_t lane_ahead;           // records of its arrival stream a group has in shared memory (32, 64 or 128)
     int32_t lane_stretch;         // bytes of that for all groups of a warp
     int32_t lanes_per_slot;       // spill rings of a warp slot
     // lane kernel, joins

@@ -39,3 +39,18 @@ def test_parity_slice_on_the_checked_build():
                           "or fan_out_parity or envelope_around or envelope_where"],
                          cwd=ROOT, env=env, capture_output=True, text=True)
     assert run.returncode == 0, run.stdout[-3000:] + run.stderr[-2000:]
+
+
+@pytest.mark.gpu
+def test_parts_and_one_pass_rows_on_the_checked_build():
+    """The streams between the parts of a pipeline, the merges of joins, root nodes on few SMs, and rows of the percentile
+    kernels that are read once."""
+    from paper_1812_01776_b200 import build
+    build.build(checked=True)
+    env = dict(os.environ, IL_ESTIMATOR_CHECKED="1")
+    run = subprocess.run([sys.executable, "-m", "pytest", "tests/test_parts.py", "tests/test_select_one_pass.py", "tests/test_threads.py",
+                          "tests/test_feasible.py", "-m", "gpu", "-x", "-q", "-k",
+                          "trace_lengths or other_forms or small_workspace or few_sms or (merges and not 20000) or one_pass "
+                          "or threads_of_their_own or decided"],
+                         cwd=ROOT, env=env, capture_output=True, text=True)
+    assert run.returncode == 0, run.stdout[-3000:] + run.stderr[-2000:]
