@@ -49,20 +49,20 @@ NCU_CAPTURES = {
     # chains of up to one warp per scheduler (workloads 1, 2): 4,096 candidates x 20,000 queries of workload 2
     "des_lane_kernel": {
         "source": "paper_1812_01776_b200/csrc/des_lane_kernel.cu",
-        "source_sha256": "2f5d3b2d4bd8c86b7e9ef66bb74e0dcdcb77e46a9e087ffd738b95a016c2c05d",
-        "dram_bytes_per_query_event": 1.84, "warp_inst_per_query_event": 3.82,
+        "source_sha256": "934d632f9d627360035cf7397193ea55d440c76066d3697047a446a2739b2669",
+        "dram_bytes_per_query_event": 1.85, "warp_inst_per_query_event": 3.82,
         "summary": "profiles/des_lane_kernel.md"},
     # two to three warps per scheduler (workload 4): 4,096 candidates x 20,000 queries of workload 4
     "des_lane_kernel:long": {
         "source": "paper_1812_01776_b200/csrc/des_lane_kernel.cu",
-        "source_sha256": "2f5d3b2d4bd8c86b7e9ef66bb74e0dcdcb77e46a9e087ffd738b95a016c2c05d",
+        "source_sha256": "934d632f9d627360035cf7397193ea55d440c76066d3697047a446a2739b2669",
         "dram_bytes_per_query_event": 0.74, "warp_inst_per_query_event": 3.66,
         "summary": "profiles/des_lane_kernel.md"},
     # pipelines with branch points (workloads 3, 5; des_part_kernel): 7,001 candidates x 20,000 queries of workload 3
     "des_lane_kernel:tree": {
         "source": "paper_1812_01776_b200/csrc/des_lane_kernel.cu",
-        "source_sha256": "2f5d3b2d4bd8c86b7e9ef66bb74e0dcdcb77e46a9e087ffd738b95a016c2c05d",
-        "dram_bytes_per_query_event": 2.14, "warp_inst_per_query_event": 4.31,
+        "source_sha256": "934d632f9d627360035cf7397193ea55d440c76066d3697047a446a2739b2669",
+        "dram_bytes_per_query_event": 2.14, "warp_inst_per_query_event": 4.29,
         "summary": "profiles/des_lane_kernel.md"},
     "des_packed_kernel": {
         "source": "paper_1812_01776_b200/csrc/des_packed_kernel.cu",
